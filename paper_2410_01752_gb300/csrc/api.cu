@@ -89,7 +89,13 @@ void free_all(sisso_ctx* c) {
         if (c->pooled.count(p)) cudaFreeAsync(p, c->stream);    // back to the library's pool
         else cudaFree(p);
     }
+    for (void* p : c->bufs) {
+        if (c->pooled.count(p)) cudaFreeAsync(p, c->stream);
+        else cudaFree(p);
+    }
     c->pooled.clear();
+    c->bufs.clear();
+    pair_tc_free(c);
     tc_screen_free(c);
     whiten_free(c);
     if (c->walk_h) cudaFreeHost(c->walk_h);
@@ -133,6 +139,34 @@ sisso_status validate(int N, int d, uint32_t ops, int rung, int k, int max_dim, 
 }
 
 }  // namespace
+
+namespace sg {
+bool zcache_fits(sisso_ctx* c, int64_t n) {
+    if (n <= c->zcap) return true;
+    if (n > c->zcap_max) return false;
+    n = std::min(c->zcap_max, std::max(n, c->zcap + c->zcap / 2));
+    double* p = nullptr;
+    const std::string err = c->err;
+    if (dalloc(c, p, (size_t)n * (size_t)c->N, "zcache")) {        // no room: the window evaluates on the fly
+        cudaGetLastError();
+        c->err = err;
+        return false;
+    }
+    if (c->pooled.erase(c->zcache)) cudaFreeAsync(c->zcache, c->stream);
+    else cudaFree(c->zcache);
+    c->zcache = p;
+    c->zcap = n;
+    return true;
+}
+
+sisso_status ctx_alloc(sisso_ctx* c, void** p, size_t bytes, const char* what) {
+    unsigned char* b = nullptr;
+    const sisso_status st = dalloc(c, b, bytes, what);
+    if (!st) c->bufs.push_back(b);
+    *p = b;
+    return st;
+}
+}  // namespace sg
 
 extern "C" {
 
@@ -249,9 +283,11 @@ sisso_status sisso_create(const double* X, const double* y, int N, int d, uint32
         return bail(st);
     cudaMemcpyAsync(c->space_dev, &c->space, sizeof(Space), cudaMemcpyHostToDevice, c->stream);
     if ((st = ensure_tile_buffers(c, c->n_cap))) return bail(st);
-    // standardised FP64 vectors of the screening window, for the duplicate rule: up to
-    // 4 GB (the walk evaluates on the fly when a window does not fit)
-    c->zcap = std::min<int64_t>(c->surv_cap, ((int64_t)16 << 30) / ((int64_t)8 * N));
+    // standardised FP64 vectors of the screening window, for the duplicate rule: room for the
+    // first window and S, grown with the window up to 16 GB (the walk evaluates on the fly when
+    // a window does not fit)
+    c->zcap_max = std::min<int64_t>(c->surv_cap, ((int64_t)16 << 30) / ((int64_t)8 * N));
+    c->zcap = std::min<int64_t>(c->zcap_max, first_window(c, sis_size) + c->n_cap);
     if ((st = dalloc(c, c->zcache, (size_t)c->zcap * Nn, "zcache")) ||
         (st = dalloc(c, c->subvalid, (size_t)c->space.phi[rung - 1], "subvalid")) ||
         (st = dalloc(c, c->dup_list, (size_t)c->sort_cap * kDupSlots, "dup_list")) ||
@@ -307,10 +343,13 @@ sisso_status sisso_create(const double* X, const double* y, int N, int d, uint32
     const bool mixed_form = o.precision == SISSO_PREC_MIXED_BF16 || o.precision == SISSO_PREC_MIXED_FP16;
     if (!st && mixed_form && o.screen != SISSO_SCREEN_CORES && c->opval64 && tc_screen_possible(c, o.screen))
         st = tc_screen_alloc(c);
+    if (!st && o.precision != SISSO_PREC_FP64 && !c->tc_on && !(mixed_form && o.screen == SISSO_SCREEN_CORES) &&
+        pair_tc_possible(c))
+        st = pair_tc_alloc(c);
     if (!st && o.whiten) {
         // whitening (§2.4) runs row by row from the FP64 operand values and keeps every
         // window vector
-        if (!c->opval64 || c->zcap < c->surv_cap)
+        if (!c->opval64 || c->zcap_max < c->surv_cap)
             st = fail(c, SISSO_ERR_CAPACITY, "whitening: FP64 operand values or window vectors do not fit");
         else
             st = whiten_setup(c, o.whiten);
@@ -340,6 +379,7 @@ sisso_status sisso_fit(sisso_ctx* c) {
     const bool tc_gram = mixed || (prec == SISSO_PREC_FP32 && c->opts.gram == SISSO_GRAM_TF32X3);
     c->stats = sisso_stats{};
     c->tc_ready = false;
+    pair_tc_reset(c);
     c->S.clear(); c->n_sis.clear(); c->res_ids.clear(); c->res_coef.clear(); c->res_rmse.clear(); c->res_r2.clear();
     c->n_dims = 0;
     c->fitted = false;
@@ -545,6 +585,7 @@ sisso_status sisso_score_all(sisso_ctx* c, const double* target, int precision, 
     if (!c || !target || !scores) return SISSO_ERR_ARG;
     cudaSetDevice(c->opts.device);
     cudaMemcpyAsync(c->target64, target, sizeof(double) * c->N, cudaMemcpyDefault, c->stream);
+    pair_tc_reset(c);
     sisso_status st = prepare_target(c, c->target64);
     if (!st) st = score_all(c, precision);
     if (!st) {
@@ -562,6 +603,7 @@ sisso_status sisso_sis_step(sisso_ctx* c, const double* target, const int64_t* S
     cudaSetDevice(c->opts.device);
     std::vector<int64_t> prev(S_prev, S_prev + n_prev);
     cudaMemcpyAsync(c->target64, target, sizeof(double) * c->N, cudaMemcpyDefault, c->stream);
+    pair_tc_reset(c);
     sisso_status st = prepare_target(c, c->target64);
     if (!st) st = score_all(c, c->opts.precision);
     std::vector<int64_t> out;

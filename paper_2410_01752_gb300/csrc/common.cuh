@@ -9,6 +9,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <string>
@@ -319,7 +320,9 @@ struct TargetStats {
     double mean, sd;        // FP64 mean and population std of the target
     double tsum;            // FP64 sum of the centred target (rounding-level, kept exact)
     double sum32, srr32;    // sum and centred sum of squares of the FP32 copy
-    float sd32, pad;
+    float sd32;
+    float rscale;           // 2^-e >= 1 / (sd sqrt(N)): scales the centred target into [-1, 1]
+    float inv_sdr, pad;     // 1 / (sd rscale)
 };
 
 // small result block of one SIS walk, copied back to the host
@@ -346,6 +349,8 @@ struct Winner {
 };
 
 }  // namespace sg
+
+namespace sg { struct PairTc; }
 
 struct sisso_ctx {
     int N, d, rung, k, max_dim;
@@ -383,6 +388,7 @@ struct sisso_ctx {
     double* surv_probe = nullptr;      // kProbes standardised values per entry
     double* zcache = nullptr;          // standardised FP64 vectors of the window (zcap x N)
     int64_t zcap = 0;
+    int64_t zcap_max = 0;              // ... and the most they may grow to
     unsigned char* subvalid = nullptr; // FP64 validity (recursive) of every id of phi_{L-1}
     float* opcache32 = nullptr;        // values of phi_{L-1}, sample-major (N x id), or null
     double* opcache64 = nullptr;       // ... FP64 copy (FP64 screening only)
@@ -491,9 +497,34 @@ struct sisso_ctx {
     double* opinv64 = nullptr;         // 1/x of every FP64 operand value (division in the FP64 re-score)
     int* tc_err = nullptr;
     unsigned long long* tc_raised = nullptr;
+
+    sg::PairTc* pt = nullptr;          // fused tensor-core pair scores (pair_tc.cu)
+    std::vector<void*> bufs;           // buffers of ctx_alloc
 };
 
 namespace sg {
+
+// pair_tc.cu: top-level pair scores from fused tensor-core products
+bool pair_tc_possible(const sisso_ctx* c);
+sisso_status pair_tc_alloc(sisso_ctx* c);
+void pair_tc_reset(sisso_ctx* c);
+void pair_tc_free(sisso_ctx* c);
+sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow);
+
+// room for the standardised vectors of n window entries (grown on demand; false: they do not fit)
+bool zcache_fits(sisso_ctx* c, int64_t n);
+// first screening window of a step: max(4096, 32 k) candidates, but at most about 2^26 sample
+// evaluations of FP64 re-scoring (the re-score costs M x N) and never below 5 k
+inline int64_t first_window(const sisso_ctx* c, int k);
+
+// a device buffer owned by the context (released with it)
+sisso_status ctx_alloc(sisso_ctx* c, void** p, size_t bytes, const char* what);
+
+inline int64_t first_window(const sisso_ctx* c, int k) {
+    return c->opts.survivors > 0
+               ? c->opts.survivors
+               : std::max<int64_t>(5LL * k, std::min<int64_t>(std::max<int64_t>(4096, 32LL * k), (1LL << 26) / c->N));
+}
 
 // host-side helpers implemented in the .cu files
 bool plan_space(int d, uint32_t ops, int rung, int grammar, Space& sp);

@@ -1470,7 +1470,15 @@ sisso_status score_all(sisso_ctx* c, int precision) {
         if ((st = tc_screen_pairs(c, A.sec))) return st;
         c->stats.screen_pair_launches++;
         c->stats.screen_tc = 1;
-    } else if (any) {
+    }
+    bool cores = any && !tc;
+    if (cores && c->pt && !fp64) {
+        bool overflow = false;
+        if ((st = pair_tc_scores(c, A.sec, &overflow))) return st;
+        c->stats.screen_pair_launches++;
+        cores = overflow;
+    }
+    if (cores) {
         std::vector<int2> tiles;
         pair_tiles(A.P, A.Q, A.nxp, tiles);
         int2* d_tiles = nullptr;
@@ -1589,11 +1597,7 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
         cudaMemcpyAsync(c->S_sorted, Ss.data(), sizeof(int64_t) * n_prev, cudaMemcpyHostToDevice, c->stream);
     const bool fp_kernel64 = c->opts.precision == SISSO_PREC_FP64;
     const double eps = fp_kernel64 ? kScoreErr64 : kScoreErr32;   // bound on |score_kernel - score_FP64|
-    // default window: max(4096, 32 k) candidates, but at most about 2^26 sample evaluations of
-    // FP64 re-scoring (the re-score costs M x N) and never below 5 k
-    int64_t M = c->opts.survivors > 0
-                    ? c->opts.survivors
-                    : std::max<int64_t>(5LL * k, std::min<int64_t>(std::max<int64_t>(4096, 32LL * k), (1LL << 26) / c->N));
+    int64_t M = first_window(c, k);
     const int64_t n = c->n_feat;
     const int gridS = std::max(1, c->sms * 8);
     cudaEvent_t q[5];
@@ -1629,7 +1633,7 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
             cudaMemcpyAsync(c->surv_ids + ns, S_prev_host, sizeof(int64_t) * n_prev, cudaMemcpyHostToDevice, c->stream);
         const int nr = ns + n_prev;
         cudaEventRecord(q[1], c->stream);
-        double* zc = (int64_t)nr <= c->zcap ? c->zcache : nullptr;   // cache the vectors if they fit
+        double* zc = zcache_fits(c, nr) ? c->zcache : nullptr;   // cache the vectors if they fit
         if (c->Wm) {            // whitened data: every window vector cached (checked at creation)
             if (!zc) { st = fail(c, SISSO_ERR_CAPACITY, "whitened window exceeds the vector cache"); break; }
             if ((st = whiten_rescore(c, c->surv_ids, nr, c->surv_score, c->surv_mean, c->surv_sd, c->surv_valid,

@@ -258,6 +258,10 @@ __device__ void prepare_target_block(const double* t, int N, double* tc64, float
         st->sum32 = s32;
         st->srr32 = ss32 - s32 * s32 / N;
         st->sd32 = (float)sqrt(st->srr32 / N);
+        int e;
+        frexp(st->sd * sqrt((double)N), &e);
+        st->rscale = (float)ldexp(1.0, -e);
+        st->inv_sdr = (float)(1.0 / ldexp(st->sd, -e));
     }
 }
 
