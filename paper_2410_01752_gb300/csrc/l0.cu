@@ -567,14 +567,13 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
     TileArgs A{};
     A.G = c->tile_G + kTC; A.b = c->tile_b; A.diag = c->tile_diag; A.ldp = ldp; A.n = n; A.N = c->N; A.D = D;
     A.syy = (float)syy; A.tau = kPivotMin32; A.sst = sst; A.sqrt_syy = std::sqrt(syy);
-    // filter: coefficient 1-norm bound Smax = 16 sqrt(syy); E1 = twice the a posteriori bound
-    // at Smax (|RSS| <= 2 SST) plus the rounding of the filter's own comparison
+    // filter: twice the a posteriori bound on RSS / N (|RSS| <= 2 SST) plus the rounding of the
+    // filter's own comparison
     {
         const double u = 5.9604644775390625e-8, c1 = 1.0 + 3.1 * (D + 1);
-        const double smax = 16.0 * std::sqrt(syy);
-        const double err = 2.0 * u * (c->N * (2.0 * std::sqrt(syy) * smax + c1 * smax * smax) + (D + 3) * 4.0 * sst);
-        A.Smax = (float)smax;
-        A.E1 = (float)(2.0 * err + 64.0 * u * sst);
+        A.e0 = (float)(4.0 * u * (D + 3) * 4.0 * syy + 64.0 * u * syy);
+        A.e1 = (float)(4.0 * u * 2.0 * std::sqrt(syy));
+        A.e2 = (float)(4.0 * u * c1);
     }
     A.tiles = reinterpret_cast<const TileInfo*>(c->tile_info); A.n_tiles = (int)tiles.size(); A.n_items = items;
     A.counter = c->work; A.ub_key = ub_key; A.tie64 = 2.0 * kRssTie * sst;

@@ -12,16 +12,23 @@
 // subset, with 1/d1 and w1/sqrt(d1) precomputed per row:
 //     g = G[i1][i2] - sum_m R[m][i1] R[m][i2],   d2 = dp[i2] - g^2 / d1,
 //     num = np[i2] - g w1 / sqrt(d1),   RSS = N (c - num^2 / d2),  c = syy - |w_prefix|^2 - w1^2
-// as in the two-pass enumerator, but the decision is a division-free filter:
-//     candidate  <=>  not ( num^2 - cB d2 < 0   and   S1 |num| - Rk d2 <= 0   and  d2 > tau )
-// cB puts the FP32 RSS above B + tie + E1 (B the running bound, below), and the second
-// test bounds the subset's coefficient 1-norm s = |gamma|_1 by Smax: with a = L_P^-T w_P,
-// a1 = L_P^-T R[.][i1], a2 = L_P^-T R[.][i2] (prefix back substitutions),
+// as in the two-pass enumerator, but the decision is a division-free filter on t = |num| / d2
+// (the coefficient of i2).  The a posteriori bound of the FP32 RSS per sample is
+// e0 + e1 s + e2 s^2 with s = |gamma|_1 the subset's coefficient 1-norm, and with
+// a = L_P^-T w_P, a1 = L_P^-T R[.][i1], a2 = L_P^-T R[.][i2] (prefix back substitutions)
 //     s <= |a|_1 + (1 + |a1|_1) |w1| / sqrt(d1)
-//            + ((1 + |a1|_1) |r| / sqrt(d1) + 1 + |a2|_1) |num| / d2,   |r| <= 1,
-// i.e. s <= S0 + S1' |num| / d2, and s <= Smax keeps the a posteriori FP32 error below E1/2.
-// So a subset that is not a candidate has RSS_FP32 - err > B + tie: it cannot be the
-// minimum nor tie with it.  Candidates (a fraction of a percent on screened subspaces)
+//            + ((1 + |a1|_1) |r| / sqrt(d1) + 1 + |a2|_1) |num| / d2 = S0 + S1 t,   |r| <= 1.
+// With K = c - (B + tie)/N - e0 - S0 (e1 + e2 S0), beta = S1 (e1 + 2 e2 S0), gamma = e2 S1^2
+// per row (e0, e1, e2 twice the bound's), a subset is dismissed when
+//     K - beta t - (d2 + gamma) t^2 > 0, that is (times d2^2, d2 > tau)
+//     d2 (num^2 - K d2 + beta |num|) + gamma num^2 < 0:
+// RSS_FP32 less its error bound at the subset's own coefficients then exceeds B + tie, so it
+// cannot be the minimum nor tie with it.  (A bound taken at one largest s for every subset
+// sent 1.7% of the C(300, 5) subsets of a 1%-noise problem to the exact test, where their
+// FP64 solves took as long as the sweep.)  The sweep keeps only the largest left-hand side and
+// the smallest d2 of a lane's columns: rows in which no lane has one to keep, almost all of
+// them, need no per-column decision.
+// Candidates (a fraction of a percent on screened subspaces)
 // go through a per-warp queue to the exact test of the two-pass form: the FP32 RSS and
 // its a posteriori bound from the back-substituted coefficients, then an FP64 solve from
 // the FP64 Gram; a subset whose FP64 RSS is within B + tie enters the band and lowers B.
@@ -77,7 +84,7 @@ struct TileArgs {
     int ldp, n, N, D;
     float syy, tau;
     double sst, sqrt_syy;
-    float E1, Smax;                      // filter window and coefficient bound (FP32 RSS units / sqrt(syy) units)
+    float e0, e1, e2;                    // filter: FP32 error of RSS / N at coefficient 1-norm s, e0 + e1 s + e2 s^2
     const TileInfo* tiles;
     int n_tiles;
     int64_t n_items;
@@ -175,8 +182,8 @@ __device__ __forceinline__ float back_l1(const float (&L)[DP > 0 ? DP : 1][DP > 
     return s;
 }
 
-// per-warp row record: R[.][i1], 1/sqrt(d1), w1, c, S1, Rk, flags (bit 1: pivots of the
-// prefix and of i1 are above tau), padded to a multiple of 4 words
+// per-warp row record: R[.][i1], 1/sqrt(d1), w1, c, K before the threshold (-inf where a pivot
+// of the prefix or of i1 is not above tau), beta, gamma, padded to a multiple of 4 words
 __host__ __device__ constexpr int row_words(int DP) { return ((DP + 6) + 3) & ~3; }
 
 template <int DP>
@@ -215,7 +222,7 @@ __device__ __noinline__ double tile_exact(const TileArgs& A, const PrefixSm* Ps,
 #pragma unroll
     for (int m = 0; m < DP; ++m) r1[m] = rr_[m];
     const float isd1 = rr_[DP], w1 = rr_[DP + 1], base_c = rr_[DP + 2];
-    const int flags = __float_as_int(rr_[DP + 5]);
+    const bool piv = rr_[DP + 3] > -INFINITY;
     float rt[DP > 0 ? DP : 1];
 #pragma unroll
     for (int m = 0; m < DP; ++m) rt[m] = colv[m * kTC + off];
@@ -229,7 +236,7 @@ __device__ __noinline__ double tile_exact(const TileArgs& A, const PrefixSm* Ps,
     pos[DP] = i1;
     pos[DP + 1] = x;
     float r32 = __int_as_float(0x7fc00000);
-    if ((flags & 2) && d2 > A.tau) {
+    if (piv && d2 > A.tau) {
         const float rss = (float)A.N * (base_c - num * num / d2);
         r32 = rss;
         if (!(rss <= thr32)) {
@@ -296,7 +303,7 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
     unsigned short* q = reinterpret_cast<unsigned short*>(reinterpret_cast<PrefixSm*>(
                             reinterpret_cast<float*>(tile_smem) + (size_t)kTW * (kTR * RW + (DP + 2) * kTC + kTQ)) +
                         kTW) + (size_t)w * kTQ;
-    const float N = (float)A.N;
+    const double inv_n = 1.0 / (double)A.N;
     double B = INFINITY;                            // fmin ignores an unset (NaN) key
     B = fmin(B, okey_inv(*(volatile unsigned long long*)A.ub_key));
     unsigned long long my_examined = 0, my_cand = 0;
@@ -389,13 +396,13 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int x = cb + lane + 32 * j;
-                if (j >= j_lo && x >= c && x < A.n) {
+                if (x > row_lo && x >= c && x < A.n) {
                     prefix_reduce<DP>(A, pre, L, invd, wv, x, rt[j], dp2[j], np2[j]);
                     q2 = fmaxf(q2, back_l1<DP>(L, invd, rt[j]));
                 } else {
 #pragma unroll
                     for (int m = 0; m < DP; ++m) rt[j][m] = 0.f;
-                    dp2[j] = 1.f;
+                    dp2[j] = 1e15f;              // never kept by the sweep: d2 huge
                     np2[j] = 0.f;
                 }
 #pragma unroll
@@ -415,16 +422,16 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
                 const float isd1 = 1.f / sqrtf(d1 > 0.f ? d1 : 1.f);
                 const float w1 = n1 * isd1;
                 const float a1 = back_l1<DP>(L, invd, r1);
-                const float S0 = A0 + (1.f + a1) * fabsf(w1) * isd1;
+                const float S0 = 1.02f * (A0 + (1.f + a1) * fabsf(w1) * isd1);
                 const float S1 = 1.02f * ((1.f + a1) * isd1 * 1.0001f + 1.f + q2);
 #pragma unroll
                 for (int m = 0; m < DP; ++m) rr_[m] = r1[m];
                 rr_[DP] = isd1;
                 rr_[DP + 1] = w1;
                 rr_[DP + 2] = A.syy - (pw2 + w1 * w1);
-                rr_[DP + 3] = S1;
-                rr_[DP + 4] = piv ? A.Smax - 1.02f * S0 : -INFINITY;
-                rr_[DP + 5] = __int_as_float(piv ? 2 : 0);
+                rr_[DP + 3] = piv ? rr_[DP + 2] - (A.e0 + S0 * fmaf(A.e2, S0, A.e1)) : -INFINITY;
+                rr_[DP + 4] = S1 * fmaf(2.f * A.e2, S0, A.e1);
+                rr_[DP + 5] = A.e2 * S1 * S1;
                 const int lo_c = max(c, i1 + 1), hi_c = min(c + kTC, A.n);
                 if (hi_c > lo_c) my_examined += (unsigned long long)(hi_c - lo_c);
             }
@@ -450,7 +457,7 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
             nmask |= (x >= c && x < A.n) ? (1u << j) : 0u;
         }
         int qn = 0;                                     // queue length (warp-uniform)
-        float thrN = (float)((B + A.tie64) / (double)A.N) + A.E1 / N;
+        float thrN = __fmul_ru((float)((B + A.tie64) * inv_n), 1.0000002f);
         int i1 = row_lo;
         // rows in segments of equal first live group J (the groups holding a column right
         // of i1 are J .. 7), so that every segment's group range is fixed at compile time
@@ -470,25 +477,15 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
                 // d2 = dp2 - g^2/d1, num = np2 - g w1/sqrt(d1)
                 const float isd1 = rec[DP], w1 = rec[DP + 1];
                 const float id1 = isd1 * isd1, w1s = w1 * isd1;
-                const float S1 = rec[DP + 3], Rk = rec[DP + 4];
-                const float cB = rec[DP + 2] - thrN;
-                // columns right of i1: j >= js, js the smallest j with cb + lane + 32 j > i1
-                const int dj = i1 - cb - lane;
-                const int js = dj < 0 ? 0 : (dj >> 5) + 1;
-                const unsigned vmask = nmask & (js >= 8 ? 0u : (0xFFu << js));
+                const float nK = thrN - rec[DP + 3], beta = rec[DP + 4], gamma = rec[DP + 5];
+                const int dj = i1 - cb - lane;             // column i1 is this lane's group dj / 32
                 const float* grow = A.G + (size_t)i1 * A.ldp + cb + lane;
                 float gv[8];
 #pragma unroll
                 for (int j = J; j < 8; ++j) gv[j] = grow[32 * j];
-                unsigned mask = 0;
                 // per column: g = G - sum R R, d2 = dp2 - g^2 / d1, num = np2 - g w1 / sqrt(d1),
-                // f = num^2 - cB d2, e = S1 |num| - Rk d2 (as fma(-a, b, c) and fma(a, a, -(c d)))
-                // dismissed <=> f < 0 and e <= 0 and d2 > tau, evaluated without branches
-                auto decide = [&](int j, float d2, float num, float f) {
-                    const float e = fmaf(S1, fabsf(num), -(Rk * d2));
-                    const bool dismiss = (f < 0.f) & (e <= 0.f) & (d2 > A.tau);
-                    mask |= (unsigned)(!dismiss) << j;
-                };
+                // n2 = num^2, z = d2 (n2 - K d2 + beta |num|) + gamma n2: dismissed where z < 0 and d2 > tau
+                float zmax = -INFINITY, dmin = INFINITY;
                 if (J & 1) {           // a first group without its pair partner
                     float g = gv[J];
                     float rtJ[DPa], dJ, nJ, u;
@@ -500,14 +497,15 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
                     for (int m = 0; m < DP; ++m) g = fmaf(-rec[m], rtJ[m], g);
                     gv[J] = g;
                     const float d2 = fmaf(-(g * g), id1, dJ);
-                    const float num = fmaf(-g, w1s, nJ);
-                    decide(J, d2, num, fmaf(num, num, -(cB * d2)));
+                    const float num = fmaf(-g, w1s, nJ), n2 = num * num;
+                    const float z = fmaf(fmaf(beta, fabsf(num), fmaf(nK, d2, n2)), d2, gamma * n2);
+                    if (dj != 32 * J) { zmax = z; dmin = d2; }       // not the row's own column
                 }
                 {
                     p2 nrec[DPa];
 #pragma unroll
                     for (int m = 0; m < DP; ++m) nrec[m] = pk2(-rec[m], -rec[m]);
-                    const p2 nid1 = pk2(-id1, -id1), nw1s = pk2(-w1s, -w1s), ncB = pk2(-cB, -cB);
+                    const p2 nid1 = pk2(-id1, -id1), nw1s = pk2(-w1s, -w1s), nK2 = pk2(nK, nK), gm2 = pk2(gamma, gamma);
 #pragma unroll
                     for (int jp = (J + 1) >> 1; jp < 4; ++jp) {
                         p2 g = pk2(gv[2 * jp], gv[2 * jp + 1]);
@@ -515,15 +513,35 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
                         for (int m = 0; m < DP; ++m) g = fma2(nrec[m], rtp[jp][m], g);
                         const p2 d2 = fma2(mul2(g, g), nid1, dpp[jp]);
                         const p2 num = fma2(g, nw1s, npp[jp]);
-                        const p2 f = fma2(num, num, mul2(ncB, d2));
-                        float ga, gb, da, db, na, nb, fa, fb;
-                        up2(g, ga, gb); up2(d2, da, db); up2(num, na, nb); up2(f, fa, fb);
+                        const p2 n2 = mul2(num, num);
+                        const p2 h = fma2(nK2, d2, n2);
+                        float ga, gb, da, db, na, nb, ha, hb, za, zb;
+                        up2(g, ga, gb); up2(d2, da, db); up2(num, na, nb); up2(h, ha, hb);
                         gv[2 * jp] = ga; gv[2 * jp + 1] = gb;
-                        decide(2 * jp, da, na, fa);
-                        decide(2 * jp + 1, db, nb, fb);
+                        const p2 z = fma2(pk2(fmaf(beta, fabsf(na), ha), fmaf(beta, fabsf(nb), hb)), d2, mul2(gm2, n2));
+                        up2(z, za, zb);
+                        if (2 * jp == J && dj == 32 * J) { za = -INFINITY; da = INFINITY; }
+                        zmax = fmaxf(fmaxf(zmax, za), zb);
+                        dmin = fminf(fminf(dmin, da), db);
                     }
                 }
-                mask &= vmask;
+                if (__any_sync(0xffffffffu, !(zmax < 0.f) || !(dmin > A.tau))) {
+                // a lane has something to keep: the decisions column by column, from the same g
+                // columns right of i1: j >= js, js the smallest j with cb + lane + 32 j > i1
+                const int js = dj < 0 ? 0 : (dj >> 5) + 1;
+                unsigned mask = 0;
+#pragma unroll
+                for (int j = J; j < 8; ++j) {
+                    const float g = gv[j];
+                    float dlo, dhi, nlo, nhi;
+                    up2(dpp[j >> 1], dlo, dhi);
+                    up2(npp[j >> 1], nlo, nhi);
+                    const float d2 = fmaf(-(g * g), id1, (j & 1) ? dhi : dlo);
+                    const float num = fmaf(-g, w1s, (j & 1) ? nhi : nlo), n2 = num * num;
+                    const float z = fmaf(fmaf(beta, fabsf(num), fmaf(nK, d2, n2)), d2, gamma * n2);
+                    mask |= (unsigned)(!((z < 0.f) & (d2 > A.tau))) << j;
+                }
+                mask &= nmask & (js >= 8 ? 0u : (0xFFu << js));
                 if (__any_sync(0xffffffffu, mask != 0)) {
                     const int cnt = __popc(mask);
                     int off = cnt;
@@ -547,8 +565,9 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
                         B = tile_flush<DP>(A, Ps, rowrec, colv, q, qg, qn, a, cb, lane, B);
                         my_cand += qn;
                         qn = 0;
-                        thrN = (float)((B + A.tie64) / (double)A.N) + A.E1 / N;
+                        thrN = __fmul_ru((float)((B + A.tie64) * inv_n), 1.0000002f);
                     }
+                }
                 }
             }
         }
