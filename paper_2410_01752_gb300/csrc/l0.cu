@@ -23,6 +23,7 @@
 //  minimum and pass 2 the tie window directly.
 #include "l0_device.cuh"
 #include "l0_tile.cuh"
+#include "l0_block.cuh"
 
 #include <algorithm>
 #include <cfloat>
@@ -588,7 +589,33 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
         cudaFuncSetAttribute(k_l0_tile<DPV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);   \
         k_l0_tile<DPV><<<grid, kTW * 32, sm, c->stream>>>(A);                                          \
     } while (0)
-    switch (DP) {
+    // D = 4 and 5 without a prefix mask: the prefix's first D - 3 features eliminated once per
+    // CTA when the triangle of the rest fits shared memory and there are enough prefixes to
+    // fill the SMs (a slice of a prefix's features at D = 4, which has only n of them)
+    const int DC = D - 3;
+    const int m_max = n - DC;
+    if (DC >= 1 && DC <= 2 && !prefix_mask && m_max >= 3 && m_max <= kBMaxM) {
+        // two launches: the prefixes with many features to their right, then those with few
+        const int slices = DC == 1 ? 4 : 1;
+        const int64_t all = DC == 1 ? n - 3 : binom_host(n - 3, 2);
+        const int last_big = n - 1 - kBSmallM;                 // a prefix's last feature below it: m > kBSmallM
+        const int64_t big = std::min(all, last_big <= 0 ? 0 : DC == 1 ? (int64_t)last_big : binom_host(last_big, 2));
+#define SG_BLOCK(DCV, WV, ITEM0, END, MV)                                                               \
+    do {                                                                                                \
+        const size_t sm = block_smem_bytes(MV, WV);                                                     \
+        A.n_items = (END) * slices;                                                                     \
+        cudaFuncSetAttribute(k_l0_block<DCV, WV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
+        k_l0_block<DCV, WV><<<c->sms * (16 / WV), WV * 32, sm, c->stream>>>(A, slices, (int)((ITEM0) * slices), MV); \
+    } while (0)
+        if (big > 0) { if (DC == 1) SG_BLOCK(1, kBWarpsBig, 0, big, m_max); else SG_BLOCK(2, kBWarpsBig, 0, big, m_max); }
+        A.counter = c->work + 1;
+        if (all > big) {
+            const int ms = std::min(m_max, kBSmallM);
+            if (DC == 1) SG_BLOCK(1, kBWarpsSmall, big, all, ms); else SG_BLOCK(2, kBWarpsSmall, big, all, ms);
+        }
+#undef SG_BLOCK
+        c->stats.launches += big > 0 && all > big;
+    } else switch (DP) {
         case 0: SG_TILE(0); break;
         case 1: SG_TILE(1); break;
         case 2: SG_TILE(2); break;

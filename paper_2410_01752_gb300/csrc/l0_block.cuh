@@ -1,0 +1,424 @@
+// l0_block.cuh — the tiled l0 enumeration (l0_tile.cuh) for D = 4 and 5 with the prefix split in
+// two: a CTA eliminates the first D - 3 features from the Gram once, in shared memory, and its
+// warps sweep every (p, i1, i2) of the rest.
+//
+// k_l0_tile re-derives a prefix's reduced columns and rows in every warp's work unit; at D = 5 a
+// prefix of three has on average only C(n, 5) / C(n, 3) = 4400 subsets at n = 300, and the unit's
+// set-up and its short rows cost several times the sweep (1.4 warp instructions a subset, 0.25 in
+// the sweep itself).  Here a work unit is a prefix of D - 3 features: the CTA forms
+//     G'[x][y] = G[x][y] - sum R R   (y < x, packed strict lower triangle, shared memory)
+// once for C(m, 3) subsets (m features to the right), and adding the next feature p needs one
+// value per feature: r = G'[x][p] / sqrt(d'_p), dp = d' - r^2, np = n' - r w_p.  The warps take
+// the p of a unit in turn and need no barrier.  Lanes are the rows i1 (their constants of the
+// filter stay in registers); a column x > i1 costs two broadcast reads, three operations for its
+// values and one row of G'.  The subset test is the filter of l0_tile.cuh with one fused
+// multiply-add in the place of D - 2.
+// Measured at n = 300, D = 5 (1.96e10 subsets): see the figures at the launch (l0.cu).  Forms
+// that took longer than k_l0_tile's 43 ms: lanes as columns with the row constants shuffled in
+// (89 ms), and four warps sharing a p through a record table and a barrier (46 ms).
+#pragma once
+
+#include "l0_tile.cuh"
+
+#include <type_traits>
+
+namespace sg {
+namespace {
+
+// warps of a CTA (one p each at a time): sixteen and one CTA per SM while the triangle is large;
+// up to kBSmallM features, four and four CTAs per SM, so that a unit's barriers hold up few warps
+// (three quarters of the prefixes of n = 300 have that few features to the right)
+constexpr int kBWarpsBig = 16, kBWarpsSmall = 4, kBSmallM = 150;
+constexpr int kBRow = 6;                  // row groups of 32 swept together (their constants are 36 registers)
+constexpr int kBQ = 64;                   // per-warp candidate queue
+constexpr int kBMaxM = 320;               // features right of the CTA's prefix (204 KB triangle)
+
+__host__ __device__ constexpr size_t block_smem_bytes(int m, int warps) {
+    return sizeof(float) * ((size_t)m * (m - 1) / 2 + 36) + 2 * sizeof(float2) * (size_t)m +
+           sizeof(unsigned) * kBQ * warps;
+}
+
+// prefix of the CTA, in feature coordinates (shared memory)
+struct BlockPre {
+    int pre[2], last, ok;        // features, the last of them, pivots above tau
+    float l10, inv[2], w[2];     // factor, 1 / diagonal, forward-solved moments
+    float u[2], pw2;             // back-substituted coefficients L^-T w, |w|^2
+};
+
+// the exact decision of one subset (positions ascending): FP32 solve with its a posteriori
+// bound, then FP64; returns the lane's new bound
+template <int D>
+__device__ __noinline__ double block_exact(const TileArgs& A, const int (&pos)[D], double B, double thr, float thr32) {
+    float L[D][D], inv[D], wv[D], q = 0.f;
+    bool piv = true;
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+        float d = A.diag[pos[j]];
+#pragma unroll
+        for (int m = 0; m < j; ++m) d -= L[j][m] * L[j][m];
+        piv = piv && d > A.tau;
+        const float l = sqrtf(d > 0.f ? d : 1.f);
+        inv[j] = 1.f / l;
+#pragma unroll
+        for (int i = j + 1; i < D; ++i) {
+            float v = A.G[(size_t)pos[i] * A.ldp + pos[j]];
+#pragma unroll
+            for (int m = 0; m < j; ++m) v -= L[i][m] * L[j][m];
+            L[i][j] = v * inv[j];
+        }
+        float v = A.b[pos[j]];
+#pragma unroll
+        for (int m = 0; m < j; ++m) v -= L[j][m] * wv[m];
+        wv[j] = v * inv[j];
+        q += wv[j] * wv[j];
+    }
+    float r32 = __int_as_float(0x7fc00000);
+    if (piv) {
+        const float rss = (float)A.N * (A.syy - q);
+        r32 = rss;
+        if (!(rss <= thr32)) {
+            float s = 0.f, gm[D];
+#pragma unroll
+            for (int j = D - 1; j >= 0; --j) {
+                float v = wv[j];
+#pragma unroll
+                for (int m = j + 1; m < D; ++m) v -= L[m][j] * gm[m];
+                gm[j] = v * inv[j];
+                s += fabsf(gm[j]);
+            }
+            if (!(rss - tile_apost_err(A, s, rss) <= thr32)) return B;
+        }
+    }
+    const double r64 = rss64(A.G64, A.b64, A.ld64, A.syy64, A.N, D, pos, nullptr);
+    if (!(r64 <= thr)) return B;
+    add_band<D - 2>(A, pos, r32);
+    if (r64 < B) {
+        atomicMin(A.ub_key, okey(r64));
+        return r64;
+    }
+    return B;
+}
+
+// the warp's queued candidates (local positions p, i1, x in ten bits each)
+template <int DC>
+__device__ __noinline__ double block_flush(const TileArgs& A, const BlockPre* P, const unsigned* q, int qn, double B) {
+    const int lane = threadIdx.x & 31;
+    const double thr = B + A.tie64;
+    const float thr32 = __double2float_ru(thr);
+    for (int e = lane; e < qn; e += 32) {
+        const unsigned v = q[e];
+        int pos[DC + 3];
+#pragma unroll
+        for (int m = 0; m < DC; ++m) pos[m] = P->pre[m];
+        pos[DC] = P->last + 1 + (int)(v & 1023u);
+        pos[DC + 1] = P->last + 1 + (int)((v >> 10) & 1023u);
+        pos[DC + 2] = P->last + 1 + (int)(v >> 20);
+        B = block_exact<DC + 3>(A, pos, B, thr, thr32);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) B = fmin(B, __shfl_xor_sync(0xffffffffu, B, o));
+    return fmin(B, okey_inv(*(volatile unsigned long long*)A.ub_key));
+}
+
+// the filter's row constants of a lane (l0_tile.cuh), row groups j and j + 1 per register pair:
+// -R[p][i1], -1/d1, -w1/sqrt(d1), -K, beta, gamma
+struct RowsC { p2 nr[kBRow / 2], nid[kBRow / 2], nw[kBRow / 2], nK[kBRow / 2], be[kBRow / 2], gm[kBRow / 2]; };
+
+// the test of one subset: z < 0 and d2 > tau dismiss it
+__device__ __forceinline__ void block_test(float gv, float r, float d, float n, float nr, float nid, float nw, float nK,
+                                           float beta, float gamma, float& z, float& d2) {
+    const float g = fmaf(nr, r, gv);
+    d2 = fmaf(g * g, nid, d);
+    const float num = fmaf(g, nw, n), n2 = num * num;
+    z = fmaf(fmaf(beta, fabsf(num), fmaf(nK, d2, n2)), d2, gamma * n2);
+}
+
+// one column (r, d, n; gx its row of G' at this lane's rows) against C row groups: the largest z
+// and the smallest d2 are folded into zmax and dmin.  dead: this lane's row of the last group is
+// not left of x
+template <int C>
+__device__ __forceinline__ void block_col(const float* gx, float r, float d, float n, bool dead, const RowsC& R,
+                                          float& zmax, float& dmin) {
+    float gv[C];
+#pragma unroll
+    for (int j = 0; j < C; ++j) gv[j] = gx[32 * j];
+    if (C > 1) {
+        const p2 rx = pk2(r, r), dx = pk2(d, d), nx = pk2(n, n);
+#pragma unroll
+        for (int jp = 0; jp < C / 2; ++jp) {
+            const p2 g = fma2(R.nr[jp], rx, pk2(gv[2 * jp], gv[2 * jp + 1]));
+            const p2 d2 = fma2(mul2(g, g), R.nid[jp], dx);
+            const p2 num = fma2(g, R.nw[jp], nx);
+            const p2 n2 = mul2(num, num);
+            const p2 h = fma2(R.nK[jp], d2, n2);
+            float da, db, na, nb, ha, hb, za, zb, ba, bb;
+            up2(d2, da, db); up2(num, na, nb); up2(h, ha, hb); up2(R.be[jp], ba, bb);
+            const p2 z = fma2(pk2(fmaf(ba, fabsf(na), ha), fmaf(bb, fabsf(nb), hb)), d2, mul2(R.gm[jp], n2));
+            up2(z, za, zb);
+            if (2 * jp + 1 == C - 1 && dead) { zb = -INFINITY; db = INFINITY; }
+            zmax = fmaxf(fmaxf(zmax, za), zb);
+            dmin = fminf(fminf(dmin, da), db);
+        }
+    }
+    if (C & 1) {
+        constexpr int h = C / 2;
+        float nr, nid, nw, nK, be, gm, u, z, d2;
+        up2(R.nr[h], nr, u); up2(R.nid[h], nid, u); up2(R.nw[h], nw, u);
+        up2(R.nK[h], nK, u); up2(R.be[h], be, u); up2(R.gm[h], gm, u);
+        block_test(gv[C - 1], r, d, n, nr, nid, nw, nK, be, gm, z, d2);
+        if (!dead) { zmax = fmaxf(zmax, z); dmin = fminf(dmin, d2); }
+    }
+}
+
+// one warp's p: the CTA's prefix plus p
+struct BlockP {
+    int p, m;
+    bool ok;                     // pivots of the prefix and of p above tau
+    float invd, w, v0, v1;       // 1 / sqrt(d'_p), w_p, p's back-substituted coefficients
+    float A0, base, q2, thrN;    // |L^-T w|_1, syy - |w|^2, largest |a2|_1, (B + tie) / N
+};
+struct BlockRow { float r, d, n, l1; };      // R[p][x], dp, np, |L_P^-T R[.][x]|_1
+
+template <int DC>
+__device__ __forceinline__ BlockRow block_feature(const BlockP& Q, const float* Gp, const float2* dn, const float2* vv, int x) {
+    const float r = Gp[x * (x - 1) / 2 + Q.p] * Q.invd, c = r * Q.invd;
+    const float2 f = dn[x], v = vv[x];
+    float l1 = fabsf(c) + fabsf(fmaf(-c, Q.v0, v.x));
+    if (DC == 2) l1 += fabsf(fmaf(-c, Q.v1, v.y));
+    return BlockRow{r, fmaf(-r, r, f.x), fmaf(-r, Q.w, f.y), l1};
+}
+
+// the filter's constants of one row
+struct RowC { float nr, nid, nw, nK, be, gm; };
+__device__ __forceinline__ RowC block_row(const TileArgs& A, const BlockP& Q, const BlockRow& f) {
+    const bool piv = Q.ok && f.d > A.tau;
+    const float isd = __frsqrt_rn(f.d > 0.f ? f.d : 1.f), w1 = f.n * isd;
+    const float S0 = 1.02f * (Q.A0 + (1.f + f.l1) * fabsf(w1) * isd);
+    const float S1 = 1.02f * ((1.f + f.l1) * isd * 1.0001f + 1.f + Q.q2);
+    const float Kc = piv ? (Q.base - w1 * w1) - (A.e0 + S0 * fmaf(A.e2, S0, A.e1)) : -INFINITY;
+    return RowC{-f.r, -(isd * isd), -(w1 * isd), Q.thrN - Kc, S1 * fmaf(2.f * A.e2, S0, A.e1), A.e2 * S1 * S1};
+}
+
+struct BlockQueue { double B; int qn, taken; };
+
+// a column some lane may keep: the decisions row group by row group, into the warp's queue
+template <int DC>
+__device__ __noinline__ BlockQueue block_take(const TileArgs& A, const BlockPre* P, const BlockP Q, const float* Gp,
+                                              const float2* dn, const float2* vv, int rb, int x, unsigned* q, int qn,
+                                              double B) {
+    const int lane = threadIdx.x & 31;
+    int taken = 0;
+    const BlockRow f = block_feature<DC>(Q, Gp, dn, vv, x);
+    const int end = min(x, rb + 32 * kBRow);            // the rows of this sweep
+    for (int i = rb; i < end; i += 32) {
+        const int i1 = i + lane;
+        bool take = false;
+        if (i1 < x) {
+            const RowC c = block_row(A, Q, block_feature<DC>(Q, Gp, dn, vv, i1));
+            float z, d2;
+            block_test(Gp[x * (x - 1) / 2 + i1], f.r, f.d, f.n, c.nr, c.nid, c.nw, c.nK, c.be, c.gm, z, d2);
+            take = !((z < 0.f) & (d2 > A.tau));
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, take);
+        if (!mask) continue;
+        if (take)
+            q[qn + __popc(mask & ((1u << lane) - 1u))] = (unsigned)Q.p | ((unsigned)i1 << 10) | ((unsigned)x << 20);
+        qn += __popc(mask);
+        taken += __popc(mask);
+        __syncwarp();
+        if (qn >= 32) {
+            B = block_flush<DC>(A, P, q, qn, B);
+            qn = 0;
+        }
+    }
+    return BlockQueue{B, qn, taken};
+}
+
+// prefixes item0 .. of the colex order, M the most features right of one of them
+template <int DC, int W>
+__global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int slices, int item0, int M) {
+    extern __shared__ __align__(16) unsigned char block_smem[];
+    __shared__ BlockPre P;
+    __shared__ int s_item, s_p;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    float2* dn = reinterpret_cast<float2*>(block_smem);           // d', n' per feature
+    float2* vv = dn + M;                                          // its coefficients L^-T R[.][x]
+    float* Gp = reinterpret_cast<float*>(vv + M);                 // (x, y < x) at x (x - 1) / 2 + y
+    unsigned* q = reinterpret_cast<unsigned*>(Gp + ((size_t)M * (M - 1) / 2 + 36)) + w * kBQ;
+    const double inv_n = 1.0 / (double)A.N;
+    double B = fmin((double)INFINITY, okey_inv(*(volatile unsigned long long*)A.ub_key));
+    unsigned long long my_examined = 0, my_cand = 0;
+    while (true) {
+        __syncthreads();                                          // the last unit's buffers are free
+        if (tid == 0) {
+            s_item = item0 + atomicAdd(A.counter, 1);
+            s_p = s_item % slices;
+        }
+        __syncthreads();
+        const int item = s_item;
+        if (item >= A.n_items) break;
+        const int pre_rank = item / slices;
+        if (tid == 0) {
+            int pre[2] = {pre_rank, -1};
+            if (DC == 2) {
+                const int64_t m = top2_fast(pre_rank);
+                pre[1] = (int)m;
+                pre[0] = (int)(pre_rank - binom2(m));
+            }
+            P.last = pre[DC - 1];
+            P.pre[0] = pre[0]; P.pre[1] = pre[1];
+            const float d0 = A.diag[pre[0]];
+            bool ok = d0 > A.tau;
+            P.inv[0] = 1.f / sqrtf(d0 > 0.f ? d0 : 1.f);
+            P.w[0] = A.b[pre[0]] * P.inv[0];
+            P.pw2 = P.w[0] * P.w[0];
+            P.l10 = 0.f; P.inv[1] = 0.f; P.w[1] = 0.f; P.u[1] = 0.f;
+            if (DC == 2) {
+                P.l10 = A.G[(size_t)pre[1] * A.ldp + pre[0]] * P.inv[0];
+                const float d1 = A.diag[pre[1]] - P.l10 * P.l10;
+                ok = ok && d1 > A.tau;
+                P.inv[1] = 1.f / sqrtf(d1 > 0.f ? d1 : 1.f);
+                P.w[1] = (A.b[pre[1]] - P.l10 * P.w[0]) * P.inv[1];
+                P.pw2 += P.w[1] * P.w[1];
+                P.u[1] = P.w[1] * P.inv[1];
+            }
+            P.u[0] = (P.w[0] - P.l10 * P.u[1]) * P.inv[0];
+            P.ok = ok;
+        }
+        __syncthreads();
+        const int x0 = P.last + 1, m = A.n - x0;                  // local feature x is x0 + x
+        if (m < 3) continue;
+        // ---- features right of the prefix, then the reduced triangle ---------------------
+        for (int x = tid; x < m; x += W * 32) {
+            const float r0 = A.G[(size_t)P.pre[0] * A.ldp + x0 + x] * P.inv[0];
+            float r1 = 0.f, v1 = 0.f;
+            if (DC == 2) {
+                r1 = (A.G[(size_t)P.pre[1] * A.ldp + x0 + x] - r0 * P.l10) * P.inv[1];
+                v1 = r1 * P.inv[1];
+            }
+            vv[x] = make_float2(r0, r1);                          // R until the triangle is formed
+            dn[x] = make_float2(A.diag[x0 + x] - r0 * r0 - r1 * r1, A.b[x0 + x] - r0 * P.w[0] - r1 * P.w[1]);
+        }
+        __syncthreads();
+        for (int i = 1 + w; i < m; i += W) {
+            const float2 ri = vv[i];
+            float* row = Gp + i * (i - 1) / 2;
+            const float* src = A.G + (size_t)(x0 + i) * A.ldp + x0;
+            for (int y = lane; y < i; y += 32) {
+                const float2 ry = vv[y];
+                float v = fmaf(-ri.x, ry.x, src[y]);
+                if (DC == 2) v = fmaf(-ri.y, ry.y, v);
+                row[y] = v;
+            }
+        }
+        __syncthreads();
+        for (int x = tid; x < m; x += W * 32) {
+            const float2 r = vv[x];
+            const float v1 = DC == 2 ? r.y * P.inv[1] : 0.f;
+            vv[x] = make_float2((r.x - P.l10 * v1) * P.inv[0], v1);
+        }
+        __syncthreads();
+        // ---- sweep: this warp's p ---------------------------------------------------------
+        // (handed out largest triangle first: the warps finish together)
+        int qn = 0;
+        while (true) {
+            int p = 0;
+            if (lane == 0) p = atomicAdd(&s_p, slices);
+            p = __shfl_sync(0xffffffffu, p, 0);
+            if (p >= m - 2) break;
+            const unsigned long long next_key = *(volatile unsigned long long*)A.ub_key;     // in flight
+            BlockP Q;
+            {
+                const float2 f = dn[p], v = vv[p];
+                Q.p = p; Q.m = m;
+                Q.ok = P.ok && f.x > A.tau;
+                Q.invd = __frsqrt_rn(f.x > 0.f ? f.x : 1.f);
+                Q.w = f.y * Q.invd;
+                Q.v0 = v.x; Q.v1 = v.y;
+                const float cp = Q.w * Q.invd;
+                Q.A0 = fabsf(cp) + fabsf(fmaf(-cp, v.x, P.u[0]));
+                if (DC == 2) Q.A0 += fabsf(fmaf(-cp, v.y, P.u[1]));
+                Q.base = A.syy - (P.pw2 + Q.w * Q.w);
+                Q.thrN = __fmul_ru((float)((B + A.tie64) * inv_n), 1.0000002f);
+            }
+            const float invd = Q.invd, wp = Q.w, tau = A.tau;
+            float q2 = 0.f;
+            for (int x = p + 1 + lane; x < m; x += 32) q2 = fmaxf(q2, block_feature<DC>(Q, Gp, dn, vv, x).l1);
+            Q.q2 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(q2)));
+            // rows p + 1 .. m - 2, kBRow groups of 32 at a time: this lane's are i0 + 32 j
+            for (int rb = p + 1; rb < m - 1; rb += 32 * kBRow) {
+            const int i0 = rb + lane, groups = (m - 1 - rb + 31) >> 5;
+            RowsC R;
+#pragma unroll
+            for (int jp = 0; jp < kBRow / 2; ++jp) {
+                RowC c[2] = {{0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}};
+                if (2 * jp < groups) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int i1 = i0 + 32 * (2 * jp + h);
+                        if (i1 < m) c[h] = block_row(A, Q, block_feature<DC>(Q, Gp, dn, vv, i1));
+                    }
+                }
+                R.nr[jp] = pk2(c[0].nr, c[1].nr); R.nid[jp] = pk2(c[0].nid, c[1].nid); R.nw[jp] = pk2(c[0].nw, c[1].nw);
+                R.nK[jp] = pk2(c[0].nK, c[1].nK); R.be[jp] = pk2(c[0].be, c[1].be); R.gm[jp] = pk2(c[0].gm, c[1].gm);
+            }
+            // columns rb + 1 .. m - 1 in segments of equal row group count C, two at a time
+            int x = rb + 1;
+            const float* gx = Gp + x * (x - 1) / 2;               // row x of G'
+            auto segment = [&](auto cc) {
+                constexpr int C = decltype(cc)::value;
+                const int end = C == kBRow ? m : min(m, rb + 1 + 32 * C);           // x - rb <= 32 C
+                auto column = [&](const float* gr, int xc, float& zmax, float& dmin) {
+                    const float r = gr[p] * invd;
+                    const float2 f = dn[xc];
+                    block_col<C>(gr + i0, r, fmaf(-r, r, f.x), fmaf(-r, wp, f.y), i0 + 32 * (C - 1) >= xc, R, zmax, dmin);
+                };
+                auto take = [&](int xc) {
+                    const BlockQueue t = block_take<DC>(A, &P, Q, Gp, dn, vv, rb, xc, q, qn, B);
+                    B = t.B;
+                    qn = t.qn;
+                    my_cand += t.taken;
+                };
+                for (; x + 1 < end; x += 2) {
+                    float zmax = -INFINITY, dmin = INFINITY;
+                    column(gx, x, zmax, dmin);
+                    column(gx + x, x + 1, zmax, dmin);
+                    gx += 2 * x + 1;
+                    if (__any_sync(0xffffffffu, !(zmax < 0.f) || !(dmin > tau))) {
+                        take(x);
+                        take(x + 1);
+                    }
+                }
+                if (x < end) {
+                    float zmax = -INFINITY, dmin = INFINITY;
+                    column(gx, x, zmax, dmin);
+                    gx += x;
+                    if (__any_sync(0xffffffffu, !(zmax < 0.f) || !(dmin > tau))) take(x);
+                    ++x;
+                }
+            };
+            segment(std::integral_constant<int, 1>{});
+            segment(std::integral_constant<int, 2>{});
+            segment(std::integral_constant<int, 3>{});
+            segment(std::integral_constant<int, 4>{});
+            segment(std::integral_constant<int, 5>{});
+            segment(std::integral_constant<int, 6>{});
+            }
+            // rows p + 1 .. x - 1 of every column
+            if (lane == 0) my_examined += (unsigned long long)(m - 1 - p) * (unsigned long long)(m - 2 - p) / 2;
+            B = fmin(B, okey_inv(next_key));
+        }
+        if (qn > 0) {                                      // the queue's entries are relative to this prefix
+            B = block_flush<DC>(A, &P, q, qn, B);
+        }
+    }
+    my_examined = l0_warp_sum(my_examined);
+    if (lane == 0) {
+        atomicAdd(A.examined, my_examined);
+        atomicAdd(A.candidates, my_cand);
+    }
+}
+
+}  // namespace
+}  // namespace sg
