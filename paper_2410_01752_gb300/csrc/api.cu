@@ -267,6 +267,11 @@ sisso_status sisso_create(const double* X, const double* y, int N, int d, uint32
         (st = dalloc(c, c->sort_score, (size_t)c->sort_cap, "sort")) ||
         (st = dalloc(c, c->sort_id, (size_t)c->sort_cap, "sort_id")) ||
         (st = dalloc(c, c->sort_src, (size_t)c->sort_cap, "sort_src")) ||
+        (st = ctx_alloc(c, (void**)&c->rank_key, sizeof(unsigned long long) * (size_t)std::min<int64_t>(c->sort_cap, 32768), "rank keys")) ||
+        (st = ctx_alloc(c, (void**)&c->rank_id, sizeof(int64_t) * (size_t)std::min<int64_t>(c->sort_cap, 32768), "rank ids")) ||
+        (st = ctx_alloc(c, (void**)&c->dup_pairs, sizeof(int) * (size_t)c->sort_cap * kDupSlots, "dup_pairs")) ||
+        (st = ctx_alloc(c, (void**)&c->dup_np, sizeof(unsigned), "dup_np")) ||
+        (st = ctx_alloc(c, (void**)&c->tpart, sizeof(double) * (5 * 64 + 1), "target sums")) ||
         (st = dalloc(c, c->removed, (size_t)c->sort_cap, "removed")) || (st = dalloc(c, c->walk, 1, "walk")) ||
         (st = dalloc(c, c->S_dev, (size_t)c->n_cap, "S")) || (st = dalloc(c, c->S_sorted, (size_t)c->n_cap, "S_sorted")) ||
         (st = dalloc(c, c->Z, (size_t)c->n_cap * Nn, "Z")) || (st = dalloc(c, c->Zmean, (size_t)c->n_cap, "Zmean")) ||

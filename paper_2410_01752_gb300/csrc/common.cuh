@@ -55,6 +55,18 @@ struct Space {
 // Largest u with u*m - u(u-1)/2 <= r: the row of rank r in a triangle whose rows have
 // m, m-1, ..., 1 entries.
 __host__ __device__ inline int64_t tri_row(int64_t r, int64_t m) {
+#ifdef __CUDA_ARCH__
+    // the estimate in FP32 (the FP64 pipe is narrow), exact integer steps to the row
+    if (m < (1 << 30)) {
+        const int64_t b2 = 2 * m + 1, d2 = b2 * b2 - 8 * r;
+        int64_t v = (int64_t)(((float)b2 - sqrtf(d2 > 0 ? (float)d2 : 0.f)) * 0.5f);
+        if (v < 0) v = 0;
+        if (v > m) v = m;
+        while (v > 0 && v * m - v * (v - 1) / 2 > r) --v;
+        while ((v + 1) * m - (v + 1) * v / 2 <= r) ++v;
+        return v;
+    }
+#endif
     double b = 2.0 * (double)m + 1.0;
     double disc = b * b - 8.0 * (double)r;
     int64_t u = (int64_t)((b - sqrt(disc > 0 ? disc : 0.0)) * 0.5);
@@ -272,7 +284,7 @@ __device__ __forceinline__ double opref_val(const OpRef& r, const double* __rest
     if (r.b < 0) { const double v = op_unary<double>(r.op, x); mag = fabs(v); return v; }
     if (r.op == DIV && r.inv) {       // one rounding more than x / y (relative 1.1e-16); x / y where 1/y overflows
         const double q = r.inv[(size_t)r.b * N + s];
-        const double v = isfinite(q) ? x * q : x / V[(size_t)r.b * N + s];
+        const double v = (__double2hiint(q) & 0x7ff00000) != 0x7ff00000 ? x * q : x / V[(size_t)r.b * N + s];
         mag = fabs(v);
         return v;
     }
@@ -413,6 +425,11 @@ struct sisso_ctx {
     int64_t sort_cap = 0;
     double* sort_score = nullptr;      // sort buffers (power of two)
     int64_t* sort_id = nullptr;
+    unsigned long long* rank_key = nullptr;   // unsorted keys and ids of windows sorted by rank
+    int64_t* rank_id = nullptr;
+    int* dup_pairs = nullptr;          // (entry, slot) pairs to confirm; dup_np: their number
+    unsigned* dup_np = nullptr;
+    double* tpart = nullptr;           // target sums per block (many samples)
     int* sort_src = nullptr;           // index into the survivor arrays
     unsigned char* removed = nullptr;  // walk: visited flags (sort_cap)
     sg::WalkResult* walk = nullptr;    // device

@@ -32,6 +32,53 @@ __global__ void k_prepare_target(const double* __restrict__ t, int N, double* __
     prepare_target_block(t, N, tc64, tc32, st, red);
 }
 
+// the same for many samples in two launches of kTargetBlocks blocks: one block's share of the
+// SM's FP64 pipe took 220 us at 65536 samples.  Partial sums are added in block order.
+constexpr int kTargetBlocks = 64, kTargetMany = 4096;
+__global__ void __launch_bounds__(256) k_target_sum(const double* __restrict__ t, int N, double* __restrict__ part) {
+    __shared__ double red[32];
+    double s = 0.0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) s += t[i];
+    s = block_sum(s, red);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<unsigned*>(part + 5 * kTargetBlocks) = 0u;
+}
+__global__ void __launch_bounds__(256) k_target_stats(const double* __restrict__ t, int N, double* __restrict__ part,
+                                                      double* __restrict__ tc64, float* __restrict__ tc32, TargetStats* st) {
+    __shared__ double red[32];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31;
+    auto total = [&](const double* p) { return warp_sum(__ldcg(p + lane) + __ldcg(p + lane + 32)); };
+    const double mean = total(part) / N;
+    double ss = 0.0, tsum = 0.0, s32 = 0.0, ss32 = 0.0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        const double c = t[i] - mean;
+        const float f = (float)c;
+        tc64[i] = c;
+        tc32[i] = f;
+        ss += c * c;
+        tsum += c;
+        s32 += (double)f;
+        ss32 += (double)f * (double)f;
+    }
+    ss = block_sum(ss, red);
+    tsum = block_sum(tsum, red);
+    s32 = block_sum(s32, red);
+    ss32 = block_sum(ss32, red);
+    if (threadIdx.x == 0) {
+        double* p = part + kTargetBlocks + blockIdx.x;
+        p[0] = ss; p[kTargetBlocks] = tsum; p[2 * kTargetBlocks] = s32; p[3 * kTargetBlocks] = ss32;
+        __threadfence();
+        last = atomicAdd(reinterpret_cast<unsigned*>(part + 5 * kTargetBlocks), 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    const double* p = part + kTargetBlocks;
+    ss = total(p); tsum = total(p + kTargetBlocks); s32 = total(p + 2 * kTargetBlocks); ss32 = total(p + 3 * kTargetBlocks);
+    if (lane == 0) finish_target(st, N, mean, ss, tsum, s32, ss32);
+}
+
 // FP64 validity of ids [lo, hi) (one level), one warp per id: the value rules (finite,
 // |v| <= 1e12, not identically zero, std > 1e-6 max|v|) and the operands' validity
 // (lower levels, already computed)
@@ -586,8 +633,8 @@ k_rescore_cta(const Space* __restrict__ sp, int N, const double* __restrict__ tc
               const double* __restrict__ Vinv, double* score, double* mean_out, double* sd_out, int* valid_out,
               double* __restrict__ probe, double* __restrict__ zc) {
     constexpr int W = kRescoreThreads / 32;
-    __shared__ double red[W][5];
-    __shared__ int red_bad[W];
+    __shared__ double red[W][3];
+    __shared__ unsigned long long redb[W][2];
     const int w = blockIdx.x, t = threadIdx.x, lane = t & 31, wp = t >> 5;
     const int64_t id = ids[w];
     int level, op; int64_t a, b;
@@ -605,20 +652,19 @@ k_rescore_cta(const Space* __restrict__ sp, int N, const double* __restrict__ tc
     double* z = zc ? zc + (size_t)w * N : nullptr;
     double mag0;
     const double v0 = opref_val(ref, V, N, 0, mag0);
-    double s1 = 0.0, s2 = 0.0, sc = 0.0, mx = 0.0, mo = 0.0;
-    int bad = 0;
-    // one comparison per sample catches non-finite values and the cap; the operands'
+    double s1 = 0.0, s2 = 0.0, sc = 0.0;
+    unsigned long long bx = 0, bo = 0;
+    // the largest |v| as an integer catches non-finite values and the cap; the operands'
     // magnitude (the cancellation rule) only for a top-level + or -
     const bool need_mag = id >= Pbot && (op == ADD || op == SUB);
     auto body = [&](int i, double v, double mag, bool with_mag) {
-        const double av = fabs(v);
-        if (!(av <= kValueCap)) bad = 1;
+        const unsigned long long av = abs_bits(v);
         const double u = v - v0;
         s1 += u;
         s2 = fma(u, u, s2);
         sc = fma(u, tc[i], sc);
-        mx = fmax(mx, av);
-        if (with_mag) mo = fmax(mo, mag);
+        bx = av > bx ? av : bx;
+        if (with_mag) { const unsigned long long am = abs_bits(mag); bo = am > bo ? am : bo; }
         if (z) z[i] = v;
     };
     if (need_mag)
@@ -633,15 +679,18 @@ k_rescore_cta(const Space* __restrict__ sp, int N, const double* __restrict__ tc
             const double v = opref_val(ref, V, N, i, mag);
             body(i, v, 0.0, false);
         }
-    bad = warp_or(bad);
-    s1 = warp_sum(s1); s2 = warp_sum(s2); sc = warp_sum(sc); mx = warp_max(mx); mo = warp_max(mo);
-    if (lane == 0) { red[wp][0] = s1; red[wp][1] = s2; red[wp][2] = sc; red[wp][3] = mx; red[wp][4] = mo; red_bad[wp] = bad; }
+    s1 = warp_sum(s1); s2 = warp_sum(s2); sc = warp_sum(sc);
+    bx = warp_max_bits(bx);
+    bo = warp_max_bits(bo);
+    if (lane == 0) { red[wp][0] = s1; red[wp][1] = s2; red[wp][2] = sc; redb[wp][0] = bx; redb[wp][1] = bo; }
     __syncthreads();
-    s1 = red[0][0]; s2 = red[0][1]; sc = red[0][2]; mx = red[0][3]; mo = red[0][4]; bad = red_bad[0];
+    s1 = red[0][0]; s2 = red[0][1]; sc = red[0][2]; bx = redb[0][0]; bo = redb[0][1];
     for (int q = 1; q < W; ++q) {
         s1 += red[q][0]; s2 += red[q][1]; sc += red[q][2];
-        mx = fmax(mx, red[q][3]); mo = fmax(mo, red[q][4]); bad |= red_bad[q];
+        bx = max(bx, redb[q][0]); bo = max(bo, redb[q][1]);
     }
+    const int bad = bx > abs_bits(kValueCap);
+    const double mx = __longlong_as_double((long long)bx), mo = __longlong_as_double((long long)bo);
     const bool cancelled = need_mag && mx <= kCancelRel * mo;
     const double mean = v0 + s1 / N;
     const double var = s2 / N - (s1 / N) * (s1 / N);
@@ -670,8 +719,9 @@ k_rescore_cta(const Space* __restrict__ sp, int N, const double* __restrict__ tc
 __global__ void k_sort_keys(const int64_t* __restrict__ ids, const double* __restrict__ score,
                             const int* __restrict__ valid, int n, const int64_t* __restrict__ S_sorted,
                             int nS, int n_pad, const unsigned* __restrict__ unit_mask, double* sk, int64_t* sid,
-                            int* ssrc) {
+                            int* ssrc, unsigned* np) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *np = 0u;
     if (i >= n_pad) return;
     if (i >= n) { sk[i] = -2.0; sid[i] = INT64_MAX; ssrc[i] = -1; return; }
     const int64_t id = ids[i];
@@ -704,35 +754,63 @@ __global__ void k_bitonic(double* sk, int64_t* sid, int* ssrc, int n, int k, int
     }
 }
 
-// the same network in one CTA's shared memory (windows of up to kSortBlock entries):
-// one launch instead of one per stage
-constexpr int kSortBlock = 8192;
-constexpr size_t kSortSmem = (size_t)kSortBlock * (sizeof(double) + sizeof(int64_t) + sizeof(int));
+// Windows of up to kRankMax entries: an entry's place is the number of entries before it (keys
+// are distinct ids), counted by comparing it with every other on the integer pipe.  n^2 / 32 warp
+// comparisons spread over every SM: 4 us at 4096 entries and 14 us at 8192, where the bitonic
+// network in one CTA's shared memory took 209 and 428 us.
+constexpr int kRankMax = 32768;
+__device__ __forceinline__ unsigned long long rank_key_of(double s) {        // ascending in s; negative scores equal
+    return s < 0.0 ? 0ull : (unsigned long long)__double_as_longlong(s) | 0x8000000000000000ull;
+}
 
-__global__ void __launch_bounds__(1024) k_sort_block(double* sk, int64_t* sid, int* ssrc, int n) {
-    extern __shared__ __align__(16) unsigned char ssm[];
-    double* k_ = reinterpret_cast<double*>(ssm);
-    int64_t* id_ = reinterpret_cast<int64_t*>(k_ + n);
-    int* src_ = reinterpret_cast<int*>(id_ + n);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) { k_[i] = sk[i]; id_[i] = sid[i]; src_[i] = ssrc[i]; }
-    __syncthreads();
-    for (int k = 2; k <= n; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                const int l = i ^ j;
-                if (l <= i) continue;
-                const bool up = (i & k) == 0;
-                const double si = k_[i], sl = k_[l];
-                const int64_t ii = id_[i], il = id_[l];
-                if (up ? before(sl, il, si, ii) : before(si, ii, sl, il)) {
-                    k_[i] = sl; k_[l] = si;
-                    id_[i] = il; id_[l] = ii;
-                    const int t = src_[i]; src_[i] = src_[l]; src_[l] = t;
-                }
-            }
-            __syncthreads();
+// keys of the window's entries: valid survivors not in S (and, with units, dimensionally
+// consistent) by their FP64 score, others below every score
+__global__ void k_rank_keys(const int64_t* __restrict__ ids, const double* __restrict__ score,
+                            const int* __restrict__ valid, int n, const int64_t* __restrict__ S_sorted, int nS,
+                            const unsigned* __restrict__ unit_mask, unsigned long long* __restrict__ key,
+                            int64_t* __restrict__ kid, unsigned* __restrict__ np) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *np = 0u;
+    if (i >= n) return;
+    const int64_t id = ids[i];
+    int lo = 0, hi = nS;            // binary search in S (ascending)
+    while (lo < hi) { const int m = (lo + hi) >> 1; if (S_sorted[m] < id) lo = m + 1; else hi = m; }
+    const bool inS = lo < nS && S_sorted[lo] == id;
+    const bool units = !unit_mask || ((unit_mask[id >> 5] >> (id & 31)) & 1u);
+    key[i] = valid[i] && !inS && units ? rank_key_of(score[i]) : 0ull;
+    kid[i] = id;
+}
+
+__global__ void __launch_bounds__(256) k_rank_sort(const unsigned long long* __restrict__ key,
+                                                   const int64_t* __restrict__ kid, int n, double* __restrict__ sk,
+                                                   int64_t* __restrict__ sid, int* __restrict__ ssrc) {
+    __shared__ ulonglong2 sh[8][32];
+    __shared__ int rank[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
+    const unsigned long long ki = i < n ? key[i] : 0ull;
+    const int64_t di = i < n ? kid[i] : 0;
+    int r = 0;
+    for (int j0 = w * 32; j0 < n; j0 += 256) {
+        const int j = j0 + lane;
+        // padding sorts after everything
+        sh[w][lane] = j < n ? make_ulonglong2(key[j], (unsigned long long)kid[j]) : make_ulonglong2(0ull, ~0ull >> 1);
+        __syncwarp();
+#pragma unroll 8
+        for (int q = 0; q < 32; ++q) {
+            const ulonglong2 o = sh[w][q];
+            r += o.x > ki || (o.x == ki && (int64_t)o.y < di);
         }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) { sk[i] = k_[i]; sid[i] = id_[i]; ssrc[i] = src_[i]; }
+        __syncwarp();
+    }
+    rank[w][lane] = r;
+    __syncthreads();
+    if (w == 0 && i < n) {
+        for (int q = 1; q < 8; ++q) r += rank[q][lane];
+        sk[r] = ki ? __longlong_as_double((long long)(ki & 0x7fffffffffffffffull)) : -1.0;
+        sid[r] = di;
+        ssrc[r] = i;
+    }
 }
 
 // ---------------------------------------------------------------------------------
@@ -766,8 +844,8 @@ __device__ __forceinline__ bool probes_match(const double* a, const double* b) {
 __global__ void k_dup_find(const double* __restrict__ sk, const int* __restrict__ ssrc,
                            const int64_t* __restrict__ sid, int n_sorted,
                            const double* __restrict__ sv_score, const double* __restrict__ sv_sd,
-                           const double* __restrict__ probe, int s_off, int nS, int* __restrict__ dup_list,
-                           int* __restrict__ dup_cnt) {
+                           const double* __restrict__ probe, int s_off, int nS, int n_conf, int* __restrict__ dup_list,
+                           int* __restrict__ dup_cnt, int* __restrict__ pairs, unsigned* __restrict__ n_pairs) {
     __shared__ int64_t s_key[8][kDupSlots];
     __shared__ int s_val[8][kDupSlots];
     const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
@@ -776,19 +854,23 @@ __global__ void k_dup_find(const double* __restrict__ sk, const int* __restrict_
     const double s = sk[i];
     if (s < 0.0) { if (lane == 0) dup_cnt[i] = 0; return; }
     const int src = ssrc[i];
-    double pc[kProbes];
-#pragma unroll
-    for (int r = 0; r < kProbes; ++r) pc[r] = probe[(size_t)src * kProbes + r];
+    // probe comparisons only where a lane's score is close (their FP64 work is what bounds the
+    // kernel); the entry's own probes are read then
+    auto match = [&](bool close, int m) {
+        if (!__any_sync(0xffffffffu, close)) return false;
+        return close && probes_match(probe + (size_t)src * kProbes, probe + (size_t)m * kProbes);
+    };
     int64_t* key = s_key[wb];
     int* val = s_val[wb];
     // keep the kDupSlots partners with the smallest keys: S members first (key -1), then
     // window entries by id (a cluster's earliest-visited member is its smallest id)
     int n = 0, total = 0;
     int64_t last = 0;                                    // key[n - 1] once the list is full
-    auto offer = [&](bool match, int m, int64_t k) {
-        const unsigned all = __ballot_sync(0xffffffffu, match);
+    auto offer = [&](bool hit, int m, int64_t k) {
+        const unsigned all = __ballot_sync(0xffffffffu, hit);
+        if (!all) return;
         total += __popc(all);
-        unsigned b = __ballot_sync(0xffffffffu, match && (n < kDupSlots || k < last));
+        unsigned b = __ballot_sync(0xffffffffu, hit && (n < kDupSlots || k < last));
         while (b) {
             const int l = __ffs(b) - 1;
             b &= b - 1;
@@ -809,45 +891,47 @@ __global__ void k_dup_find(const double* __restrict__ sk, const int* __restrict_
     };
     for (int q0 = 0; q0 < nS; q0 += 32) {
         const int q = q0 + lane, m = s_off + q;
-        const bool c = q < nS && sv_sd[m] > 0.0 && fabs(sv_score[m] - s) <= kDupScore &&
-                       probes_match(pc, probe + (size_t)m * kProbes);
-        offer(c, m, -1);
+        offer(match(q < nS && sv_sd[m] > 0.0 && fabs(sv_score[m] - s) <= kDupScore, m), m, -1);
     }
     for (int b0 = 0;; b0 += 32) {                        // higher scores (sorted descending)
         const int j = i - 1 - b0 - lane;
         const bool in = j >= 0 && sk[j] - s <= kDupScore;
         const int mj = in ? ssrc[j] : 0;
-        offer(in && probes_match(pc, probe + (size_t)mj * kProbes), mj, in ? sid[j] : 0);
+        offer(match(in, mj), mj, in ? sid[j] : 0);
         if (__ballot_sync(0xffffffffu, in) != 0xffffffffu) break;
     }
     for (int b0 = 0;; b0 += 32) {                        // lower scores
         const int j = i + 1 + b0 + lane;
         const bool in = j < n_sorted && sk[j] >= 0.0 && s - sk[j] <= kDupScore;
         const int mj = in ? ssrc[j] : 0;
-        offer(in && probes_match(pc, probe + (size_t)mj * kProbes), mj, in ? sid[j] : 0);
+        offer(match(in, mj), mj, in ? sid[j] : 0);
         if (__ballot_sync(0xffffffffu, in) != 0xffffffffu) break;
     }
     if (lane < n) dup_list[(size_t)i * kDupSlots + lane] = val[lane];
     // overflow: n partners kept, more exist (the walk falls back to a full check)
     if (lane == 0) dup_cnt[i] = total > kDupSlots ? -n - 1 : n;
+    const int nc = min(n, n_conf);                       // partners confirmed ahead of the walk
+    if (nc > 0) {
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(n_pairs, (unsigned)nc);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (lane < nc) pairs[at + lane] = i * kDupSlots + lane;
+    }
 }
 
 // one warp per sorted entry: every listed partner compared on all samples
 __global__ void k_dup_confirm(const Space* __restrict__ sp, const double* __restrict__ Xc, int N,
-                              const int* __restrict__ ssrc, const int64_t* __restrict__ sid, int n_sorted,
+                              const int* __restrict__ ssrc, const int64_t* __restrict__ sid,
                               const int64_t* __restrict__ sv_ids, const double* __restrict__ sv_mean,
                               const double* __restrict__ sv_sd, const double* __restrict__ zc,
                               const double* __restrict__ V, const int* __restrict__ dup_list,
-                              const int* __restrict__ dup_cnt, unsigned char* __restrict__ dup_ok,
-                              const double* __restrict__ Vinv) {
+                              const int* __restrict__ pairs, const unsigned* __restrict__ n_pairs,
+                              unsigned char* __restrict__ dup_ok, const double* __restrict__ Vinv) {
     const int lane = threadIdx.x & 31;
-    // one warp per (sorted entry, listed partner)
-    for (int64_t wi = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; wi < (int64_t)n_sorted * kDupSlots;
-         wi += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const int i = (int)(wi / kDupSlots), q = (int)(wi % kDupSlots);
-        const int raw = dup_cnt[i];
-        const int cnt = min(raw < 0 ? -raw - 1 : raw, n_confirm(N));
-        if (q >= cnt) continue;
+    const unsigned np = *n_pairs;
+    // one warp per listed (sorted entry, partner slot)
+    for (unsigned wi = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; wi < np; wi += (gridDim.x * blockDim.x) >> 5) {
+        const int i = pairs[wi] / kDupSlots, q = pairs[wi] % kDupSlots;
         const int src = ssrc[i];
         Prog pc;
         OpRef rc{};
@@ -921,7 +1005,7 @@ __global__ void k_dup_confirm(const Space* __restrict__ sp, const double* __rest
 // ---------------------------------------------------------------------------------
 constexpr int kWalkThreads = 1024;
 constexpr int kHeapCap = 2048;          // tie-window entries held in the shared-memory heap
-constexpr int kWalkStage = 4096;        // sorted entries staged in shared memory
+constexpr int kWalkStage = 6144;        // sorted entries staged in shared memory
 constexpr size_t kWalkSmem = (size_t)kWalkStage * (sizeof(double) + sizeof(int64_t) + 2 * sizeof(int) + 2);
 
 __global__ void __launch_bounds__(kWalkThreads)
@@ -1339,8 +1423,14 @@ sisso_status fill_opcache(sisso_ctx* c) {
 }
 
 sisso_status prepare_target(sisso_ctx* c, const double* target_dev) {
-    k_prepare_target<<<1, 1024, 0, c->stream>>>(target_dev, c->N, c->tc64, c->tc32, c->tstats);
-    c->stats.launches++;
+    if (c->N > kTargetMany) {
+        k_target_sum<<<kTargetBlocks, 256, 0, c->stream>>>(target_dev, c->N, c->tpart);
+        k_target_stats<<<kTargetBlocks, 256, 0, c->stream>>>(target_dev, c->N, c->tpart, c->tc64, c->tc32, c->tstats);
+        c->stats.launches += 2;
+    } else {
+        k_prepare_target<<<1, c->N > 128 ? 256 : 128, 0, c->stream>>>(target_dev, c->N, c->tc64, c->tc32, c->tstats);
+        c->stats.launches++;
+    }
     return check_cuda(c, cudaGetLastError(), "prepare_target");
 }
 
@@ -1649,17 +1739,21 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
                                                                      c->surv_ids, nr, c->subvalid, c->opval64,
                                                                      c->surv_score, c->surv_mean, c->surv_sd,
                                                                      c->surv_valid, c->surv_probe, zc, c->opinv64);
+        const bool ranked = ns > 0 && ns <= kRankMax;
         int n_pad = 1;
         while (n_pad < std::max(ns, 1)) n_pad <<= 1;
+        if (ranked) n_pad = ns;
+        if (ranked)
+            k_rank_keys<<<(n_pad + 255) / 256, 256, 0, c->stream>>>(c->surv_ids, c->surv_score, c->surv_valid, ns, c->S_sorted,
+                                                                    n_prev, c->unit_mask, c->rank_key, c->rank_id, c->dup_np);
+        else
         k_sort_keys<<<(n_pad + 255) / 256, 256, 0, c->stream>>>(c->surv_ids, c->surv_score, c->surv_valid, ns,
                                                                  c->S_sorted, n_prev, n_pad, c->unit_mask,
-                                                                 c->sort_score, c->sort_id, c->sort_src);
+                                                                 c->sort_score, c->sort_id, c->sort_src, c->dup_np);
         c->stats.launches += 2;
         cudaEventRecord(q[2], c->stream);
-        if (n_pad <= kSortBlock) {
-            const size_t sm = (size_t)n_pad * (sizeof(double) + sizeof(int64_t) + sizeof(int));
-            cudaFuncSetAttribute(k_sort_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSortSmem);
-            k_sort_block<<<1, 1024, sm, c->stream>>>(c->sort_score, c->sort_id, c->sort_src, n_pad);
+        if (ranked) {
+            k_rank_sort<<<(ns + 31) / 32, 256, 0, c->stream>>>(c->rank_key, c->rank_id, ns, c->sort_score, c->sort_id, c->sort_src);
             c->stats.launches++;
         } else {
             for (int kk = 2; kk <= n_pad; kk <<= 1)
@@ -1673,11 +1767,11 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
         cudaMemsetAsync(c->removed, 0, (size_t)n_pad, c->stream);
         cudaMemsetAsync(c->accepted, 0, (size_t)ns, c->stream);
         k_dup_find<<<(int)(((int64_t)n_pad * 32 + 255) / 256), 256, 0, c->stream>>>(c->sort_score, c->sort_src, c->sort_id, n_pad, c->surv_score,
-                                                               c->surv_sd, c->surv_probe, ns, n_prev, c->dup_list,
-                                                               c->dup_cnt);
-        k_dup_confirm<<<(int)std::max<int64_t>(1, std::min<int64_t>((int64_t)c->sms * 32, ((int64_t)n_pad * kDupSlots * 32 + 255) / 256)), 256, 0, c->stream>>>(
-            c->space_dev, c->Xc64, c->N, c->sort_src, c->sort_id, n_pad, c->surv_ids, c->surv_mean, c->surv_sd, zc,
-            c->opval64, c->dup_list, c->dup_cnt, c->dup_ok, c->opinv64);
+                                                               c->surv_sd, c->surv_probe, ns, n_prev, n_confirm(c->N), c->dup_list,
+                                                               c->dup_cnt, c->dup_pairs, c->dup_np);
+        k_dup_confirm<<<(int)std::max<int64_t>(1, std::min<int64_t>((int64_t)c->sms * 8, ((int64_t)n_pad + 7) / 8)), 256, 0, c->stream>>>(
+            c->space_dev, c->Xc64, c->N, c->sort_src, c->sort_id, c->surv_ids, c->surv_mean, c->surv_sd, zc,
+            c->opval64, c->dup_list, c->dup_pairs, c->dup_np, c->dup_ok, c->opinv64);
         cudaFuncSetAttribute(k_walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkSmem);
         const size_t wsm = n_pad <= kWalkStage && ns <= kWalkStage ? kWalkSmem : 0;
         k_walk<<<1, kWalkThreads, wsm, c->stream>>>(c->space_dev, c->Xc64, c->N, c->sort_score, c->sort_id, c->sort_src,

@@ -26,15 +26,22 @@ template <typename T> __device__ __forceinline__ T warp_max(T v) {
 }
 __device__ __forceinline__ int warp_or(int v) { return __any_sync(0xffffffffu, v); }
 
-// sum over a block of blockDim.x threads (multiple of 32); result valid in all threads
+// sum over a block of blockDim.x threads (multiple of 32); result valid in all threads.  The
+// warps' sums are combined by one warp: on this part an FP64 warp instruction occupies the SM's
+// FP64 pipe for about 18 cycles, so a loop over them in every warp took longer than the sums
+// (1024 threads: five sums 60 us)
 template <typename T> __device__ T block_sum(T v, T* red) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     v = warp_sum(v);
     __syncthreads();
     if (lane == 0) red[w] = v;
     __syncthreads();
-    T r = 0;
-    for (int i = 0; i < nw; ++i) r += red[i];
+    if (w == 0) {
+        v = warp_sum(lane < nw ? red[lane] : T(0));
+        if (lane == 0) red[0] = v;
+    }
+    __syncthreads();
+    const T r = red[0];
     __syncthreads();
     return r;
 }
@@ -44,10 +51,28 @@ template <typename T> __device__ T block_max(T v, T* red) {
     __syncthreads();
     if (lane == 0) red[w] = v;
     __syncthreads();
-    T r = red[0];
-    for (int i = 1; i < nw; ++i) r = max(r, red[i]);
+    if (w == 0) {
+        v = warp_max(red[lane < nw ? lane : 0]);
+        if (lane == 0) red[0] = v;
+    }
+    __syncthreads();
+    const T r = red[0];
     __syncthreads();
     return r;
+}
+
+// |x| as an integer: ordered as the values are, infinities and NaN above every finite value (a
+// maximum or a cap test on it keeps off the FP64 pipe)
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+    return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long t = __shfl_xor_sync(0xffffffffu, v, o);
+        v = t > v ? t : v;
+    }
+    return v;
 }
 
 // score from shifted sums (v' = v - v0): Pearson |rho| with population moments, or -1
@@ -228,6 +253,22 @@ __device__ __forceinline__ void stage_store(PairSmem<T>& S, int b, const T (&v)[
 }
 
 
+// the target's moments from its sums: s of the values' FP64 squares, FP64 values, FP32 copies
+// and their squares (all centred)
+__device__ __forceinline__ void finish_target(TargetStats* st, int N, double mean, double ss, double tsum, double s32,
+                                              double ss32) {
+    st->mean = mean;
+    st->sd = sqrt(ss / N);
+    st->tsum = tsum;
+    st->sum32 = s32;
+    st->srr32 = ss32 - s32 * s32 / N;
+    st->sd32 = (float)sqrt(st->srr32 / N);
+    int e;
+    frexp(st->sd * sqrt((double)N), &e);
+    st->rscale = (float)ldexp(1.0, -e);
+    st->inv_sdr = (float)(1.0 / ldexp(st->sd, -e));
+}
+
 // moments of a screening target t (one block of any multiple of 32 threads): the centred
 // copies in FP64 and FP32 and their sums
 __device__ void prepare_target_block(const double* t, int N, double* tc64, float* tc32, TargetStats* st,
@@ -235,34 +276,22 @@ __device__ void prepare_target_block(const double* t, int N, double* tc64, float
     double s = 0.0;
     for (int i = threadIdx.x; i < N; i += blockDim.x) s += t[i];
     const double mean = block_sum(s, red) / N;
-    double ss = 0.0, s32 = 0.0, ss32 = 0.0;
+    double ss = 0.0, tsum = 0.0, s32 = 0.0, ss32 = 0.0;
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
         const double c = t[i] - mean;
         const float f = (float)c;
         tc64[i] = c;
         tc32[i] = f;
         ss += c * c;
+        tsum += c;
         s32 += (double)f;
         ss32 += (double)f * (double)f;
     }
     ss = block_sum(ss, red);
-    double tsum = 0.0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tsum += tc64[i];
     tsum = block_sum(tsum, red);
     s32 = block_sum(s32, red);
     ss32 = block_sum(ss32, red);
-    if (threadIdx.x == 0) {
-        st->mean = mean;
-        st->sd = sqrt(ss / N);
-        st->tsum = tsum;
-        st->sum32 = s32;
-        st->srr32 = ss32 - s32 * s32 / N;
-        st->sd32 = (float)sqrt(st->srr32 / N);
-        int e;
-        frexp(st->sd * sqrt((double)N), &e);
-        st->rscale = (float)ldexp(1.0, -e);
-        st->inv_sdr = (float)(1.0 / ldexp(st->sd, -e));
-    }
+    if (threadIdx.x == 0) finish_target(st, N, mean, ss, tsum, s32, ss32);
 }
 
 // one id below the top level scored from the sample-major cache (row stride P)
@@ -357,9 +386,8 @@ __device__ __forceinline__ void rescore_one(const Space* sp, const double* Xc, i
     Prog p;
     int level, op; int64_t a, b;
     const int64_t Pbot = sp->phi[sp->rung - 1];
-    OpRef ref{};
-    bool built = decode(*sp, id, level, op, a, b) && (V ? make_opref(*sp, id, ref) : build_prog(*sp, id, p));
-    ref.inv = Vinv;
+    bool built = decode(*sp, id, level, op, a, b) && (V || build_prog(*sp, id, p));
+    OpRef ref = id < Pbot ? OpRef{id, -1, -1, Vinv} : OpRef{a, b, op, Vinv};
     if (built && id < Pbot && !subvalid[id]) built = false;                                  // exact, recursive
     if (built && id >= Pbot && (!subvalid[a] || (b >= 0 && !subvalid[b]))) built = false;   // invalid operand
     if (!built) {
@@ -375,28 +403,29 @@ __device__ __forceinline__ void rescore_one(const Space* sp, const double* Xc, i
     // inside the 1e-9 tie window of the walk)
     double mag0;
     const double v0 = value(0, mag0);
-    double s1 = 0.0, s2 = 0.0, sc = 0.0, mx = 0.0, mo = 0.0;
-    int bad = 0;
+    double s1 = 0.0, s2 = 0.0, sc = 0.0;
+    unsigned long long bx = 0, bo = 0;       // largest |v| and operand magnitude
+    // identically zero: a top-level + or - whose operands cancel (lower ids: in subvalid)
+    const bool top_addsub = id >= Pbot && (op == ADD || op == SUB);
     for (int i = lane; i < N; i += 32) {
         double mag;
         const double v = value(i, mag);
-        if (!isfinite(v) || fabs(v) > kValueCap) bad = 1;
         const double u = v - v0;
         s1 += u;
         s2 += u * u;
         sc += u * tc[i];
-        mx = fmax(mx, fabs(v));
-        mo = fmax(mo, mag);
+        const unsigned long long av = abs_bits(v);
+        bx = av > bx ? av : bx;
+        if (top_addsub) { const unsigned long long am = abs_bits(mag); bo = am > bo ? am : bo; }
         if (z) z[i] = v;
     }
-    bad = warp_or(bad);
     s1 = warp_sum(s1);
     s2 = warp_sum(s2);
     sc = warp_sum(sc);
-    mx = warp_max(mx);
-    mo = warp_max(mo);
-    // identically zero: a top-level + or - whose operands cancel (lower ids: in subvalid)
-    const bool top_addsub = id >= Pbot && (op == ADD || op == SUB);
+    bx = warp_max_bits(bx);
+    if (top_addsub) bo = warp_max_bits(bo);
+    const int bad = bx > abs_bits(kValueCap);          // above the cap, infinite or NaN
+    const double mx = __longlong_as_double((long long)bx), mo = __longlong_as_double((long long)bo);
     const bool cancelled = top_addsub && mx <= kCancelRel * mo;
     const double mean = v0 + s1 / N;
     const double var = s2 / N - (s1 / N) * (s1 / N);
