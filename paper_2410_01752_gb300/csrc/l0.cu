@@ -170,7 +170,7 @@ __global__ void k_refit(const double* __restrict__ G, const double* __restrict__
 
 // one block: among refit entries within the tie window of the minimum, the smallest
 // ascending global-id tuple (block-strided scan, then a pairwise reduction)
-__global__ void k_winner(const uint64_t* __restrict__ band, const double* __restrict__ rss,
+__global__ void __launch_bounds__(1024) k_winner(const uint64_t* __restrict__ band, const double* __restrict__ rss,
                          const unsigned* __restrict__ count, int64_t cap, const unsigned long long* min_key,
                          double tie, const int64_t* __restrict__ gid, int D, Winner* W) {
     __shared__ int64_t best_e[1024];
@@ -216,7 +216,7 @@ __global__ void k_winner(const uint64_t* __restrict__ band, const double* __rest
 }
 
 // winner's coefficients (original units), residual r* = y~ - Z_E gamma, RMSE, R^2
-__global__ void k_model(const double* __restrict__ G, const double* __restrict__ b, int ld, double syy, int N,
+__global__ void __launch_bounds__(1024) k_model(const double* __restrict__ G, const double* __restrict__ b, int ld, double syy, int N,
                         int D, const double* __restrict__ Z, const double* __restrict__ Zmean,
                         const double* __restrict__ Zsd, const double* __restrict__ yc, double ybar,
                         const int64_t* __restrict__ gid, Winner* W, double* __restrict__ resid) {
@@ -358,7 +358,7 @@ __global__ void k_refit_z(const double* __restrict__ Z, const double* __restrict
 }
 
 // the winner's model from Z rows (one block): coefficients in original units, residual
-__global__ void k_model_z(const double* __restrict__ Z, const double* __restrict__ Zmean,
+__global__ void __launch_bounds__(1024) k_model_z(const double* __restrict__ Z, const double* __restrict__ Zmean,
                           const double* __restrict__ Zsd, const double* __restrict__ yc, double ybar, int N, double syy,
                           int D, const int64_t* __restrict__ gid, Winner* W, double* __restrict__ resid) {
     __shared__ double g[kMaxDim][kMaxDim], bv[kMaxDim], gamma[kMaxDim];
@@ -859,7 +859,8 @@ sisso_status winner_model_z(sisso_ctx* c, int n, int D, Winner& w) {
                                          c->resid);
     c->stats.launches++;
     cudaMemcpyAsync(c->win_h, c->win, sizeof(Winner), cudaMemcpyDeviceToHost, c->stream);
-    sisso_status st = check_cuda(c, cudaStreamSynchronize(c->stream), "winner_model_z");
+    sisso_status st = check_cuda(c, cudaGetLastError(), "winner_model_z");
+    if (!st) st = check_cuda(c, cudaStreamSynchronize(c->stream), "winner_model_z");
     if (st) return st;
     w = *c->win_h;
     return SISSO_OK;
@@ -871,7 +872,8 @@ sisso_status winner_model(sisso_ctx* c, int n, int D, Winner& w) {
                                        c->ybar, c->S_dev, c->win, c->resid);
     c->stats.launches++;
     cudaMemcpyAsync(c->win_h, c->win, sizeof(Winner), cudaMemcpyDeviceToHost, c->stream);
-    sisso_status st = check_cuda(c, cudaStreamSynchronize(c->stream), "winner_model");
+    sisso_status st = check_cuda(c, cudaGetLastError(), "winner_model");
+    if (!st) st = check_cuda(c, cudaStreamSynchronize(c->stream), "winner_model");
     if (st) return st;
     w = *c->win_h;
     return SISSO_OK;

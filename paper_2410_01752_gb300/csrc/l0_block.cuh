@@ -89,6 +89,7 @@ __device__ __noinline__ double block_exact(const TileArgs& A, const int (&pos)[D
             if (!(rss - tile_apost_err(A, s, rss) <= thr32)) return B;
         }
     }
+    if (clears64<D>(A.G64, A.b64, A.ld64, A.syy64, A.N, thr, pos)) return B;
     const double r64 = rss64(A.G64, A.b64, A.ld64, A.syy64, A.N, D, pos, nullptr);
     if (!(r64 <= thr)) return B;
     add_band<D - 2>(A, pos, r32);
@@ -176,7 +177,8 @@ struct BlockP {
     int p, m;
     bool ok;                     // pivots of the prefix and of p above tau
     float invd, w, v0, v1;       // 1 / sqrt(d'_p), w_p, p's back-substituted coefficients
-    float A0, base, q2, thrN;    // |L^-T w|_1, syy - |w|^2, largest |a2|_1, (B + tie) / N
+    float A0, base, thrN;        // |L^-T w|_1, syy - |w|^2, (B + tie) / N
+    float q2, rmax;              // largest |a2|_1 and root of the largest dp
 };
 struct BlockRow { float r, d, n, l1; };      // R[p][x], dp, np, |L_P^-T R[.][x]|_1
 
@@ -195,7 +197,7 @@ __device__ __forceinline__ RowC block_row(const TileArgs& A, const BlockP& Q, co
     const bool piv = Q.ok && f.d > A.tau;
     const float isd = __frsqrt_rn(f.d > 0.f ? f.d : 1.f), w1 = f.n * isd;
     const float S0 = 1.02f * (Q.A0 + (1.f + f.l1) * fabsf(w1) * isd);
-    const float S1 = 1.02f * ((1.f + f.l1) * isd * 1.0001f + 1.f + Q.q2);
+    const float S1 = 1.02f * ((1.f + f.l1) * isd * Q.rmax * 1.0001f + 1.f + Q.q2);
     const float Kc = piv ? (Q.base - w1 * w1) - (A.e0 + S0 * fmaf(A.e2, S0, A.e1)) : -INFINITY;
     return RowC{-f.r, -(isd * isd), -(w1 * isd), Q.thrN - Kc, S1 * fmaf(2.f * A.e2, S0, A.e1), A.e2 * S1 * S1};
 }
@@ -343,9 +345,14 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int sli
                 Q.thrN = __fmul_ru((float)((B + A.tie64) * inv_n), 1.0000002f);
             }
             const float invd = Q.invd, wp = Q.w, tau = A.tau;
-            float q2 = 0.f;
-            for (int x = p + 1 + lane; x < m; x += 32) q2 = fmaxf(q2, block_feature<DC>(Q, Gp, dn, vv, x).l1);
+            float q2 = 0.f, dmax = 0.f;
+            for (int x = p + 1 + lane; x < m; x += 32) {
+                const BlockRow f = block_feature<DC>(Q, Gp, dn, vv, x);
+                q2 = fmaxf(q2, f.l1);
+                dmax = fmaxf(dmax, f.d);
+            }
             Q.q2 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(q2)));
+            Q.rmax = sqrtf(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(dmax))));
             // rows p + 1 .. m - 2, kBRow groups of 32 at a time: this lane's are i0 + 32 j
             for (int rb = p + 1; rb < m - 1; rb += 32 * kBRow) {
             const int i0 = rb + lane, groups = (m - 1 - rb + 31) >> 5;

@@ -113,35 +113,108 @@ template <int DP> __device__ __forceinline__ void colex_unrank(int64_t r, int (&
 
 // MODE 0: bound (min of RSS + err); MODE 1: band collection
 
-__device__ double rss64(const double* G, const double* b, int ld, double syy, int N, int D, const int* pos,
-                        double* gamma) {
-    double L[kMaxDim][kMaxDim], w[kMaxDim];
+// FP64 RSS of one subset by Cholesky (infinite when a pivot is at or below kPivotMin), and its
+// coefficients in gamma when given.  The dimension is fixed at compile time: with a runtime one
+// the factor lives in local memory
+template <int D>
+__device__ __noinline__ double rss64_fixed(const double* G, const double* b, int ld, double syy, int N, const int* pos_,
+                                           double* gamma) {
+    double L[D][D], w[D];
+    int pos[D];
+#pragma unroll
+    for (int j = 0; j < D; ++j) pos[j] = pos_[j];
+#pragma unroll
     for (int j = 0; j < D; ++j) {
         double dj = G[(size_t)pos[j] * ld + pos[j]];
+#pragma unroll
         for (int m = 0; m < j; ++m) dj -= L[j][m] * L[j][m];
         if (!(dj > kPivotMin)) return INFINITY;
         L[j][j] = sqrt(dj);
+#pragma unroll
         for (int i = j + 1; i < D; ++i) {
             double v = G[(size_t)pos[i] * ld + pos[j]];
+#pragma unroll
             for (int m = 0; m < j; ++m) v -= L[i][m] * L[j][m];
             L[i][j] = v / L[j][j];
         }
     }
     double q = 0.0;
+#pragma unroll
     for (int j = 0; j < D; ++j) {
         double v = b[pos[j]];
+#pragma unroll
         for (int m = 0; m < j; ++m) v -= L[j][m] * w[m];
         w[j] = v / L[j][j];
         q += w[j] * w[j];
     }
     if (gamma) {   // back substitution L^T gamma = w
+        double g[D];
+#pragma unroll
         for (int j = D - 1; j >= 0; --j) {
             double v = w[j];
-            for (int m = j + 1; m < D; ++m) v -= L[m][j] * gamma[m];
-            gamma[j] = v / L[j][j];
+#pragma unroll
+            for (int m = j + 1; m < D; ++m) v -= L[m][j] * g[m];
+            g[j] = v / L[j][j];
+            gamma[j] = g[j];
         }
     }
     return (double)N * (syy - q);
+}
+
+__device__ __forceinline__ double rss64(const double* G, const double* b, int ld, double syy, int N, int D, const int* pos,
+                                        double* gamma) {
+    switch (D) {
+        case 1: return rss64_fixed<1>(G, b, ld, syy, N, pos, gamma);
+        case 2: return rss64_fixed<2>(G, b, ld, syy, N, pos, gamma);
+        case 3: return rss64_fixed<3>(G, b, ld, syy, N, pos, gamma);
+        case 4: return rss64_fixed<4>(G, b, ld, syy, N, pos, gamma);
+        default: return rss64_fixed<5>(G, b, ld, syy, N, pos, gamma);
+    }
+}
+
+// Whether rss64 of a subset is certainly above thr (or infinite): an LDL^T solve, one reciprocal
+// per pivot and no square root or division (a quarter of rss64's FP64 instructions on a pipe that
+// takes about 18 cycles for each), with the a posteriori bound of the FP32 form at FP64's unit
+// roundoff for both solves.  On strongly collinear subspaces, where FP32 cannot decide up to a
+// sixth of all subsets, these solves are most of the search.
+template <int D>
+__device__ __forceinline__ bool clears64(const double* G, const double* b, int ld, double syy, int N, double thr,
+                                         const int (&pos)[D]) {
+    double l[D][D], inv[D], z[D], q = 0.0;
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+        double u[D];
+        double dj = G[(size_t)pos[j] * ld + pos[j]];
+        const double slack = 1e-13 + 4e-15 * dj;
+#pragma unroll
+        for (int m = 0; m < j; ++m) {
+            double v = G[(size_t)pos[j] * ld + pos[m]];
+#pragma unroll
+            for (int k = 0; k < m; ++k) v -= u[k] * l[m][k];
+            u[m] = v;
+            l[j][m] = v * inv[m];
+            dj -= v * l[j][m];
+        }
+        if (!(dj > kPivotMin + slack)) return dj < kPivotMin - slack;
+        inv[j] = 1.0 / dj;
+        double v = b[pos[j]];
+#pragma unroll
+        for (int m = 0; m < j; ++m) v -= l[j][m] * z[m];
+        z[j] = v;
+        q += v * v * inv[j];
+    }
+    double s = 0.0, g[D];
+#pragma unroll
+    for (int j = D - 1; j >= 0; --j) {
+        double v = z[j] * inv[j];
+#pragma unroll
+        for (int m = j + 1; m < D; ++m) v -= l[m][j] * g[m];
+        g[j] = v;
+        s += fabs(v);
+    }
+    const double sst = syy * N, r = sst - N * q, c1 = 1.0 + 3.1 * (D + 1);
+    const double err = 4.0 * 1.1102230246251565e-16 * (N * (2.0 * sqrt(syy) * s + c1 * s * s) + (D + 3) * (2.0 * sst + fabs(r)));
+    return r - 2.0 * err > thr;
 }
 
 __device__ __forceinline__ void unpack(uint64_t key, int D, int* pos) {

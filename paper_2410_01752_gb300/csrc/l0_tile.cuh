@@ -17,7 +17,9 @@
 // e0 + e1 s + e2 s^2 with s = |gamma|_1 the subset's coefficient 1-norm, and with
 // a = L_P^-T w_P, a1 = L_P^-T R[.][i1], a2 = L_P^-T R[.][i2] (prefix back substitutions)
 //     s <= |a|_1 + (1 + |a1|_1) |w1| / sqrt(d1)
-//            + ((1 + |a1|_1) |r| / sqrt(d1) + 1 + |a2|_1) |num| / d2 = S0 + S1 t,   |r| <= 1.
+//            + ((1 + |a1|_1) |r| / sqrt(d1) + 1 + |a2|_1) |num| / d2 = S0 + S1 t,
+// with |r| = |g| / sqrt(d1) <= sqrt(dp[i2]), taken at the largest dp of the unit's columns (where
+// the prefix explains most of every feature that is far below 1).
 // With K = c - (B + tie)/N - e0 - S0 (e1 + e2 S0), beta = S1 (e1 + 2 e2 S0), gamma = e2 S1^2
 // per row (e0, e1, e2 twice the bound's), a subset is dismissed when
 //     K - beta t - (d2 + gamma) t^2 > 0, that is (times d2^2, d2 > tau)
@@ -42,6 +44,8 @@
 #pragma once
 
 #include "l0_device.cuh"
+
+#include <climits>
 
 namespace sg {
 namespace {
@@ -257,6 +261,7 @@ __device__ __noinline__ double tile_exact(const TileArgs& A, const PrefixSm* Ps,
         }
     }
     // FP64 confirmation from the FP64 Gram
+    if (clears64<DP + 2>(A.G64, A.b64, A.ld64, A.syy64, A.N, thr, pos)) return B;
     const double r64 = rss64(A.G64, A.b64, A.ld64, A.syy64, A.N, DP + 2, pos, nullptr);
     if (!(r64 <= thr)) return B;
     add_band<DP>(A, pos, r32);
@@ -337,7 +342,7 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
         // column groups j (columns c + 32 j + lane) and rows of this unit
         int pm = -1;
         int row_lo, row_hi, j_lo, jc, cb;
-        float q2 = 0.f, pw2 = 0.f;
+        float q2 = 0.f, pw2 = 0.f, dmax = 0.f;
         float rt[8][DPa], dp2[8], np2[8];
         {
             // ---- prefix factor (warp-uniform, redundant in every lane) ---------------
@@ -399,6 +404,7 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
                 if (x > row_lo && x >= c && x < A.n) {
                     prefix_reduce<DP>(A, pre, L, invd, wv, x, rt[j], dp2[j], np2[j]);
                     q2 = fmaxf(q2, back_l1<DP>(L, invd, rt[j]));
+                    dmax = fmaxf(dmax, dp2[j]);
                 } else {
 #pragma unroll
                     for (int m = 0; m < DP; ++m) rt[j][m] = 0.f;
@@ -411,7 +417,11 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
                 colv[(DP + 1) * kTC + lane + 32 * j] = np2[j];
             }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) q2 = fmaxf(q2, __shfl_xor_sync(0xffffffffu, q2, o));
+            for (int o = 16; o > 0; o >>= 1) {
+                q2 = fmaxf(q2, __shfl_xor_sync(0xffffffffu, q2, o));
+                dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+            }
+            const float rmax = sqrtf(dmax);
 
             // ---- rows: record per row in shared memory --------------------------------
             for (int i1 = row_lo + lane; i1 <= row_hi; i1 += 32) {
@@ -423,7 +433,7 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
                 const float w1 = n1 * isd1;
                 const float a1 = back_l1<DP>(L, invd, r1);
                 const float S0 = 1.02f * (A0 + (1.f + a1) * fabsf(w1) * isd1);
-                const float S1 = 1.02f * ((1.f + a1) * isd1 * 1.0001f + 1.f + q2);
+                const float S1 = 1.02f * ((1.f + a1) * isd1 * rmax * 1.0001f + 1.f + q2);
 #pragma unroll
                 for (int m = 0; m < DP; ++m) rr_[m] = r1[m];
                 rr_[DP] = isd1;
@@ -713,8 +723,8 @@ __global__ void k_prefix_sq(const double* __restrict__ w, int n, const int* __re
 // greedy forward selection in FP64: its D-subset's RSS is an upper bound of the minimum
 __global__ void k_greedy_bound(const double* __restrict__ G, const double* __restrict__ b, int ld, double syy, int N,
                                int n, int D, unsigned long long* ub_key) {
-    __shared__ double s_val[256];
-    __shared__ int s_idx[256];
+    __shared__ unsigned long long s_key[8];
+    __shared__ int s_idx[8];
     __shared__ int sel[kMaxDim];
     int pos[kMaxDim];
     for (int t = 0; t < D; ++t) {
@@ -729,20 +739,24 @@ __global__ void k_greedy_bound(const double* __restrict__ G, const double* __res
             const double r = rss64(G, b, ld, syy, N, t + 1, pos, nullptr);
             if (r < best) { best = r; bi = x; }
         }
-        s_val[threadIdx.x] = best;
-        s_idx[threadIdx.x] = bi;
+        // the lowest RSS of the block, ties to the lowest thread: warps, then the warps' best
+        unsigned long long key = okey(best);
+        int at = bi >= 0 ? (int)threadIdx.x : INT_MAX;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, o);
+            const int b2 = __shfl_xor_sync(0xffffffffu, bi, o), a2 = __shfl_xor_sync(0xffffffffu, at, o);
+            if (a2 != INT_MAX && (at == INT_MAX || k2 < key || (k2 == key && a2 < at))) { key = k2; bi = b2; at = a2; }
+        }
+        if ((threadIdx.x & 31) == 0) { s_key[threadIdx.x >> 5] = key; s_idx[threadIdx.x >> 5] = at == INT_MAX ? -1 : bi; }
         __syncthreads();
         if (threadIdx.x == 0) {
-            double bv = INFINITY;
             int bx = -1;
-            for (int q = 0; q < (int)blockDim.x; ++q)
-                if (s_idx[q] >= 0 && s_val[q] < bv) { bv = s_val[q]; bx = s_idx[q]; }
-            if (bx < 0) {                       // every extension singular: give up (bound stays)
-                sel[t] = -1;
-            } else {
-                sel[t] = bx;
-                if (t == D - 1) atomicMin(ub_key, okey(bv));
-            }
+            unsigned long long bk = 0;
+            for (int q = 0; q < (int)(blockDim.x >> 5); ++q)
+                if (s_idx[q] >= 0 && (bx < 0 || s_key[q] < bk)) { bk = s_key[q]; bx = s_idx[q]; }
+            sel[t] = bx;                        // -1: every extension singular, give up (the bound stays)
+            if (bx >= 0 && t == D - 1) atomicMin(ub_key, bk);
         }
         __syncthreads();
         if (sel[t] < 0) return;
