@@ -24,6 +24,7 @@
 #include "l0_device.cuh"
 #include "l0_tile.cuh"
 #include "l0_block.cuh"
+#include "l0_pair64.cuh"
 
 #include <algorithm>
 #include <cfloat>
@@ -527,6 +528,8 @@ sisso_status ensure_tile_buffers(sisso_ctx* c, int n) {
 // tie-broken winner.
 __global__ void k_set_bound(unsigned long long* key, double v) { *key = okey(v); }
 
+constexpr int64_t kPair64Max = 200000000;     // D = 2 and 3: most subsets enumerated in FP64
+
 // prefix_mask (optional): only the prefixes whose bit is set are enumerated; bound0 >= 0:
 // the search starts from this FP64 RSS (an upper bound of the minimum) instead of the greedy one
 static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* b, int ld, double syy, int n, int D,
@@ -568,7 +571,8 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
     cudaMemsetAsync(cand, 0, sizeof(unsigned long long), c->stream);
     cudaMemsetAsync(c->band_count, 0, sizeof(unsigned), c->stream);
     const int64_t tot = (int64_t)n * ldp;
-    k_pad_gram<<<std::max(1, (int)std::min<int64_t>(c->sms * 8, (tot + 255) / 256)), 256, 0, c->stream>>>(
+    const bool pair64 = DP <= 1 && !prefix_mask && binom_host(n, D) <= kPair64Max && pair64_smem(n) <= ((size_t)200 << 10);
+    if (!pair64) k_pad_gram<<<std::max(1, (int)std::min<int64_t>(c->sms * 8, (tot + 255) / 256)), 256, 0, c->stream>>>(
         G, b, ld, n, ldp, c->tile_G, c->tile_b, c->tile_diag);
     if (bound0 >= 0.0) k_set_bound<<<1, 1, 0, c->stream>>>(ub_key, bound0);
     else k_greedy_bound<<<1, 256, 0, c->stream>>>(G, b, ld, syy, c->N, n, D, ub_key);
@@ -596,12 +600,24 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
         cudaFuncSetAttribute(k_l0_tile<DPV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);   \
         k_l0_tile<DPV><<<grid, kTW * 32, sm, c->stream>>>(A);                                          \
     } while (0)
+    // D = 2 and 3 in FP64 while their FP64 work (six operations a subset, 0.52e12 a second) stays
+    // below about 2.3 ms and the tables fit shared memory
+    if (pair64) {
+        const size_t sm = pair64_smem(n);
+        if (DP == 0) {
+            cudaFuncSetAttribute(k_l0_pair64<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            k_l0_pair64<2><<<dim3(1, (unsigned)std::max(1, std::min(c->sms, (n + 7) / 8))), kPairThreads, sm, c->stream>>>(A);
+        } else {
+            // rows of a p cut so that every SM has about four CTAs
+            const int cut = std::max(1, std::min((n + 15) / 16, 4 * c->sms / n));
+            cudaFuncSetAttribute(k_l0_pair64<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            k_l0_pair64<3><<<dim3((unsigned)(n - 2), (unsigned)cut), kPairThreads, sm, c->stream>>>(A);
+        }
+    } else
     // D = 4 and 5 without a prefix mask: the prefix's first D - 3 features eliminated once per
     // CTA when the triangle of the rest fits shared memory and there are enough prefixes to
     // fill the SMs (a slice of a prefix's features at D = 4, which has only n of them)
-    const int DC = D - 3;
-    const int m_max = n - DC;
-    if (DC >= 1 && DC <= 2 && !prefix_mask && m_max >= 3 && m_max <= kBMaxM) {
+    if (const int DC = D - 3, m_max = n - DC; DC >= 1 && DC <= 2 && !prefix_mask && m_max >= 3 && m_max <= kBMaxM) {
         // two launches: the prefixes with many features to their right, then those with few
         const int slices = DC == 1 ? 4 : 1;
         const int64_t all = DC == 1 ? n - 3 : binom_host(n - 3, 2);
