@@ -82,7 +82,7 @@ void free_all(sisso_ctx* c) {
                     c->band, c->band_rss, c->band_count, c->prefixes, c->work, c->win, c->blk_best,
                     c->space_dev, c->surv_probe, c->zcache, c->subvalid, c->dup_list, c->dup_ok,
                     c->dup_cnt, c->accepted, c->opcache32, c->opcache64, c->opsum, c->opval64,
-                    c->band_r32, c->band_sel, c->tile_G, c->tile_b, c->tile_diag, c->tile_info,
+                    c->band_r32, c->band_sel, c->l0_perm, c->l0_Gq, c->tile_G, c->tile_b, c->tile_diag, c->tile_info,
                     c->unit_ok, c->unit_mask, c->opinv64, c->fix_ids, c->fix_count};
     for (void* p : bufs) {
         if (!p) continue;

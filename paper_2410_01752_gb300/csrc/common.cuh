@@ -159,6 +159,18 @@ struct Prog {
     int16_t code[kProgLen];
 };
 
+// c 2^k rounded to nearest FP32 (ties to even; below FP32's normal range zero), |result| < 2^127,
+// on the integer pipe: the conversion instruction runs at the FP64 pipe's rate
+__device__ __forceinline__ float scaled_f32(double c, int k) {
+    const unsigned hi = (unsigned)__double2hiint(c), lo = (unsigned)__double2loint(c);
+    const int fe = (int)((hi >> 20) & 0x7ffu) - (1023 - 127) + k;
+    if (fe <= 0) return 0.f;
+    unsigned b = ((unsigned)fe << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned rest = lo & 0x1fffffffu;
+    b += (rest > 0x10000000u) | ((rest == 0x10000000u) & b);
+    return __uint_as_float(b | (hi & 0x80000000u));
+}
+
 // Postfix program of feature id: children first (a, then b), then the operator.
 // Iterative depth-first walk with an explicit stack (a rung-3 tree has at most 7
 // pending entries); no recursion, so the per-thread stack stays small and static.
@@ -473,6 +485,8 @@ struct sisso_ctx {
     float* tile_G = nullptr;
     float* tile_b = nullptr;
     float* tile_diag = nullptr;
+    int* l0_perm = nullptr;            // features in the greedy search's order
+    double* l0_Gq = nullptr;           // FP64 Gram and moments in that order
     int tile_rows = 0, tile_ld = 0;
     void* tile_info = nullptr;
     int tile_info_cap = 0;

@@ -509,12 +509,17 @@ sisso_status ensure_tile_buffers(sisso_ctx* c, int n) {
     const int n_tiles = ((n + kTR - 1) / kTR) * ((n + kTC - 1) / kTC);
     if (n <= c->tile_rows && ld <= c->tile_ld && n_tiles <= c->tile_info_cap) return SISSO_OK;
     cudaStreamSynchronize(c->stream);
+    cudaFree(c->l0_perm); cudaFree(c->l0_Gq);
+    c->l0_perm = nullptr;
+    c->l0_Gq = nullptr;
     cudaFree(c->tile_G); cudaFree(c->tile_b); cudaFree(c->tile_diag); cudaFree(c->tile_info);
     c->tile_G = c->tile_b = c->tile_diag = nullptr;
     c->tile_info = nullptr;
     c->tile_rows = c->tile_ld = c->tile_info_cap = 0;
     sisso_status st;
     if ((st = check_cuda(c, cudaMalloc(&c->tile_G, sizeof(float) * (size_t)n * ld), "tile_G")) ||
+        (st = check_cuda(c, cudaMalloc(&c->l0_perm, sizeof(int) * (size_t)n), "l0 order")) ||
+        (st = check_cuda(c, cudaMalloc(&c->l0_Gq, sizeof(double) * (size_t)std::min(n, kBMaxM + 2) * (std::min(n, kBMaxM + 2) + 1)), "l0 reordered Gram")) ||
         (st = check_cuda(c, cudaMalloc(&c->tile_b, sizeof(float) * (size_t)ld), "tile_b")) ||
         (st = check_cuda(c, cudaMalloc(&c->tile_diag, sizeof(float) * (size_t)ld), "tile_diag")) ||
         (st = check_cuda(c, cudaMalloc(&c->tile_info, sizeof(TileInfo) * (size_t)n_tiles), "tile_info")))
@@ -572,10 +577,11 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
     cudaMemsetAsync(c->band_count, 0, sizeof(unsigned), c->stream);
     const int64_t tot = (int64_t)n * ldp;
     const bool pair64 = DP <= 1 && !prefix_mask && binom_host(n, D) <= kPair64Max && pair64_smem(n) <= ((size_t)200 << 10);
-    if (!pair64) k_pad_gram<<<std::max(1, (int)std::min<int64_t>(c->sms * 8, (tot + 255) / 256)), 256, 0, c->stream>>>(
+    const bool block = D >= 4 && !prefix_mask && n >= D && n - (D - 3) <= kBMaxM;
+    if (!pair64 && !block) k_pad_gram<<<std::max(1, (int)std::min<int64_t>(c->sms * 8, (tot + 255) / 256)), 256, 0, c->stream>>>(
         G, b, ld, n, ldp, c->tile_G, c->tile_b, c->tile_diag);
     if (bound0 >= 0.0) k_set_bound<<<1, 1, 0, c->stream>>>(ub_key, bound0);
-    else k_greedy_bound<<<1, 256, 0, c->stream>>>(G, b, ld, syy, c->N, n, D, ub_key);
+    else k_greedy_bound<<<1, 256, 0, c->stream>>>(G, b, ld, syy, c->N, n, D, ub_key, block ? c->l0_perm : nullptr);
     TileArgs A{};
     A.G = c->tile_G + kTC; A.b = c->tile_b; A.diag = c->tile_diag; A.ldp = ldp; A.n = n; A.N = c->N; A.D = D;
     A.syy = (float)syy; A.tau = kPivotMin32; A.sst = sst; A.sqrt_syy = std::sqrt(syy);
@@ -591,7 +597,7 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
     A.counter = c->work; A.ub_key = ub_key; A.tie64 = 2.0 * kRssTie * sst;
     A.G64 = G; A.b64 = b; A.ld64 = ld; A.syy64 = syy;
     A.band = c->band; A.band_count = c->band_count; A.band_cap = c->band_cap; A.band_r32 = nullptr;
-    A.examined = examined; A.candidates = cand; A.prefix_mask = prefix_mask;
+    A.examined = examined; A.candidates = cand; A.prefix_mask = prefix_mask; A.perm = c->l0_perm;
     cudaEventRecord(e1, c->stream);
     const int grid = c->sms * 2;
 #define SG_TILE(DPV)                                                                                   \
@@ -617,7 +623,12 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
     // D = 4 and 5 without a prefix mask: the prefix's first D - 3 features eliminated once per
     // CTA when the triangle of the rest fits shared memory and there are enough prefixes to
     // fill the SMs (a slice of a prefix's features at D = 4, which has only n of them)
-    if (const int DC = D - 3, m_max = n - DC; DC >= 1 && DC <= 2 && !prefix_mask && m_max >= 3 && m_max <= kBMaxM) {
+    if (block) {
+        k_l0_reorder<<<std::max(1, std::min(c->sms * 2, (n * n + 255) / 256)), 256, 0, c->stream>>>(G, b, ld, n, c->l0_perm, c->l0_Gq,
+                                                                                                 c->l0_Gq + (size_t)n * n);
+        c->stats.launches++;
+        A.Gq = c->l0_Gq; A.bq = c->l0_Gq + (size_t)n * n;
+        const int DC = D - 3, m_max = n - DC;
         // two launches: the prefixes with many features to their right, then those with few
         const int slices = DC == 1 ? 4 : 1;
         const int64_t all = DC == 1 ? n - 3 : binom_host(n - 3, 2);

@@ -13,6 +13,15 @@
 // filter stay in registers); a column x > i1 costs two broadcast reads, three operations for its
 // values and one row of G'.  The subset test is the filter of l0_tile.cuh with one fused
 // multiply-add in the place of D - 2.
+//
+// The prefix is eliminated in FP64, its reduced features scaled to unit variance and then rounded
+// to FP32, so that the FP32 error of a subset is relative to what the prefix leaves unexplained
+// (syy' = syy - |w|^2 in the filter's e0 and e1, coefficients of the reduced features), not to the
+// whole target.  The features are taken by their largest correlation with a feature of the greedy
+// search: where a few features, or others that could stand in for them, reach the noise and every
+// subset that holds them nearly ties, they are the prefix, and FP32 still tells those subsets
+// apart (eliminated in FP32 and in the order of screening, up to 5.4e7 of the 1.96e10 subsets of
+// such problems went to FP64 solves, which then took longer than the sweep).
 // Measured at n = 300, D = 5 (1.96e10 subsets): see the figures at the launch (l0.cu).  Forms
 // that took longer than k_l0_tile's 43 ms: lanes as columns with the row constants shuffled in
 // (89 ms), and four warps sharing a p through a record table and a barrier (46 ms).
@@ -34,65 +43,25 @@ constexpr int kBQ = 64;                   // per-warp candidate queue
 constexpr int kBMaxM = 320;               // features right of the CTA's prefix (204 KB triangle)
 
 __host__ __device__ constexpr size_t block_smem_bytes(int m, int warps) {
-    return sizeof(float) * ((size_t)m * (m - 1) / 2 + 36) + 2 * sizeof(float2) * (size_t)m +
+    return sizeof(float) * ((size_t)m * (m - 1) / 2 + 36) + (sizeof(double2) + sizeof(float2)) * (size_t)m +
            sizeof(unsigned) * kBQ * warps;
 }
 
-// prefix of the CTA, in feature coordinates (shared memory)
+// prefix of the CTA
 struct BlockPre {
-    int pre[2], last, ok;        // features, the last of them, pivots above tau
-    float l10, inv[2], w[2];     // factor, 1 / diagonal, forward-solved moments
-    float u[2], pw2;             // back-substituted coefficients L^-T w, |w|^2
+    int pre[2], last, ok;        // positions, the last of them; pivots usable
+    double l10, inv[2], w[2];    // factor, 1 / diagonal, forward-solved moments
+    float low;                   // the least pivot
+    float base, e0, e1;          // syy' and the filter's errors at its scale
 };
 
-// the exact decision of one subset (positions ascending): FP32 solve with its a posteriori
-// bound, then FP64; returns the lane's new bound
+// the exact decision of one subset (feature positions ascending); returns the lane's new bound
 template <int D>
-__device__ __noinline__ double block_exact(const TileArgs& A, const int (&pos)[D], double B, double thr, float thr32) {
-    float L[D][D], inv[D], wv[D], q = 0.f;
-    bool piv = true;
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-        float d = A.diag[pos[j]];
-#pragma unroll
-        for (int m = 0; m < j; ++m) d -= L[j][m] * L[j][m];
-        piv = piv && d > A.tau;
-        const float l = sqrtf(d > 0.f ? d : 1.f);
-        inv[j] = 1.f / l;
-#pragma unroll
-        for (int i = j + 1; i < D; ++i) {
-            float v = A.G[(size_t)pos[i] * A.ldp + pos[j]];
-#pragma unroll
-            for (int m = 0; m < j; ++m) v -= L[i][m] * L[j][m];
-            L[i][j] = v * inv[j];
-        }
-        float v = A.b[pos[j]];
-#pragma unroll
-        for (int m = 0; m < j; ++m) v -= L[j][m] * wv[m];
-        wv[j] = v * inv[j];
-        q += wv[j] * wv[j];
-    }
-    float r32 = __int_as_float(0x7fc00000);
-    if (piv) {
-        const float rss = (float)A.N * (A.syy - q);
-        r32 = rss;
-        if (!(rss <= thr32)) {
-            float s = 0.f, gm[D];
-#pragma unroll
-            for (int j = D - 1; j >= 0; --j) {
-                float v = wv[j];
-#pragma unroll
-                for (int m = j + 1; m < D; ++m) v -= L[m][j] * gm[m];
-                gm[j] = v * inv[j];
-                s += fabsf(gm[j]);
-            }
-            if (!(rss - tile_apost_err(A, s, rss) <= thr32)) return B;
-        }
-    }
+__device__ __noinline__ double block_exact(const TileArgs& A, const int (&pos)[D], double B, double thr) {
     if (clears64<D>(A.G64, A.b64, A.ld64, A.syy64, A.N, thr, pos)) return B;
     const double r64 = rss64(A.G64, A.b64, A.ld64, A.syy64, A.N, D, pos, nullptr);
     if (!(r64 <= thr)) return B;
-    add_band<D - 2>(A, pos, r32);
+    add_band<D - 2>(A, pos, (float)r64);
     if (r64 < B) {
         atomicMin(A.ub_key, okey(r64));
         return r64;
@@ -105,16 +74,23 @@ template <int DC>
 __device__ __noinline__ double block_flush(const TileArgs& A, const BlockPre* P, const unsigned* q, int qn, double B) {
     const int lane = threadIdx.x & 31;
     const double thr = B + A.tie64;
-    const float thr32 = __double2float_ru(thr);
     for (int e = lane; e < qn; e += 32) {
         const unsigned v = q[e];
         int pos[DC + 3];
 #pragma unroll
-        for (int m = 0; m < DC; ++m) pos[m] = P->pre[m];
-        pos[DC] = P->last + 1 + (int)(v & 1023u);
-        pos[DC + 1] = P->last + 1 + (int)((v >> 10) & 1023u);
-        pos[DC + 2] = P->last + 1 + (int)(v >> 20);
-        B = block_exact<DC + 3>(A, pos, B, thr, thr32);
+        for (int m = 0; m < DC; ++m) pos[m] = A.perm[P->pre[m]];
+        pos[DC] = A.perm[P->last + 1 + (int)(v & 1023u)];
+        pos[DC + 1] = A.perm[P->last + 1 + (int)((v >> 10) & 1023u)];
+        pos[DC + 2] = A.perm[P->last + 1 + (int)(v >> 20)];
+#pragma unroll
+        for (int i = 1; i < DC + 3; ++i)                      // ascending
+#pragma unroll
+            for (int j = i; j > 0; --j) {
+                const int lo = min(pos[j - 1], pos[j]), hi = max(pos[j - 1], pos[j]);
+                pos[j - 1] = lo;
+                pos[j] = hi;
+            }
+        B = block_exact<DC + 3>(A, pos, B, thr);
     }
     __syncwarp();
 #pragma unroll
@@ -176,19 +152,17 @@ __device__ __forceinline__ void block_col(const float* gx, float r, float d, flo
 struct BlockP {
     int p, m;
     bool ok;                     // pivots of the prefix and of p above tau
-    float invd, w, v0, v1;       // 1 / sqrt(d'_p), w_p, p's back-substituted coefficients
-    float A0, base, thrN;        // |L^-T w|_1, syy - |w|^2, (B + tie) / N
-    float q2, rmax;              // largest |a2|_1 and root of the largest dp
+    float invd, w;               // 1 / sqrt(d'_p), w_p
+    float A0, base, thrN;        // |w_p| / sqrt(d'_p), syy' - w_p^2, (B + tie) / N
+    float e0, e1;                // the filter's errors at this prefix's scale
+    float q2, rmax;              // largest |a2| and root of the largest dp
 };
-struct BlockRow { float r, d, n, l1; };      // R[p][x], dp, np, |L_P^-T R[.][x]|_1
+struct BlockRow { float r, d, n, l1; };      // R[p][x], dp, np, |coefficient on p|
 
-template <int DC>
-__device__ __forceinline__ BlockRow block_feature(const BlockP& Q, const float* Gp, const float2* dn, const float2* vv, int x) {
-    const float r = Gp[x * (x - 1) / 2 + Q.p] * Q.invd, c = r * Q.invd;
-    const float2 f = dn[x], v = vv[x];
-    float l1 = fabsf(c) + fabsf(fmaf(-c, Q.v0, v.x));
-    if (DC == 2) l1 += fabsf(fmaf(-c, Q.v1, v.y));
-    return BlockRow{r, fmaf(-r, r, f.x), fmaf(-r, Q.w, f.y), l1};
+__device__ __forceinline__ BlockRow block_feature(const BlockP& Q, const float* Gp, const float2* dn, int x) {
+    const float r = Gp[x * (x - 1) / 2 + Q.p] * Q.invd;
+    const float2 f = dn[x];
+    return BlockRow{r, fmaf(-r, r, f.x), fmaf(-r, Q.w, f.y), fabsf(r * Q.invd)};
 }
 
 // the filter's constants of one row
@@ -198,8 +172,8 @@ __device__ __forceinline__ RowC block_row(const TileArgs& A, const BlockP& Q, co
     const float isd = __frsqrt_rn(f.d > 0.f ? f.d : 1.f), w1 = f.n * isd;
     const float S0 = 1.02f * (Q.A0 + (1.f + f.l1) * fabsf(w1) * isd);
     const float S1 = 1.02f * ((1.f + f.l1) * isd * Q.rmax * 1.0001f + 1.f + Q.q2);
-    const float Kc = piv ? (Q.base - w1 * w1) - (A.e0 + S0 * fmaf(A.e2, S0, A.e1)) : -INFINITY;
-    return RowC{-f.r, -(isd * isd), -(w1 * isd), Q.thrN - Kc, S1 * fmaf(2.f * A.e2, S0, A.e1), A.e2 * S1 * S1};
+    const float Kc = piv ? (Q.base - w1 * w1) - (Q.e0 + S0 * fmaf(A.e2, S0, Q.e1)) : -INFINITY;
+    return RowC{-f.r, -(isd * isd), -(w1 * isd), Q.thrN - Kc, S1 * fmaf(2.f * A.e2, S0, Q.e1), A.e2 * S1 * S1};
 }
 
 struct BlockQueue { double B; int qn, taken; };
@@ -207,17 +181,17 @@ struct BlockQueue { double B; int qn, taken; };
 // a column some lane may keep: the decisions row group by row group, into the warp's queue
 template <int DC>
 __device__ __noinline__ BlockQueue block_take(const TileArgs& A, const BlockPre* P, const BlockP Q, const float* Gp,
-                                              const float2* dn, const float2* vv, int rb, int x, unsigned* q, int qn,
+                                              const float2* dn, int rb, int x, unsigned* q, int qn,
                                               double B) {
     const int lane = threadIdx.x & 31;
     int taken = 0;
-    const BlockRow f = block_feature<DC>(Q, Gp, dn, vv, x);
+    const BlockRow f = block_feature(Q, Gp, dn, x);
     const int end = min(x, rb + 32 * kBRow);            // the rows of this sweep
     for (int i = rb; i < end; i += 32) {
         const int i1 = i + lane;
         bool take = false;
         if (i1 < x) {
-            const RowC c = block_row(A, Q, block_feature<DC>(Q, Gp, dn, vv, i1));
+            const RowC c = block_row(A, Q, block_feature(Q, Gp, dn, i1));
             float z, d2;
             block_test(Gp[x * (x - 1) / 2 + i1], f.r, f.d, f.n, c.nr, c.nid, c.nw, c.nK, c.be, c.gm, z, d2);
             take = !((z < 0.f) & (d2 > A.tau));
@@ -238,15 +212,25 @@ __device__ __noinline__ BlockQueue block_take(const TileArgs& A, const BlockPre*
 }
 
 // prefixes item0 .. of the colex order, M the most features right of one of them
+// the FP64 Gram and moments in the order of perm
+__global__ void k_l0_reorder(const double* __restrict__ G, const double* __restrict__ b, int ld, int n,
+                             const int* __restrict__ perm, double* __restrict__ Gq, double* __restrict__ bq) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n * n; e += gridDim.x * blockDim.x) {
+        const int i = e / n, j = e - i * n;
+        Gq[e] = G[(size_t)perm[i] * ld + perm[j]];
+        if (i == 0) bq[j] = b[perm[j]];
+    }
+}
+
 template <int DC, int W>
 __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int slices, int item0, int M) {
     extern __shared__ __align__(16) unsigned char block_smem[];
     __shared__ BlockPre P;
     __shared__ int s_item, s_p;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    float2* dn = reinterpret_cast<float2*>(block_smem);           // d', n' per feature
-    float2* vv = dn + M;                                          // its coefficients L^-T R[.][x]
-    float* Gp = reinterpret_cast<float*>(vv + M);                 // (x, y < x) at x (x - 1) / 2 + y
+    double2* rr = reinterpret_cast<double2*>(block_smem);         // R per feature (while the triangle is formed)
+    float2* dn = reinterpret_cast<float2*>(rr + M);               // d', n' per feature; first its scale in .x
+    float* Gp = reinterpret_cast<float*>(dn + M);                 // (x, y < x) at x (x - 1) / 2 + y
     unsigned* q = reinterpret_cast<unsigned*>(Gp + ((size_t)M * (M - 1) / 2 + 36)) + w * kBQ;
     const double inv_n = 1.0 / (double)A.N;
     double B = fmin((double)INFINITY, okey_inv(*(volatile unsigned long long*)A.ub_key));
@@ -270,55 +254,71 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int sli
             }
             P.last = pre[DC - 1];
             P.pre[0] = pre[0]; P.pre[1] = pre[1];
-            const float d0 = A.diag[pre[0]];
-            bool ok = d0 > A.tau;
-            P.inv[0] = 1.f / sqrtf(d0 > 0.f ? d0 : 1.f);
-            P.w[0] = A.b[pre[0]] * P.inv[0];
-            P.pw2 = P.w[0] * P.w[0];
-            P.l10 = 0.f; P.inv[1] = 0.f; P.w[1] = 0.f; P.u[1] = 0.f;
+            const int f0 = pre[0], f1 = max(pre[1], 0);
+            const double d0 = A.Gq[(size_t)f0 * A.n + f0];
+            bool ok = d0 >= 1e-6;
+            double low = d0;
+            P.inv[0] = ok ? 1.0 / sqrt(d0) : 0.0;
+            P.w[0] = A.bq[f0] * P.inv[0];
+            P.l10 = 0.0; P.inv[1] = 0.0; P.w[1] = 0.0;
             if (DC == 2) {
-                P.l10 = A.G[(size_t)pre[1] * A.ldp + pre[0]] * P.inv[0];
-                const float d1 = A.diag[pre[1]] - P.l10 * P.l10;
-                ok = ok && d1 > A.tau;
-                P.inv[1] = 1.f / sqrtf(d1 > 0.f ? d1 : 1.f);
-                P.w[1] = (A.b[pre[1]] - P.l10 * P.w[0]) * P.inv[1];
-                P.pw2 += P.w[1] * P.w[1];
-                P.u[1] = P.w[1] * P.inv[1];
+                P.l10 = A.Gq[(size_t)f1 * A.n + f0] * P.inv[0];
+                const double d1 = A.Gq[(size_t)f1 * A.n + f1] - P.l10 * P.l10;
+                ok = ok && d1 >= 1e-6;
+                low = fmin(low, d1);
+                P.inv[1] = ok ? 1.0 / sqrt(d1) : 0.0;
+                P.w[1] = (A.bq[f1] - P.l10 * P.w[0]) * P.inv[1];
             }
-            P.u[0] = (P.w[0] - P.l10 * P.u[1]) * P.inv[0];
-            P.ok = ok;
+            const double s2 = A.syy64 - P.w[0] * P.w[0] - P.w[1] * P.w[1], share = s2 > 0.0 ? s2 / A.syy64 : 0.0;
+            P.ok = ok && share > 1e-9;
+            P.low = ok ? (float)low : 0.f;
+            P.base = (float)s2;
+            P.e0 = A.e0 * (float)share * 1.01f;
+            P.e1 = A.e1 * (float)sqrt(share) * 1.01f;
         }
         __syncthreads();
-        const int x0 = P.last + 1, m = A.n - x0;                  // local feature x is x0 + x
+        const int x0 = P.last + 1, m = A.n - x0;                  // local feature x is position x0 + x
         if (m < 3) continue;
         // ---- features right of the prefix, then the reduced triangle ---------------------
+        const int q0 = P.pre[0], q1 = max(P.pre[1], 0);
+        // FP64 leaves an error of about 2e-16 (r1^2 / d1 + 2 |r1| / sqrt(d1) + 2) in a reduced
+        // variance h (d1 the second pivot, r1 the feature's value on it): h is resolved to FP32's
+        // rounding where that is below 4e-8 h
+        auto scale_of = [&](double h, double r1d) {
+            const float r1 = fabsf((float)r1d), hf = (float)h;
+            return P.ok && hf > 5e-9f * r1 * r1 / P.low + 1e-8f * r1 * rsqrtf(P.low) + 1e-8f ? rsqrtf(hf) : 0.f;
+        };
         for (int x = tid; x < m; x += W * 32) {
-            const float r0 = A.G[(size_t)P.pre[0] * A.ldp + x0 + x] * P.inv[0];
-            float r1 = 0.f, v1 = 0.f;
-            if (DC == 2) {
-                r1 = (A.G[(size_t)P.pre[1] * A.ldp + x0 + x] - r0 * P.l10) * P.inv[1];
-                v1 = r1 * P.inv[1];
-            }
-            vv[x] = make_float2(r0, r1);                          // R until the triangle is formed
-            dn[x] = make_float2(A.diag[x0 + x] - r0 * r0 - r1 * r1, A.b[x0 + x] - r0 * P.w[0] - r1 * P.w[1]);
+            const int f = x0 + x;
+            const double r0 = A.Gq[(size_t)q0 * A.n + f] * P.inv[0];
+            const double r1 = DC == 2 ? (A.Gq[(size_t)q1 * A.n + f] - r0 * P.l10) * P.inv[1] : 0.0;
+            rr[x] = make_double2(r0, r1);
+            double h = A.Gq[(size_t)f * A.n + f] - r0 * r0;
+            if (DC == 2) h -= r1 * r1;
+            dn[x].x = scale_of(h, r1);
         }
         __syncthreads();
         for (int i = 1 + w; i < m; i += W) {
-            const float2 ri = vv[i];
+            const double2 ri = rr[i];
+            const float si = dn[i].x;
             float* row = Gp + i * (i - 1) / 2;
-            const float* src = A.G + (size_t)(x0 + i) * A.ldp + x0;
+            const double* src = A.Gq + (size_t)(x0 + i) * A.n + x0;
             for (int y = lane; y < i; y += 32) {
-                const float2 ry = vv[y];
-                float v = fmaf(-ri.x, ry.x, src[y]);
-                if (DC == 2) v = fmaf(-ri.y, ry.y, v);
-                row[y] = v;
+                const double2 ry = rr[y];
+                double v = fma(-ri.x, ry.x, src[y]);
+                if (DC == 2) v = fma(-ri.y, ry.y, v);
+                row[y] = scaled_f32(v, 0) * (si * dn[y].x);
             }
         }
         __syncthreads();
+        // variance (one to FP32 rounding; zero: unresolved, every subset kept) and moment
         for (int x = tid; x < m; x += W * 32) {
-            const float2 r = vv[x];
-            const float v1 = DC == 2 ? r.y * P.inv[1] : 0.f;
-            vv[x] = make_float2((r.x - P.l10 * v1) * P.inv[0], v1);
+            const int f = x0 + x;
+            const double2 r = rr[x];
+            const float sc = dn[x].x;
+            double h = A.Gq[(size_t)f * A.n + f] - r.x * r.x, n = A.bq[f] - r.x * P.w[0];
+            if (DC == 2) { h -= r.y * r.y; n -= r.y * P.w[1]; }
+            dn[x] = make_float2(sc > 0.f ? (float)h * sc * sc : 0.f, (float)n * sc);
         }
         __syncthreads();
         // ---- sweep: this warp's p ---------------------------------------------------------
@@ -332,22 +332,20 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int sli
             const unsigned long long next_key = *(volatile unsigned long long*)A.ub_key;     // in flight
             BlockP Q;
             {
-                const float2 f = dn[p], v = vv[p];
+                const float2 f = dn[p];
                 Q.p = p; Q.m = m;
                 Q.ok = P.ok && f.x > A.tau;
                 Q.invd = __frsqrt_rn(f.x > 0.f ? f.x : 1.f);
                 Q.w = f.y * Q.invd;
-                Q.v0 = v.x; Q.v1 = v.y;
-                const float cp = Q.w * Q.invd;
-                Q.A0 = fabsf(cp) + fabsf(fmaf(-cp, v.x, P.u[0]));
-                if (DC == 2) Q.A0 += fabsf(fmaf(-cp, v.y, P.u[1]));
-                Q.base = A.syy - (P.pw2 + Q.w * Q.w);
+                Q.A0 = fabsf(Q.w * Q.invd);
+                Q.base = P.base - Q.w * Q.w;
+                Q.e0 = P.e0; Q.e1 = P.e1;
                 Q.thrN = __fmul_ru((float)((B + A.tie64) * inv_n), 1.0000002f);
             }
             const float invd = Q.invd, wp = Q.w, tau = A.tau;
             float q2 = 0.f, dmax = 0.f;
             for (int x = p + 1 + lane; x < m; x += 32) {
-                const BlockRow f = block_feature<DC>(Q, Gp, dn, vv, x);
+                const BlockRow f = block_feature(Q, Gp, dn, x);
                 q2 = fmaxf(q2, f.l1);
                 dmax = fmaxf(dmax, f.d);
             }
@@ -364,7 +362,7 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int sli
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int i1 = i0 + 32 * (2 * jp + h);
-                        if (i1 < m) c[h] = block_row(A, Q, block_feature<DC>(Q, Gp, dn, vv, i1));
+                        if (i1 < m) c[h] = block_row(A, Q, block_feature(Q, Gp, dn, i1));
                     }
                 }
                 R.nr[jp] = pk2(c[0].nr, c[1].nr); R.nid[jp] = pk2(c[0].nid, c[1].nid); R.nw[jp] = pk2(c[0].nw, c[1].nw);
@@ -382,7 +380,7 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int sli
                     block_col<C>(gr + i0, r, fmaf(-r, r, f.x), fmaf(-r, wp, f.y), i0 + 32 * (C - 1) >= xc, R, zmax, dmin);
                 };
                 auto take = [&](int xc) {
-                    const BlockQueue t = block_take<DC>(A, &P, Q, Gp, dn, vv, rb, xc, q, qn, B);
+                    const BlockQueue t = block_take<DC>(A, &P, Q, Gp, dn, rb, xc, q, qn, B);
                     B = t.B;
                     qn = t.qn;
                     my_cand += t.taken;

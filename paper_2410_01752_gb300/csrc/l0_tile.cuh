@@ -105,6 +105,8 @@ struct TileArgs {
     float* band_r32;
     unsigned long long* examined;
     unsigned long long* candidates;      // subsets sent to the exact test
+    const int* perm;                     // features in the greedy search's order (l0_block.cuh),
+    const double *Gq, *bq;               //   and the FP64 Gram (row stride n) and moments in that order
     const unsigned* prefix_mask;         // optional: one bit per (D-2)-prefix in colex order;
                                          //   prefixes whose bit is clear are skipped
 };
@@ -721,8 +723,10 @@ __global__ void k_prefix_sq(const double* __restrict__ w, int n, const int* __re
 }
 
 // greedy forward selection in FP64: its D-subset's RSS is an upper bound of the minimum
+constexpr int kPermMax = 512;           // features up to which the greedy search's order is asked for
+
 __global__ void k_greedy_bound(const double* __restrict__ G, const double* __restrict__ b, int ld, double syy, int N,
-                               int n, int D, unsigned long long* ub_key) {
+                               int n, int D, unsigned long long* ub_key, int* perm) {
     __shared__ unsigned long long s_key[8];
     __shared__ int s_idx[8];
     __shared__ int sel[kMaxDim];
@@ -759,7 +763,35 @@ __global__ void k_greedy_bound(const double* __restrict__ G, const double* __res
             if (bx >= 0 && t == D - 1) atomicMin(ub_key, bk);
         }
         __syncthreads();
-        if (sel[t] < 0) return;
+        if (sel[t] < 0) {
+            for (int x = threadIdx.x; perm && x < n; x += blockDim.x) perm[x] = x;
+            return;
+        }
+    }
+    // features with a near twin first (FP32 resolves a pair with 1 - rho^2 below 1e-5 only where
+    // the FP64 prefix holds one of them), then by the largest squared correlation with a chosen
+    // feature: the chosen ones and those that could stand in for them
+    if (!perm) return;
+    __shared__ float key[kPermMax];
+    for (int x = threadIdx.x; x < n; x += blockDim.x) {
+        float k = 0.f;
+        for (int j = 0; j < D; ++j) {
+            const float g = (float)G[(size_t)x * ld + sel[j]];
+            k = fmaxf(k, sel[j] == x ? 4.f - 0.1f * (float)j : g * g);
+        }
+        double twin = 0.0;
+#pragma unroll 8
+        for (int y = 0; y < n; ++y) {
+            const double g = G[(size_t)y * ld + x];
+            if (y != x) twin = fmax(twin, fabs(g));
+        }
+        key[x] = twin * twin > 1.0 - 1e-4 ? 8.f + (float)(twin * twin) : k;
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < n; x += blockDim.x) {
+        int at = 0;
+        for (int q = 0; q < n; ++q) at += key[q] > key[x] || (key[q] == key[x] && q < x);
+        perm[at] = x;
     }
 }
 

@@ -157,18 +157,6 @@ __device__ __forceinline__ float log2_abs(double x) {
     return (float)((hi >> 20) - 1023) + log2f(__int_as_float(0x3f800000 | ((hi & 0xfffff) << 3)));
 }
 
-// c 2^k rounded to nearest FP32 (ties to even; below FP32's normal range zero), |result| < 2^127,
-// on the integer pipe: the conversion instruction runs at the FP64 pipe's rate
-__device__ __forceinline__ float scaled_f32(double c, int k) {
-    const unsigned hi = (unsigned)__double2hiint(c), lo = (unsigned)__double2loint(c);
-    const int fe = (int)((hi >> 20) & 0x7ffu) - (1023 - 127) + k;
-    if (fe <= 0) return 0.f;
-    unsigned b = ((unsigned)fe << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-    const unsigned rest = lo & 0x1fffffffu;
-    b += (rest > 0x10000000u) | ((rest == 0x10000000u) & b);
-    return __uint_as_float(b | (hi & 0x80000000u));
-}
-
 // Rows of both sets of one operand: the mean (FP64), the exponent of the largest centred value
 // (from the exponent bits: no FP64 comparison), the scaled rows and their squares.  The FP64
 // pipe is the narrow one on this part (an FP64 warp instruction takes about 18 cycles of an
