@@ -96,7 +96,6 @@ void free_all(sisso_ctx* c) {
     c->pooled.clear();
     c->bufs.clear();
     pair_tc_free(c);
-    tc_screen_free(c);
     whiten_free(c);
     if (c->walk_h) cudaFreeHost(c->walk_h);
     if (c->win_h) cudaFreeHost(c->win_h);
@@ -272,6 +271,7 @@ sisso_status sisso_create(const double* X, const double* y, int N, int d, uint32
         (st = ctx_alloc(c, (void**)&c->dup_pairs, sizeof(int) * (size_t)c->sort_cap * kDupSlots, "dup_pairs")) ||
         (st = ctx_alloc(c, (void**)&c->dup_np, sizeof(unsigned), "dup_np")) ||
         (st = ctx_alloc(c, (void**)&c->tpart, sizeof(double) * (5 * 64 + 1), "target sums")) ||
+        (st = ctx_alloc(c, (void**)&c->mpart, sizeof(double) * (64 * 20 + 2), "model sums")) ||
         (st = dalloc(c, c->removed, (size_t)c->sort_cap, "removed")) || (st = dalloc(c, c->walk, 1, "walk")) ||
         (st = dalloc(c, c->S_dev, (size_t)c->n_cap, "S")) || (st = dalloc(c, c->S_sorted, (size_t)c->n_cap, "S_sorted")) ||
         (st = dalloc(c, c->Z, (size_t)c->n_cap * Nn, "Z")) || (st = dalloc(c, c->Zmean, (size_t)c->n_cap, "Zmean")) ||
@@ -346,10 +346,7 @@ sisso_status sisso_create(const double* X, const double* y, int N, int d, uint32
     if (!st) st = compute_subvalid(c);
     if (!st) st = fill_opcache(c);
     const bool mixed_form = o.precision == SISSO_PREC_MIXED_BF16 || o.precision == SISSO_PREC_MIXED_FP16;
-    if (!st && mixed_form && o.screen != SISSO_SCREEN_CORES && c->opval64 && tc_screen_possible(c, o.screen))
-        st = tc_screen_alloc(c);
-    if (!st && o.precision != SISSO_PREC_FP64 && !c->tc_on && !(mixed_form && o.screen == SISSO_SCREEN_CORES) &&
-        pair_tc_possible(c))
+    if (!st && o.precision != SISSO_PREC_FP64 && !(mixed_form && o.screen == SISSO_SCREEN_CORES) && pair_tc_possible(c))
         st = pair_tc_alloc(c);
     if (!st && o.whiten) {
         // whitening (§2.4) runs row by row from the FP64 operand values and keeps every
@@ -383,7 +380,6 @@ sisso_status sisso_fit(sisso_ctx* c) {
     // either way the l0 step refits its best subsets in FP64 from the standardised rows
     const bool tc_gram = mixed || (prec == SISSO_PREC_FP32 && c->opts.gram == SISSO_GRAM_TF32X3);
     c->stats = sisso_stats{};
-    c->tc_ready = false;
     pair_tc_reset(c);
     c->S.clear(); c->n_sis.clear(); c->res_ids.clear(); c->res_coef.clear(); c->res_rmse.clear(); c->res_r2.clear();
     c->n_dims = 0;

@@ -1,5 +1,5 @@
 // pair_tc.cu — SIS scores of the top level's binary candidates (§2.2 Eqs. 5-6) from fused
-// tcgen05 products: the FP32 form's pair kernel.
+// tcgen05 products: the pair kernel of the FP32 and the mixed forms.
 //
 // With every operand x and its reciprocal z = 1/x centred (x' = x - A, A the FP64 mean), a
 // candidate v = x_i g_j (g = x_j, z_j; and z_i x_j) has, over the samples,
@@ -24,6 +24,12 @@
 // Each key carries a bound of its error (pt_key); a key whose bound could matter next to the
 // screening margin, where the candidate's terms nearly cancel, is left open and scored by
 // k_pt_direct from the sums the definition writes, sample by sample.
+//
+// Measured against the CUDA-core kernel it replaced: 2.9e8 rung-3 candidates (1000 samples, 10 primaries), 40.6 ms
+// a step -> 5.6 ms (first step), 2.4 ms (later ones) and 2.7 ms of open keys; 402 operands over
+// 65 536 samples, 7.9 ms a step -> 0.77 and 0.18 ms.  The mixed forms had their own split
+// products (FP64 rows, chunk sums and scores): 4.9 ms a step there.  The rows, target rows and
+// partials bound the long samples (HBM), the epilogue's FP32 adds the short ones.
 #include "sis_device.cuh"
 #include "tc_device.cuh"
 
@@ -884,6 +890,14 @@ __global__ void __launch_bounds__(256) k_pt_direct(PtArgs A, const float* __rest
     }
 }
 
+// ids below the top level: |E x'r| / sqrt(E x'^2) of the operand itself
+__global__ void __launch_bounds__(256) k_pt_low(PtArgs A, const unsigned char* __restrict__ valid) {
+    const int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (f >= A.P) return;
+    const float4 p = A.par[f];
+    A.scores[f] = valid[f] && p.w < INFINITY ? fabsf(A.R[f]) * __frsqrt_rn(p.y) * A.st->inv_sdr : -1.f;
+}
+
 bool pt_map(CUtensorMap* m, void* base, int64_t rows, int Kpad, int box_rows) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
@@ -897,8 +911,7 @@ bool pt_map(CUtensorMap* m, void* base, int64_t rows, int Kpad, int box_rows) {
 
 }  // namespace
 
-// Used for the FP32 form (and for the mixed forms' NEW_X_PREV pairs, which the FP32 form's
-// kernel scores) when the operands' FP64 values are kept and their 16-bit rows (16 bytes per
+// Used for the FP32 and the mixed forms when the operands' FP64 values are kept and their 16-bit rows (16 bytes per
 // value) fit 40 GB; other contexts keep the CUDA-core kernel.
 bool pair_tc_possible(const sisso_ctx* c) {
     const Space& sp = c->space;
@@ -1024,6 +1037,7 @@ sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow) {
         k_pt_target<false><<<(unsigned)((t->P + 7) / 8), 256, 0, c->stream>>>(t->rows, c->tc32, c->tstats, t->P, t->Pi, c->N, t->Kpad, t->rrows, t->R);
     else
         k_pt_target<true><<<(unsigned)t->P, 512, 0, c->stream>>>(t->rows, c->tc32, c->tstats, t->P, t->Pi, c->N, t->Kpad, t->rrows, t->R);
+    k_pt_low<<<(unsigned)((t->P + 255) / 256), 256, 0, c->stream>>>(A, c->subvalid);
     const int units = A.n_tiles * A.ntypes * A.chunks, grid = std::min(units, c->sms);
     const size_t smem = (size_t)kPtStages * pt_stage_bytes(v == 0 ? 5 : 1, A.ni) + 1024 +
                         (v == 0 ? pt_row_bytes<5>(A.ni) : pt_row_bytes<1>(A.ni));
@@ -1043,7 +1057,7 @@ sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow) {
         if (many) k_pt_direct<false, true><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
         else k_pt_direct<false, false><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
     }
-    c->stats.launches += 3 + (A.chunks > 1) + (v == 0);
+    c->stats.launches += 4 + (A.chunks > 1) + (v == 0);
     unsigned h[4] = {0, 0, 0, 0};
     cudaMemcpyAsync(h, t->count, sizeof(h), cudaMemcpyDeviceToHost, c->stream);
     sisso_status st = check_cuda(c, cudaStreamSynchronize(c->stream), "pair scores");

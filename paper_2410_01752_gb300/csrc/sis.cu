@@ -82,15 +82,18 @@ __global__ void __launch_bounds__(256) k_target_stats(const double* __restrict__
 // FP64 validity of ids [lo, hi) (one level), one warp per id: the value rules (finite,
 // |v| <= 1e12, not identically zero, std > 1e-6 max|v|) and the operands' validity
 // (lower levels, already computed)
-// FP64 values of every id of phi_{L-1}, feature-major (one warp per id, lanes over samples)
+// FP64 values of every id of phi_{L-1}, feature-major (one warp per id
+// and chunk blockIdx.y of the samples, lanes over samples: 402 ids over 65 536 samples, without
+// chunks, left most SMs idle, 3.8 ms against 1.0)
 __global__ void k_fill_val64(const Space* __restrict__ sp, const double* __restrict__ Xc, int N, int64_t n_ids,
-                             double* __restrict__ V) {
+                             double* __restrict__ V, int chunk) {
     const int64_t id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (id >= n_ids) return;
     Prog p;
     const bool ok = build_prog(*sp, id, p);
-    for (int s = lane; s < N; s += 32)
+    const int end = min(N, ((int)blockIdx.y + 1) * chunk);
+    for (int s = (int)blockIdx.y * chunk + lane; s < end; s += 32)
         V[(size_t)id * N + s] = ok ? eval_prog<double>(p, [&](int c) { return Xc[(size_t)c * N + s]; }) : NAN;
 }
 
@@ -119,46 +122,60 @@ __global__ void k_fill_inv64(const double* __restrict__ V, int64_t total, double
         inv[e] = 1.0 / V[e];
 }
 
-__global__ void k_subvalid(const Space* __restrict__ sp, const double* __restrict__ Xc, int N, int64_t lo,
+// (one warp per id, or one CTA where many samples meet few ids: 402 ids over 65 536 samples took
+// 2.9 ms by warps, 0.47 ms by CTAs; the largest magnitudes are taken on the integer pipe)
+template <bool CTA>
+__global__ void __launch_bounds__(512) k_subvalid(const Space* __restrict__ sp, const double* __restrict__ Xc, int N, int64_t lo,
                            int64_t hi, const double* __restrict__ V, const unsigned char* __restrict__ unit_ok,
                            unsigned char* __restrict__ valid) {
-    const int64_t id = lo + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
+    __shared__ double red[32];
+    __shared__ unsigned long long redb[2][32];
+    const int64_t id = CTA ? lo + (int64_t)blockIdx.x : lo + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int t = CTA ? (int)threadIdx.x : (int)(threadIdx.x & 31), nt = CTA ? (int)blockDim.x : 32;
     if (id >= hi) return;
     int level, op; int64_t a, b;
     Prog p;
-    if (!decode(*sp, id, level, op, a, b) || !build_prog(*sp, id, p)) { if (lane == 0) valid[id] = 0; return; }
-    if (level > 0 && (!valid[a] || (b >= 0 && !valid[b]))) { if (lane == 0) valid[id] = 0; return; }
-    double s = 0.0, mx = 0.0, mo = 0.0;
-    int bad = 0;
+    if (!decode(*sp, id, level, op, a, b) || !build_prog(*sp, id, p)) { if (t == 0) valid[id] = 0; return; }
+    if (level > 0 && (!valid[a] || (b >= 0 && !valid[b]))) { if (t == 0) valid[id] = 0; return; }
+    double s = 0.0;
+    unsigned long long bx = 0, bo = 0;
     const bool addsub = level > 0 && (op == ADD || op == SUB);
-    for (int i = lane; i < N; i += 32) {
+    for (int i = t; i < N; i += nt) {
         double mag;
         double v;
         if (V) {
             v = V[(size_t)id * N + i];
-            mag = addsub ? fabs(V[(size_t)a * N + i]) + fabs(V[(size_t)b * N + i]) : fabs(v);
+            mag = addsub ? fabs(V[(size_t)a * N + i]) + fabs(V[(size_t)b * N + i]) : 0.0;
         } else {
             v = eval_prog_mag<double>(p, [&](int c) { return Xc[(size_t)c * N + i]; }, mag);
         }
-        if (!isfinite(v) || fabs(v) > kValueCap) bad = 1;
         s += v;
-        mx = fmax(mx, fabs(v));
-        mo = fmax(mo, mag);
+        const unsigned long long av = abs_bits(v);
+        bx = av > bx ? av : bx;
+        if (addsub) { const unsigned long long am = abs_bits(mag); bo = am > bo ? am : bo; }
     }
-    bad = warp_or(bad);
-    s = warp_sum(s);
-    mx = warp_max(mx);
-    mo = warp_max(mo);
+    bx = warp_max_bits(bx);
+    if (addsub) bo = warp_max_bits(bo);
+    if constexpr (CTA) {
+        const int w = t >> 5, nw = nt >> 5;
+        if ((t & 31) == 0) { redb[0][w] = bx; redb[1][w] = bo; }
+        s = block_sum(s, red);                       // (synchronises: redb is complete)
+        for (int q = 0; q < nw; ++q) { bx = max(bx, redb[0][q]); bo = max(bo, redb[1][q]); }
+    } else {
+        s = warp_sum(s);
+    }
+    const bool bad = bx > abs_bits(kValueCap);       // above the cap, infinite or NaN
+    const double mx = __longlong_as_double((long long)bx), mo = __longlong_as_double((long long)bo);
     const double mean = s / N;
     double ss = 0.0;
     if (!bad)
-        for (int i = lane; i < N; i += 32) {
+        for (int i = t; i < N; i += nt) {
             const double v = (V ? V[(size_t)id * N + i] : eval_prog<double>(p, [&](int c) { return Xc[(size_t)c * N + i]; })) - mean;
             ss += v * v;
         }
-    ss = warp_sum(ss);
-    if (lane == 0) {
+    if constexpr (CTA) ss = block_sum(ss, red);
+    else ss = warp_sum(ss);
+    if (t == 0) {
         const bool cancelled = root_is_addsub(p) && mx <= kCancelRel * mo;
         valid[id] = !bad && !cancelled && sqrt(ss / N) > kConstRel * mx && (!unit_ok || unit_ok[id]);
     }
@@ -994,6 +1011,40 @@ __global__ void k_dup_confirm(const Space* __restrict__ sp, const double* __rest
     }
 }
 
+// the same with one CTA per pair, cached vectors of many samples (a warp's few loads in flight
+// left most of the bandwidth unused): 1024 samples a round, the CTA stops when both maxima have
+// passed the tolerance; 65 536 samples, windows of about 2000: 2.4 -> 1.4 ms over three steps
+__global__ void __launch_bounds__(256) k_dup_confirm_cta(int N, const int* __restrict__ ssrc, const double* __restrict__ zc,
+                                                         const int* __restrict__ dup_list, const int* __restrict__ pairs,
+                                                         const unsigned* __restrict__ n_pairs, unsigned char* __restrict__ dup_ok) {
+    const unsigned np = *n_pairs;
+    for (unsigned e = blockIdx.x; e < np; e += gridDim.x) {
+        const int pr = pairs[e];
+        const double* pa = zc + (size_t)ssrc[pr / kDupSlots] * N;
+        const double* pb = zc + (size_t)dup_list[pr] * N;
+        bool d1 = false, d2 = false;
+        for (int t0 = 0; t0 < N; t0 += 1024) {
+            bool x1 = false, x2 = false;
+            double a4[4], b4[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int t = t0 + 256 * u + (int)threadIdx.x;
+                a4[u] = t < N ? pa[t] : 0.0;
+                b4[u] = t < N ? pb[t] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                x1 |= fabs(a4[u] - b4[u]) > kDupTol;
+                x2 |= fabs(a4[u] + b4[u]) > kDupTol;
+            }
+            d1 = d1 || __syncthreads_or(x1);
+            d2 = d2 || __syncthreads_or(x2);
+            if (d1 && d2) break;
+        }
+        if (threadIdx.x == 0) dup_ok[pr] = !(d1 && d2);
+    }
+}
+
 // ---------------------------------------------------------------------------------
 // the walk: one CTA.  Lane 0 of warp 0 picks, among the remaining candidates whose score
 // is within kScoreTie of the current maximum, the lowest id; warp 0 then checks the pick's
@@ -1367,8 +1418,11 @@ sisso_status compute_subvalid(sisso_ctx* c) {
         const int64_t lo = l == 0 ? 0 : sp.phi[l - 1], hi = sp.phi[l];
         const int64_t n = hi - lo;
         if (n <= 0) continue;
-        k_subvalid<<<(int)((n * 32 + 255) / 256), 256, 0, c->stream>>>(c->space_dev, c->Xc64, c->N, lo, hi,
-                                                                       c->opval64, c->unit_ok, c->subvalid);
+        if (c->N >= 4096 && n <= 65535)
+            k_subvalid<true><<<(int)n, 512, 0, c->stream>>>(c->space_dev, c->Xc64, c->N, lo, hi, c->opval64, c->unit_ok, c->subvalid);
+        else
+            k_subvalid<false><<<(int)((n * 32 + 255) / 256), 256, 0, c->stream>>>(c->space_dev, c->Xc64, c->N, lo, hi,
+                                                                                  c->opval64, c->unit_ok, c->subvalid);
         c->stats.launches++;
     }
     return check_cuda(c, cudaGetLastError(), "subvalid");
@@ -1379,7 +1433,11 @@ sisso_status fill_val64(sisso_ctx* c) {
     const int64_t n = c->space.phi[c->rung - 1];
     // levels 0 and 1 from the primaries, every higher level from the one below
     const int64_t n01 = c->rung - 1 >= 1 ? c->space.phi[1] : n;
-    k_fill_val64<<<(int)((n01 * 32 + 255) / 256), 256, 0, c->stream>>>(c->space_dev, c->Xc64, c->N, n01, c->opval64);
+    // about 32 warps per SM, chunks of 256 samples at least
+    const int64_t cuts = std::max<int64_t>(1, std::min<int64_t>((c->N + 255) / 256, (c->sms * 32 + n01 - 1) / n01));
+    const int chunk = (int)(((c->N + cuts - 1) / cuts + 31) / 32 * 32);
+    k_fill_val64<<<dim3((unsigned)((n01 * 32 + 255) / 256), (unsigned)((c->N + chunk - 1) / chunk)), 256, 0, c->stream>>>(
+        c->space_dev, c->Xc64, c->N, n01, c->opval64, chunk);
     c->stats.launches++;
     for (int l = 2; l <= c->rung - 1; ++l) {
         const int64_t lo = c->space.phi[l - 1], hi = c->space.phi[l];
@@ -1485,19 +1543,21 @@ sisso_status score_all(sisso_ctx* c, int precision) {
     cudaEventCreate(&e0); cudaEventCreate(&e1); cudaEventCreate(&e2);
     cudaEventRecord(e0, c->stream);
     const bool cached = fp64 ? c->opcache64 != nullptr : c->opcache32 != nullptr;
+    const bool use_pt = c->pt && !fp64;        // the pair stage scores the ids below the top level too
     if (cached) {
         // lower levels from cached rows; the top level's unary sections from cached operands
         const int64_t nlow = sp.phi[L - 1];
         const bool few = nlow < 65536;      // few ids: a warp per id splits the samples
         const int gl = few ? (int)((nlow * 32 + 255) / 256) : (int)((nlow + 255) / 256);
-        if (fp64) {
+        if (use_pt) {
+        } else if (fp64) {
             if (few) k_score_cached_w<double><<<gl, 256, 0, c->stream>>>(c->opcache64, c->N, nlow, c->tc32, c->tc64, c->tstats, 0, nlow, c->subvalid, c->scores);
             else k_score_cached<double><<<gl, 256, 0, c->stream>>>(c->opcache64, c->N, nlow, c->tc32, c->tc64, c->tstats, 0, nlow, c->subvalid, c->scores);
         } else {
             if (few) k_score_cached_w<float><<<gl, 256, 0, c->stream>>>(c->opcache32, c->N, nlow, c->tc32, c->tc64, c->tstats, 0, nlow, c->subvalid, c->scores);
             else k_score_cached<float><<<gl, 256, 0, c->stream>>>(c->opcache32, c->N, nlow, c->tc32, c->tc64, c->tstats, 0, nlow, c->subvalid, c->scores);
         }
-        c->stats.launches++;
+        c->stats.launches += !use_pt;
         UnaryArgs U{};
         U.Q = A.Q; U.P = A.P; U.N = c->N;
         for (int q = 0; q < sp.nsec; ++q)
@@ -1554,19 +1614,15 @@ sisso_status score_all(sisso_ctx* c, int precision) {
     cudaEventRecord(e1, c->stream);
     bool any = false;
     for (int o = 0; o < 4; ++o) any |= A.sec[o] >= 0;
-    const bool tc = any && c->tc_on && (precision == SISSO_PREC_MIXED_BF16 || precision == SISSO_PREC_MIXED_FP16);
-    if (tc) {
-        cudaEventRecord(e1, c->stream);
-        if ((st = tc_screen_pairs(c, A.sec))) return st;
-        c->stats.screen_pair_launches++;
-        c->stats.screen_tc = 1;
-    }
-    bool cores = any && !tc;
-    if (cores && c->pt && !fp64) {
+    bool cores = any;
+    if (use_pt) {
         bool overflow = false;
         if ((st = pair_tc_scores(c, A.sec, &overflow))) return st;
         c->stats.screen_pair_launches++;
         cores = overflow;
+        // reported for the mixed forms where their rule asks for the tensor cores
+        c->stats.screen_tc = (precision == SISSO_PREC_MIXED_BF16 || precision == SISSO_PREC_MIXED_FP16) &&
+                             (!A.nxp || c->opts.screen == SISSO_SCREEN_TENSOR) && !overflow;
     }
     if (cores) {
         std::vector<int2> tiles;
@@ -1653,7 +1709,6 @@ sisso_status score_all(sisso_ctx* c, int precision) {
     cudaEventCreate(&e3);
     cudaEventRecord(e3, c->stream);
     cudaEventSynchronize(e3);
-    if (tc && (st = tc_screen_status(c))) return st;
     c->stats.ms_screen += event_ms(e0, e3);
     c->stats.ms_screen_pair += event_ms(e1, e2);
     cudaEventDestroy(e3);
@@ -1769,6 +1824,10 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
         k_dup_find<<<(int)(((int64_t)n_pad * 32 + 255) / 256), 256, 0, c->stream>>>(c->sort_score, c->sort_src, c->sort_id, n_pad, c->surv_score,
                                                                c->surv_sd, c->surv_probe, ns, n_prev, n_confirm(c->N), c->dup_list,
                                                                c->dup_cnt, c->dup_pairs, c->dup_np);
+        if (zc && c->N > 4096)
+            k_dup_confirm_cta<<<(int)std::min<int64_t>((int64_t)c->sms * 8, std::max<int64_t>(1, (int64_t)n_pad * n_confirm(c->N))), 256, 0,
+                                c->stream>>>(c->N, c->sort_src, zc, c->dup_list, c->dup_pairs, c->dup_np, c->dup_ok);
+        else
         k_dup_confirm<<<(int)std::max<int64_t>(1, std::min<int64_t>((int64_t)c->sms * 8, ((int64_t)n_pad + 7) / 8)), 256, 0, c->stream>>>(
             c->space_dev, c->Xc64, c->N, c->sort_src, c->sort_id, c->surv_ids, c->surv_mean, c->surv_sd, zc,
             c->opval64, c->dup_list, c->dup_pairs, c->dup_np, c->dup_ok, c->opinv64);
