@@ -446,6 +446,7 @@ struct sisso_ctx {
     int* sort_src = nullptr;           // index into the survivor arrays
     unsigned char* removed = nullptr;  // walk: visited flags (sort_cap)
     sg::WalkResult* walk = nullptr;    // device
+    void* slab = nullptr;              // pinned memory of walk_h and win_h
     sg::WalkResult* walk_h = nullptr;  // pinned host
     int64_t* S_dev = nullptr;          // S ids (device, acceptance order)
     int64_t* S_sorted = nullptr;       // S ids ascending (device)
@@ -533,6 +534,10 @@ inline int64_t first_window(const sisso_ctx* c, int k);
 
 // a device buffer owned by the context (released with it)
 sisso_status ctx_alloc(sisso_ctx* c, void** p, size_t bytes, const char* what);
+// a temporary from the library's pool on the context's stream, given back with cudaFreeAsync there
+// (the default pool unmaps freed memory at every synchronisation: a step of a 1013-sample fit
+// spent 0.1 ms mapping its temporaries, the 4e6-prefix network inputs 1.5 ms)
+sisso_status tmp_alloc(sisso_ctx* c, void** p, size_t bytes, const char* what);
 
 inline int64_t first_window(const sisso_ctx* c, int k) {
     return c->opts.survivors > 0

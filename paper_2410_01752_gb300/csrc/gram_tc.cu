@@ -379,11 +379,9 @@ static sisso_status gram_tf32x3(sisso_ctx* c, const double* Z, const double* yc,
     float* P = nullptr;
     int* err = nullptr;
     sisso_status st;
-    if ((st = check_cuda(c, cudaMallocAsync((void**)&parts, (size_t)2 * Rpad * Kpad * sizeof(float), c->stream),
-                         "gram_tc tf32 parts")) ||
-        (st = check_cuda(c, cudaMallocAsync((void**)&P, (size_t)splits * pairs * TMT * TNT * sizeof(float), c->stream),
-                         "gram_tc tf32 partials")) ||
-        (st = check_cuda(c, cudaMallocAsync((void**)&err, sizeof(int), c->stream), "gram_tc err")))
+    if ((st = tmp_alloc(c, (void**)&parts, (size_t)2 * Rpad * Kpad * sizeof(float), "gram_tc tf32 parts")) ||
+        (st = tmp_alloc(c, (void**)&P, (size_t)splits * pairs * TMT * TNT * sizeof(float), "gram_tc tf32 partials")) ||
+        (st = tmp_alloc(c, (void**)&err, sizeof(int), "gram_tc err")))
         return st;
     const int g = std::max(1, std::min(c->sms * 8, (int)(((int64_t)Rpad * Kpad + 255) / 256)));
     k_to_tf32x2<<<g, 256, 0, c->stream>>>(Z, yc, 1.0 / sdy, n, N, Rpad, Kpad, parts);
@@ -437,9 +435,9 @@ sisso_status gram_tc(sisso_ctx* c, const double* Z, const double* yc, double sdy
     float* C = nullptr;
     int* err = nullptr;
     sisso_status st;
-    if ((st = check_cuda(c, cudaMallocAsync(&half, (size_t)Rpad * Kpad * 2, c->stream), "gram_tc half")) ||
-        (st = check_cuda(c, cudaMallocAsync((void**)&C, (size_t)Rpad * Rpad * sizeof(float), c->stream), "gram_tc C")) ||
-        (st = check_cuda(c, cudaMallocAsync((void**)&err, sizeof(int), c->stream), "gram_tc err")))
+    if ((st = tmp_alloc(c, (void**)&half, (size_t)Rpad * Kpad * 2, "gram_tc half")) ||
+        (st = tmp_alloc(c, (void**)&C, (size_t)Rpad * Rpad * sizeof(float), "gram_tc C")) ||
+        (st = tmp_alloc(c, (void**)&err, sizeof(int), "gram_tc err")))
         return st;
     const bool bf16 = kind == SISSO_PREC_MIXED_BF16;
     const int g = std::max(1, std::min(c->sms * 8, (int)(((int64_t)Rpad * Kpad + 255) / 256)));
@@ -491,6 +489,7 @@ extern "C" sisso_status sisso_gram_tc(const double* Z, const double* yc, double 
     c.stream = 0;
     int dev = 0;
     cudaGetDevice(&dev);
+    c.opts.device = dev;
     cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev);
     double *dZ = nullptr, *dy = nullptr;
     float *dG = nullptr, *db = nullptr;

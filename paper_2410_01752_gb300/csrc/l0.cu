@@ -676,21 +676,20 @@ sisso_status ensure_tile_buffers(sisso_ctx* c, int n) {
     const int ld = kTC + (n + 31) / 32 * 32;                  // kTC zero columns, then the row
     const int n_tiles = ((n + kTR - 1) / kTR) * ((n + kTC - 1) / kTC);
     if (n <= c->tile_rows && ld <= c->tile_ld && n_tiles <= c->tile_info_cap) return SISSO_OK;
-    cudaStreamSynchronize(c->stream);
-    cudaFree(c->l0_perm); cudaFree(c->l0_Gq);
+    for (void* p : {(void*)c->l0_perm, (void*)c->l0_Gq, (void*)c->tile_G, (void*)c->tile_b, (void*)c->tile_diag, (void*)c->tile_info})
+        if (p) cudaFreeAsync(p, c->stream);
     c->l0_perm = nullptr;
     c->l0_Gq = nullptr;
-    cudaFree(c->tile_G); cudaFree(c->tile_b); cudaFree(c->tile_diag); cudaFree(c->tile_info);
     c->tile_G = c->tile_b = c->tile_diag = nullptr;
     c->tile_info = nullptr;
     c->tile_rows = c->tile_ld = c->tile_info_cap = 0;
     sisso_status st;
-    if ((st = check_cuda(c, cudaMalloc(&c->tile_G, sizeof(float) * (size_t)n * ld), "tile_G")) ||
-        (st = check_cuda(c, cudaMalloc(&c->l0_perm, sizeof(int) * (size_t)n), "l0 order")) ||
-        (st = check_cuda(c, cudaMalloc(&c->l0_Gq, sizeof(double) * (size_t)std::min(n, kBMaxM + 2) * (std::min(n, kBMaxM + 2) + 1)), "l0 reordered Gram")) ||
-        (st = check_cuda(c, cudaMalloc(&c->tile_b, sizeof(float) * (size_t)ld), "tile_b")) ||
-        (st = check_cuda(c, cudaMalloc(&c->tile_diag, sizeof(float) * (size_t)ld), "tile_diag")) ||
-        (st = check_cuda(c, cudaMalloc(&c->tile_info, sizeof(TileInfo) * (size_t)n_tiles), "tile_info")))
+    if ((st = tmp_alloc(c, (void**)&c->tile_G, sizeof(float) * (size_t)n * ld, "tile_G")) ||
+        (st = tmp_alloc(c, (void**)&c->l0_perm, sizeof(int) * (size_t)n, "l0 order")) ||
+        (st = tmp_alloc(c, (void**)&c->l0_Gq, sizeof(double) * (size_t)std::min(n, kBMaxM + 2) * (std::min(n, kBMaxM + 2) + 1), "l0 reordered Gram")) ||
+        (st = tmp_alloc(c, (void**)&c->tile_b, sizeof(float) * (size_t)ld, "tile_b")) ||
+        (st = tmp_alloc(c, (void**)&c->tile_diag, sizeof(float) * (size_t)ld, "tile_diag")) ||
+        (st = tmp_alloc(c, (void**)&c->tile_info, sizeof(TileInfo) * (size_t)n_tiles, "tile_info")))
         return st;
     c->tile_rows = n; c->tile_ld = ld; c->tile_info_cap = n_tiles;
     return SISSO_OK;
@@ -873,12 +872,12 @@ sisso_status l0_certify(sisso_ctx* c, const double* G, const double* b, int ld, 
     unsigned long long* kept = nullptr;
     sisso_status st = SISSO_OK;
     auto ck = [&](cudaError_t e, const char* what) { if (!st && e != cudaSuccess) st = check_cuda(c, e, what); };
-    ck(cudaMallocAsync((void**)&L, sizeof(double) * (size_t)n * n, c->stream), "certificate: factor");
-    ck(cudaMallocAsync((void**)&wv, sizeof(double) * (size_t)n, c->stream), "certificate: w");
-    ck(cudaMallocAsync((void**)&q, sizeof(double) * (size_t)(n + 1), c->stream), "certificate: q");
-    ck(cudaMallocAsync((void**)&m_ok, sizeof(int), c->stream), "certificate: m");
-    ck(cudaMallocAsync((void**)&mask, sizeof(unsigned) * (size_t)words, c->stream), "certificate: mask");
-    ck(cudaMallocAsync((void**)&kept, sizeof(unsigned long long), c->stream), "certificate: count");
+    if (!st) st = tmp_alloc(c, (void**)&L, sizeof(double) * (size_t)n * n, "certificate: factor");
+    if (!st) st = tmp_alloc(c, (void**)&wv, sizeof(double) * (size_t)n, "certificate: w");
+    if (!st) st = tmp_alloc(c, (void**)&q, sizeof(double) * (size_t)(n + 1), "certificate: q");
+    if (!st) st = tmp_alloc(c, (void**)&m_ok, sizeof(int), "certificate: m");
+    if (!st) st = tmp_alloc(c, (void**)&mask, sizeof(unsigned) * (size_t)words, "certificate: mask");
+    if (!st) st = tmp_alloc(c, (void**)&kept, sizeof(unsigned long long), "certificate: count");
     if (!st) {
         const double sst = syy * c->N;
         const double thr = bound0 + 2.0 * kRssTie * sst + 1e-9 * sst + 1e-7 * std::fabs(bound0);

@@ -1009,14 +1009,14 @@ sisso_status l0_learned(sisso_ctx* c, sisso_mlp* mlp, const double* G, const dou
     unsigned* count = nullptr;
     sisso_status st = SISSO_OK;
     auto ck = [&](cudaError_t e, const char* what) { if (!st && e != cudaSuccess) st = check_cuda(c, e, what); };
-    ck(cudaMallocAsync((void**)&Gd, sizeof(double) * n * n, c->stream), "learned: G");
-    ck(cudaMallocAsync((void**)&X, sizeof(float) * np * kIn, c->stream), "learned: inputs");
-    ck(cudaMallocAsync((void**)&plist, sizeof(int) * 3 * np, c->stream), "learned: prefixes");
-    ck(cudaMallocAsync((void**)&sel, sizeof(int) * 3 * np, c->stream), "learned: selection");
+    if (!st) st = tmp_alloc(c, (void**)&Gd, sizeof(double) * n * n, "learned: G");
+    if (!st) st = tmp_alloc(c, (void**)&X, sizeof(float) * np * kIn, "learned: inputs");
+    if (!st) st = tmp_alloc(c, (void**)&plist, sizeof(int) * 3 * np, "learned: prefixes");
+    if (!st) st = tmp_alloc(c, (void**)&sel, sizeof(int) * 3 * np, "learned: selection");
     float* base = nullptr;
-    ck(cudaMallocAsync((void**)&base, sizeof(float) * np, c->stream), "learned: base");
-    ck(cudaMallocAsync((void**)&hist, sizeof(unsigned long long) * 3 * 2048, c->stream), "learned: histogram");
-    ck(cudaMallocAsync((void**)&state, sizeof(unsigned) * 8, c->stream), "learned: state");
+    if (!st) st = tmp_alloc(c, (void**)&base, sizeof(float) * np, "learned: base");
+    if (!st) st = tmp_alloc(c, (void**)&hist, sizeof(unsigned long long) * 3 * 2048, "learned: histogram");
+    if (!st) st = tmp_alloc(c, (void**)&state, sizeof(unsigned) * 8, "learned: state");
     if (st) return st;
     count = state + 4;
     ck(cudaMemcpy2DAsync(Gd, sizeof(double) * n, G, sizeof(double) * ld, sizeof(double) * n, n, cudaMemcpyDeviceToDevice,

@@ -1400,7 +1400,7 @@ sisso_status build_units(sisso_ctx* c) {
     const int64_t words = (n + 31) / 32;
     if ((st = check_cuda(c, cudaMalloc(&c->unit_ok, (size_t)P), "unit_ok")) ||
         (st = check_cuda(c, cudaMalloc(&c->unit_mask, sizeof(unsigned) * (size_t)words), "unit_mask")) ||
-        (st = check_cuda(c, cudaMallocAsync(&d_cls, sizeof(int) * (size_t)P, c->stream), "unit classes")))
+        (st = tmp_alloc(c, (void**)&d_cls, sizeof(int) * (size_t)P, "unit classes")))
         return st;
     cudaMemcpyAsync(c->unit_ok, ok.data(), (size_t)P, cudaMemcpyHostToDevice, c->stream);
     cudaMemcpyAsync(d_cls, cls.data(), sizeof(int) * (size_t)P, cudaMemcpyHostToDevice, c->stream);
@@ -1580,9 +1580,7 @@ sisso_status score_all(sisso_ctx* c, int precision) {
                 const int runs = (int)std::max<int64_t>(1, std::min<int64_t>((c->N + 1023) / 1024,
                                                                              ((int64_t)c->sms * 32 + nz - 1) / nz));
                 double* part = nullptr;
-                const sisso_status su = check_cuda(
-                    c, cudaMallocAsync((void**)&part, sizeof(double) * 3 * (size_t)runs * U.n_ops * nz, c->stream),
-                    "unary partials");
+                const sisso_status su = tmp_alloc(c, (void**)&part, sizeof(double) * 3 * (size_t)runs * U.n_ops * nz, "unary partials");
                 if (su) return su;
                 const int gw = (int)((nz * runs * 32 + 255) / 256), gf = (int)((nz * U.n_ops + 255) / 256);
                 if (fp64) {
@@ -1628,7 +1626,7 @@ sisso_status score_all(sisso_ctx* c, int precision) {
         std::vector<int2> tiles;
         pair_tiles(A.P, A.Q, A.nxp, tiles);
         int2* d_tiles = nullptr;
-        st = check_cuda(c, cudaMallocAsync(&d_tiles, sizeof(int2) * tiles.size(), c->stream), "tiles");
+        st = tmp_alloc(c, (void**)&d_tiles, sizeof(int2) * tiles.size(), "tiles");
         if (st) return st;
         cudaMemcpyAsync(d_tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice, c->stream);
         A.tiles = d_tiles;
