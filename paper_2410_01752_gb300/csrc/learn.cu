@@ -345,42 +345,67 @@ __device__ __forceinline__ int64_t c3(int64_t m) { return m * (m - 1) * (m - 2) 
 __device__ __forceinline__ int64_t c2(int64_t m) { return m * (m - 1) / 2; }
 
 __device__ __forceinline__ void prefix_of(int64_t r, int& p0, int& p1, int& p2) {
-    int64_t m = (int64_t)cbrt(6.0 * (double)r) + 1;
+    int64_t m = (int64_t)cbrtf(6.f * (float)r) + 1;       // estimates; the loops make them exact
     while (m > 2 && c3(m) > r) --m;
     while (c3(m + 1) <= r) ++m;
     p2 = (int)m;
     r -= c3(m);
-    int64_t q = (int64_t)((1.0 + sqrt(1.0 + 8.0 * (double)r)) * 0.5);
+    int64_t q = (int64_t)((1.f + sqrtf(1.f + 8.f * (float)r)) * 0.5f);
     while (q > 1 && c2(q) > r) --q;
     while (c2(q + 1) <= r) ++q;
     p1 = (int)q;
     p0 = (int)(r - c2(q));
 }
 
+// FP32 tables of the prefix features: T[j][e] = G[e][j], b and b / sqrt(syy).  (Converting at
+// every use took most of k_prefix_features: FP64 to FP32 conversions run at the FP64 rate.)
+__global__ void k_prefix_tables(const double* __restrict__ G, const double* __restrict__ b, double inv_sy, int n, int ld,
+                                float* __restrict__ T, float* __restrict__ bf, float* __restrict__ bs) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)n * n; e += (int64_t)gridDim.x * blockDim.x) {
+        const int r = (int)(e / n), c = (int)(e % n);
+        T[(size_t)c * n + r] = (float)G[(size_t)r * ld + c];
+        if (c == 0) { bf[r] = (float)b[r]; bs[r] = (float)(b[r] * inv_sy); }
+    }
+}
+
+// x / l from l's rounded reciprocal, corrected once by its remainder (Markstein): the rounded
+// quotient, without the divide's scaling of extreme exponents
+__device__ __forceinline__ float quot(float x, float l, float rl) {
+    const float q = x * rl;
+    return fmaf(fmaf(-q, l, x), rl, q);
+}
+
 // Greedy completion of a prefix: with E the current positions (m of them) and L, w its
 // Cholesky factor and forward solution, adding feature j lowers RSS / N by c_j^2 / d_j with
 // v = L^-1 G[E][j], d_j = G[j][j] - |v|^2, c_j = b[j] - v . w.  Returns the j > lo that
-// lowers it most (-1 if none) and extends L, w by it.
+// lowers it most (-1 if none) and extends L, w by it.  T is the transposed Gram: neighbouring
+// lanes hold neighbouring E[0] and the same E[1], E[2], so a row of T is read coalesced.
 template <int M>
-__device__ __forceinline__ int greedy_next(const double* __restrict__ G, const double* __restrict__ b, int n,
+__device__ __forceinline__ int greedy_next(const float* __restrict__ T, const float* __restrict__ b, int n,
                                            const int (&E)[5], float (&L)[5][5], float (&w)[5], int lo, int skip) {
     int best = -1;
-    float best_gain = -1.f, bv[5] = {0, 0, 0, 0, 0}, bd = 1.f, bc = 0.f;
+    float best_gain = -1.f, bv[5] = {0, 0, 0, 0, 0}, bd = 1.f, bc = 0.f, rl[5];
+#pragma unroll
+    for (int q = 0; q < M; ++q) rl[q] = 1.f / L[q][q];
     for (int j = lo + 1; j < n; ++j) {
         if (j == skip) continue;
+        const float* row = T + (size_t)j * n;
         float v[5];
-        float d = (float)G[(size_t)j * n + j], c = (float)b[j];
+        float d = __ldg(row + j), c = __ldg(b + j);
 #pragma unroll
         for (int q = 0; q < M; ++q) {
-            float x = (float)G[(size_t)E[q] * n + j];
+            float x = __ldg(row + E[q]);
 #pragma unroll
             for (int r = 0; r < q; ++r) x -= L[q][r] * v[r];
-            v[q] = x / L[q][q];
+            v[q] = quot(x, L[q][q], rl[q]);
             d -= v[q] * v[q];
             c -= v[q] * w[q];
         }
         if (!(d > 1e-6f)) continue;
-        const float gain = c * c / d;
+        // divided only where the quotient could exceed the best one
+        const float cc = c * c;
+        if (!(cc >= 0.999999f * (best_gain * d))) continue;
+        const float gain = cc / d;
         if (gain > best_gain) {
             best_gain = gain; best = j; bd = d; bc = c;
 #pragma unroll
@@ -401,9 +426,13 @@ __device__ __forceinline__ int greedy_next(const double* __restrict__ G, const d
 // E = (p0, p1, p2, j1, j2): the upper triangle of its standardised sub-Gram in row order,
 // then its correlations b_i / sqrt(syy).  A prefix without two such features keeps zeros
 // in the missing slots (it has no extension either).  base (optional): log10 of the
-// completion's RSS / SST, the score the network corrects.
-__global__ void k_prefix_features(const double* __restrict__ G, const double* __restrict__ b, double inv_sy, int n,
-                                  int64_t n_pre, float* __restrict__ X, int* __restrict__ plist,
+// completion's RSS / SST, the score the network corrects.  T, b, bs: k_prefix_tables.
+// X: FP32 rows of kIn values, or (Xb) the network's rows, 16-bit and padded to kInPad.
+// Bound by the FP32 pipe: about 70 instructions per prefix and feature right of it, 2 C(n, 4) of
+// them; 4.45e6 prefixes of 300 features 6.3 -> 1.66 ms (and the copy into the network's rows, 0.28 ms, saved).
+__global__ void __launch_bounds__(256) k_prefix_features(const float* __restrict__ T, const float* __restrict__ b,
+                                  const float* __restrict__ bs, double inv_sy, int n,
+                                  int64_t n_pre, float* __restrict__ X, __nv_bfloat16* __restrict__ Xb, int* __restrict__ plist,
                                   float* __restrict__ base) {
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n_pre; r += (int64_t)gridDim.x * blockDim.x) {
         int E[5] = {0, 0, 0, -1, -1};
@@ -411,39 +440,75 @@ __global__ void k_prefix_features(const double* __restrict__ G, const double* __
         // Cholesky of the prefix (FP32; a singular prefix gets no completion)
         float L[5][5] = {}, w[5] = {};
         bool ok = true;
-        for (int q = 0; q < 3 && ok; ++q) {
-            float d = (float)G[(size_t)E[q] * n + E[q]];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            float d = T[(size_t)E[q] * n + E[q]];
+#pragma unroll
             for (int m = 0; m < q; ++m) d -= L[q][m] * L[q][m];
-            if (!(d > 1e-6f)) { ok = false; break; }
+            if (!(d > 1e-6f)) { ok = false; d = 1.f; }
             L[q][q] = sqrtf(d);
+#pragma unroll
             for (int i = q + 1; i < 3; ++i) {
-                float x = (float)G[(size_t)E[i] * n + E[q]];
+                float x = T[(size_t)E[q] * n + E[i]];
+#pragma unroll
                 for (int m = 0; m < q; ++m) x -= L[i][m] * L[q][m];
                 L[i][q] = x / L[q][q];
             }
-            float v = (float)b[E[q]];
+            float v = b[E[q]];
+#pragma unroll
             for (int m = 0; m < q; ++m) v -= L[q][m] * w[m];
             w[q] = v / L[q][q];
         }
         if (ok) {
-            E[3] = greedy_next<3>(G, b, n, E, L, w, E[2], -1);
-            if (E[3] >= 0) E[4] = greedy_next<4>(G, b, n, E, L, w, E[2], E[3]);
+            E[3] = greedy_next<3>(T, b, n, E, L, w, E[2], -1);
+            if (E[3] >= 0) E[4] = greedy_next<4>(T, b, n, E, L, w, E[2], E[3]);
         }
         // base score: log10 of the greedy completion's RSS / SST = 1 - |w|^2 syy^-1
         if (base) {
             float q = 0.f;
+#pragma unroll
             for (int i = 0; i < 5; ++i) q += (ok && E[4] >= 0) ? w[i] * w[i] : 0.f;
             const float frac = (ok && E[4] >= 0) ? 1.f - q * (float)(inv_sy * inv_sy) : 1.f;
             base[r] = log10f(fmaxf(frac, 1e-12f));
         }
-        float* x = X + r * kIn;
+        float x[24] = {};
         int q = 0;
+#pragma unroll
         for (int i = 0; i < 5; ++i)
+#pragma unroll
             for (int j = i; j < 5; ++j, ++q)
-                x[q] = (E[i] >= 0 && E[j] >= 0) ? (float)G[(size_t)E[i] * n + E[j]] : 0.f;
-        for (int i = 0; i < 5; ++i) x[15 + i] = E[i] >= 0 ? (float)(b[E[i]] * inv_sy) : 0.f;
+                x[q] = (E[i] >= 0 && E[j] >= 0) ? T[(size_t)E[j] * n + E[i]] : 0.f;
+#pragma unroll
+        for (int i = 0; i < 5; ++i) x[15 + i] = E[i] >= 0 ? bs[E[i]] : 0.f;
+        if (Xb) {
+            uint4* o = reinterpret_cast<uint4*>(Xb + r * kInPad);
+#pragma unroll
+            for (int g = 0; g < kInPad / 8; ++g) {
+                __nv_bfloat162 h[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int k = 8 * g + 2 * u;
+                    h[u] = k < 24 ? __floats2bfloat162_rn(x[k], x[k + 1]) : __floats2bfloat162_rn(0.f, 0.f);
+                }
+                o[g] = *reinterpret_cast<const uint4*>(h);
+            }
+        } else {
+            float4* o = reinterpret_cast<float4*>(X + r * kIn);
+#pragma unroll
+            for (int g = 0; g < kIn / 4; ++g) o[g] = make_float4(x[4 * g], x[4 * g + 1], x[4 * g + 2], x[4 * g + 3]);
+        }
         if (plist) { plist[3 * r] = E[0]; plist[3 * r + 1] = E[1]; plist[3 * r + 2] = E[2]; }
     }
+}
+
+// the tables (n (n + 2) floats at `tab`) and the features, on one stream
+void prefix_features(cudaStream_t s, const double* G, const double* b, int ld, double syy, int n, int64_t np, float* tab,
+                     float* X, __nv_bfloat16* Xb, int* plist, float* base) {
+    float *bf = tab + (size_t)n * n, *bs = bf + n;
+    const double inv_sy = 1.0 / std::sqrt(syy);
+    k_prefix_tables<<<std::min(1024, (n * n + 255) / 256), 256, 0, s>>>(G, b, inv_sy, n, ld, tab, bf, bs);
+    k_prefix_features<<<(unsigned)std::min<int64_t>((np + 255) / 256, 65535), 256, 0, s>>>(tab, bf, bs, inv_sy, n, np, X, Xb,
+                                                                                           plist, base);
 }
 
 __device__ __forceinline__ unsigned fkey32(float v) {
@@ -508,13 +573,23 @@ __global__ void k_wsel_hist(const float* __restrict__ score, const int* __restri
 // (one 64-bit value, 8-byte aligned), [4] compacted count
 __global__ void k_wsel_find(const unsigned long long* __restrict__ hist, int pass, unsigned* state,
                             unsigned long long budget) {
-    if (threadIdx.x != 0) return;
     unsigned long long* rest = reinterpret_cast<unsigned long long*>(state + 2);
-    const int nb = pass == 2 ? 1024 : 2048;
+    const int nb = pass == 2 ? 1024 : 2048, lane = threadIdx.x, per = nb / 32;
     const unsigned long long need = pass == 0 ? budget : *rest;
-    unsigned long long cum = 0;
+    // each lane sums its run of bins, and the lane that reaches the weight walks its run
+    unsigned long long mine = 0;
+    for (int q = 0; q < per; ++q) mine += hist[pass * 2048 + lane * per + q];
+    unsigned long long incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    const unsigned hit = __ballot_sync(0xffffffffu, incl >= need);
+    if (lane != (hit ? __ffs(hit) - 1 : 31)) return;
+    unsigned long long cum = incl - mine;
     int bin = nb - 1;
-    for (int q = 0; q < nb; ++q) {
+    for (int q = lane * per; q < (lane + 1) * per; ++q) {
         const unsigned long long c = hist[pass * 2048 + q];
         if (cum + c >= need) { bin = q; break; }
         cum += c;
@@ -859,7 +934,9 @@ sisso_status sisso_prefix_features(const double* G, const double* b, double syy,
     double *dG = nullptr, *db = nullptr;
     float *dX = nullptr, *dB = nullptr;
     int* dP = nullptr;
+    float* dT = nullptr;
     bool ok = cudaMalloc((void**)&dG, sizeof(double) * n * n) == cudaSuccess &&
+              cudaMalloc((void**)&dT, sizeof(float) * n * (n + 2)) == cudaSuccess &&
               cudaMalloc((void**)&db, sizeof(double) * n) == cudaSuccess &&
               cudaMalloc((void**)&dX, sizeof(float) * np * kIn) == cudaSuccess &&
               (!prefixes || cudaMalloc((void**)&dP, sizeof(int) * 3 * np) == cudaSuccess) &&
@@ -868,15 +945,14 @@ sisso_status sisso_prefix_features(const double* G, const double* b, double syy,
     if (ok) {
         cudaMemcpy(dG, G, sizeof(double) * n * n, cudaMemcpyDefault);
         cudaMemcpy(db, b, sizeof(double) * n, cudaMemcpyDefault);
-        k_prefix_features<<<(unsigned)std::min<int64_t>((np + 255) / 256, 65535), 256>>>(dG, db, 1.0 / std::sqrt(syy), n,
-                                                                                          np, dX, dP, dB);
+        prefix_features(0, dG, db, n, syy, n, np, dT, dX, nullptr, dP, dB);
         if (cudaMemcpy(out, dX, sizeof(float) * np * kIn, cudaMemcpyDefault) != cudaSuccess) st = SISSO_ERR_CUDA;
         if (!st && prefixes && cudaMemcpy(prefixes, dP, sizeof(int) * 3 * np, cudaMemcpyDefault) != cudaSuccess)
             st = SISSO_ERR_CUDA;
         if (!st && base && cudaMemcpy(base, dB, sizeof(float) * np, cudaMemcpyDefault) != cudaSuccess) st = SISSO_ERR_CUDA;
     }
     cudaGetLastError();
-    cudaFree(dG); cudaFree(db); cudaFree(dX); cudaFree(dP); cudaFree(dB);
+    cudaFree(dG); cudaFree(db); cudaFree(dX); cudaFree(dP); cudaFree(dB); cudaFree(dT);
     return st;
 }
 
@@ -964,21 +1040,21 @@ sisso_status sisso_prefix_training(const double* G, const double* b, double syy,
         return SISSO_ERR_ARG;
     const int64_t np = (int64_t)n * (n - 1) * (n - 2) / 6;
     double *dG = nullptr, *db = nullptr;
-    float *dX = nullptr, *dB = nullptr;
+    float *dX = nullptr, *dB = nullptr, *dT = nullptr;
     sisso_status st = SISSO_OK;
-    if (cudaMalloc((void**)&dG, sizeof(double) * n * n) != cudaSuccess || cudaMalloc((void**)&db, sizeof(double) * n) != cudaSuccess ||
+    if (cudaMalloc((void**)&dT, sizeof(float) * n * (n + 2)) != cudaSuccess ||
+        cudaMalloc((void**)&dG, sizeof(double) * n * n) != cudaSuccess || cudaMalloc((void**)&db, sizeof(double) * n) != cudaSuccess ||
         cudaMalloc((void**)&dX, sizeof(float) * np * kIn) != cudaSuccess || cudaMalloc((void**)&dB, sizeof(float) * np) != cudaSuccess)
         st = SISSO_ERR_OOM;
     if (!st) {
         cudaMemcpy(dG, G, sizeof(double) * n * n, cudaMemcpyDefault);
         cudaMemcpy(db, b, sizeof(double) * n, cudaMemcpyDefault);
-        k_prefix_features<<<(unsigned)std::min<int64_t>((np + 255) / 256, 65535), 256>>>(dG, db, 1.0 / std::sqrt(syy), n,
-                                                                                          np, dX, nullptr, dB);
+        prefix_features(0, dG, db, n, syy, n, np, dT, dX, nullptr, nullptr, dB);
         if (cudaMemcpy(inputs, dX, sizeof(float) * np * kIn, cudaMemcpyDeviceToHost) != cudaSuccess) st = SISSO_ERR_CUDA;
         if (!st) st = sg::prefix_labels_dev(G, b, syy, N, n, dB, labels, targets);
     }
     cudaGetLastError();
-    cudaFree(dG); cudaFree(db); cudaFree(dX); cudaFree(dB);
+    cudaFree(dG); cudaFree(db); cudaFree(dX); cudaFree(dB); cudaFree(dT);
     return st;
 }
 
@@ -998,9 +1074,7 @@ sisso_status l0_learned(sisso_ctx* c, sisso_mlp* mlp, const double* G, const dou
                         int64_t* n_selected) {
     if (n < 5 || n > 1400) return fail(c, SISSO_ERR_ARG, "learned l0: n must be in 5..1400");
     const int64_t np = (int64_t)n * (n - 1) * (n - 2) / 6;
-    // the network reads a dense n x n Gram
-    double* Gd = nullptr;
-    float* X = nullptr;
+    float* tab = nullptr;
     int* plist = nullptr;
     int* sel = nullptr;
     float* score = nullptr;
@@ -1009,8 +1083,7 @@ sisso_status l0_learned(sisso_ctx* c, sisso_mlp* mlp, const double* G, const dou
     unsigned* count = nullptr;
     sisso_status st = SISSO_OK;
     auto ck = [&](cudaError_t e, const char* what) { if (!st && e != cudaSuccess) st = check_cuda(c, e, what); };
-    if (!st) st = tmp_alloc(c, (void**)&Gd, sizeof(double) * n * n, "learned: G");
-    if (!st) st = tmp_alloc(c, (void**)&X, sizeof(float) * np * kIn, "learned: inputs");
+    if (!st) st = tmp_alloc(c, (void**)&tab, sizeof(float) * n * (n + 2), "learned: tables");
     if (!st) st = tmp_alloc(c, (void**)&plist, sizeof(int) * 3 * np, "learned: prefixes");
     if (!st) st = tmp_alloc(c, (void**)&sel, sizeof(int) * 3 * np, "learned: selection");
     float* base = nullptr;
@@ -1019,11 +1092,7 @@ sisso_status l0_learned(sisso_ctx* c, sisso_mlp* mlp, const double* G, const dou
     if (!st) st = tmp_alloc(c, (void**)&state, sizeof(unsigned) * 8, "learned: state");
     if (st) return st;
     count = state + 4;
-    ck(cudaMemcpy2DAsync(Gd, sizeof(double) * n, G, sizeof(double) * ld, sizeof(double) * n, n, cudaMemcpyDeviceToDevice,
-                         c->stream), "learned: G copy");
-    k_prefix_features<<<(unsigned)std::min<int64_t>((np + 255) / 256, 65535), 256, 0, c->stream>>>(
-        Gd, b, 1.0 / std::sqrt(syy), n, np, X, plist, base);
-    // network scores (on the network's stream, ordered after the features)
+    // features straight into the network's rows, and its scores (on the network's stream)
     sisso_status sm = mlp_reserve(mlp, np, false);
     if (sm) return fail(c, sm, "learned: network buffers");
     cudaEvent_t ev;
@@ -1031,8 +1100,8 @@ sisso_status l0_learned(sisso_ctx* c, sisso_mlp* mlp, const double* G, const dou
     cudaEventRecord(ev, c->stream);
     cudaStreamWaitEvent(mlp->stream, ev, 0);
     const int64_t Mpad = pad128(np);
-    k_pack_x<<<(unsigned)std::min<int64_t>((Mpad * kInPad + 255) / 256, 65535), 256, 0, mlp->stream>>>(X, np, Mpad,
-                                                                                                          mlp->Xb, nullptr);
+    prefix_features(mlp->stream, G, b, ld, syy, n, np, tab, nullptr, mlp->Xb, plist, base);
+    cudaMemsetAsync(mlp->Xb + np * kInPad, 0, sizeof(__nv_bfloat16) * (size_t)(Mpad - np) * kInPad, mlp->stream);
     ck(mlp_forward_dev(mlp, np, false), "learned: network");
     score = mlp->out;
     cudaEventRecord(ev, mlp->stream);
@@ -1051,7 +1120,7 @@ sisso_status l0_learned(sisso_ctx* c, sisso_mlp* mlp, const double* G, const dou
         k_wsel_find<<<1, 32, 0, c->stream>>>(hist, pass, state, budget);
     }
     k_wsel_compact<<<gs, 256, 0, c->stream>>>(score, plist, np, state, sel, count, np, nullptr);
-    c->stats.launches += 13;   // features, pack, 2 layers + head, add, 3 x (histogram, find), compact
+    c->stats.launches += 13;   // tables, features, 2 layers + head, add, 3 x (histogram, find), compact
     unsigned h_count = 0;
     cudaMemcpyAsync(&h_count, count, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream);
     ck(cudaStreamSynchronize(c->stream), "learned: selection");
@@ -1064,7 +1133,7 @@ sisso_status l0_learned(sisso_ctx* c, sisso_mlp* mlp, const double* G, const dou
         *n_selected = h_count;
         st = l0_solve(c, G, b, G32, b32, ld, syy, n, 5, gid_dev, SISSO_PREC_FP32, w, sel, (int64_t)h_count);
     }
-    cudaFreeAsync(Gd, c->stream); cudaFreeAsync(X, c->stream); cudaFreeAsync(plist, c->stream);
+    cudaFreeAsync(tab, c->stream); cudaFreeAsync(plist, c->stream);
     cudaFreeAsync(sel, c->stream); cudaFreeAsync(hist, c->stream); cudaFreeAsync(state, c->stream);
     cudaFreeAsync(base, c->stream);
     return st;

@@ -621,6 +621,74 @@ __global__ void k_compact(const float* __restrict__ scores, int64_t n, const uns
     }
 }
 
+// narrows a window of n <= kNarrowMax entries before its FP64 work: keeps the entries whose key
+// is within `margin` of the key of rank `want` or above it (the rank found to within an eighth,
+// by bisection on the keys' bits), and lowers nothing else -- the threshold key in state[2]
+// rises to the smallest kept, and state[3] (every candidate is in the window) is cleared.  A walk
+// that visits at most `want` candidates then proves its selection with this window; one that
+// does not is repeated with the whole window.
+constexpr int kNarrowMax = 8192, kNarrowThreads = 1024, kNarrowPer = kNarrowMax / kNarrowThreads;
+__global__ void __launch_bounds__(kNarrowThreads) k_narrow(const float* __restrict__ scores, int64_t* __restrict__ ids,
+                                                           unsigned* count, unsigned* state, int want, float margin) {
+    __shared__ unsigned red[2][32];
+    __shared__ unsigned kept;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const unsigned n = *count;
+    if (n > (unsigned)kNarrowMax || n <= 2u * (unsigned)want) return;
+    const unsigned thr = max(state[2], 1u);
+    int64_t id[kNarrowPer];
+    unsigned key[kNarrowPer], top = 0;
+#pragma unroll
+    for (int q = 0; q < kNarrowPer; ++q) {
+        const unsigned i = q * kNarrowThreads + t;
+        id[q] = i < n ? ids[i] : -1;
+        key[q] = i < n ? key_of(scores[id[q]]) : 0u;
+        top = max(top, key[q]);
+    }
+    if (t == 0) kept = 0;
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0) red[1][w] = top;
+    __syncthreads();
+    top = __reduce_max_sync(0xffffffffu, red[1][lane]);
+    int buf = 0;
+    auto above = [&](unsigned v) {                  // entries with a key of v or more
+        unsigned c = 0;
+#pragma unroll
+        for (int q = 0; q < kNarrowPer; ++q) c += key[q] >= v;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) red[buf][w] = c;
+        __syncthreads();
+        c = __reduce_add_sync(0xffffffffu, red[buf][lane]);
+        buf ^= 1;
+        return c;
+    };
+    unsigned lo = thr, hi = top + 1u;               // above(lo) >= want > above(hi)
+    while (hi - lo > 1u) {
+        const unsigned mid = lo + (hi - lo) / 2u, c = above(mid);
+        if (c >= (unsigned)want) {
+            lo = mid;
+            if (c <= (unsigned)(want + want / 8)) break;
+        } else {
+            hi = mid;
+        }
+    }
+    const float low = __uint_as_float(lo) - margin;
+    const unsigned cut = max(low > 0.f ? __float_as_uint(low) : 1u, thr);
+    if (cut <= thr) return;
+    const unsigned keep = above(cut);
+    if (keep > n - n / 4u) return;
+#pragma unroll
+    for (int q = 0; q < kNarrowPer; ++q) {
+        const bool in = key[q] >= cut;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        unsigned base = 0;
+        if (lane == 0 && m) base = atomicAdd(&kept, (unsigned)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (in) ids[base + __popc(m & ((1u << lane) - 1u))] = id[q];
+    }
+    if (t == 0) { *count = keep; state[2] = cut; state[3] = 0; }
+}
+
 // ---------------------------------------------------------------------------------
 // FP64 re-score: one warp per id, lanes over samples.  Applies the exact validity rules
 // (every |v| <= 1e12 and finite, not identically zero, std > 1e-6 max|v|), computes the
@@ -1741,6 +1809,11 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
     const bool fp_kernel64 = c->opts.precision == SISSO_PREC_FP64;
     const double eps = fp_kernel64 ? kScoreErr64 : kScoreErr32;   // bound on |score_kernel - score_FP64|
     int64_t M = first_window(c, k);
+    // the default window holds thousands of candidates so that it proves dense selections too; the
+    // FP64 work of most steps needs the best few hundred: walks visit 1.2 to 4.4 k candidates, so
+    // rank 5 k (at 3 k one step in twelve was repeated).  1013 samples, k = 50: 12 438 -> 636 candidates
+    // re-scored over three steps, 3.1 -> 2.6 ms a fit
+    bool narrow = c->opts.survivors <= 0;
     const int64_t n = c->n_feat;
     const int gridS = std::max(1, c->sms * 8);
     cudaEvent_t q[5];
@@ -1759,6 +1832,11 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
         k_compact<<<gridS, kBlock, 0, c->stream>>>(c->scores, n, c->sel_state, c->surv_ids, c->surv_count,
                                                    c->surv_cap - n_prev);
         c->stats.launches++;
+        if (narrow && M <= kNarrowMax) {
+            k_narrow<<<1, kNarrowThreads, 0, c->stream>>>(c->scores, c->surv_ids, c->surv_count, c->sel_state, 5 * k,
+                                                          (float)(2.25 * eps + 8.0 * kScoreTie));
+            c->stats.launches++;
+        }
         unsigned h_state[4], h_count = 0;
         cudaMemcpyAsync(h_state, c->sel_state, sizeof(h_state), cudaMemcpyDeviceToHost, c->stream);
         cudaMemcpyAsync(&h_count, c->surv_count, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream);
@@ -1855,6 +1933,7 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
         const double thr = c->opts.sis_threshold;
         const bool safe = all || (w.n_acc == k && w.last_score - kScoreTie > (double)t32 + eps) ||
                           (w.thr_stop && (double)t32 + eps < thr - kScoreTie);
+        if (!safe && narrow) { narrow = false; continue; }
         const bool can_grow = M < c->surv_cap - n_prev;
         if (safe || !can_grow) {
             if (!safe) c->stats.window_saturated = 1;
