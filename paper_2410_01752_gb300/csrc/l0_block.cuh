@@ -22,9 +22,14 @@
 // subset that holds them nearly ties, they are the prefix, and FP32 still tells those subsets
 // apart (eliminated in FP32 and in the order of screening, up to 5.4e7 of the 1.96e10 subsets of
 // such problems went to FP64 solves, which then took longer than the sweep).
-// Measured at n = 300, D = 5 (1.96e10 subsets): see the figures at the launch (l0.cu).  Forms
-// that took longer than k_l0_tile's 43 ms: lanes as columns with the row constants shuffled in
-// (89 ms), and four warps sharing a p through a record table and a barrier (46 ms).
+// The sweep runs a shorter test that implies the filter (block_sweep_row) and only marks the
+// columns it does not dismiss; they are decided after the sweep, so that no call stands between the
+// row constants and their registers (with the calls inside, a third of the instructions were
+// spills' and their operands').
+// Measured at n = 300, D = 5 (1.96e10 subsets) over five problems: 20 to 25 ms (30 to 36 with the
+// filter itself in the sweep, 43 and more by k_l0_tile); 0.6 warp instructions a subset at 56% of
+// the issue slots.  Forms that took longer than k_l0_tile: lanes as columns with the row constants
+// shuffled in (89 ms), and four warps sharing a p through a record table and a barrier (46 ms).
 #pragma once
 
 #include "l0_tile.cuh"
@@ -38,7 +43,7 @@ namespace {
 // up to kBSmallM features, four and four CTAs per SM, so that a unit's barriers hold up few warps
 // (three quarters of the prefixes of n = 300 have that few features to the right)
 constexpr int kBWarpsBig = 16, kBWarpsSmall = 4, kBSmallM = 150;
-constexpr int kBRow = 6;                  // row groups of 32 swept together (their constants are 36 registers)
+constexpr int kBRow = 6;                  // row groups of 32 swept together (their constants are 30 registers)
 constexpr int kBQ = 64;                   // per-warp candidate queue
 constexpr int kBMaxM = 320;               // features right of the CTA's prefix (204 KB triangle)
 
@@ -98,9 +103,9 @@ __device__ __noinline__ double block_flush(const TileArgs& A, const BlockPre* P,
     return fmin(B, okey_inv(*(volatile unsigned long long*)A.ub_key));
 }
 
-// the filter's row constants of a lane (l0_tile.cuh), row groups j and j + 1 per register pair:
-// -R[p][i1], -1/d1, -w1/sqrt(d1), -K, beta, gamma
-struct RowsC { p2 nr[kBRow / 2], nid[kBRow / 2], nw[kBRow / 2], nK[kBRow / 2], be[kBRow / 2], gm[kBRow / 2]; };
+// the sweep's row constants of a lane, row groups j and j + 1 per register pair: -R[p][i1],
+// -1/d1, -w1/sqrt(d1), -K2 and c (block_sweep_row)
+struct RowsC { p2 nr[kBRow / 2], nid[kBRow / 2], nw[kBRow / 2], nK[kBRow / 2], c[kBRow / 2]; };
 
 // the test of one subset: z < 0 and d2 > tau dismiss it
 __device__ __forceinline__ void block_test(float gv, float r, float d, float n, float nr, float nid, float nw, float nK,
@@ -111,40 +116,33 @@ __device__ __forceinline__ void block_test(float gv, float r, float d, float n, 
     z = fmaf(fmaf(beta, fabsf(num), fmaf(nK, d2, n2)), d2, gamma * n2);
 }
 
-// one column (r, d, n; gx its row of G' at this lane's rows) against C row groups: the largest z
-// and the smallest d2 are folded into zmax and dmin.  dead: this lane's row of the last group is
-// not left of x
+// one column (r, d, n; gx its row of G' at this lane's rows) against C row groups with the sweep's
+// test, num^2 - K2 d2 + c < 0: the largest value is folded into zmax.  dead: this lane's row of
+// the last group is not left of x
 template <int C>
 __device__ __forceinline__ void block_col(const float* gx, float r, float d, float n, bool dead, const RowsC& R,
-                                          float& zmax, float& dmin) {
+                                          float& zmax) {
     float gv[C];
 #pragma unroll
     for (int j = 0; j < C; ++j) gv[j] = gx[32 * j];
-    if (C > 1) {
-        const p2 rx = pk2(r, r), dx = pk2(d, d), nx = pk2(n, n);
+    const p2 rx = pk2(r, r), dx = pk2(d, d), nx = pk2(n, n);
 #pragma unroll
-        for (int jp = 0; jp < C / 2; ++jp) {
-            const p2 g = fma2(R.nr[jp], rx, pk2(gv[2 * jp], gv[2 * jp + 1]));
-            const p2 d2 = fma2(mul2(g, g), R.nid[jp], dx);
-            const p2 num = fma2(g, R.nw[jp], nx);
-            const p2 n2 = mul2(num, num);
-            const p2 h = fma2(R.nK[jp], d2, n2);
-            float da, db, na, nb, ha, hb, za, zb, ba, bb;
-            up2(d2, da, db); up2(num, na, nb); up2(h, ha, hb); up2(R.be[jp], ba, bb);
-            const p2 z = fma2(pk2(fmaf(ba, fabsf(na), ha), fmaf(bb, fabsf(nb), hb)), d2, mul2(R.gm[jp], n2));
-            up2(z, za, zb);
-            if (2 * jp + 1 == C - 1 && dead) { zb = -INFINITY; db = INFINITY; }
-            zmax = fmaxf(fmaxf(zmax, za), zb);
-            dmin = fminf(fminf(dmin, da), db);
-        }
+    for (int jp = 0; jp < C / 2; ++jp) {
+        const p2 g = fma2(R.nr[jp], rx, pk2(gv[2 * jp], gv[2 * jp + 1]));
+        const p2 d2 = fma2(mul2(g, g), R.nid[jp], dx);
+        const p2 num = fma2(g, R.nw[jp], nx);
+        float za, zb;
+        up2(fma2(num, num, fma2(R.nK[jp], d2, R.c[jp])), za, zb);
+        if (2 * jp + 1 == C - 1 && dead) zb = -INFINITY;
+        zmax = fmaxf(fmaxf(zmax, za), zb);
     }
     if (C & 1) {
         constexpr int h = C / 2;
-        float nr, nid, nw, nK, be, gm, u, z, d2;
-        up2(R.nr[h], nr, u); up2(R.nid[h], nid, u); up2(R.nw[h], nw, u);
-        up2(R.nK[h], nK, u); up2(R.be[h], be, u); up2(R.gm[h], gm, u);
-        block_test(gv[C - 1], r, d, n, nr, nid, nw, nK, be, gm, z, d2);
-        if (!dead) { zmax = fmaxf(zmax, z); dmin = fminf(dmin, d2); }
+        float nr, nid, nw, nK, c, u;
+        up2(R.nr[h], nr, u); up2(R.nid[h], nid, u); up2(R.nw[h], nw, u); up2(R.nK[h], nK, u); up2(R.c[h], c, u);
+        const float g = fmaf(nr, r, gv[C - 1]), d2 = fmaf(g * g, nid, d), num = fmaf(g, nw, n);
+        const float z = fmaf(num, num, fmaf(nK, d2, c));
+        if (!dead) zmax = fmaxf(zmax, z);
     }
 }
 
@@ -176,11 +174,26 @@ __device__ __forceinline__ RowC block_row(const TileArgs& A, const BlockP& Q, co
     return RowC{-f.r, -(isd * isd), -(w1 * isd), Q.thrN - Kc, S1 * fmaf(2.f * A.e2, S0, Q.e1), A.e2 * S1 * S1};
 }
 
+// The sweep's test of the same row: six operations of two subsets each instead of ten and the
+// smallest d2.  The filter dismisses a subset when
+//     num^2 (d2 + gamma) + beta |num| d2 < K d2^2  and  d2 > tau,
+// and with K > 0, t = max(gamma, tau) and d2 <= rmax^2 that follows from
+//     num^2 + K t + beta sqrt(K) rmax < K d2:
+// then num^2 < K d2, so gamma num^2 <= gamma K d2 and |num| < sqrt(K) rmax, and d2 > t.  Tested as
+// num^2 - K2 d2 + c < 0 with room for the rounding of these expressions in K2 and c.  A column it
+// does not dismiss is decided by the filter (block_take).
+struct SweepC { float nK, c; };
+__device__ __forceinline__ SweepC block_sweep_row(float tau, float rmax, const RowC& r) {
+    const float K2 = -0.9999f * r.nK;
+    const float c = 1.001f * (K2 * fmaxf(tau, r.gm) + r.be * sqrtf(fmaxf(K2, 0.f)) * rmax);
+    return K2 > 0.f && c < INFINITY ? SweepC{-K2, c} : SweepC{0.f, 1.f};
+}
+
 struct BlockQueue { double B; int qn, taken; };
 
 // a column some lane may keep: the decisions row group by row group, into the warp's queue
 template <int DC>
-__device__ __noinline__ BlockQueue block_take(const TileArgs& A, const BlockPre* P, const BlockP Q, const float* Gp,
+__device__ __noinline__ BlockQueue block_take(const TileArgs& A, const BlockPre* P, const BlockP& Q, const float* Gp,
                                               const float2* dn, int rb, int x, unsigned* q, int qn,
                                               double B) {
     const int lane = threadIdx.x & 31;
@@ -223,18 +236,24 @@ __global__ void k_l0_reorder(const double* __restrict__ G, const double* __restr
 }
 
 template <int DC, int W>
-__global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int slices, int item0, int M) {
+__global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(const __grid_constant__ TileArgs A, int slices, int item0, int M) {
     extern __shared__ __align__(16) unsigned char block_smem[];
     __shared__ BlockPre P;
     __shared__ int s_item, s_p;
+    __shared__ BlockP s_q[W];                                     // the warp's p, bound and subsets
+    __shared__ double s_b[W];
+    __shared__ unsigned long long s_seen[W];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     double2* rr = reinterpret_cast<double2*>(block_smem);         // R per feature (while the triangle is formed)
     float2* dn = reinterpret_cast<float2*>(rr + M);               // d', n' per feature; first its scale in .x
     float* Gp = reinterpret_cast<float*>(dn + M);                 // (x, y < x) at x (x - 1) / 2 + y
     unsigned* q = reinterpret_cast<unsigned*>(Gp + ((size_t)M * (M - 1) / 2 + 36)) + w * kBQ;
     const double inv_n = 1.0 / (double)A.N;
-    double B = fmin((double)INFINITY, okey_inv(*(volatile unsigned long long*)A.ub_key));
-    unsigned long long my_examined = 0, my_cand = 0;
+    if (lane == 0) {
+        s_b[w] = fmin((double)INFINITY, okey_inv(*(volatile unsigned long long*)A.ub_key));
+        s_seen[w] = 0;
+    }
+    __syncwarp();
     while (true) {
         __syncthreads();                                          // the last unit's buffers are free
         if (tid == 0) {
@@ -340,7 +359,7 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int sli
                 Q.A0 = fabsf(Q.w * Q.invd);
                 Q.base = P.base - Q.w * Q.w;
                 Q.e0 = P.e0; Q.e1 = P.e1;
-                Q.thrN = __fmul_ru((float)((B + A.tie64) * inv_n), 1.0000002f);
+                Q.thrN = __fmul_ru((float)((s_b[w] + A.tie64) * inv_n), 1.0000002f);
             }
             const float invd = Q.invd, wp = Q.w, tau = A.tau;
             float q2 = 0.f, dmax = 0.f;
@@ -351,6 +370,9 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int sli
             }
             Q.q2 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(q2)));
             Q.rmax = sqrtf(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(dmax))));
+            __syncwarp();
+            if (lane == 0) s_q[w] = Q;
+            __syncwarp();
             // rows p + 1 .. m - 2, kBRow groups of 32 at a time: this lane's are i0 + 32 j
             for (int rb = p + 1; rb < m - 1; rb += 32 * kBRow) {
             const int i0 = rb + lane, groups = (m - 1 - rb + 31) >> 5;
@@ -358,48 +380,45 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int sli
 #pragma unroll
             for (int jp = 0; jp < kBRow / 2; ++jp) {
                 RowC c[2] = {{0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}};
+                SweepC k[2] = {{0.f, 0.f}, {0.f, 0.f}};
                 if (2 * jp < groups) {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int i1 = i0 + 32 * (2 * jp + h);
-                        if (i1 < m) c[h] = block_row(A, Q, block_feature(Q, Gp, dn, i1));
+                        if (i1 < m) {
+                            c[h] = block_row(A, Q, block_feature(Q, Gp, dn, i1));
+                            k[h] = block_sweep_row(tau, Q.rmax, c[h]);
+                        }
                     }
                 }
                 R.nr[jp] = pk2(c[0].nr, c[1].nr); R.nid[jp] = pk2(c[0].nid, c[1].nid); R.nw[jp] = pk2(c[0].nw, c[1].nw);
-                R.nK[jp] = pk2(c[0].nK, c[1].nK); R.be[jp] = pk2(c[0].be, c[1].be); R.gm[jp] = pk2(c[0].gm, c[1].gm);
+                R.nK[jp] = pk2(k[0].nK, k[1].nK); R.c[jp] = pk2(k[0].c, k[1].c);
             }
+            // columns to decide, one bit each: lane l holds those of rb + 1 + 32 l ..
+            unsigned open = 0;
             // columns rb + 1 .. m - 1 in segments of equal row group count C, two at a time
             int x = rb + 1;
             const float* gx = Gp + x * (x - 1) / 2;               // row x of G'
             auto segment = [&](auto cc) {
                 constexpr int C = decltype(cc)::value;
                 const int end = C == kBRow ? m : min(m, rb + 1 + 32 * C);           // x - rb <= 32 C
-                auto column = [&](const float* gr, int xc, float& zmax, float& dmin) {
+                auto column = [&](const float* gr, int xc, float& zmax) {
                     const float r = gr[p] * invd;
                     const float2 f = dn[xc];
-                    block_col<C>(gr + i0, r, fmaf(-r, r, f.x), fmaf(-r, wp, f.y), i0 + 32 * (C - 1) >= xc, R, zmax, dmin);
+                    block_col<C>(gr + i0, r, fmaf(-r, r, f.x), fmaf(-r, wp, f.y), i0 + 32 * (C - 1) >= xc, R, zmax);
                 };
-                auto take = [&](int xc) {
-                    const BlockQueue t = block_take<DC>(A, &P, Q, Gp, dn, rb, xc, q, qn, B);
-                    B = t.B;
-                    qn = t.qn;
-                    my_cand += t.taken;
-                };
-                for (; x + 1 < end; x += 2) {
-                    float zmax = -INFINITY, dmin = INFINITY;
-                    column(gx, x, zmax, dmin);
-                    column(gx + x, x + 1, zmax, dmin);
+                for (; x + 1 < end; x += 2) {                     // (an even number of columns from rb + 1: one word)
+                    float zmax = -INFINITY;
+                    column(gx, x, zmax);
+                    column(gx + x, x + 1, zmax);
                     gx += 2 * x + 1;
-                    if (__any_sync(0xffffffffu, !(zmax < 0.f) || !(dmin > tau))) {
-                        take(x);
-                        take(x + 1);
-                    }
+                    if (__any_sync(0xffffffffu, !(zmax < 0.f)) && lane == ((x - rb - 1) >> 5)) open |= 3u << ((x - rb - 1) & 31);
                 }
                 if (x < end) {
-                    float zmax = -INFINITY, dmin = INFINITY;
-                    column(gx, x, zmax, dmin);
+                    float zmax = -INFINITY;
+                    column(gx, x, zmax);
                     gx += x;
-                    if (__any_sync(0xffffffffu, !(zmax < 0.f) || !(dmin > tau))) take(x);
+                    if (__any_sync(0xffffffffu, !(zmax < 0.f)) && lane == ((x - rb - 1) >> 5)) open |= 1u << ((x - rb - 1) & 31);
                     ++x;
                 }
             };
@@ -409,20 +428,34 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(TileArgs A, int sli
             segment(std::integral_constant<int, 4>{});
             segment(std::integral_constant<int, 5>{});
             segment(std::integral_constant<int, 6>{});
+            for (unsigned words = __ballot_sync(0xffffffffu, open != 0u); words; words &= words - 1u) {
+                const int l = __ffs(words) - 1;
+                for (unsigned o = __shfl_sync(0xffffffffu, open, l); o; o &= o - 1u) {
+                    const BlockQueue t = block_take<DC>(A, &P, s_q[w], Gp, dn, rb, rb + 32 * l + __ffs(o), q, qn, s_b[w]);
+                    qn = t.qn;
+                    __syncwarp();
+                    if (lane == 0) {
+                        s_b[w] = t.B;
+                        if (t.taken) atomicAdd(A.candidates, (unsigned long long)t.taken);
+                    }
+                    __syncwarp();
+                }
+            }
             }
             // rows p + 1 .. x - 1 of every column
-            if (lane == 0) my_examined += (unsigned long long)(m - 1 - p) * (unsigned long long)(m - 2 - p) / 2;
-            B = fmin(B, okey_inv(next_key));
+            if (lane == 0) {
+                s_seen[w] += (unsigned long long)(m - 1 - p) * (unsigned long long)(m - 2 - p) / 2;
+                s_b[w] = fmin(s_b[w], okey_inv(next_key));
+            }
+            __syncwarp();
         }
         if (qn > 0) {                                      // the queue's entries are relative to this prefix
-            B = block_flush<DC>(A, &P, q, qn, B);
+            const double B = block_flush<DC>(A, &P, q, qn, s_b[w]);
+            __syncwarp();
+            if (lane == 0) s_b[w] = B;
         }
     }
-    my_examined = l0_warp_sum(my_examined);
-    if (lane == 0) {
-        atomicAdd(A.examined, my_examined);
-        atomicAdd(A.candidates, my_cand);
-    }
+    if (lane == 0) atomicAdd(A.examined, s_seen[w]);
 }
 
 }  // namespace
