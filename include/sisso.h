@@ -347,6 +347,11 @@ sisso_status sisso_gram_tc(const double* Z, const double* yc, double sdy, int n,
  * Errors: SISSO_ERR_ARG, SISSO_ERR_CUDA, SISSO_ERR_TIMEOUT (a bounded wait ran out). */
 sisso_status sisso_bilinear_tc(const double* L, const double* R, int m, int n, int N, int kind, double* out);
 
+/* G = Z Z^T / N and b = Z yc / N (Z: n rows of N samples) by the exact tensor-core products that
+ * long samples' FP64 Grams take: rows as 55-bit integers in base 256, digit products summed as
+ * integers.  N up to 2^23. */
+sisso_status sisso_gram_fp64(const double* Z, const double* yc, int n, int N, double* G, double* b);
+
 /* Measured FMA throughput of the current device in TFLOP/s, the denominator of the ALU-bound
  * kernels' roofline: kind 0 FP32 (fma.rn.f32, 2 flop), 1 paired FP32 (fma.rn.f32x2, 4 flop),
  * 2 FP64.  Every SM busy with independent chains; best of five timed launches of about

@@ -442,6 +442,9 @@ struct sisso_ctx {
     int* dup_pairs = nullptr;          // (entry, slot) pairs to confirm; dup_np: their number
     unsigned* dup_np = nullptr;
     double* tpart = nullptr;           // target sums per block (many samples)
+    void* gram_sl = nullptr;           // digits of the rows of Z (gram64_tc.cu), their exponents
+    int* gram_ex = nullptr;
+    int gram_rows = 0;                 // rows [0, gram_rows) have digits
     double* mpart = nullptr;           // the winner's sums per block (many samples)
     int* sort_src = nullptr;           // index into the survivor arrays
     unsigned char* removed = nullptr;  // walk: visited flags (sort_cap)
@@ -592,6 +595,12 @@ sisso_status winner_model(sisso_ctx* c, int n, int D, Winner& w);
 sisso_status l0_learned(sisso_ctx* c, sisso_mlp* mlp, const double* G, const double* b, const float* G32,
                         const float* b32, int ld, double syy, int n, const int64_t* gid_dev, double frac, Winner& w,
                         int64_t* n_selected);
+
+// FP64 Gram from exact tensor-core products (gram64_tc.cu)
+bool gram64_tc_possible(int N, int n_new, int n, int n_cap);
+size_t gram64_tc_bytes(int N, int n_cap);
+sisso_status gram64_tc(sisso_ctx* c, const double* Z, const double* yc, int N, int first, int n_old, int n, int n_cap, int ld,
+                       void* sl, int* ex, double* G, double* b, float* G32, float* b32);
 
 // tensor-core Gram (gram_tc.cu)
 sisso_status gram_tc(sisso_ctx* c, const double* Z, const double* yc, double sdy, int n, int N, int kind,

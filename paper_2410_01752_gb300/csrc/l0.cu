@@ -630,7 +630,18 @@ sisso_status append_subspace(sisso_ctx* c, int n_old, int n_new, bool gram64) {
                                                      c->Zmean, c->Zsd);
         c->stats.launches++;
     }
-    if (gram64) {
+    if (n_old < c->gram_rows) c->gram_rows = n_old;
+    // FP64 sums, or exact integer ones on the tensor cores where the FP64 pipe would take longer
+    if (gram64 && gram64_tc_possible(c->N, n_new, n, c->n_cap)) {
+        sisso_status st;
+        if (!c->gram_sl && ((st = ctx_alloc(c, &c->gram_sl, gram64_tc_bytes(c->N, c->n_cap), "gram digits")) ||
+                            (st = ctx_alloc(c, (void**)&c->gram_ex, sizeof(int) * (size_t)c->n_cap, "gram exponents"))))
+            return st;
+        if ((st = gram64_tc(c, c->Z, c->yc64, c->N, c->gram_rows, n_old, n, c->n_cap, c->n_cap, c->gram_sl, c->gram_ex, c->G64,
+                            c->b64, c->G32, c->b32)))
+            return st;
+        c->gram_rows = n;
+    } else if (gram64) {
         dim3 grid(n_new, std::max(1, std::min(64, (n + 1 + kWarps - 1) / kWarps)));
         k_gram_rows<<<grid, kWarps * 32, 0, c->stream>>>(c->Z, c->yc64, c->N, n_old, n, c->n_cap, c->G64, c->b64,
                                                           c->G32, c->b32);

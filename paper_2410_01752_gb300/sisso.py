@@ -43,7 +43,7 @@ EXPORTS = [
     "sisso_mlp_gradients", "sisso_mlp_train", "sisso_prefix_features", "sisso_prefix_labels", "sisso_l0_learned",
     "sisso_set_proposal", "sisso_get_primaries", "sisso_prescreen", "sisso_prefix_training",
     "sisso_batch_set_wait_limit", "sisso_l0_learned_certified", "sisso_set_proposal_ex",
-    "sisso_bilinear_tc", "sisso_measure_alu_peak", "sisso_release_memory",
+    "sisso_bilinear_tc", "sisso_gram_fp64", "sisso_measure_alu_peak", "sisso_release_memory",
 ]
 MLP_IN, MLP_HIDDEN = 20, 256
 MLP_PARAMS = MLP_HIDDEN * MLP_IN + MLP_HIDDEN + MLP_HIDDEN * MLP_HIDDEN + MLP_HIDDEN + MLP_HIDDEN + 1
@@ -149,6 +149,7 @@ def load() -> C.CDLL:
                                   C.POINTER(C.c_int), dp, i64p]
     L.sisso_space_sizes.argtypes = [C.c_int, C.c_uint32, C.c_int, C.c_int, i64p]
     L.sisso_gram_tc.argtypes = [vp, vp, C.c_double, C.c_int, C.c_int, C.c_int, vp, vp]
+    L.sisso_gram_fp64.argtypes = [vp, vp, C.c_int, C.c_int, vp, vp]
     L.sisso_bilinear_tc.argtypes = [vp, vp, C.c_int, C.c_int, C.c_int, C.c_int, vp]
     L.sisso_measure_alu_peak.argtypes = [C.c_int, C.POINTER(C.c_double)]
     L.sisso_release_memory.argtypes = [C.c_int]
@@ -259,6 +260,19 @@ def gram_tc(Z, yc, sdy: float, kind: int = PREC_MIXED_BF16):
                               C.c_void_p(G.ctypes.data), C.c_void_p(b.ctypes.data))
     if st:
         raise SissoError(st, "gram_tc")
+    return G, b
+
+
+def gram_fp64(Z, yc):
+    """(Z Z^T / N, Z yc / N) from exact tensor-core products (sisso_gram_fp64)."""
+    Z = np.ascontiguousarray(Z, dtype=np.float64)
+    yc = np.ascontiguousarray(yc, dtype=np.float64)
+    n, N = Z.shape
+    G, b = np.zeros((n, n)), np.zeros(n)
+    st = load().sisso_gram_fp64(C.c_void_p(Z.ctypes.data), C.c_void_p(yc.ctypes.data), n, N,
+                                C.c_void_p(G.ctypes.data), C.c_void_p(b.ctypes.data))
+    if st:
+        raise SissoError(st, "gram_fp64")
     return G, b
 
 
