@@ -430,7 +430,7 @@ sisso_status sisso_fit(sisso_ctx* c) {
         if ((st = prepare_target(c, target))) break;
         if ((st = score_all(c, prec))) break;
         std::vector<int64_t> acc;
-        if ((st = sis_select(c, c->k, c->S.data(), (int)c->S.size(), acc))) break;
+        if ((st = sis_select(c, c->k, c->S.data(), (int)c->S.size(), acc, true))) break;
         const int n_old = (int)c->S.size();
         if (!acc.empty())
             cudaMemcpyAsync(c->S_dev + n_old, acc.data(), sizeof(int64_t) * acc.size(), cudaMemcpyHostToDevice, c->stream);

@@ -569,7 +569,7 @@ sisso_status whiten_rescore(sisso_ctx* c, const int64_t* ids, int n, double* sco
                             int* valid, double* probe, double* zc);
 sisso_status whiten_standardise(sisso_ctx* c, const int64_t* ids, int n, double* Z, double* Zmean, double* Zsd);
 sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_prev,
-                        std::vector<int64_t>& acc);
+                        std::vector<int64_t>& acc, bool S_rows = false);
 sisso_status eval_features(sisso_ctx* c, const int64_t* ids_dev, int64_t n, int precision,
                            double* out_dev);
 // 32 x 32 operand-pair tiles of the top level's binary sections (upper left corners)

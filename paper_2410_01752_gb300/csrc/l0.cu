@@ -87,6 +87,60 @@ __global__ void __launch_bounds__(1024) k_standardise(const Space* __restrict__ 
     for (int i = threadIdx.x; i < N; i += blockDim.x) z[i] = (z[i] - m) * inv;
 }
 
+// the same over many samples, each row cut into gridDim.y runs: values and their sums, squares
+// about the mean, standardised values (a CTA a row left the device half idle: 200 rows of 65 536
+// samples 0.37 -> 0.1 ms).  part: [2][rows][runs], combined in order
+__device__ __forceinline__ double std_block_sum(double s, double* red) {
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    for (int q = 1; q < (int)(blockDim.x >> 5); ++q) s += red[q];
+    return s;                                              // thread 0
+}
+__device__ __forceinline__ double std_total(const double* p, int runs) {
+    double s = 0.0;
+    for (int q = 0; q < runs; ++q) s += p[q];
+    return s;
+}
+__global__ void __launch_bounds__(256) k_std_values(const Space* __restrict__ sp, int N, const int64_t* __restrict__ ids, int row0,
+                                                    const double* __restrict__ V, double* __restrict__ Z, int run,
+                                                    double* __restrict__ part) {
+    __shared__ double red[8];
+    const int row = row0 + blockIdx.x, end = min(N, ((int)blockIdx.y + 1) * run);
+    OpRef ref{};
+    const bool ok = make_opref(*sp, ids[row], ref);
+    double* z = Z + (size_t)row * N;
+    double s = 0.0;
+    for (int i = blockIdx.y * run + threadIdx.x; i < end; i += 256) {
+        double mg;
+        const double v = ok ? opref_val(ref, V, N, i, mg) : 0.0;
+        z[i] = v;
+        s += v;
+    }
+    s = std_block_sum(s, red);
+    if (threadIdx.x == 0) part[blockIdx.x * gridDim.y + blockIdx.y] = s;
+}
+__global__ void __launch_bounds__(256) k_std_squares(int N, int row0, const double* __restrict__ Z, int run, double* __restrict__ part) {
+    __shared__ double red[8];
+    const int row = row0 + blockIdx.x, end = min(N, ((int)blockIdx.y + 1) * run);
+    const double m = std_total(part + blockIdx.x * gridDim.y, gridDim.y) / N;
+    const double* z = Z + (size_t)row * N;
+    double s = 0.0;
+    for (int i = blockIdx.y * run + threadIdx.x; i < end; i += 256) { const double v = z[i] - m; s += v * v; }
+    s = std_block_sum(s, red);
+    if (threadIdx.x == 0) part[(gridDim.x + blockIdx.x) * gridDim.y + blockIdx.y] = s;
+}
+__global__ void __launch_bounds__(256) k_std_write(int N, int row0, double* __restrict__ Z, int run, const double* __restrict__ part,
+                                                   double* __restrict__ mean_out, double* __restrict__ sd_out) {
+    const int row = row0 + blockIdx.x, end = min(N, ((int)blockIdx.y + 1) * run);
+    const double m = std_total(part + blockIdx.x * gridDim.y, gridDim.y) / N;
+    const double sd = sqrt(std_total(part + (gridDim.x + blockIdx.x) * gridDim.y, gridDim.y) / N);
+    const double inv = sd > 0.0 ? 1.0 / sd : 0.0;
+    double* z = Z + (size_t)row * N;
+    for (int i = blockIdx.y * run + threadIdx.x; i < end; i += 256) z[i] = (z[i] - m) * inv;
+    if (blockIdx.y == 0 && threadIdx.x == 0) { mean_out[row] = m; sd_out[row] = sd; }
+}
+
 // G[i][j] = G[j][i] = Z_i . Z_j / N for i in [n_old, n), j in [0, n); b[i] = Z_i . y~ / N
 __global__ void k_gram_rows(const double* __restrict__ Z, const double* __restrict__ yc, int N, int n_old,
                             int n, int ld, double* __restrict__ G, double* __restrict__ b,
@@ -626,7 +680,20 @@ sisso_status append_subspace(sisso_ctx* c, int n_old, int n_new, bool gram64) {
                                              c->Zmean + n_old, c->Zsd + n_old);
         if (st) return st;
     } else {
-        k_standardise<<<n_new, c->N > 4096 ? 1024 : 256, 0, c->stream>>>(c->space_dev, c->Xc64, c->N, c->S_dev, n_old, c->opval64, c->Z,
+        if (c->N > 4096 && c->opval64) {
+            const int runs = std::max(1, std::min({c->N / 2048, 32, c->sms * 16 / n_new}));
+            const int run = (c->N + runs - 1) / runs;
+            const dim3 grid((unsigned)n_new, (unsigned)((c->N + run - 1) / run));
+            double* part = nullptr;
+            const sisso_status st = tmp_alloc(c, (void**)&part, sizeof(double) * 2 * grid.x * grid.y, "row sums");
+            if (st) return st;
+            k_std_values<<<grid, 256, 0, c->stream>>>(c->space_dev, c->N, c->S_dev, n_old, c->opval64, c->Z, run, part);
+            k_std_squares<<<grid, 256, 0, c->stream>>>(c->N, n_old, c->Z, run, part);
+            k_std_write<<<grid, 256, 0, c->stream>>>(c->N, n_old, c->Z, run, part, c->Zmean, c->Zsd);
+            c->stats.launches += 2;
+            cudaFreeAsync(part, c->stream);
+        } else
+        k_standardise<<<n_new, 256, 0, c->stream>>>(c->space_dev, c->Xc64, c->N, c->S_dev, n_old, c->opval64, c->Z,
                                                      c->Zmean, c->Zsd);
         c->stats.launches++;
     }

@@ -716,11 +716,34 @@ __global__ void __launch_bounds__(kRescoreThreads)
 k_rescore_cta(const Space* __restrict__ sp, int N, const double* __restrict__ tc, const TargetStats* __restrict__ st,
               const int64_t* __restrict__ ids, const unsigned char* __restrict__ subvalid, const double* __restrict__ V,
               const double* __restrict__ Vinv, double* score, double* mean_out, double* sd_out, int* valid_out,
-              double* __restrict__ probe, double* __restrict__ zc) {
+              double* __restrict__ probe, double* __restrict__ zc, const double* __restrict__ Zs,
+              const double* __restrict__ Zmean, const double* __restrict__ Zsd, int ns) {
     constexpr int W = kRescoreThreads / 32;
     __shared__ double red[W][3];
     __shared__ unsigned long long redb[W][2];
     const int w = blockIdx.x, t = threadIdx.x, lane = t & 31, wp = t >> 5;
+    if (Zs && w >= ns) {            // a member of S: its standardised row is at hand
+        const double* zr = Zs + (size_t)(w - ns) * N;
+        double* z = zc ? zc + (size_t)w * N : nullptr;
+        double sc = 0.0;
+        for (int i = t; i < N; i += kRescoreThreads) {
+            const double v = zr[i];
+            sc = fma(v, tc[i], sc);
+            if (z) z[i] = v;
+        }
+        sc = warp_sum(sc);
+        if (lane == 0) red[wp][0] = sc;
+        __syncthreads();
+        if (t < kProbes) probe[(size_t)w * kProbes + t] = zr[(int)(((int64_t)t * N) / kProbes)];
+        if (t == 0) {
+            for (int q = 1; q < W; ++q) sc += red[q][0];
+            valid_out[w] = 1;
+            mean_out[w] = Zmean[w - ns];
+            sd_out[w] = Zsd[w - ns];
+            score[w] = fabs(sc) / ((double)N * st->sd);
+        }
+        return;
+    }
     const int64_t id = ids[w];
     int level, op; int64_t a, b;
     const int64_t Pbot = sp->phi[sp->rung - 1];
@@ -1795,8 +1818,9 @@ sisso_status eval_features(sisso_ctx* c, const int64_t* ids_dev, int64_t n, int 
 
 // One SIS step on the scores already in c->scores (against the target prepared by
 // prepare_target).  S_prev_host: S_{t-1} in acceptance order.
+// S_rows: the standardised rows of S_{t-1} are the first n_prev of c->Z.
 sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_prev,
-                        std::vector<int64_t>& acc) {
+                        std::vector<int64_t>& acc, bool S_rows) {
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0); cudaEventCreate(&e1);
     cudaEventRecord(e0, c->stream);
@@ -1811,7 +1835,8 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
     int64_t M = first_window(c, k);
     // the default window holds thousands of candidates so that it proves dense selections too; the
     // FP64 work of most steps needs the best few hundred: walks visit 1.2 to 4.4 k candidates, so
-    // rank 5 k (at 3 k one step in twelve was repeated).  1013 samples, k = 50: 12 438 -> 636 candidates
+    // rank 5 k (at 3 k one step in twelve was repeated); half of that for long samples, whose FP64
+    // work dwarfs a repeated step's kernels (65 536 samples, k = 200: 1.6 -> 0.9 ms a step).  1013 samples, k = 50: 12 438 -> 636 candidates
     // re-scored over three steps, 3.1 -> 2.6 ms a fit
     bool narrow = c->opts.survivors <= 0;
     const int64_t n = c->n_feat;
@@ -1833,7 +1858,7 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
                                                    c->surv_cap - n_prev);
         c->stats.launches++;
         if (narrow && M <= kNarrowMax) {
-            k_narrow<<<1, kNarrowThreads, 0, c->stream>>>(c->scores, c->surv_ids, c->surv_count, c->sel_state, 5 * k,
+            k_narrow<<<1, kNarrowThreads, 0, c->stream>>>(c->scores, c->surv_ids, c->surv_count, c->sel_state, c->N > 4096 ? 5 * k / 2 : 5 * k,
                                                           (float)(2.25 * eps + 8.0 * kScoreTie));
             c->stats.launches++;
         }
@@ -1864,7 +1889,8 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
             k_rescore_cta<<<nr, kRescoreThreads, 0, c->stream>>>(c->space_dev, c->N, c->tc64, c->tstats, c->surv_ids,
                                                                  c->subvalid, c->opval64, c->opinv64, c->surv_score,
                                                                  c->surv_mean, c->surv_sd, c->surv_valid,
-                                                                 c->surv_probe, zc);
+                                                                 c->surv_probe, zc, S_rows ? c->Z : nullptr, c->Zmean,
+                                                                 c->Zsd, ns);
         else
             k_rescore<<<(nr * 32 + 255) / 256, 256, 0, c->stream>>>(c->space_dev, c->Xc64, c->N, c->tc64, c->tstats,
                                                                      c->surv_ids, nr, c->subvalid, c->opval64,
