@@ -126,6 +126,7 @@ struct BTask {
     double* Z;                  // standardised subspace members (kMaxSub rows, stride ldv)
     double* zraw;               // FP64 values of the first kZRaw window entries (stride N)
     double* A1;                 // per operand: sum_s (x_s - x_0) (P), written with the step-1 sums
+    float* keep;                // per pair tile: the candidates' std and mean of step 1 (null: not kept)
     BDim dim[kMaxDim + 1];      // index t = 1..max_dim
 };
 
@@ -459,8 +460,15 @@ __device__ __forceinline__ void run_score(const BatchArgs& B, int task, int t, l
             PairArgs A = T.pa;
             A.scores = D.scores;
             const int2 tl = T.tiles[u - T.n_low - T.n_un];
-            pair_tile<float, true>(A, nullptr, D.tc32, D.tc64, D.ts, T.valid, T.cache, T.A1, D.AR,
-                                    *reinterpret_cast<PairSmem<float>*>(smem), tl.x, tl.y);
+            PairSmem<float>& PS = *reinterpret_cast<PairSmem<float>*>(smem);
+            float* keep = T.keep ? T.keep + (u - T.n_low - T.n_un) * kPairKeepTile : nullptr;
+            if (!keep)
+                pair_tile<float, true>(A, nullptr, D.tc32, D.tc64, D.ts, T.valid, T.cache, T.A1, D.AR, PS, tl.x, tl.y);
+            else if (t == 1)
+                pair_tile<float, true, false, true>(A, nullptr, D.tc32, D.tc64, D.ts, T.valid, T.cache, T.A1, D.AR, PS, tl.x,
+                                                    tl.y, keep);
+            else
+                pair_tile_cov(A, D.tc32, D.ts, T.valid, T.cache, T.A1, D.AR, PS, tl.x, tl.y, keep);
             __syncthreads();
         }
     }
@@ -623,6 +631,64 @@ __device__ void standardise_from(const BTask& T, Ctl& C, const double* raw, doub
     __syncthreads();
 }
 
+// the window's entries down to those within the screening margin of rank `want` (to within an
+// eighth, by bisection on the keys), or above it: the FP64 re-score is one CTA's, about 1.3 us an
+// entry at 100 samples and 6.5 at 1000, and walks visit 1.5 k candidates.  A walk that visits at
+// most `want` proves its selection with them; one that does not is repeated with the whole window.
+__device__ bool narrow_window(const BatchArgs& B, SelectSmem& M, Ctl& C, const BDim& D, int want, unsigned thr, int& ns,
+                              float& t32) {
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    unsigned* key = M.u.hist;
+    int* cnt = reinterpret_cast<int*>(M.u.hist + kWinMax);
+    unsigned top = 0;
+    for (int e = tid; e < ns; e += kBT) {
+        key[e] = rkey(__ldcg(D.scores + D.w_ids[e]));
+        top = max(top, key[e]);
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0) cnt[w] = (int)top;
+    __syncthreads();
+    for (int q = 0; q < kBT / 32; ++q) top = max(top, (unsigned)cnt[q]);
+    __syncthreads();
+    auto above = [&](unsigned v) {
+        int c = 0;
+        for (int e = tid; e < ns; e += kBT) c += key[e] >= v;
+        c = __reduce_add_sync(0xffffffffu, c);
+        __syncthreads();
+        if (lane == 0) cnt[w] = c;
+        __syncthreads();
+        c = 0;
+        for (int q = 0; q < kBT / 32; ++q) c += cnt[q];
+        return c;
+    };
+    unsigned lo = max(thr, 1u), hi = top + 1u;
+    while (hi - lo > 1u) {
+        const unsigned mid = lo + (hi - lo) / 2u;
+        const int c = above(mid);
+        if (c >= want) {
+            lo = mid;
+            if (c <= want + want / 8) break;
+        } else {
+            hi = mid;
+        }
+    }
+    const float low = __uint_as_float(lo) - (float)(2.25 * kScoreErr32 + 8.0 * kScoreTie);
+    const unsigned cut = max(low > 0.f ? __float_as_uint(low) : 1u, max(thr, 1u));
+    if (above(cut) > ns - ns / 8) return false;
+    if (tid == 0) C.n = 0;
+    for (int base = 0; base < ns; base += kBT) {
+        const int e = base + tid;
+        const bool in = e < ns && key[e] >= cut;
+        const int64_t id = in ? D.w_ids[e] : 0;
+        __syncthreads();                                  // this run's ids are read: the slots lie at or before it
+        if (in) D.w_ids[atomicAdd(&C.n, 1)] = id;
+        __syncthreads();
+    }
+    ns = C.n;
+    t32 = __uint_as_float(cut);
+    return true;
+}
+
 // returns SISSO_OK, or an error status for the task
 __device__ __noinline__ int run_select(const BatchArgs& B, Ctl& C, int task, int t, unsigned char* smem) {
     const BTask& T = B.tasks[task];
@@ -635,18 +701,16 @@ __device__ __noinline__ int run_select(const BatchArgs& B, Ctl& C, int task, int
     const int k = B.k;
     // S, ascending, for the membership test; previous members carried into this step's lists
     for (int i = tid; i < n_prev; i += kBT) {
-        M.S_sorted[i] = gprev[i];
+        const int64_t id = __ldcg(gprev + i);
+        int rank = 0;
+        for (int e = 0; e < n_prev; ++e) rank += __ldcg(gprev + e) < id;
+        M.S_sorted[rank] = id;
         D.gid[i] = gprev[i];
         D.zmean[i] = T.dim[t - 1].zmean[i];
         D.zsd[i] = T.dim[t - 1].zsd[i];
     }
     __syncthreads();
-    if (tid == 0)
-        for (int a = 1; a < n_prev; ++a)
-            for (int c = a; c > 0 && M.S_sorted[c - 1] > M.S_sorted[c]; --c) {
-                const int64_t x = M.S_sorted[c]; M.S_sorted[c] = M.S_sorted[c - 1]; M.S_sorted[c - 1] = x;
-            }
-    __syncthreads();
+    bool narrow = true;
     int Mw = B.win0 < k ? k : B.win0;
     if (Mw > kWinMax) Mw = kWinMax;
     int n_acc = 0;
@@ -654,7 +718,7 @@ __device__ __noinline__ int run_select(const BatchArgs& B, Ctl& C, int task, int
         unsigned long long ts0 = gtimer();
         radix_select(M, C, D.scores, T.n_feat, (unsigned)Mw);
         const unsigned thr = (unsigned)C.ukey;
-        const int all = C.flag;
+        int all = C.flag;
         float t32 = 0.f;
         if (!all) t32 = __uint_as_float(thr);
         // compact the window
@@ -668,8 +732,11 @@ __device__ __noinline__ int run_select(const BatchArgs& B, Ctl& C, int task, int
             }
         }
         __syncthreads();
-        const int ns = C.n;
+        int ns = C.n;
         if (ns > kWinMax) return SISSO_ERR_CAPACITY;    // tied scores overflow the window
+        bool narrowed = false;
+        if (narrow && ns > 5 * k) narrowed = narrow_window(B, M, C, D, 5 * k / 2, thr, ns, t32);
+        if (narrowed) all = 0;
         unsigned long long ts1 = gtimer();
         if (tid == 0) prof_add(B.prof, PS_SEL_RADIX, ts1 - ts0);
         // FP64 re-score, one warp per entry
@@ -782,6 +849,7 @@ __device__ __noinline__ int run_select(const BatchArgs& B, Ctl& C, int task, int
         // exact iff every candidate outside the window scores below the last visited one by
         // more than the tie tolerance (FP32 scores within kScoreErr32 of FP64)
         const bool safe = all || (n_acc == k && last - kScoreTie > (double)t32 + kScoreErr32);
+        if (!safe && narrowed) { narrow = false; __syncthreads(); continue; }
         if (safe || Mw >= kWinMax) {
             if (!safe && tid == 0) St.saturated = 1;
             break;
@@ -1490,9 +1558,19 @@ sisso_status sisso_batch_create(const sisso_task* tasks, int n_tasks, uint32_t o
             f.AR[t] = region(sizeof(double) * P.P);
         }
     }
-    b->arena_bytes = total;
+    // the pair tiles' kept values behind the rest, left out when they do not fit
+    std::vector<size_t> keep_off(n_tasks);
+    const size_t without = total;
+    if (max_dim > 1)
+        for (int i = 0; i < n_tasks; ++i) keep_off[i] = region(sizeof(float) * kPairKeepTile * plans[i].tiles.size());
     sisso_status st;
-    if ((st = bcuda(b, cudaMalloc(&b->arena, total), "batch arena"))) return bail(st, "");
+    if (total > without && cudaMalloc(&b->arena, total) != cudaSuccess) {
+        cudaGetLastError();
+        b->arena = nullptr;
+        total = without;
+    }
+    b->arena_bytes = total;
+    if (!b->arena && (st = bcuda(b, cudaMalloc(&b->arena, total), "batch arena"))) return bail(st, "");
     size_t n_tiles_all = 0;
     for (auto& P : plans) n_tiles_all += P.tiles.size();
     if ((st = bcuda(b, cudaMalloc(&b->plans, sizeof(Space) * n_tasks), "plans")) ||
@@ -1557,6 +1635,7 @@ sisso_status sisso_batch_create(const sisso_task* tasks, int n_tasks, uint32_t o
         T.Z = reinterpret_cast<double*>(A + f.Z);
         T.zraw = reinterpret_cast<double*>(A + f.zraw);
         T.A1 = reinterpret_cast<double*>(A + f.A1);
+        T.keep = total > without ? reinterpret_cast<float*>(A + keep_off[i]) : nullptr;
         for (int t = 1; t <= max_dim; ++t) {
             BDim& D = T.dim[t];
             D.scores = reinterpret_cast<float*>(A + f.scores[t]);

@@ -79,8 +79,12 @@ __device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long v
 // when the feature is certainly invalid.  The exact validity rule (every |v| <= 1e12,
 // std > 1e-6 max|v|) is applied by the FP64 re-score; here a feature is rejected only
 // if it must fail it (non-finite sums, |v0| > 1e12, std <= 1e-6 max(|v0|, |mean|)).
+// keep_sd, keep_ms (optional): the std (-1: rejected) and the mean of v - v0, for a later target's
+// score (finalize_cov)
 template <typename T>
-__device__ __forceinline__ float finalize(T s1, T s2, T sr, T v0, int N, T sum_t, T sd_t) {
+__device__ __forceinline__ float finalize(T s1, T s2, T sr, T v0, int N, T sum_t, T sd_t, T* keep_sd = nullptr,
+                                          T* keep_ms = nullptr) {
+    if (keep_sd) *keep_sd = T(-1);
     const T inv_n = T(1) / T(N);
     const T ms = s1 * inv_n;
     const T var = s2 * inv_n - ms * ms;
@@ -91,15 +95,25 @@ __device__ __forceinline__ float finalize(T s1, T s2, T sr, T v0, int N, T sum_t
     const T sd = sqrt(var);
     const T mx = fabs(v0) > fabs(mean) ? fabs(v0) : fabs(mean);
     if (!(sd > T(kConstRel) * mx)) return -1.f;
+    if (keep_sd) *keep_sd = sd;
+    if (keep_ms) *keep_ms = ms;
     return (float)(fabs(cov) / (sd * sd_t));
+}
+
+// the score against another target from its sum of v' r and the kept std and mean: the operations
+// finalize applies to them
+__device__ __forceinline__ float finalize_cov(float ms, float sd, float sr, int N, float sum_t, float sd_t) {
+    const float inv_n = 1.f / (float)N;
+    const float cov = sr * inv_n - ms * (sum_t * inv_n);
+    return sd > 0.f && isfinite(sr) ? fabsf(cov) / (sd * sd_t) : -1.f;
 }
 
 // the same, for + and -: the sums of v' and v' r come from per-operand FP64 sums; only
 // their combination is done in FP64 (where a and b nearly cancel), the rest in T (FP64
 // throughput is a small fraction of FP32 on this part)
 template <typename T>
-__device__ __forceinline__ float finalize_lin(double s1, T s2, double sr, T v0, int N, T sum_t, T sd_t) {
-    return finalize<T>((T)s1, s2, (T)sr, v0, N, sum_t, sd_t);
+__device__ __forceinline__ float finalize_lin(double s1, T s2, double sr, T v0, int N, T sum_t, T sd_t, T* keep_sd = nullptr) {
+    return finalize<T>((T)s1, s2, (T)sr, v0, N, sum_t, sd_t, keep_sd);
 }
 
 // + and - from the cross sum (FP32 form): the sum of v'^2 is q2 = A2[a] + A2[b] +/- 2 X with
@@ -476,12 +490,17 @@ __device__ __forceinline__ f2 f2sub(f2 a, f2 b) {
 // One 32 x 32 tile of operand pairs (i0.., j0..): stage operands chunk by chunk, accumulate
 // the shifted sums of + - * a/b b/a for 4 pairs per thread, write the scores.  Called by
 // every thread of an 8-warp CTA; S is that CTA's shared memory.
-template <typename T, bool LIN, bool XS = false>
+// KEEP: the candidates' std and mean go to keep (kPairKeep values per pair, by tile and thread) for
+// pair_tile_cov
+constexpr int kPairKeep = 8;              // std of + - * a/b b/a, mean shift of * a/b b/a
+constexpr size_t kPairKeepTile = (size_t)kPairKeep * TI * TJ;
+
+template <typename T, bool LIN, bool XS = false, bool KEEP = false>
 __device__ __forceinline__ void pair_tile(const PairArgs& A, const T* __restrict__ Xc, const float* __restrict__ tc32,
                                           const double* __restrict__ tc64, const TargetStats* __restrict__ st,
                                           const unsigned char* __restrict__ subvalid, const T* __restrict__ cache,
                                           const double* __restrict__ A1, const double* __restrict__ AR, PairSmem<T>& S,
-                                          int64_t i0, int64_t j0) {
+                                          int64_t i0, int64_t j0, float* keep = nullptr) {
     const int tid = threadIdx.x, lane = tid & 31, g = tid >> 5;
     const int N = A.N;
     const T* tc = TgtView<T>::tc(tc32, tc64);
@@ -651,6 +670,11 @@ __device__ __forceinline__ void pair_tile(const PairArgs& A, const T* __restrict
         const T keq = kPair ? b0 * rcp<T>(a0) : Ke[q];
         const bool opv = okj && S.ok[g * RI + q];   // both operands valid
         const double a1i = lin ? A1[i] : 0.0, ari = lin ? AR[i] : 0.0;
+        [[maybe_unused]] T ks[kPairKeep];
+        if constexpr (KEEP) {
+#pragma unroll
+            for (int o = 0; o < kPairKeep; ++o) ks[o] = T(-1);
+        }
         if constexpr (kX) {
             if (A.sec[0] >= 0 || A.sec[1] >= 0) {
                 // rounding bound of X: (TS + runs + 2) u per unit of sum |a'b'| <= sqrt(A2[i] A2[j]),
@@ -682,26 +706,134 @@ __device__ __forceinline__ void pair_tile(const PairArgs& A, const T* __restrict
         if (A.sec[0] >= 0) {
             const Section& sc = A.sp->sec[A.sec[0]];
             float v = -1.f;
-            if (opv) v = lin ? finalize_lin<T>(a1i + a1j, q2[0][q], ari + arj, a0 + b0, N, sum_t, sd_t)
+            if (opv) v = lin ? finalize_lin<T>(a1i + a1j, q2[0][q], ari + arj, a0 + b0, N, sum_t, sd_t, KEEP ? &ks[0] : nullptr)
                              : finalize<T>(l1[0][q], q2[0][q], lr[0][q], a0 + b0, N, sum_t, sd_t);
             A.scores[sc.base + rank_of(sc, i, j)] = v;
         }
         if (A.sec[1] >= 0) {
             const Section& sc = A.sp->sec[A.sec[1]];
             float v = -1.f;
-            if (opv) v = lin ? finalize_lin<T>(a1i - a1j, q2[1][q], ari - arj, a0 - b0, N, sum_t, sd_t)
+            if (opv) v = lin ? finalize_lin<T>(a1i - a1j, q2[1][q], ari - arj, a0 - b0, N, sum_t, sd_t, KEEP ? &ks[1] : nullptr)
                              : finalize<T>(l1[1][q], q2[1][q], lr[1][q], a0 - b0, N, sum_t, sd_t);
             A.scores[sc.base + rank_of(sc, i, j)] = v;
         }
         }
         if (A.sec[2] >= 0) {
             const Section& sc = A.sp->sec[A.sec[2]];
-            A.scores[sc.base + rank_of(sc, i, j)] = opv ? finalize<T>(s1[0][q], s2[0][q], sr[0][q], kmq, N, sum_t, sd_t) : -1.f;
+            A.scores[sc.base + rank_of(sc, i, j)] = opv ? finalize<T>(s1[0][q], s2[0][q], sr[0][q], kmq, N, sum_t, sd_t, KEEP ? &ks[2] : nullptr, KEEP ? &ks[5] : nullptr) : -1.f;
         }
         if (A.sec[3] >= 0) {
             const Section& sc = A.sp->sec[A.sec[3]];
-            A.scores[sc.base + rank_of(sc, i, j)] = opv ? finalize<T>(s1[1][q], s2[1][q], sr[1][q], kdq, N, sum_t, sd_t) : -1.f;
-            A.scores[sc.base + rank_of(sc, j, i)] = opv ? finalize<T>(s1[2][q], s2[2][q], sr[2][q], keq, N, sum_t, sd_t) : -1.f;
+            A.scores[sc.base + rank_of(sc, i, j)] = opv ? finalize<T>(s1[1][q], s2[1][q], sr[1][q], kdq, N, sum_t, sd_t, KEEP ? &ks[3] : nullptr, KEEP ? &ks[6] : nullptr) : -1.f;
+            A.scores[sc.base + rank_of(sc, j, i)] = opv ? finalize<T>(s1[2][q], s2[2][q], sr[2][q], keq, N, sum_t, sd_t, KEEP ? &ks[4] : nullptr, KEEP ? &ks[7] : nullptr) : -1.f;
+        }
+        if constexpr (KEEP) {
+#pragma unroll
+            for (int o = 0; o < kPairKeep; ++o) keep[(o * RI + q) * (TI * TJ / RI) + tid] = ks[o];
+        }
+    }
+}
+
+// the tile's scores against a later target (FP32, per-operand sums and kept values of the first):
+// + and - need the operands' sums alone, * a/b b/a the one sum of v' r.  Six packed operations per
+// two pairs and sample against sixteen; the values are the ones pair_tile computes, bit for bit
+__device__ __forceinline__ void pair_tile_cov(const PairArgs& A, const float* __restrict__ tc, const TargetStats* __restrict__ st,
+                                              const unsigned char* __restrict__ subvalid, const float* __restrict__ cache,
+                                              const double* __restrict__ A1, const double* __restrict__ AR, PairSmem<float>& S,
+                                              int64_t i0, int64_t j0, const float* __restrict__ keep) {
+    const int tid = threadIdx.x, lane = tid & 31, g = tid >> 5;
+    const int N = A.N;
+    const float sum_t = TgtView<float>::sum(st), sd_t = TgtView<float>::sd(st);
+    __syncthreads();
+    if (tid < TI + TJ) {
+        const int64_t f = tid < TI ? i0 + tid : j0 + (tid - TI);
+        S.prog[tid].n = 0;
+        S.ok[tid] = f < A.P && subvalid[f];
+        const float v = f < A.P ? cache[f] : 0.f;
+        if (tid < TI) S.a0[tid] = v; else S.b0[tid - TI] = v;
+    }
+    __syncthreads();
+    const int64_t j = j0 + lane;
+    constexpr int RH = RI / 2;
+    const f2 zero = f2pk(0.f, 0.f);
+    f2 SR[3][RH] = {{zero, zero}, {zero, zero}, {zero, zero}}, NKM[RH], NKD[RH], NKE[RH];
+    static_assert(RH == 2, "two pairs of i operands per thread");
+    if (A.sec[2] >= 0 || A.sec[3] >= 0) {
+        const float b0 = S.b0[lane], rb0 = rcp<float>(b0);
+#pragma unroll
+        for (int h = 0; h < RH; ++h) {
+            const float p = S.a0[g * RI + 2 * h], q = S.a0[g * RI + 2 * h + 1];
+            NKM[h] = f2pk(-(p * b0), -(q * b0));
+            NKD[h] = f2pk(-(p * rb0), -(q * rb0));
+            NKE[h] = f2pk(-(b0 * rcp<float>(p)), -(b0 * rcp<float>(q)));
+        }
+        float pf[kStageSlots], py[kStageSlots / 2];
+        stage_load<float>(A, nullptr, cache, tc, S, i0, j0, 0, g, lane, pf, py);
+        stage_store<float>(S, 0, pf, py, g, lane);
+        __syncthreads();
+        int b = 0;
+        for (int s0 = 0; s0 < N; s0 += TS, b ^= 1) {
+            const bool more = s0 + TS < N;
+            if (more) stage_load<float>(A, nullptr, cache, tc, S, i0, j0, s0 + TS, g, lane, pf, py);
+            const PairBuf<float>& B = S.buf[b];
+            const int ns = min(TS, N - s0);
+            auto step = [&](int s) {
+                const Quad<float> bq = B.bq[s][lane];
+                const f2 r2 = f2pk(bq.y, bq.y), bv2 = f2pk(bq.v, bq.v), br2 = f2pk(bq.r, bq.r);
+                const ulonglong2 av = *reinterpret_cast<const ulonglong2*>(&B.av[s][g * RI]);
+                const ulonglong2 ar = *reinterpret_cast<const ulonglong2*>(&B.ar[s][g * RI]);
+                const f2 avp[RH] = {av.x, av.y}, arp[RH] = {ar.x, ar.y};
+#pragma unroll
+                for (int h = 0; h < RH; ++h) {
+                    SR[0][h] = f2fma(f2fma(avp[h], bv2, NKM[h]), r2, SR[0][h]);
+                    SR[1][h] = f2fma(f2fma(avp[h], br2, NKD[h]), r2, SR[1][h]);
+                    SR[2][h] = f2fma(f2fma(bv2, arp[h], NKE[h]), r2, SR[2][h]);
+                }
+            };
+            if (ns == TS) {
+#pragma unroll 8
+                for (int s = 0; s < TS; ++s) step(s);
+            } else {
+                for (int s = 0; s < ns; ++s) step(s);
+            }
+            if (more) stage_store<float>(S, b ^ 1, pf, py, g, lane);
+            __syncthreads();
+        }
+    }
+    float sr[3][RI];
+#pragma unroll
+    for (int o = 0; o < 3; ++o)
+#pragma unroll
+        for (int h = 0; h < RH; ++h) f2up(SR[o][h], sr[o][2 * h], sr[o][2 * h + 1]);
+    const bool okj = S.ok[TI + lane];
+    const double a1j = j < A.P ? A1[j] : 0.0, arj = j < A.P ? AR[j] : 0.0;
+    const float inv_n = 1.f / (float)N;
+#pragma unroll
+    for (int q = 0; q < RI; ++q) {
+        const int64_t i = i0 + g * RI + q;
+        if (!pair_ok(i, j, A.P, A.Q, A.nxp)) continue;
+        const bool opv = okj && S.ok[g * RI + q];
+        auto kept = [&](int o) { return __ldcg(keep + (o * RI + q) * (TI * TJ / RI) + tid); };
+        if (A.sec[0] >= 0 || A.sec[1] >= 0) {
+            const double a1i = A1[i], ari = AR[i];
+#pragma unroll
+            for (int o = 0; o < 2; ++o) {
+                if (A.sec[o] < 0) continue;
+                const Section& sc = A.sp->sec[A.sec[o]];
+                A.scores[sc.base + rank_of(sc, i, j)] =
+                    !opv ? -1.f
+                         : finalize_cov((float)(o ? a1i - a1j : a1i + a1j) * inv_n, kept(o), (float)(o ? ari - arj : ari + arj), N,
+                                        sum_t, sd_t);
+            }
+        }
+        if (A.sec[2] >= 0) {
+            const Section& sc = A.sp->sec[A.sec[2]];
+            A.scores[sc.base + rank_of(sc, i, j)] = opv ? finalize_cov(kept(5), kept(2), sr[0][q], N, sum_t, sd_t) : -1.f;
+        }
+        if (A.sec[3] >= 0) {
+            const Section& sc = A.sp->sec[A.sec[3]];
+            A.scores[sc.base + rank_of(sc, i, j)] = opv ? finalize_cov(kept(6), kept(3), sr[1][q], N, sum_t, sd_t) : -1.f;
+            A.scores[sc.base + rank_of(sc, j, i)] = opv ? finalize_cov(kept(7), kept(4), sr[2][q], N, sum_t, sd_t) : -1.f;
         }
     }
 }
