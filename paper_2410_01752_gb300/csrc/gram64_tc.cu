@@ -48,17 +48,6 @@ struct Gram64Smem {
     int failed;
 };
 
-// K-major tile of rows of 64 bytes, 64-byte swizzle: 8-row groups 512 B apart
-__device__ __forceinline__ uint64_t desc_sw64(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(512 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)4 << 61;
-    return d;
-}
-
 // digits of rows [row0, row0 + gridDim.x): one CTA per row, all on the integer pipe
 __global__ void __launch_bounds__(512) k_gram_slices(const double* __restrict__ Z, int N, int Kpad, int row0, int R,
                                                      __half* __restrict__ sl, int* __restrict__ ex) {

@@ -183,6 +183,175 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN) : "memory");
 }
 
+// The network's forward pass, both layers and the head in one kernel: out[r] =
+// w3 . relu(W2 relu(W1 x + b1) + b2) + b3, the hidden values rounded to BF16 as the layers' own
+// kernels store them.  Layer by layer it was bound by the activations' way through HBM (4.6 GB
+// for 4.45e6 prefixes, 3.1 ms); here they stay on the SM and the TMEM reads and the activation's
+// arithmetic bound it, 1.04 ms.  A CTA keeps both weight matrices in shared memory and takes
+// tiles of 128 rows: warp 8 streams the rows (two buffers), warp 9 issues layer 1 (K = 32) into
+// TMEM columns 0 .. 255 and layer 2 into 256 .. 511, and eight warps (rows 32 (w % 4) ..,
+// columns 128 (w / 4) ..) turn layer 1's sums into layer 2's operand, in the 128-byte swizzle, and
+// layer 2's into the output.  Layer 1 of the next tile runs behind layer 2's epilogue.
+struct MlpSmem {
+    uint8_t w2[4][kHid * 128];
+    uint8_t h1[4][GT * 128];
+    uint8_t w1[kHid * 64];
+    uint8_t x[2][GT * 64];
+    uint64_t w_full, x_full[2], x_empty[2], d1_full, d1_empty, h1_full, d2_full, d2_empty;
+    uint32_t tmem_base;
+    int failed, stop;             // stop: the epilogue warps' own, set before their first barrier of a tile
+    float part[GT];
+};
+constexpr int kMlpThreads = 320;
+
+__global__ void __launch_bounds__(kMlpThreads, 1)
+k_mlp_fwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w1,
+          const __grid_constant__ CUtensorMap map_w2, const float* __restrict__ p, int64_t M, int64_t tiles,
+          float* __restrict__ out, int* err) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    MlpSmem& S = *reinterpret_cast<MlpSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        mbar_init(&S.w_full, 1);
+        for (int s = 0; s < 2; ++s) { mbar_init(&S.x_full[s], 1); mbar_init(&S.x_empty[s], 1); }
+        mbar_init(&S.d1_full, 1); mbar_init(&S.d1_empty, 8); mbar_init(&S.h1_full, 8);
+        mbar_init(&S.d2_full, 1); mbar_init(&S.d2_empty, 8);
+        S.failed = S.stop = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem_base)), "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = S.tmem_base;
+    const int64_t first = blockIdx.x, step = gridDim.x;
+    auto arrive = [&](uint64_t* bar) {
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+    };
+    if (warp == 8 && lane == 0) {
+        mbar_expect_tx(&S.w_full, sizeof(S.w1) + sizeof(S.w2));
+        tma_load_2d(S.w1, &map_w1, 0, 0, &S.w_full);
+        for (int kb = 0; kb < 4; ++kb) tma_load_2d(S.w2[kb], &map_w2, kb * 64, 0, &S.w_full);
+        bool ok = true;
+        int n = 0;
+        for (int64_t t = first; t < tiles; t += step, ++n) {
+            const int s = n & 1;
+            if (n >= 2 && !mbar_wait(&S.x_empty[s], (uint32_t)((n >> 1) - 1) & 1u)) { ok = false; break; }
+            mbar_expect_tx(&S.x_full[s], GT * 64);
+            tma_load_2d(S.x[s], &map_x, 0, (int)(t * GT), &S.x_full[s]);
+        }
+        // the copies land before the CTA goes
+        ok = mbar_wait(&S.w_full, 0) && ok;
+        for (int q = n > 2 ? n - 2 : 0; q < n; ++q) ok = mbar_wait(&S.x_full[q & 1], (uint32_t)(q >> 1) & 1u) && ok;
+        if (!ok) S.failed = 1;
+    } else if (warp == 9 && lane == 0) {
+        constexpr uint32_t idesc = idesc_f16(1u, GT, kHid);
+        bool ok = mbar_wait(&S.w_full, 0);
+        int n = 0;
+        auto layer1 = [&](int q) {                    // tile q of this CTA
+            const int s = q & 1;
+            if (!mbar_wait(&S.x_full[s], (uint32_t)(q >> 1) & 1u)) return false;
+            if (q > 0 && !mbar_wait(&S.d1_empty, (uint32_t)(q - 1) & 1u)) return false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint64_t a = desc_sw64(smem_u32(S.x[s])), b = desc_sw64(smem_u32(S.w1));
+#pragma unroll
+            for (int k = 0; k < 2; ++k) mma_f16(tmem, a + (uint64_t)(2 * k), b + (uint64_t)(2 * k), idesc, k > 0 ? 1u : 0u);
+            mma_commit(&S.x_empty[s]);
+            mma_commit(&S.d1_full);
+            return true;
+        };
+        if (first < tiles) ok = ok && layer1(0);
+        for (int64_t t = first; t < tiles && ok; t += step, ++n) {
+            ok = mbar_wait(&S.h1_full, (uint32_t)n & 1u) && (n == 0 || mbar_wait(&S.d2_empty, (uint32_t)(n - 1) & 1u));
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+            for (int kb = 0; kb < 4; ++kb) {
+                const uint64_t a = desc_sw128(smem_u32(S.h1[kb])), b = desc_sw128(smem_u32(S.w2[kb]));
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    mma_f16(tmem + kHid, a + (uint64_t)(2 * k), b + (uint64_t)(2 * k), idesc, kb > 0 || k > 0 ? 1u : 0u);
+            }
+            mma_commit(&S.d2_full);
+            if (t + step < tiles) ok = layer1(n + 1);
+        }
+        if (!ok) S.failed = 1;
+    } else if (warp < 8) {
+        const int quad = warp & 3, half = warp >> 2, row = quad * 32 + lane;
+        const uint32_t base = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * 128);
+        const float* b1 = p + oB1 + half * 128;
+        const float* b2 = p + oB2 + half * 128;
+        const float* w3 = p + oW3 + half * 128;
+        int n = 0;
+        for (int64_t t = first; t < tiles; t += step, ++n) {
+            const uint32_t ph = (uint32_t)n & 1u;
+            bool ok = mbar_wait(&S.d1_full, ph);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+            for (int cb = 0; cb < 4; ++cb) {
+                uint32_t r[32];
+                tmem_ld32(base + (uint32_t)(cb * 32), r);
+                uint8_t* dst = S.h1[half * 2 + (cb >> 1)] + row * 128;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    uint32_t pk[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int k = 8 * c + 2 * u;
+                        const float2 bb = __ldg(reinterpret_cast<const float2*>(b1 + cb * 32 + k));
+                        const __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(__uint_as_float(r[k]) + bb.x, 0.f),
+                                                                      fmaxf(__uint_as_float(r[k + 1]) + bb.y, 0.f));
+                        pk[u] = *reinterpret_cast<const uint32_t*>(&h);
+                    }
+                    *reinterpret_cast<uint4*>(dst + (((cb & 1) * 4 + c) ^ (row & 7)) * 16) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            arrive(&S.d1_empty);
+            arrive(&S.h1_full);
+            ok = mbar_wait(&S.d2_full, ph) && ok;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            float s4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+            for (int cb = 0; cb < 4; ++cb) {
+                uint32_t r[32];
+                tmem_ld32(base + (uint32_t)(kHid + cb * 32), r);
+#pragma unroll
+                for (int k = 0; k < 32; k += 2) {
+                    const float2 bb = __ldg(reinterpret_cast<const float2*>(b2 + cb * 32 + k));
+                    const float2 ww = __ldg(reinterpret_cast<const float2*>(w3 + cb * 32 + k));
+                    const float2 h = __bfloat1622float2(__floats2bfloat162_rn(fmaxf(__uint_as_float(r[k]) + bb.x, 0.f),
+                                                                             fmaxf(__uint_as_float(r[k + 1]) + bb.y, 0.f)));
+                    s4[k & 2] = fmaf(h.x, ww.x, s4[k & 2]);
+                    s4[(k & 2) + 1] = fmaf(h.y, ww.y, s4[(k & 2) + 1]);
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            arrive(&S.d2_empty);
+            const float s = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+            // the two halves of a row meet in shared memory (both barriers: the eight warps)
+            if (half) S.part[row] = s;
+            if (!ok) *(volatile int*)&S.stop = 1;
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            const bool stop = *(volatile int*)&S.stop != 0;         // the same for all eight warps
+            if (!half && !stop && t * GT + row < M) out[t * GT + row] = s + S.part[row] + __ldg(p + oB3);
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            if (stop) { S.failed = 1; break; }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0 && S.failed) atomicExch(err, 1);
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
 // ---------------------------------------------------------------------------------
 // CUDA-core parts of the network
 // ---------------------------------------------------------------------------------
@@ -620,16 +789,16 @@ __global__ void k_wsel_compact(const float* __restrict__ score, const int* __res
 // ---------------------------------------------------------------------------------
 // host: GEMM launch
 // ---------------------------------------------------------------------------------
-bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows) {
+bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows, int box_cols = GBK) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
     const cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     const cuuint64_t gstride[1] = {(cuuint64_t)cols * 2};
-    const cuuint32_t box[2] = {GBK, (cuuint32_t)box_rows};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     const cuuint32_t es[2] = {1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), gdim, gstride, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+               CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <int EPI, int BN>
@@ -704,10 +873,10 @@ sisso_status mlp_reserve(sisso_mlp* m, int64_t rows, bool train) {
     auto al = [&](void** q, size_t bytes) { if (ok && cudaMalloc(q, bytes) != cudaSuccess) ok = false; };
     al((void**)&m->xin, sizeof(float) * R * kIn);
     al((void**)&m->Xb, 2 * R * kInPad);
-    al((void**)&m->H1, 2 * R * kHid);
-    al((void**)&m->H2, 2 * R * kHid);
     al((void**)&m->out, sizeof(float) * R);
     if (train) {
+        al((void**)&m->H1, 2 * R * kHid);
+        al((void**)&m->H2, 2 * R * kHid);
         al((void**)&m->XT, 2 * (size_t)GT * R);
         al((void**)&m->H1T, 2 * (size_t)kHid * R);
         al((void**)&m->dZ2, 2 * R * kHid);
@@ -723,12 +892,27 @@ sisso_status mlp_reserve(sisso_mlp* m, int64_t rows, bool train) {
     return SISSO_OK;
 }
 
-// forward on rows already packed in m->Xb (Mpad rows); train: keep H1^T for the backward
+// forward on rows already packed in m->Xb (Mpad rows); train: layer by layer, the hidden values and
+// H1^T kept for the backward
 cudaError_t mlp_forward_dev(sisso_mlp* m, int64_t M, bool train) {
     const int64_t Mpad = pad128(M);
+    if (!train) {
+        CUtensorMap mx, m1, m2;
+        if (!make_map(&mx, m->Xb, Mpad, kInPad, GT, 32) || !make_map(&m1, m->W1b, kHid, kInPad, kHid, 32) ||
+            !make_map(&m2, m->W2b, kHid, kHid, kHid))
+            return cudaErrorInvalidValue;
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
+        const int64_t tiles = Mpad / GT;
+        const size_t smem = sizeof(MlpSmem) + 1024;
+        cudaFuncSetAttribute(k_mlp_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k_mlp_fwd<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, sms)), kMlpThreads, smem, m->stream>>>(
+            mx, m1, m2, m->p, M, tiles, m->out, m->err);
+        return cudaGetLastError();
+    }
     GemmArgs g{};
     g.rows = (int)std::min<int64_t>(M, INT32_MAX); g.err = m->err;
-    g.bias = m->p + oB1; g.H = m->H1; g.ldh = kHid; g.HT = train ? m->H1T : nullptr; g.ldt = (int)Mpad;
+    g.bias = m->p + oB1; g.H = m->H1; g.ldh = kHid; g.HT = m->H1T; g.ldt = (int)Mpad;
     cudaError_t e = gemm(m->stream, m->Xb, Mpad, m->W1b, kHid, kInPad, EPI_RELU, g);
     if (e) return e;
     g.bias = m->p + oB2; g.H = m->H2; g.HT = nullptr;
@@ -1120,7 +1304,7 @@ sisso_status l0_learned(sisso_ctx* c, sisso_mlp* mlp, const double* G, const dou
         k_wsel_find<<<1, 32, 0, c->stream>>>(hist, pass, state, budget);
     }
     k_wsel_compact<<<gs, 256, 0, c->stream>>>(score, plist, np, state, sel, count, np, nullptr);
-    c->stats.launches += 13;   // tables, features, 2 layers + head, add, 3 x (histogram, find), compact
+    c->stats.launches += 11;   // tables, features, network, add, 3 x (histogram, find), compact
     unsigned h_count = 0;
     cudaMemcpyAsync(&h_count, count, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream);
     ck(cudaStreamSynchronize(c->stream), "learned: selection");

@@ -58,6 +58,17 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
     return d;
 }
 
+// K-major tile of rows of 64 bytes, 64-byte swizzle: 8-row groups 512 B apart
+__device__ __forceinline__ uint64_t desc_sw64(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(512 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;
+    return d;
+}
+
 // instruction descriptor of tcgen05.mma kind::f16 / kind::tf32: FP32 accumulator, A and B of
 // the same type (kind::f16: 0 FP16, 1 BF16; kind::tf32: 2 TF32), both K-major, tile M x N
 __host__ __device__ constexpr uint32_t idesc_f16(uint32_t ab_type, int M = 128, int N = 128) {
