@@ -873,6 +873,10 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
                                                                                                  c->l0_Gq + (size_t)n * n);
         c->stats.launches++;
         A.Gq = c->l0_Gq; A.bq = c->l0_Gq + (size_t)n * n;
+        A.conf_cap = (int64_t)1 << 21;
+        if ((st = tmp_alloc(c, (void**)&A.conf, sizeof(uint64_t) * (size_t)(A.conf_cap + 1), "l0 candidates"))) return st;
+        A.conf_count = reinterpret_cast<unsigned long long*>(A.conf + A.conf_cap);
+        cudaMemsetAsync(A.conf_count, 0, sizeof(unsigned long long), c->stream);
         const int DC = D - 3, m_max = n - DC;
         // two launches: the prefixes with many features to their right, then those with few
         const int slices = DC == 1 ? 4 : 1;
@@ -893,7 +897,10 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
             if (DC == 1) SG_BLOCK(1, kBWarpsSmall, big, all, ms); else SG_BLOCK(2, kBWarpsSmall, big, all, ms);
         }
 #undef SG_BLOCK
-        c->stats.launches += big > 0 && all > big;
+        if (DC == 1) k_l0_confirm<4><<<c->sms * 4, 128, 0, c->stream>>>(A);
+        else k_l0_confirm<5><<<c->sms * 4, 128, 0, c->stream>>>(A);
+        cudaFreeAsync(A.conf, c->stream);
+        c->stats.launches += 1 + (big > 0 && all > big);
     } else switch (DP) {
         case 0: SG_TILE(0); break;
         case 1: SG_TILE(1); break;

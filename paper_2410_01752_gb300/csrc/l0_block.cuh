@@ -26,7 +26,7 @@
 // columns it does not dismiss; they are decided after the sweep, so that no call stands between the
 // row constants and their registers (with the calls inside, a third of the instructions were
 // spills' and their operands').
-// Measured at n = 300, D = 5 (1.96e10 subsets) over five problems: 20 to 25 ms (30 to 36 with the
+// Measured at n = 300, D = 5 (1.96e10 subsets) over five problems: 20 to 25.5 ms (30 to 36 with the
 // filter itself in the sweep, 43 and more by k_l0_tile); 0.6 warp instructions a subset at 56% of
 // the issue slots.  Forms that took longer than k_l0_tile: lanes as columns with the row constants
 // shuffled in (89 ms), and four warps sharing a p through a record table and a barrier (46 ms).
@@ -74,11 +74,24 @@ __device__ __noinline__ double block_exact(const TileArgs& A, const int (&pos)[D
     return B;
 }
 
-// the warp's queued candidates (local positions p, i1, x in ten bits each)
+// the warp's queued candidates (local positions p, i1, x in ten bits each), decided here or, with
+// defer and while the list has room, left for k_l0_confirm: a p whose every extension nearly ties
+// held one warp for milliseconds while the other SMs had nothing left to do (C(300, 4) with
+// 22 000 candidates around one feature: 3.3 ms, 1.07 with the list, 0.5 where there are few)
 template <int DC>
-__device__ __noinline__ double block_flush(const TileArgs& A, const BlockPre* P, const unsigned* q, int qn, double B) {
+__device__ __noinline__ double block_flush(const TileArgs& A, const BlockPre* P, const unsigned* q, int qn, double B, bool defer) {
     const int lane = threadIdx.x & 31;
     const double thr = B + A.tie64;
+    int64_t at = -1;
+    if (defer) {
+        if (lane == 0) at = (int64_t)atomicAdd(A.conf_count, (unsigned long long)qn);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (at + qn > A.conf_cap) {                               // full: the slots taken hold nothing
+            for (int e = lane; e < qn; e += 32)
+                if (at + e < A.conf_cap) A.conf[at + e] = ~0ull;
+            at = -1;
+        }
+    }
     for (int e = lane; e < qn; e += 32) {
         const unsigned v = q[e];
         int pos[DC + 3];
@@ -95,12 +108,34 @@ __device__ __noinline__ double block_flush(const TileArgs& A, const BlockPre* P,
                 pos[j - 1] = lo;
                 pos[j] = hi;
             }
-        B = block_exact<DC + 3>(A, pos, B, thr);
+        if (at >= 0) {
+            uint64_t k = 0;
+#pragma unroll
+            for (int m = 0; m < DC + 3; ++m) k |= (uint64_t)pos[m] << (12 * m);
+            A.conf[at + e] = k;
+        } else {
+            B = block_exact<DC + 3>(A, pos, B, thr);
+        }
     }
     __syncwarp();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) B = fmin(B, __shfl_xor_sync(0xffffffffu, B, o));
     return fmin(B, okey_inv(*(volatile unsigned long long*)A.ub_key));
+}
+
+// the deferred candidates, a thread each
+template <int D>
+__global__ void __launch_bounds__(128) k_l0_confirm(const __grid_constant__ TileArgs A) {
+    const int64_t n = min((int64_t)*A.conf_count, A.conf_cap);
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = A.conf[e];
+        if (k == ~0ull) continue;
+        int pos[D];
+#pragma unroll
+        for (int m = 0; m < D; ++m) pos[m] = (int)((k >> (12 * m)) & 4095u);
+        const double B = okey_inv(*(volatile unsigned long long*)A.ub_key);
+        block_exact<D>(A, pos, B, B + A.tie64);
+    }
 }
 
 // the sweep's row constants of a lane, row groups j and j + 1 per register pair: -R[p][i1],
@@ -154,6 +189,7 @@ struct BlockP {
     float A0, base, thrN;        // |w_p| / sqrt(d'_p), syy' - w_p^2, (B + tie) / N
     float e0, e1;                // the filter's errors at this prefix's scale
     float q2, rmax;              // largest |a2| and root of the largest dp
+    int flushes;                 // full queues of this p (the first is decided at once, for its bound)
 };
 struct BlockRow { float r, d, n, l1; };      // R[p][x], dp, np, |coefficient on p|
 
@@ -193,7 +229,7 @@ struct BlockQueue { double B; int qn, taken; };
 
 // a column some lane may keep: the decisions row group by row group, into the warp's queue
 template <int DC>
-__device__ __noinline__ BlockQueue block_take(const TileArgs& A, const BlockPre* P, const BlockP& Q, const float* Gp,
+__device__ __noinline__ BlockQueue block_take(const TileArgs& A, const BlockPre* P, BlockP& Q, const float* Gp,
                                               const float2* dn, int rb, int x, unsigned* q, int qn,
                                               double B) {
     const int lane = threadIdx.x & 31;
@@ -217,8 +253,10 @@ __device__ __noinline__ BlockQueue block_take(const TileArgs& A, const BlockPre*
         taken += __popc(mask);
         __syncwarp();
         if (qn >= 32) {
-            B = block_flush<DC>(A, P, q, qn, B);
+            B = block_flush<DC>(A, P, q, qn, B, Q.flushes > 0);
             qn = 0;
+            if (lane == 0) ++Q.flushes;
+            __syncwarp();
         }
     }
     return BlockQueue{B, qn, taken};
@@ -352,7 +390,7 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(const __grid_consta
             BlockP Q;
             {
                 const float2 f = dn[p];
-                Q.p = p; Q.m = m;
+                Q.p = p; Q.m = m; Q.flushes = 0;
                 Q.ok = P.ok && f.x > A.tau;
                 Q.invd = __frsqrt_rn(f.x > 0.f ? f.x : 1.f);
                 Q.w = f.y * Q.invd;
@@ -450,7 +488,7 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(const __grid_consta
             __syncwarp();
         }
         if (qn > 0) {                                      // the queue's entries are relative to this prefix
-            const double B = block_flush<DC>(A, &P, q, qn, s_b[w]);
+            const double B = block_flush<DC>(A, &P, q, qn, s_b[w], false);
             __syncwarp();
             if (lane == 0) s_b[w] = B;
         }

@@ -105,6 +105,9 @@ struct TileArgs {
     float* band_r32;
     unsigned long long* examined;
     unsigned long long* candidates;      // subsets sent to the exact test
+    uint64_t* conf;                      // deferred candidates (l0_block.cuh), their count and room
+    unsigned long long* conf_count;
+    int64_t conf_cap;
     const int* perm;                     // features in the greedy search's order (l0_block.cuh),
     const double *Gq, *bq;               //   and the FP64 Gram (row stride n) and moments in that order
     const unsigned* prefix_mask;         // optional: one bit per (D-2)-prefix in colex order;
