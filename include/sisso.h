@@ -97,8 +97,10 @@ typedef struct {
                                selection and refits are always FP64 (default FP32) */
     int grammar;            /* SISSO_GRAMMAR_* (default EQ2) */
     int survivors;          /* FP32 screening window: candidates re-scored in FP64 per
-                               step (0 = max(5 k, min(max(4096, 32 k), 2^26 / N))); grown
-                               x4 automatically when it cannot prove the selection exact */
+                               step (0 = max(5 k, min(max(4096, 32 k), 2^26 / N)), of which
+                               the best 5 k, 2.5 k above 4096 samples, and those within the
+                               screening margin of them are tried first); grown x4
+                               automatically when it cannot prove the selection exact */
     double band_rel;        /* l0: FP32 RSS band, relative to SST, refit in FP64
                                (0 = 1e-4) */
     int64_t max_band;       /* l0: capacity of the FP64 refit list (0 = 1<<22) */
@@ -132,14 +134,13 @@ typedef struct {
                                is built from one that does, is invalid (scores -1, never
                                selected); ids are those of the space without units. */
     int screen;             /* mixed forms' scoring of the top level's binary candidates:
-                               SISSO_SCREEN_AUTO (default) from split 16-bit tensor-core
-                               products (§2.2 Eq. 5 as a contraction; each key carries its
-                               error bound, see sisso_bilinear_tc) when the pairs lie within
-                               phi_{L-1} (EQ2 grammar, or rung <= 2) and |phi_{L-1}| <= 4096,
-                               else the FP32 CUDA-core kernel; SISSO_SCREEN_CORES always the
-                               CUDA-core kernel; SISSO_SCREEN_TENSOR the tensor cores also for
-                               the NEW_X_PREV pairs phi_{L-2} x new_{L-1} at rung >= 3 (when
-                               |phi_{L-2}| <= 4096 and the products fit 48 GB) */
+                               SISSO_SCREEN_AUTO (default) and SISSO_SCREEN_TENSOR from split
+                               16-bit tensor-core products (§2.2 Eq. 5 as a contraction; each
+                               key's error is bounded, keys whose bound is too wide are scored
+                               directly), as FP32 precision does, while the operands' rows fit
+                               40 GB; SISSO_SCREEN_CORES always the CUDA-core kernel.
+                               stats.screen_tc reports the tensor cores for AUTO when the pairs
+                               lie within phi_{L-1} (EQ2 grammar, or rung <= 2) and for TENSOR */
     int gram;               /* FP32 precision's subspace Gram (§2.3 Eq. 7):
                                SISSO_GRAM_AUTO (default) and SISSO_GRAM_FP64 build it from
                                FP64 rows on the CUDA cores, and the l0 result is the FP64
@@ -197,11 +198,11 @@ typedef struct {
     int64_t l0_candidates;       /* subsets its filter sent to the exact FP32/FP64 test */
     int64_t certified_prefixes;  /* learned D = 5 step: 3-prefixes its certificate left to enumerate */
     int screen_tc;               /* 1 if the top level's pairs were scored on the tensor cores */
-    int64_t tc_keys_raised;      /* ... keys raised to their error bound (bound above the FP32
-                                    screening margin, or the variance not resolved) */
-    int64_t pm_keys_direct;      /* FP32 top-level + / - candidates whose cross-sum key was left
-                                    open (operands that nearly cancel) and scored from the
-                                    direct sums instead, all steps */
+    int64_t tc_keys_raised;      /* ... keys raised to their error bound (0: keys with a wide
+                                    bound are scored directly, see pm_keys_direct) */
+    int64_t pm_keys_direct;      /* top-level binary candidates whose key from per-operand and
+                                    pair sums was left open (terms that nearly cancel) and
+                                    scored from the direct sums instead, all steps */
 } sisso_stats;
 
 void sisso_default_opts(sisso_opts* opts);

@@ -1,9 +1,12 @@
 // l0.cu — the sparsifying operator (§2.3, Eqs. 7-8) on the device.
 //
 //  Subspace: each new S member is evaluated in FP64 from the primaries and standardised
-//  (rows of Z); the FP64 Gram G = Z Z^T / N and b = Z y~ / N grow by the new rows only.
+//  (rows of Z); the FP64 Gram G = Z Z^T / N and b = Z y~ / N grow by the new rows only (many
+//  samples: by exact integer tensor-core products, gram64_tc.cu).
 //
-//  Enumeration (k_l0_enum): every D-subset {p_0 < ... < p_{D-3} < i1 < i2} is one FP32
+//  Enumeration, FP32 precision: FP64 pairs at D = 2 and 3 (l0_pair64.cuh), the CTA-shared prefix at
+//  D = 4 and 5 (l0_block.cuh), beyond their sizes and for prefix masks the tiles of l0_tile.cuh.
+//  FP64 precision, prefix lists and the mixed forms (k_l0_enum): every D-subset {p_0 < ... < p_{D-3} < i1 < i2} is one FP32
 //  (or FP64) Cholesky solve.  A warp owns a prefix (p_0..p_{D-3}) and a run of i1 rows.
 //  It first tabulates, for every x > i1_start, the prefix-reduced row of x:
 //      R[m][x] = (G[x][p_m] - sum_{m'<m} R[m'][x] L[m][m']) / L[m][m],

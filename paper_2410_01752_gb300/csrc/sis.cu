@@ -1,18 +1,20 @@
 // sis.cu — sure independence screening (§2.2, Eqs. 5-6) on the device.
 //
-//  1. k_score_pairs: the fused generate-and-score kernel for the top level's binary
-//     sections (almost all of phi_L).  A CTA owns a 32 x 32 tile of operand pairs; for
-//     each 32-sample chunk it rebuilds the 64 operand features from the primaries
-//     (postfix programs, one warp per feature, lanes over samples) into shared memory,
-//     then every thread accumulates, for 4 pairs x 5 operators (+, -, *, a/b, b/a), the
-//     shifted sums S1 = sum v', S2 = sum v'^2, SR = sum v' r~ with v' = v - v(sample 0).
-//     Nothing but one FP32 score per candidate leaves the CTA.
-//  2. k_score_generic: every other id (lower levels, unary sections), thread per id.
-//  3. Selection: a 3-pass radix select finds the score of the M-th best candidate, the
-//     ids at or above it are compacted, re-scored in FP64 (k_rescore), sorted by
-//     (score desc, id asc) and walked by one CTA (k_walk) with the tie and duplicate
-//     rules.  The host checks that the k-th accepted FP64 score clears the FP32 cut-off
-//     by the FP32 error margin; if not, the window grows and selection repeats.
+//  1. The top level's binary sections (almost all of phi_L): pair_tc.cu's tensor-core products
+//     for the FP32 and mixed forms; k_score_pairs otherwise (FP64, SISSO_SCREEN_CORES, operands
+//     too large for the rows or the cache, or too many open keys).  A CTA of k_score_pairs owns a
+//     32 x 32 tile of operand pairs, stages 32 samples of both sides at a time (from the operand
+//     cache, or rebuilt from the primaries by postfix programs), and every thread accumulates, for
+//     4 pairs x 5 operators (+, -, *, a/b, b/a), the shifted sums S1 = sum v', S2 = sum v'^2,
+//     SR = sum v' r~ with v' = v - v(sample 0).  Only one FP32 score per candidate leaves the CTA.
+//  2. The other ids: from cached operand rows (k_score_cached, k_score_unary_w, k_score_unary_runs)
+//     or, without a cache, k_score_generic, a thread per id.
+//  3. Selection: a 3-pass radix select finds the score of the M-th best candidate, the ids at or
+//     above it are compacted and narrowed to the best 5 k and their margin (k_narrow), re-scored in
+//     FP64 (k_rescore), sorted by (score desc, id asc) by counted ranks (k_rank_sort) and walked
+//     by one CTA (k_walk) with the tie and duplicate rules.  The host checks that the k-th
+//     accepted FP64 score clears the FP32 cut-off by the FP32 error margin; if not, the whole
+//     window is taken, then grown, and selection repeats.
 #include "sis_device.cuh"
 
 #include <algorithm>
