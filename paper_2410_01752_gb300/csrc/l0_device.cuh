@@ -292,6 +292,10 @@ template <typename T> __device__ __forceinline__ T round_up(double x);
 template <> __device__ __forceinline__ float round_up<float>(double x) { return __double2float_ru(x); }
 template <> __device__ __forceinline__ double round_up<double>(double x) { return x; }
 
+// 1 / sqrt(x), rounded once in FP32 (a root and a division there took as long as the sweep of a row)
+__device__ __forceinline__ float rsq(float x) { return __frsqrt_rn(x); }
+__device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
+
 template <typename T, int DP, int MODE>
 __device__ __forceinline__ void enum_item(const EnumArgs<T>& A, T* tab, int64_t item, T& best,
                                           unsigned long long& best_key, double thr, unsigned long long& my_examined) {
@@ -381,7 +385,7 @@ __device__ __forceinline__ void enum_item(const EnumArgs<T>& A, T* tab, int64_t 
             const T d1 = dpart[ic];
             ok1[k] = pre_ok && d1 > T(A.tau);
             if (!A.fp32 && !ok1[k]) live[k] = false;          // FP64: singular, every extension skipped
-            isd1[k] = T(1) / sqrt(d1 > T(0) ? d1 : T(1));
+            isd1[k] = rsq(d1 > T(0) ? d1 : T(1));
             w1[k] = npart[ic] * isd1[k];
             base_c[k] = A.syy - (pw2 + w1[k] * w1[k]);
             // rss < best (MODE 0) or rss <= thr_eff (MODE 1)  <=>  num^2 - c d2 > 0 (>= 0)
