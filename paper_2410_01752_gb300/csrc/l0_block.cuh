@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(const __grid_consta
         if (tid == 0) {
             int pre[2] = {pre_rank, -1};
             if (DC == 2) {
-                const int64_t m = top2_fast(pre_rank);
+                const int64_t m = colex_top2(pre_rank);
                 pre[1] = (int)m;
                 pre[0] = (int)(pre_rank - binom2(m));
             }

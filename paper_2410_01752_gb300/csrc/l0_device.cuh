@@ -80,15 +80,19 @@ __device__ __forceinline__ int64_t binom3(int64_t m) { return m * (m - 1) * (m -
 
 __device__ __forceinline__ int64_t binom4(int64_t m) { return m * (m - 1) * (m - 2) * (m - 3) / 24; }
 
-// largest m with C(m, 2) <= r
+// largest m with C(m, 2) <= r, and C(m, 3): FP32 estimates (within a step or two at any rank of
+// 65535 features) corrected by exact 64-bit integer steps.  The FP64 root of a rank held the SM's
+// FP64 pipe for 700 cycles an item, most of what a small enumeration took
 __device__ __forceinline__ int64_t colex_top2(int64_t r) {
-    int64_t m = (int64_t)((1.0 + sqrt(1.0 + 8.0 * (double)r)) * 0.5);
+    int64_t m = (int64_t)((1.f + sqrtf(1.f + 8.f * (float)r)) * 0.5f);
+    if (m < 1) m = 1;
     while (m > 1 && binom2(m) > r) --m;
     while (binom2(m + 1) <= r) ++m;
     return m;
 }
 __device__ __forceinline__ int64_t colex_top3(int64_t r) {
-    int64_t m = (int64_t)cbrt(6.0 * (double)r) + 1;
+    int64_t m = (int64_t)cbrtf(6.f * (float)r) + 1;
+    if (m < 2) m = 2;
     while (m > 2 && binom3(m) > r) --m;
     while (binom3(m + 1) <= r) ++m;
     return m;
@@ -311,8 +315,8 @@ __device__ __forceinline__ void enum_item(const EnumArgs<T>& A, T* tab, int64_t 
     // item -> (prefix in colex order, chunk): prefixes are the (D-2)-combinations of
     // [0, n-2) ordered by their largest element, so the longest sweeps come first
     int pre[DP > 0 ? DP : 1];
-    const int64_t prank = item / A.cpp;
-    const int chunk = (int)(item % A.cpp);
+    const int64_t prank = (item >> 32) == 0 ? (int64_t)((unsigned)item / (unsigned)A.cpp) : item / A.cpp;
+    const int chunk = (int)(item - prank * A.cpp);
     if (A.prefix_list) {
 #pragma unroll
         for (int m = 0; m < DP; ++m) pre[m] = A.prefix_list[prank * (DP > 0 ? DP : 1) + m];

@@ -122,33 +122,6 @@ __device__ __forceinline__ float tile_apost_err(const TileArgs& A, float s, floa
                       (float)(A.D + 3) * (2.f * (float)A.sst + fabsf(rss)));
 }
 
-// r-th DP-combination in colex order, as colex_unrank but from FP32 estimates of the
-// largest element (sqrt / cbrt of the rank) corrected by exact 64-bit integer steps: the
-// GB300 FP64 pipe runs at a small fraction of the FP32 rate
-__device__ __forceinline__ int64_t top2_fast(int64_t r) {
-    int64_t m = (int64_t)((1.f + sqrtf(1.f + 8.f * (float)r)) * 0.5f);
-    if (m < 1) m = 1;
-    while (m > 1 && binom2(m) > r) --m;
-    while (binom2(m + 1) <= r) ++m;
-    return m;
-}
-__device__ __forceinline__ int64_t top3_fast(int64_t r) {
-    int64_t m = (int64_t)cbrtf(6.f * (float)r) + 1;
-    if (m < 2) m = 2;
-    while (m > 2 && binom3(m) > r) --m;
-    while (binom3(m + 1) <= r) ++m;
-    return m;
-}
-template <int DP> __device__ __forceinline__ void colex_unrank_fast(int64_t r, int (&p)[DP > 0 ? DP : 1]) {
-    if (DP == 0) return;
-    if (DP == 1) { p[0] = (int)r; return; }
-    int64_t m;
-    if (DP >= 3) { m = top3_fast(r); p[DP > 2 ? 2 : 0] = (int)m; r -= binom3(m); }
-    m = top2_fast(r);
-    p[1] = (int)m;
-    p[0] = (int)(r - binom2(m));
-}
-
 // prefix factor of one warp's current prefix, in shared memory (read by the exact test)
 struct PrefixSm {
     int pre[4];
@@ -353,7 +326,7 @@ __global__ void __launch_bounds__(kTW * 32, 2) k_l0_tile(TileArgs A) {
             // ---- prefix factor (warp-uniform, redundant in every lane) ---------------
             int pre[DPa];
             float L[DPa][DPa], invd[DPa], wv[DPa];
-            colex_unrank_fast<DP>(prank, pre);
+            colex_unrank<DP>(prank, pre);
             bool ok = true;
 #pragma unroll
             for (int j = 0; j < DP; ++j) {
