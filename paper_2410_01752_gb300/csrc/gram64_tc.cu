@@ -19,8 +19,8 @@
 // warps read an accumulator as soon as its weight is complete, while the next block's products of
 // the weights already read proceed.
 // Measured: 200, 400 and 600 features over 65 536 samples, 200 new each, 19.8 -> 3.0 ms (2.55 the
-// products, 0.29 the digits, 0.15 the moments); the operands' shared-memory reads bound a
-// 128 x 64 tile, at about half the cuBLAS rate of FP16.
+// products, 0.29 the digits, 0.15 the moments); the tensor pipe is 27% active, the epilogue
+// warps wait for TMEM: eight accumulators of 64 columns leave none to double-buffer.
 #include "tc_device.cuh"
 
 #include <cuda_fp16.h>
