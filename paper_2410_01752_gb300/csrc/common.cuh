@@ -529,6 +529,16 @@ void pair_tc_reset(sisso_ctx* c);
 void pair_tc_free(sisso_ctx* c);
 sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow);
 
+// Allows `kernel` `bytes` of dynamic shared memory.  The limit belongs to the function, shared by
+// every thread of the process, so `bytes` is the kernel's largest and the same at every call (a
+// context that set its own smaller size between another thread's call and launch made that launch
+// fail); the size of a launch is its own argument.
+template <typename K> inline void allow_smem(K* kernel, size_t bytes) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+// dynamic shared memory of a CTA at most, for kernels without static shared memory
+constexpr size_t kSmemMax = (size_t)227 << 10;
+
 // room for the standardised vectors of n window entries (grown on demand; false: they do not fit)
 bool zcache_fits(sisso_ctx* c, int64_t n);
 // first screening window of a step: max(4096, 32 k) candidates, but at most about 2^26 sample

@@ -736,7 +736,7 @@ static sisso_status run_enum(sisso_ctx* c, EnumArgs<T> A, int D, int mode) {
     cudaMemsetAsync(A.counter, 0, sizeof(int), c->stream);
 #define SG_LAUNCH(DPV, MV)                                                                              \
     do {                                                                                                \
-        cudaFuncSetAttribute(k_l0_enum<T, DPV, MV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+        allow_smem(k_l0_enum<T, DPV, MV>, kSmemMax);                                                    \
         k_l0_enum<T, DPV, MV><<<grid, kWarps * 32, smem, c->stream>>>(A);                               \
     } while (0)
     if (D == 1) {
@@ -824,7 +824,7 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
     cudaMemsetAsync(cand, 0, sizeof(unsigned long long), c->stream);
     cudaMemsetAsync(c->band_count, 0, sizeof(unsigned), c->stream);
     const int64_t tot = (int64_t)n * ldp;
-    const bool pair64 = DP <= 1 && !prefix_mask && binom_host(n, D) <= kPair64Max && pair64_smem(n) <= ((size_t)200 << 10);
+    const bool pair64 = DP <= 1 && !prefix_mask && binom_host(n, D) <= kPair64Max && pair64_smem(n) <= kPair64Smem;
     const bool block = D >= 4 && !prefix_mask && n >= D && n - (D - 3) <= kBMaxM;
     if (!pair64 && !block) k_pad_gram<<<std::max(1, (int)std::min<int64_t>(c->sms * 8, (tot + 255) / 256)), 256, 0, c->stream>>>(
         G, b, ld, n, ldp, c->tile_G, c->tile_b, c->tile_diag);
@@ -859,12 +859,12 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
     if (pair64) {
         const size_t sm = pair64_smem(n);
         if (DP == 0) {
-            cudaFuncSetAttribute(k_l0_pair64<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            allow_smem(k_l0_pair64<2>, kPair64Smem);
             k_l0_pair64<2><<<dim3(1, (unsigned)std::max(1, std::min(c->sms, (n + 7) / 8))), kPairThreads, sm, c->stream>>>(A);
         } else {
             // rows of a p cut so that every SM has about four CTAs
             const int cut = std::max(1, std::min((n + 15) / 16, 4 * c->sms / n));
-            cudaFuncSetAttribute(k_l0_pair64<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            allow_smem(k_l0_pair64<3>, kPair64Smem);
             k_l0_pair64<3><<<dim3((unsigned)(n - 2), (unsigned)cut), kPairThreads, sm, c->stream>>>(A);
         }
     } else
@@ -890,7 +890,7 @@ static sisso_status l0_solve_tiled(sisso_ctx* c, const double* G, const double* 
     do {                                                                                                \
         const size_t sm = block_smem_bytes(MV, WV);                                                     \
         A.n_items = (END) * slices;                                                                     \
-        cudaFuncSetAttribute(k_l0_block<DCV, WV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
+        allow_smem(k_l0_block<DCV, WV>, block_smem_bytes(WV == kBWarpsBig ? kBMaxM : kBSmallM, WV));    \
         k_l0_block<DCV, WV><<<c->sms * (16 / WV), WV * 32, sm, c->stream>>>(A, slices, (int)((ITEM0) * slices), MV); \
     } while (0)
         if (big > 0) { if (DC == 1) SG_BLOCK(1, kBWarpsBig, 0, big, m_max); else SG_BLOCK(2, kBWarpsBig, 0, big, m_max); }
@@ -1234,7 +1234,7 @@ cudaError_t na_enum(const EnumArgs<T>& A, int D, int mode, int sms, cudaStream_t
     const int grid = sms * 2;
 #define SG_NA(DPV, MV)                                                                                   \
     do {                                                                                                 \
-        cudaFuncSetAttribute(k_l0_enum<T, DPV, MV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+        allow_smem(k_l0_enum<T, DPV, MV>, kSmemMax);                                                    \
         k_l0_enum<T, DPV, MV><<<grid, kWarps * 32, smem, st>>>(A);                                       \
     } while (0)
     if (D == 1) {

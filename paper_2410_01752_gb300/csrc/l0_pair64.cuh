@@ -27,6 +27,8 @@ constexpr int kPairThreads = 256;
 // per feature: reduced values, then its constants as a row
 struct PairTab { double *r, *d, *n, *id, *nK; };       // 1/d1; -K before the threshold, in units of RSS / N
 
+constexpr size_t kPair64Smem = (size_t)200 << 10;      // tables of up to 5120 features
+
 __host__ __device__ constexpr size_t pair64_smem(int m) { return (size_t)m * 5 * sizeof(double); }
 
 template <int D>

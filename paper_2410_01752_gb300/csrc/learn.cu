@@ -1194,7 +1194,7 @@ static sisso_status prefix_labels_dev(const double* G, const double* b, double s
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_prefix_labels<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k_prefix_labels<0>, kSmemMax);
         k_prefix_labels<0><<<sms * 2, kWarps * 32, smem>>>(A, lab);
         // prefixes of [0, n-2) only have extensions; the rest keep the +inf key
         k_prefix_targets<<<(unsigned)std::min<int64_t>((np + 255) / 256, 4096), 256>>>(lab, np, syy * N, base_dev, dl,

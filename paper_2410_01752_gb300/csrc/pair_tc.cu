@@ -464,6 +464,11 @@ template <int F> __host__ __device__ constexpr uint32_t pt_row_bytes(int ni) {
     return (uint32_t)sizeof(PtRow<F>) * kPtEpiWarps * (uint32_t)(ni / 3);
 }
 
+// dynamic shared memory of k_pair_tc<F> with i tiles of ni
+template <int F> constexpr size_t pt_smem_bytes(int ni) {
+    return (size_t)kPtStages * pt_stage_bytes(F, ni) + 1024 + pt_row_bytes<F>(ni);
+}
+
 // Persistent: one CTA per SM walks the work units (tile of 128 j x ni i operands, product form,
 // sample chunk).  A TMA warp stages a run's rows (two stages), an MMA warp issues its products
 // into one of two TMEM buffers of 240 columns, twelve warps add the run's sums to their
@@ -1039,19 +1044,18 @@ sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow) {
         k_pt_target<true><<<(unsigned)t->P, 512, 0, c->stream>>>(t->rows, c->tc32, c->tstats, t->P, t->Pi, c->N, t->Kpad, t->rrows, t->R);
     k_pt_low<<<(unsigned)((t->P + 255) / 256), 256, 0, c->stream>>>(A, c->subvalid);
     const int units = A.n_tiles * A.ntypes * A.chunks, grid = std::min(units, c->sms);
-    const size_t smem = (size_t)kPtStages * pt_stage_bytes(v == 0 ? 5 : 1, A.ni) + 1024 +
-                        (v == 0 ? pt_row_bytes<5>(A.ni) : pt_row_bytes<1>(A.ni));
+    const size_t smem = v == 0 ? pt_smem_bytes<5>(A.ni) : pt_smem_bytes<1>(A.ni);
     const bool many = t->Kpad > 4096;
     const unsigned gr = (unsigned)(A.n_tiles * A.ntypes * A.ni);
     if (v == 0) {
-        cudaFuncSetAttribute(k_pair_tc<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k_pair_tc<5>, pt_smem_bytes<5>(kPtI5));
         k_pair_tc<5><<<grid, kPtThreads, smem, c->stream>>>(t->mapM, t->mapN[0], t->mapR[0], A);
         if (A.chunks > 1) k_pt_reduce<5><<<gr, kPtM, 0, c->stream>>>(A);
         k_pt_open<<<(unsigned)std::max<size_t>(1, std::min<size_t>((size_t)c->sms * 8, (t->n_w + 1023) / 1024)), 256, 0, c->stream>>>(A, (int64_t)t->n_w);
         if (many) k_pt_direct<true, true><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
         else k_pt_direct<true, false><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
     } else {
-        cudaFuncSetAttribute(k_pair_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k_pair_tc<1>, pt_smem_bytes<1>(kPtI1));
         k_pair_tc<1><<<grid, kPtThreads, smem, c->stream>>>(t->mapM, t->mapN[1], t->mapR[1], A);
         if (A.chunks > 1) k_pt_reduce<1><<<gr, kPtM, 0, c->stream>>>(A);
         if (many) k_pt_direct<false, true><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
