@@ -82,6 +82,7 @@ sisso_status fail(sisso_ctx* c, sisso_status st, const std::string& msg) {
 
 sisso_status check_cuda(sisso_ctx* c, cudaError_t e, const char* what) {
     if (e == cudaSuccess) return SISSO_OK;
+    cudaGetLastError();        // reported here: the thread's next call must not read it as its own
     return fail(c, e == cudaErrorMemoryAllocation ? SISSO_ERR_OOM : SISSO_ERR_CUDA,
                 std::string(what) + ": " + cudaGetErrorString(e));
 }
