@@ -1062,10 +1062,12 @@ sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow) {
         else k_pt_direct<false, false><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
     }
     c->stats.launches += 4 + (A.chunks > 1) + (v == 0);
+    // a launch that was refused leaves the last step's keys: waiting alone would not tell
+    sisso_status st = check_cuda(c, cudaGetLastError(), "pair scores");
+    if (st) return st;
     unsigned h[4] = {0, 0, 0, 0};
     cudaMemcpyAsync(h, t->count, sizeof(h), cudaMemcpyDeviceToHost, c->stream);
-    sisso_status st = check_cuda(c, cudaStreamSynchronize(c->stream), "pair scores");
-    if (st) return st;
+    if ((st = check_cuda(c, cudaStreamSynchronize(c->stream), "pair scores"))) return st;
     if (h[2]) return fail(c, SISSO_ERR_TIMEOUT, "pair scores: a bounded wait ran out");
     c->stats.pm_keys_direct += (int64_t)h[v == 0 ? 0 : 1];
     if ((int64_t)h[0] > t->cap) *overflow = true;

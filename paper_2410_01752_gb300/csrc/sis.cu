@@ -1864,6 +1864,7 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
                                                           (float)(2.25 * eps + 8.0 * kScoreTie));
             c->stats.launches++;
         }
+        if ((st = check_cuda(c, cudaGetLastError(), "select"))) break;
         unsigned h_state[4], h_count = 0;
         cudaMemcpyAsync(h_state, c->sel_state, sizeof(h_state), cudaMemcpyDeviceToHost, c->stream);
         cudaMemcpyAsync(&h_count, c->surv_count, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream);
@@ -1943,6 +1944,7 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
                                                   ns, n_prev, k, c->opts.sis_threshold, c->removed, c->accepted,
                                                   c->walk);
         c->stats.launches += 3;
+        if ((st = check_cuda(c, cudaGetLastError(), "walk"))) break;
         cudaEventRecord(q[4], c->stream);
         cudaMemcpyAsync(c->walk_h, c->walk, sizeof(WalkResult), cudaMemcpyDeviceToHost, c->stream);
         if ((st = check_cuda(c, cudaStreamSynchronize(c->stream), "walk"))) break;
