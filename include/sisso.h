@@ -137,8 +137,9 @@ typedef struct {
                                SISSO_SCREEN_AUTO (default) and SISSO_SCREEN_TENSOR from split
                                16-bit tensor-core products (§2.2 Eq. 5 as a contraction; each
                                key's error is bounded, keys whose bound is too wide are scored
-                               directly), as FP32 precision does, while the operands' rows fit
-                               40 GB; SISSO_SCREEN_CORES always the CUDA-core kernel.
+                               directly), as FP32 precision does, where the buffers for them
+                               take at most half of the device memory left; SISSO_SCREEN_CORES
+                               always the CUDA-core kernel.
                                stats.screen_tc reports the tensor cores for AUTO when the pairs
                                lie within phi_{L-1} (EQ2 grammar, or rung <= 2) and for TENSOR */
     int gram;               /* FP32 precision's subspace Gram (§2.3 Eq. 7):

@@ -184,6 +184,24 @@ bool zcache_fits(sisso_ctx* c, int64_t n) {
     return true;
 }
 
+void ctx_free(sisso_ctx* c, void* p) {
+    if (!p) return;
+    c->bufs.erase(std::find(c->bufs.begin(), c->bufs.end(), p));
+    if (c->pooled.erase(p)) cudaFreeAsync(p, c->stream);
+    else cudaFree(p);
+}
+
+size_t memory_left(const sisso_ctx* c) {
+    size_t left = 0, total = 0;
+    if (cudaMemGetInfo(&left, &total) != cudaSuccess) { cudaGetLastError(); return 0; }
+    uint64_t held = 0, used = 0;
+    cudaMemPool_t pool = ctx_pool(c->opts.device, false);
+    if (pool && cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && held > used)
+        left += (size_t)(held - used);
+    return left;
+}
+
 sisso_status tmp_alloc(sisso_ctx* c, void** p, size_t bytes, const char* what) {
     cudaMemPool_t pool = ctx_pool(c->opts.device, true);
     return check_cuda(c, pool ? cudaMallocFromPoolAsync(p, std::max<size_t>(bytes, 1), pool, c->stream)
@@ -394,11 +412,7 @@ sisso_status sisso_create(const double* X, const double* y, int N, int d, uint32
     TargetStats ts{};
     cudaMemcpyAsync(&ts, c->tstats, sizeof(ts), cudaMemcpyDeviceToHost, c->stream);
     sisso_status st2 = check_cuda(c, cudaStreamSynchronize(c->stream), "create");
-    for (void* p : {(void*)Xraw, (void*)yraw, (void*)bad}) {
-        c->bufs.erase(std::find(c->bufs.begin(), c->bufs.end(), p));
-        if (c->pooled.erase(p)) cudaFreeAsync(p, c->stream);
-        else cudaFree(p);
-    }
+    for (void* p : {(void*)Xraw, (void*)yraw, (void*)bad}) ctx_free(c, p);
     if (st || st2) return bail(st ? st : st2);
     if (h_bad) return bail(SISSO_ERR_ARG);
     if (!(ts.sd > 0.0)) return bail(SISSO_ERR_ARG);     // constant target

@@ -545,8 +545,11 @@ bool zcache_fits(sisso_ctx* c, int64_t n);
 // evaluations of FP64 re-scoring (the re-score costs M x N) and never below 5 k
 inline int64_t first_window(const sisso_ctx* c, int k);
 
-// a device buffer owned by the context (released with it)
+// a device buffer owned by the context (released with it, or by ctx_free)
 sisso_status ctx_alloc(sisso_ctx* c, void** p, size_t bytes, const char* what);
+void ctx_free(sisso_ctx* c, void* p);
+// device memory that a context could still take: free, or kept unused by the library's pool
+size_t memory_left(const sisso_ctx* c);
 // a temporary from the library's pool on the context's stream, given back with cudaFreeAsync there
 // (the default pool unmaps freed memory at every synchronisation: a step of a 1013-sample fit
 // spent 0.1 ms mapping its temporaries, the 4e6-prefix network inputs 1.5 ms)

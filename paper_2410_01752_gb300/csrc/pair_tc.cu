@@ -57,9 +57,11 @@ struct PairTc {
     unsigned* count = nullptr;     // [0] open keys, [1] keys open at every step, [2] error flag
     int64_t cap = 0;
     size_t n_w = 0;
-    float* part = nullptr;         // chunk partials (long samples)
+    float* part = nullptr;         // chunk partials (long samples) of `batch` tiles
     int2* tiles[2] = {nullptr, nullptr};   // (i0, j0) per tile: five-sum and one-sum shapes
-    int n_tiles[2] = {0, 0}, ni[2] = {0, 0}, chunks[2] = {1, 1}, run_len[2] = {0, 0};
+    int64_t n_tiles[2] = {0, 0}, batch[2] = {0, 0};
+    int ni[2] = {0, 0}, chunks[2] = {1, 1}, run_len[2] = {0, 0};
+    size_t part_bytes = 0;
     CUtensorMap mapM, mapN[2], mapR[2];
     std::vector<int2> tile_list[2];   // host copies of the tiles (the source of an asynchronous copy)
     bool ready = false;            // w and the lists hold this fit's operands
@@ -916,63 +918,103 @@ bool pt_map(CUtensorMap* m, void* base, int64_t rows, int Kpad, int box_rows) {
 
 }  // namespace
 
-// Used for the FP32 and the mixed forms when the operands' FP64 values are kept and their 16-bit rows (16 bytes per
-// value) fit 40 GB; other contexts keep the CUDA-core kernel.
+namespace {
+
+// Partial sums of long samples are kept for at most this much at a time, whole tiles of all chunks
+// (one tile at least): 402 operands over 65 536 samples have 0.35 GB, 2355 over 16 384 would have 1.5.
+constexpr size_t kPtPart = (size_t)1 << 30;
+// The buffers may take this much, or half of what is left of the device beside the context's
+// others: they make a fit faster, and the scores alone are as large as the deviations kept for
+// later steps (half as large in the EQ2 grammar).
+constexpr size_t kPtSmall = (size_t)1 << 30;
+
+// i0 of the tiles of one row of j tiles: [0, end), every ni
+int64_t pt_i_end(const PairTc& t, int64_t j0) { return std::min(t.Pi, std::min(j0 + kPtM, t.P) - 1); }
+
+// sizes, tiles and chunks of a context's pair stage
+void pt_layout(const sisso_ctx* c, PairTc& t) {
+    const Space& sp = c->space;
+    const int L = c->rung;
+    t.P = sp.phi[L - 1];
+    t.Q = L >= 2 ? sp.phi[L - 2] : 0;
+    t.Pi = sp.grammar == SISSO_GRAMMAR_NEW_X_PREV && L >= 3 ? t.Q : t.P;
+    t.runs = (c->N + kPtK - 1) / kPtK;
+    t.Kpad = t.runs * kPtK;
+    t.cap = (int64_t)1 << 22;
+    t.n_w = 5 * (size_t)t.Pi * (size_t)(t.P - t.Q);
+    t.part_bytes = 0;
+    for (int v = 0; v < 2; ++v) {
+        // i tiles: 48 for the five sums; for the one sum the multiple of 48 up to 240 that pads
+        // the i operands least, the largest of those that leave every SM two units (long samples
+        // are cut into chunks, so there a unit is a tile's chunk)
+        t.ni[v] = kPtI5;
+        if (v == 1) {
+            auto padded = [&](int ni) { return (t.Pi + ni - 1) / ni * ni; };
+            const int64_t nj = (t.P - t.Q + kPtM - 1) / kPtM, cuts = t.runs > kMaxRuns ? (t.runs + 15) / 16 : 1;
+            for (int ni = 2 * kPtI5; ni <= kPtI1; ni += kPtI5)
+                if (padded(ni) <= padded(t.ni[v]) && 3 * nj * ((t.Pi + ni - 1) / ni) * cuts >= 2 * c->sms) t.ni[v] = ni;
+        }
+        t.n_tiles[v] = 0;
+        for (int64_t j0 = t.Q; j0 < t.P; j0 += kPtM) t.n_tiles[v] += (std::max<int64_t>(0, pt_i_end(t, j0)) + t.ni[v] - 1) / t.ni[v];
+        // sample chunks: at most kMaxRuns runs each (the runs are added in FP32); a chunk of 16
+        // runs or more costs the partials' round trip little, so long samples are cut until
+        // every SM has about four units
+        const int64_t units = std::max<int64_t>(1, 3 * t.n_tiles[v]);
+        int64_t ch = (t.runs + kMaxRuns - 1) / kMaxRuns;
+        if (ch > 1) ch = std::max(ch, std::min<int64_t>((t.runs + 15) / 16, (4 * c->sms + units - 1) / units));
+        t.run_len[v] = (int)((t.runs + ch - 1) / ch);
+        t.chunks[v] = (t.runs + t.run_len[v] - 1) / t.run_len[v];
+        t.batch[v] = std::max<int64_t>(1, t.n_tiles[v]);
+        if (t.chunks[v] > 1) {
+            const size_t tile = sizeof(float) * 3 * (size_t)t.chunks[v] * (v == 0 ? 5 : 1) * t.ni[v] * kPtM;
+            t.batch[v] = std::max<int64_t>(1, std::min<int64_t>(t.batch[v], (int64_t)(kPtPart / tile)));
+            t.part_bytes = std::max(t.part_bytes, tile * (size_t)t.batch[v]);
+        }
+    }
+}
+
+size_t pt_bytes(const PairTc& t) {
+    const size_t K = (size_t)t.Kpad, P = (size_t)t.P;
+    return 20 * P * K + 8 * (size_t)t.Pi * K + 48 * P + sizeof(float) * t.n_w + sizeof(unsigned long long) * 2 * t.cap +
+           t.part_bytes + sizeof(int2) * (size_t)(t.n_tiles[0] + t.n_tiles[1]);
+}
+
+}  // namespace
+
+// Used for the FP32 and the mixed forms when the operands' FP32 and FP64 values are kept (8 GB of
+// the former at most) and the buffers, 20 to 28 bytes per padded operand value and 20 per pair,
+// fit; other contexts keep the CUDA-core kernel.
 bool pair_tc_possible(const sisso_ctx* c) {
     const Space& sp = c->space;
     const int64_t P = sp.phi[c->rung - 1];
     const int64_t Kpad = ((int64_t)c->N + kPtK - 1) / kPtK * kPtK;
     bool any = false;
     for (int s = 0; s < sp.nsec; ++s) any |= sp.sec[s].level == c->rung && sp.sec[s].op <= DIV;
-    return any && c->opcache32 && c->opval64 && P >= 2 && P <= ((int64_t)1 << 27) &&
-           P * Kpad * 16 <= ((int64_t)40 << 30) && encode_fn() != nullptr;
+    if (!any || !c->opcache32 || !c->opval64 || P < 2 || P > ((int64_t)1 << 27) || P * Kpad * 16 > ((int64_t)40 << 30) ||
+        encode_fn() == nullptr)
+        return false;
+    PairTc t;
+    pt_layout(c, t);
+    const size_t need = pt_bytes(t);
+    return need <= kPtSmall || need <= memory_left(c) / 2;
 }
 
-// per-operand rows, tiles and buffers of a context (they depend on X only)
+// per-operand rows, tiles and buffers of a context (they depend on X only); without them
+// (c->pt null) where the device has no room
 sisso_status pair_tc_alloc(sisso_ctx* c) {
-    const Space& sp = c->space;
-    const int L = c->rung;
     PairTc* t = new (std::nothrow) PairTc();
     if (!t) return SISSO_ERR_OOM;
     c->pt = t;
-    t->P = sp.phi[L - 1];
-    t->Q = L >= 2 ? sp.phi[L - 2] : 0;
-    const bool nxp = sp.grammar == SISSO_GRAMMAR_NEW_X_PREV && L >= 3;
-    t->Pi = nxp ? t->Q : t->P;
-    t->runs = (c->N + kPtK - 1) / kPtK;
-    t->Kpad = t->runs * kPtK;
-    t->cap = (int64_t)1 << 22;
-    sisso_status st;
-    size_t part = 0;
+    pt_layout(c, *t);
     std::vector<int2>* tiles = t->tile_list;
     for (int v = 0; v < 2; ++v) {
-        // i tiles: 48 for the five sums; for the one sum the multiple of 48 up to 240 that pads
-        // the i operands least, the largest of those that leave every SM two units (long samples
-        // are cut into chunks, so there a unit is a tile's chunk)
-        t->ni[v] = kPtI5;
-        if (v == 1) {
-            auto padded = [&](int ni) { return (t->Pi + ni - 1) / ni * ni; };
-            const int64_t nj = (t->P - t->Q + kPtM - 1) / kPtM, cuts = t->runs > kMaxRuns ? (t->runs + 15) / 16 : 1;
-            for (int ni = 2 * kPtI5; ni <= kPtI1; ni += kPtI5)
-                if (padded(ni) <= padded(t->ni[v]) && 3 * nj * ((t->Pi + ni - 1) / ni) * cuts >= 2 * c->sms) t->ni[v] = ni;
-        }
+        tiles[v].reserve((size_t)t->n_tiles[v]);
         for (int64_t j0 = t->Q; j0 < t->P; j0 += kPtM)
-            for (int64_t i0 = 0; i0 < t->Pi && i0 < std::min(j0 + kPtM, t->P) - 1; i0 += t->ni[v])
-                tiles[v].push_back(make_int2((int)i0, (int)j0));
-        t->n_tiles[v] = (int)tiles[v].size();
-        // sample chunks: at most kMaxRuns runs each (the runs are added in FP32); a chunk of 16
-        // runs or more costs the partials' round trip little, so long samples are cut until
-        // every SM has about four units
-        const int64_t units = std::max<int64_t>(1, 3 * t->n_tiles[v]);
-        int64_t ch = (t->runs + kMaxRuns - 1) / kMaxRuns;
-        if (ch > 1) ch = std::max(ch, std::min<int64_t>((t->runs + 15) / 16, (4 * c->sms + units - 1) / units));
-        t->run_len[v] = (int)((t->runs + ch - 1) / ch);
-        t->chunks[v] = (t->runs + t->run_len[v] - 1) / t->run_len[v];
-        if (t->chunks[v] > 1)
-            part = std::max(part, (size_t)t->chunks[v] * units * (v == 0 ? 5 : 1) * t->ni[v] * kPtM);
+            for (int64_t i0 = 0; i0 < pt_i_end(*t, j0); i0 += t->ni[v]) tiles[v].push_back(make_int2((int)i0, (int)j0));
     }
     const size_t K = (size_t)t->Kpad, P = (size_t)t->P;
-    t->n_w = 5 * (size_t)t->Pi * (size_t)(t->P - t->Q);
+    const std::string err = c->err;
+    sisso_status st;
     if ((st = ctx_alloc(c, (void**)&t->rows, 16 * P * K, "pair rows")) ||
         (st = ctx_alloc(c, (void**)&t->rrows, 8 * (size_t)t->Pi * K, "pair target rows")) ||
         (st = ctx_alloc(c, (void**)&t->val32, 4 * P * K, "pair FP32 values")) ||
@@ -982,10 +1024,17 @@ sisso_status pair_tc_alloc(sisso_ctx* c) {
         (st = ctx_alloc(c, (void**)&t->w, sizeof(float) * t->n_w, "pair 1/sd")) ||
         (st = ctx_alloc(c, (void**)&t->list, sizeof(unsigned long long) * 2 * t->cap, "pair open keys")) ||
         (st = ctx_alloc(c, (void**)&t->count, sizeof(unsigned) * 4, "pair counts")) ||
-        (st = ctx_alloc(c, (void**)&t->part, sizeof(float) * part, "pair partials")))
+        (st = ctx_alloc(c, (void**)&t->part, t->part_bytes, "pair partials")) ||
+        (st = ctx_alloc(c, (void**)&t->tiles[0], sizeof(int2) * tiles[0].size(), "pair tiles")) ||
+        (st = ctx_alloc(c, (void**)&t->tiles[1], sizeof(int2) * tiles[1].size(), "pair tiles"))) {
+        for (void* p : {(void*)t->rows, (void*)t->rrows, (void*)t->val32, (void*)t->par, (void*)t->ex, (void*)t->R, (void*)t->w,
+                        (void*)t->list, (void*)t->count, (void*)t->part, (void*)t->tiles[0], (void*)t->tiles[1]})
+            ctx_free(c, p);
+        pair_tc_free(c);
+        if (st == SISSO_ERR_OOM) { c->err = err; return SISSO_OK; }
         return st;
+    }
     for (int v = 0; v < 2; ++v) {
-        if ((st = ctx_alloc(c, (void**)&t->tiles[v], sizeof(int2) * tiles[v].size(), "pair tiles"))) return st;
         cudaMemcpyAsync(t->tiles[v], tiles[v].data(), sizeof(int2) * tiles[v].size(), cudaMemcpyHostToDevice, c->stream);
         if (!pt_map(&t->mapN[v], t->rows, 8 * t->P, t->Kpad, t->ni[v]) ||
             !pt_map(&t->mapR[v], t->rrows, 4 * t->Pi, t->Kpad, t->ni[v]))
@@ -1023,7 +1072,7 @@ sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow) {
     A.nxp = c->space.grammar == SISSO_GRAMMAR_NEW_X_PREV && c->rung >= 3;
     if (sec[0] >= 0 || sec[1] >= 0 || sec[2] >= 0) A.type[A.ntypes++] = 0;
     if (sec[3] >= 0) { A.type[A.ntypes++] = 1; A.type[A.ntypes++] = 2; }
-    A.tiles = t->tiles[v]; A.n_tiles = t->n_tiles[v]; A.ni = t->ni[v];
+    A.ni = t->ni[v];
     A.chunks = t->chunks[v]; A.run_len = t->run_len[v]; A.runs = t->runs;
     A.N = c->N; A.Kpad = t->Kpad; A.rows = t->rows; A.val32 = t->val32;
     A.scale = (float)(1.0 / (1073741824.0 * c->N));
@@ -1043,25 +1092,34 @@ sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow) {
     else
         k_pt_target<true><<<(unsigned)t->P, 512, 0, c->stream>>>(t->rows, c->tc32, c->tstats, t->P, t->Pi, c->N, t->Kpad, t->rrows, t->R);
     k_pt_low<<<(unsigned)((t->P + 255) / 256), 256, 0, c->stream>>>(A, c->subvalid);
-    const int units = A.n_tiles * A.ntypes * A.chunks, grid = std::min(units, c->sms);
     const size_t smem = v == 0 ? pt_smem_bytes<5>(A.ni) : pt_smem_bytes<1>(A.ni);
     const bool many = t->Kpad > 4096;
-    const unsigned gr = (unsigned)(A.n_tiles * A.ntypes * A.ni);
+    if (v == 0) allow_smem(k_pair_tc<5>, pt_smem_bytes<5>(kPtI5));
+    else allow_smem(k_pair_tc<1>, pt_smem_bytes<1>(kPtI1));
+    for (int64_t t0 = 0; t0 < t->n_tiles[v]; t0 += t->batch[v]) {          // (one batch unless the samples are cut)
+        A.tiles = t->tiles[v] + t0;
+        A.n_tiles = (int)std::min(t->batch[v], t->n_tiles[v] - t0);
+        const int64_t units = (int64_t)A.n_tiles * A.ntypes * A.chunks;
+        const int grid = (int)std::min<int64_t>(units, c->sms);
+        const unsigned gr = (unsigned)(A.n_tiles * A.ntypes * A.ni);
+        if (v == 0) {
+            k_pair_tc<5><<<grid, kPtThreads, smem, c->stream>>>(t->mapM, t->mapN[0], t->mapR[0], A);
+            if (A.chunks > 1) k_pt_reduce<5><<<gr, kPtM, 0, c->stream>>>(A);
+        } else {
+            k_pair_tc<1><<<grid, kPtThreads, smem, c->stream>>>(t->mapM, t->mapN[1], t->mapR[1], A);
+            if (A.chunks > 1) k_pt_reduce<1><<<gr, kPtM, 0, c->stream>>>(A);
+        }
+        c->stats.launches += 1 + (A.chunks > 1);
+    }
     if (v == 0) {
-        allow_smem(k_pair_tc<5>, pt_smem_bytes<5>(kPtI5));
-        k_pair_tc<5><<<grid, kPtThreads, smem, c->stream>>>(t->mapM, t->mapN[0], t->mapR[0], A);
-        if (A.chunks > 1) k_pt_reduce<5><<<gr, kPtM, 0, c->stream>>>(A);
         k_pt_open<<<(unsigned)std::max<size_t>(1, std::min<size_t>((size_t)c->sms * 8, (t->n_w + 1023) / 1024)), 256, 0, c->stream>>>(A, (int64_t)t->n_w);
         if (many) k_pt_direct<true, true><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
         else k_pt_direct<true, false><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
     } else {
-        allow_smem(k_pair_tc<1>, pt_smem_bytes<1>(kPtI1));
-        k_pair_tc<1><<<grid, kPtThreads, smem, c->stream>>>(t->mapM, t->mapN[1], t->mapR[1], A);
-        if (A.chunks > 1) k_pt_reduce<1><<<gr, kPtM, 0, c->stream>>>(A);
         if (many) k_pt_direct<false, true><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
         else k_pt_direct<false, false><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
     }
-    c->stats.launches += 4 + (A.chunks > 1) + (v == 0);
+    c->stats.launches += 3 + (v == 0);
     // a launch that was refused leaves the last step's keys: waiting alone would not tell
     sisso_status st = check_cuda(c, cudaGetLastError(), "pair scores");
     if (st) return st;
