@@ -675,6 +675,20 @@ __global__ void __launch_bounds__(1024) k_model_z(const double* __restrict__ Z, 
 // host side
 // ===================================================================================
 
+// room for the digits of the exact Gram's rows, 14 bytes a value; false where the device has none
+static bool gram_digits(sisso_ctx* c) {
+    if (c->gram_sl) return true;
+    const std::string err = c->err;
+    if (ctx_alloc(c, &c->gram_sl, gram64_tc_bytes(c->N, c->n_cap), "gram digits") ||
+        ctx_alloc(c, (void**)&c->gram_ex, sizeof(int) * (size_t)c->n_cap, "gram exponents")) {
+        ctx_free(c, c->gram_sl);
+        c->gram_sl = nullptr;
+        c->err = err;
+        return false;
+    }
+    return true;
+}
+
 sisso_status append_subspace(sisso_ctx* c, int n_old, int n_new, bool gram64) {
     if (n_new <= 0) return SISSO_OK;
     const int n = n_old + n_new;
@@ -702,11 +716,8 @@ sisso_status append_subspace(sisso_ctx* c, int n_old, int n_new, bool gram64) {
     }
     if (n_old < c->gram_rows) c->gram_rows = n_old;
     // FP64 sums, or exact integer ones on the tensor cores where the FP64 pipe would take longer
-    if (gram64 && gram64_tc_possible(c->N, n_new, n, c->n_cap)) {
+    if (gram64 && gram64_tc_possible(c->N, n_new, n, c->n_cap) && gram_digits(c)) {
         sisso_status st;
-        if (!c->gram_sl && ((st = ctx_alloc(c, &c->gram_sl, gram64_tc_bytes(c->N, c->n_cap), "gram digits")) ||
-                            (st = ctx_alloc(c, (void**)&c->gram_ex, sizeof(int) * (size_t)c->n_cap, "gram exponents"))))
-            return st;
         if ((st = gram64_tc(c, c->Z, c->yc64, c->N, c->gram_rows, n_old, n, c->n_cap, c->n_cap, c->gram_sl, c->gram_ex, c->G64,
                             c->b64, c->G32, c->b32)))
             return st;

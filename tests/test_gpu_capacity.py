@@ -118,3 +118,13 @@ def test_partial_sums_in_bounded_batches():
     cells, K = 2355, 16384
     room = 28 * cells * K + 20 * cells * cells + GB + GB // 4
     assert _memory_of(S, lambda: make(S.SCREEN_AUTO)) - _memory_of(S, lambda: make(S.SCREEN_CORES)) <= room
+
+
+def test_gram_digits_that_do_not_fit():
+    """600 features over 65 536 samples: 0.55 GB of digits for the exact Gram, asked for in the fit."""
+    from paper_2410_01752_gb300 import sisso as S
+    X, y = _problem(65536, 3)
+    with S.Sisso(X, y, inputs.OPS9, 2, 200, 3) as c:
+        ref = _fit(c)
+    with S.Sisso(X, y, inputs.OPS9, 2, 200, 3) as c, _Held(S, GB // 3):
+        _same(_fit(c), ref)
