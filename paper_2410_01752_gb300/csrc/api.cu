@@ -306,7 +306,7 @@ sisso_status sisso_create(const double* X, const double* y, int N, int d, uint32
         (st = dalloc(c, c->scores, (size_t)c->n_feat, "scores")) || (st = dalloc(c, c->target64, Nn, "target")) ||
         (st = dalloc(c, c->tc64, Nn, "tc64")) || (st = dalloc(c, c->tc32, Nn, "tc32")) ||
         (st = dalloc(c, c->tstats, 1, "tstats")) || (st = dalloc(c, c->hist, 3 * 4096, "hist")) ||
-        (st = dalloc(c, c->sel_state, 4, "sel")) || (st = dalloc(c, c->surv_ids, (size_t)c->surv_cap, "surv")) ||
+        (st = dalloc(c, c->sel_state, kSelState, "sel")) || (st = dalloc(c, c->surv_ids, (size_t)c->surv_cap, "surv")) ||
         (st = dalloc(c, c->surv_count, 1, "surv_count")) ||
         (st = dalloc(c, c->surv_score, (size_t)c->surv_cap, "surv_score")) ||
         (st = dalloc(c, c->surv_mean, (size_t)c->surv_cap, "surv_mean")) ||

@@ -349,6 +349,10 @@ struct TargetStats {
     float inv_sdr, pad;     // 1 / (sd rscale)
 };
 
+// words of the radix select's state: [2] key of the last rank, [3] every candidate is in the window,
+// [4] entries were left out of it (k_narrow)
+constexpr int kSelState = 5;
+
 // small result block of one SIS walk, copied back to the host
 struct WalkResult {
     int n_acc;              // accepted ids
@@ -401,7 +405,7 @@ struct sisso_ctx {
     float* tc32 = nullptr;             // centred target FP32
     sg::TargetStats* tstats = nullptr;
     unsigned int* hist = nullptr;      // radix-select histograms (3 x 4096)
-    unsigned int* sel_state = nullptr; // radix-select state
+    unsigned int* sel_state = nullptr; // radix-select state (kSelState words)
     int64_t surv_cap = 0;              // capacity of the survivor buffers
     int64_t* surv_ids = nullptr;
     unsigned int* surv_count = nullptr;

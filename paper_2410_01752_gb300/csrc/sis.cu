@@ -626,9 +626,9 @@ __global__ void k_compact(const float* __restrict__ scores, int64_t n, const uns
 // narrows a window of n <= kNarrowMax entries before its FP64 work: keeps the entries whose key
 // is within `margin` of the key of rank `want` or above it (the rank found to within an eighth,
 // by bisection on the keys' bits), and lowers nothing else -- the threshold key in state[2]
-// rises to the smallest kept, and state[3] (every candidate is in the window) is cleared.  A walk
-// that visits at most `want` candidates then proves its selection with this window; one that
-// does not is repeated with the whole window.
+// rises to the smallest kept, state[3] (every candidate is in the window) is cleared, and state[4]
+// tells that entries were left out.  A walk that visits at most `want` candidates then proves its
+// selection with this window; one that does not is repeated with the whole window.
 constexpr int kNarrowMax = 8192, kNarrowThreads = 1024, kNarrowPer = kNarrowMax / kNarrowThreads;
 __global__ void __launch_bounds__(kNarrowThreads) k_narrow(const float* __restrict__ scores, int64_t* __restrict__ ids,
                                                            unsigned* count, unsigned* state, int want, float margin) {
@@ -688,7 +688,7 @@ __global__ void __launch_bounds__(kNarrowThreads) k_narrow(const float* __restri
         base = __shfl_sync(0xffffffffu, base, 0);
         if (in) ids[base + __popc(m & ((1u << lane) - 1u))] = id[q];
     }
-    if (t == 0) { *count = keep; state[2] = cut; state[3] = 0; }
+    if (t == 0) { *count = keep; state[2] = cut; state[3] = 0; state[4] = 1; }
 }
 
 // ---------------------------------------------------------------------------------
@@ -1849,7 +1849,7 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
         M = std::min<int64_t>(M, c->surv_cap - n_prev);
         cudaEventRecord(q[0], c->stream);
         cudaMemsetAsync(c->hist, 0, sizeof(unsigned) * 3 * 4096, c->stream);
-        cudaMemsetAsync(c->sel_state, 0, sizeof(unsigned) * 4, c->stream);
+        cudaMemsetAsync(c->sel_state, 0, sizeof(unsigned) * kSelState, c->stream);
         cudaMemsetAsync(c->surv_count, 0, sizeof(unsigned), c->stream);
         for (int pass = 0; pass < 3; ++pass) {
             k_hist<<<gridS, kBlock, 0, c->stream>>>(c->scores, n, pass, c->sel_state, c->hist);
@@ -1865,7 +1865,7 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
             c->stats.launches++;
         }
         if ((st = check_cuda(c, cudaGetLastError(), "select"))) break;
-        unsigned h_state[4], h_count = 0;
+        unsigned h_state[kSelState], h_count = 0;
         cudaMemcpyAsync(h_state, c->sel_state, sizeof(h_state), cudaMemcpyDeviceToHost, c->stream);
         cudaMemcpyAsync(&h_count, c->surv_count, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream);
         if ((st = check_cuda(c, cudaStreamSynchronize(c->stream), "select"))) break;
@@ -1963,7 +1963,8 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
         const double thr = c->opts.sis_threshold;
         const bool safe = all || (w.n_acc == k && w.last_score - kScoreTie > (double)t32 + eps) ||
                           (w.thr_stop && (double)t32 + eps < thr - kScoreTie);
-        if (!safe && narrow) { narrow = false; continue; }
+        // the same window again only where entries were left out of it
+        if (!safe && h_state[4]) { narrow = false; continue; }
         const bool can_grow = M < c->surv_cap - n_prev;
         if (safe || !can_grow) {
             if (!safe) c->stats.window_saturated = 1;
