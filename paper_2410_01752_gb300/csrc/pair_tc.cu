@@ -33,6 +33,7 @@
 #include "sis_device.cuh"
 #include "tc_device.cuh"
 
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -53,8 +54,8 @@ struct PairTc {
     int* ex = nullptr;             // [set][P]: scale exponents (scaled = value 2^-ex)
     float* R = nullptr;            // [set][P]: E x'r, scaled
     float* w = nullptr;            // [+, -, i j, i / j, j / i][Pi][P - Q]: 1 / sd (scaled), negative where invalid
-    unsigned long long* list = nullptr;   // open keys of the first step, then those of every step
-    unsigned* count = nullptr;     // [0] open keys, [1] keys open at every step, [2] error flag
+    unsigned long long* list = nullptr;   // open keys of the first step, those of every step, those left to FP64
+    unsigned* count = nullptr;     // [0] open keys, [1] keys open at every step, [2] error flag, [3] left to FP64
     int64_t cap = 0;
     size_t n_w = 0;
     float* part = nullptr;         // chunk partials (long samples) of `batch` tiles
@@ -101,6 +102,10 @@ struct PtArgs {
     int N, Kpad, nxp, ntypes;
     const __half* rows;
     const float* val32;
+    const double* val64;       // operand values and reciprocals (or null), feature-major, N samples
+    const double* inv64;
+    const double* tc64;
+    double inv_n;
     int type[3];               // 0: x_i x_j and x_i +/- x_j, 1: x_i / x_j, 2: x_j / x_i
     const int2* tiles;
     int n_tiles, ni, chunks, run_len, runs;
@@ -807,12 +812,38 @@ __global__ void __launch_bounds__(256) k_pt_open(PtArgs A, int64_t n) {
     }
 }
 
+// an open candidate, and where its key and 1/sd go
+struct PtOpen { int op, type; int64_t i, j; };           // +, -, x_i x_j, x_i / x_j, x_j / x_i; product form
+__device__ __forceinline__ PtOpen pt_open(unsigned long long word) {
+    const int op = (int)(word >> 61);
+    return PtOpen{op, op < 2 ? 0 : op - 2, (int64_t)((word >> 31) & 0x3FFFFFFFull), (int64_t)(word & 0x7FFFFFFFull)};
+}
+// exponent of the units of its 1/sd
+__device__ __forceinline__ int pt_scale(const PtArgs& A, const PtOpen& o) {
+    return o.op < 2 ? max(__ldg(A.ex + o.i), __ldg(A.ex + o.j))
+                    : __ldg(A.ex + (o.type == 2 ? A.P : 0) + o.i) + __ldg(A.ex + (o.type == 1 ? A.P : 0) + o.j);
+}
+template <bool FIRST> __device__ __forceinline__ void pt_close(const PtArgs& A, unsigned long long word, const PtOpen& o, const PtKey& k) {
+    const int64_t rank = o.type == 0 ? sym_base(A.nxp, A.P, A.Q, o.i) + o.j
+                         : o.type == 1 ? div_base(A.nxp, A.P, A.Q, o.i) + o.j : rdiv_base(A.nxp, A.P, A.Q, o.j) + o.i;
+    A.scores[A.sp->sec[A.sec[o.op < 3 ? o.op : 3]].base + rank] = k.key;
+    if (FIRST) {
+        const size_t wi = w_index(A, o.op, o.i, o.j);
+        const float dc = -A.w[wi];
+        if (k.w > 0.f && !(dc * k.w <= 0.5f * A.tol))
+            A.list[A.cap + atomicAdd(A.count + 1, 1u)] = word;      // at most one entry per listed key
+        A.w[wi] = k.w > 0.f ? k.w : -INFINITY;
+    }
+}
+
 // open keys: one warp per candidate (one CTA, many samples), the sums of its definition sample by sample, in FP32 with
 // runs of 32 samples per lane.  Products from the FP32 values, shifted by sample 0's product (a
 // value near zero keeps its relative precision beside a reciprocal that is huge there); + and -
-// from the centred values (hi + lo), which cancel without the values' own rounding.  FIRST:
-// stores 1/sd and lists the candidates whose covariance stays open at every step; later steps
-// run those alone.
+// from the centred values (hi + lo), which cancel without the values' own rounding.  A candidate
+// that cancels so far that the operands' FP32 rounding or that of the shifted sums could move its
+// key by more than three quarters of the screening margin, or that these sums reject, is left to
+// k_pt_exact.  FIRST: stores 1/sd and lists the candidates whose covariance stays open at every
+// step; later steps run those alone.
 template <bool FIRST, bool CTA>
 __global__ void __launch_bounds__(256) k_pt_direct(PtArgs A, const float* __restrict__ r) {
     __shared__ float sh[16];
@@ -826,9 +857,9 @@ __global__ void __launch_bounds__(256) k_pt_direct(PtArgs A, const float* __rest
     for (int64_t e = CTA ? (int64_t)blockIdx.x : ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < n;
          e += CTA ? (int64_t)gridDim.x : ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const unsigned long long word = list[e];
-        const int op = (int)(word >> 61);               // +, -, x_i x_j, x_i / x_j, x_j / x_i
-        const int64_t i = (int64_t)((word >> 31) & 0x3FFFFFFFull), j = (int64_t)(word & 0x7FFFFFFFull);
-        const int type = op < 2 ? 0 : op - 2;
+        const PtOpen o = pt_open(word);
+        const int op = o.op, scale = pt_scale(A, o);
+        const int64_t i = o.i, j = o.j;
         float t1 = 0.f, t2 = 0.f, tr = 0.f, s1 = 0.f, s2 = 0.f, sr = 0.f;
         int q = 0;
         auto add = [&](float u0, float u1, float y0, float y1) {
@@ -841,12 +872,12 @@ __global__ void __launch_bounds__(256) k_pt_direct(PtArgs A, const float* __rest
             t1 = group_sum<CTA>(t1 + s1, sh); t2 = group_sum<CTA>(t2 + s2, sh); tr = group_sum<CTA>(tr + sr, sh);
         };
         PtKey k{-1.f, -INFINITY};
-        const size_t wi = w_index(A, op, i, j);
+        bool sure = false;
         if (op < 2) {
             const PtSide a = pt_side(A, 0, i), b = pt_side(A, 0, j);
             const __half* xa = A.rows + (size_t)i * A.Kpad;
             const __half* xb = A.rows + (size_t)j * A.Kpad;
-            const int em = max(a.ex, b.ex);
+            const int em = scale;
             const float ca = pow2f(a.ex - em), cb = op == 1 ? -pow2f(b.ex - em) : pow2f(b.ex - em), g = 3.0517578125e-5f;
             for (int s = 2 * lane; s < A.Kpad; s += stride) {                      // padding: all zero
                 const float2 ah = __half22float2(*reinterpret_cast<const __half2*>(xa + s));
@@ -859,9 +890,13 @@ __global__ void __launch_bounds__(256) k_pt_direct(PtArgs A, const float* __rest
             total();
             const float v0 = ca * a.x0 + cb * b.x0;
             t1 *= inv_n;
-            k = pt_key(t2 * inv_n - t1 * t1, 0.f, tr * inv_n, 0.f, v0, ca * a.m + cb * b.m,
+            const float var = t2 * inv_n - t1 * t1;
+            k = pt_key(var, 0.f, tr * inv_n, 0.f, v0, ca * a.m + cb * b.m,
                        a.lg < INFINITY && b.lg < INFINITY && fabsf(v0) * pow2f(em) <= (float)kValueCap,
                        exp2f(kLogRms - 2.f * (float)em), A.tol, inv_sdr);
+            // values 3 2^-24 and 2^-39 off, in the sums of v r and of v^2
+            const float off = 6.f * kU * (ca * a.s + fabsf(cb) * b.s) + 4.f * kFloor * (ca + fabsf(cb));
+            sure = k.key >= 0.f && off * off <= kTolMany * kTolMany * var;
         } else {
             const bool quot = op > 2;
             const float* xa = A.val32 + (size_t)(op == 4 ? j : i) * A.Kpad;      // numerator
@@ -877,23 +912,74 @@ __global__ void __launch_bounds__(256) k_pt_direct(PtArgs A, const float* __rest
             total();
             k.key = finalize<float>(t1, t2, tr, v0, A.N, sum_t, sd_t);
             if (k.key >= 0.f) {
-                const int ex = __ldg(A.ex + (type == 2 ? A.P : 0) + i) + __ldg(A.ex + (type == 1 ? A.P : 0) + j);
                 t1 *= inv_n;
-                k.w = __frsqrt_rn(t2 * inv_n - t1 * t1) * pow2f(ex / 2) * pow2f(ex - ex / 2);
+                t2 *= inv_n;
+                const float var = t2 - t1 * t1, mean = v0 + t1, half = 0.5f * kTolMany;
+                k.w = __frsqrt_rn(var) * pow2f(scale / 2) * pow2f(scale - scale / 2);
+                // values 3 2^-24 off (two operands, the reciprocal), in the sums of v r and of v^2; sums of
+                // u = v - v0 about 40 2^-24 of E u^2 off
+                sure = k.w > 0.f && 36.f * kU * kU * (var + mean * mean) <= kTolMany * kTolMany * var && 60.f * kU * t2 <= half * var;
             }
         }
         if (lane == 0) {
-            const int64_t rank = type == 0 ? sym_base(A.nxp, A.P, A.Q, i) + j
-                                 : type == 1 ? div_base(A.nxp, A.P, A.Q, i) + j : rdiv_base(A.nxp, A.P, A.Q, j) + i;
-            const int64_t id = A.sp->sec[A.sec[op < 3 ? op : 3]].base + rank;
-            A.scores[id] = k.key;
-            if (FIRST) {
-                const float dc = -A.w[wi];
-                if (k.w > 0.f && !(dc * k.w <= 0.5f * A.tol))
-                    A.list[A.cap + atomicAdd(A.count + 1, 1u)] = word;      // at most one entry per listed key
-                A.w[wi] = k.w > 0.f ? k.w : -INFINITY;
-            }
+            if (sure) pt_close<FIRST>(A, word, o, k);
+            else A.list[2 * A.cap + atomicAdd(A.count + 3, 1u)] = word;
         }
+    }
+}
+
+// key and 1/sd from the sums of u = v - v0: moments in FP64, root and quotients in FP32 (in FP64
+// they took twice as long as 333 samples' sums).  Rejected where finalize<double> rejects.
+__device__ __forceinline__ PtKey pt_key64(const PtArgs& A, double s1, double s2, double sr, double v0, int scale) {
+    const double ms = s1 * A.inv_n, var = fma(s2, A.inv_n, -ms * ms), cov = fma(sr, A.inv_n, -ms * (A.st->tsum * A.inv_n));
+    const double mean = v0 + ms, mx = fmax(fabs(v0), fabs(mean));
+    const int hv = __double2hiint(var), hc = __double2hiint(cov) & 0x7fffffff;
+    if (!(fabs(v0) <= kValueCap) || !(var > kConstRel * kConstRel * (1.0 - 1e-9) * mx * mx) || hv >= 0x7ff00000 || hc >= 0x7ff00000)
+        return PtKey{-1.f, -INFINITY};
+    const int h = ((hv >> 20) - 1023) >> 1;                            // var = m 4^h, m in [1, 4)
+    const float rm = __frsqrt_rn(scaled_f32(var, -2 * h));
+    const int er = 127 - (__float_as_int(A.st->rscale) >> 23);         // rscale = 2^-er
+    return PtKey{fabsf(scaled_f32(cov, -h - er)) * rm * A.st->inv_sdr, rm * pow2f(scale - h)};
+}
+
+// ... and those from the FP64 operand values, summed in FP64: the margin that the selection relies
+// on holds for every key.  Bound by the FP64 pipe, five operations a sample; there are few (0.1 to
+// 6% of the open keys), so long samples take a cluster of four CTAs each.
+constexpr int kExactCtas = 4;
+template <bool FIRST, bool CTA>
+__global__ void __launch_bounds__(256) k_pt_exact(PtArgs A) {
+    __shared__ double sh[16], part[3];
+    const int64_t n = min((int64_t)A.count[3], A.cap);
+    namespace cg = cooperative_groups;
+    const int rank = CTA ? (int)cg::this_cluster().block_rank() : 0;
+    const int t = CTA ? rank * (int)blockDim.x + (int)threadIdx.x : (int)(threadIdx.x & 31);
+    const int nt = CTA ? kExactCtas * (int)blockDim.x : 32;
+    for (int64_t e = CTA ? (int64_t)blockIdx.x / kExactCtas : ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < n;
+         e += CTA ? (int64_t)gridDim.x / kExactCtas : ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const unsigned long long word = A.list[2 * A.cap + e];
+        const PtOpen o = pt_open(word);
+        const OpRef ref{o.op == 4 ? o.j : o.i, o.op == 4 ? o.i : o.j, o.op < 3 ? o.op : DIV, A.inv64};
+        double mag;
+        const double v0 = opref_val(ref, A.val64, A.N, 0, mag);
+        double s1 = 0.0, s2 = 0.0, sr = 0.0;
+        for (int s = t; s < A.N; s += nt) {
+            const double u = opref_val(ref, A.val64, A.N, s, mag) - v0;
+            s1 += u;
+            s2 = fma(u, u, s2);
+            sr = fma(u, A.tc64[s], sr);
+        }
+        s1 = group_sum<CTA>(s1, sh); s2 = group_sum<CTA>(s2, sh); sr = group_sum<CTA>(sr, sh);
+        if constexpr (CTA) {
+            if (threadIdx.x == 0) { part[0] = s1; part[1] = s2; part[2] = sr; }
+            cg::this_cluster().sync();
+            if (t == 0)
+                for (int q = 1; q < kExactCtas; ++q) {
+                    const double* p = cg::this_cluster().map_shared_rank(part, q);
+                    s1 += p[0]; s2 += p[1]; sr += p[2];
+                }
+            cg::this_cluster().sync();             // read before the next candidate's, and before a CTA ends
+        }
+        if (t == 0) pt_close<FIRST>(A, word, o, pt_key64(A, s1, s2, sr, v0, pt_scale(A, o)));
     }
 }
 
@@ -975,7 +1061,7 @@ void pt_layout(const sisso_ctx* c, PairTc& t) {
 
 size_t pt_bytes(const PairTc& t) {
     const size_t K = (size_t)t.Kpad, P = (size_t)t.P;
-    return 20 * P * K + 8 * (size_t)t.Pi * K + 48 * P + sizeof(float) * t.n_w + sizeof(unsigned long long) * 2 * t.cap +
+    return 20 * P * K + 8 * (size_t)t.Pi * K + 48 * P + sizeof(float) * t.n_w + sizeof(unsigned long long) * 3 * t.cap +
            t.part_bytes + sizeof(int2) * (size_t)(t.n_tiles[0] + t.n_tiles[1]);
 }
 
@@ -1022,7 +1108,7 @@ sisso_status pair_tc_alloc(sisso_ctx* c) {
         (st = ctx_alloc(c, (void**)&t->ex, sizeof(int) * 2 * P, "pair exponents")) ||
         (st = ctx_alloc(c, (void**)&t->R, sizeof(float) * 2 * P, "pair R")) ||
         (st = ctx_alloc(c, (void**)&t->w, sizeof(float) * t->n_w, "pair 1/sd")) ||
-        (st = ctx_alloc(c, (void**)&t->list, sizeof(unsigned long long) * 2 * t->cap, "pair open keys")) ||
+        (st = ctx_alloc(c, (void**)&t->list, sizeof(unsigned long long) * 3 * t->cap, "pair open keys")) ||
         (st = ctx_alloc(c, (void**)&t->count, sizeof(unsigned) * 4, "pair counts")) ||
         (st = ctx_alloc(c, (void**)&t->part, t->part_bytes, "pair partials")) ||
         (st = ctx_alloc(c, (void**)&t->tiles[0], sizeof(int2) * tiles[0].size(), "pair tiles")) ||
@@ -1075,6 +1161,7 @@ sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow) {
     A.ni = t->ni[v];
     A.chunks = t->chunks[v]; A.run_len = t->run_len[v]; A.runs = t->runs;
     A.N = c->N; A.Kpad = t->Kpad; A.rows = t->rows; A.val32 = t->val32;
+    A.val64 = c->opval64; A.inv64 = c->opinv64; A.tc64 = c->tc64; A.inv_n = 1.0 / c->N;
     A.scale = (float)(1.0 / (1073741824.0 * c->N));
     // a run's sums: at most four last-place units from its hi hi MMAs (2^-23 each), the parts'
     // rounding and the dropped lo lo (3 2^-24); one rounding per run added
@@ -1082,6 +1169,7 @@ sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow) {
     A.tol = t->runs <= kFewRuns ? kTolFew : kTolMany;
     A.par = t->par; A.ex = t->ex; A.R = t->R; A.w = t->w; A.scores = c->scores; A.st = c->tstats;
     A.list = t->list; A.count = t->count; A.cap = t->cap; A.part = t->part;
+    cudaMemsetAsync(t->count + 3, 0, sizeof(unsigned), c->stream);
     if (v == 0) {
         cudaMemsetAsync(t->count, 0, sizeof(unsigned) * 4, c->stream);
         // entries no unit writes (pairs i >= j of one set, disabled operators) read as not open
@@ -1111,15 +1199,34 @@ sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow) {
         }
         c->stats.launches += 1 + (A.chunks > 1);
     }
+    cudaLaunchAttribute cluster{};
+    cluster.id = cudaLaunchAttributeClusterDimension;
+    cluster.val.clusterDim.x = kExactCtas;
+    cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(256);
+    cfg.stream = c->stream;
+    cfg.attrs = &cluster;
+    cfg.numAttrs = 1;
+#define SG_PT_DIRECT(FIRST)                                                                              \
+    do {                                                                                                  \
+        if (many) {                                                                                       \
+            k_pt_direct<FIRST, true><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);                      \
+            cfg.gridDim = dim3((unsigned)(c->sms * 8 / kExactCtas * kExactCtas));                         \
+            cudaLaunchKernelEx(&cfg, k_pt_exact<FIRST, true>, A);                                         \
+        } else {                                                                                          \
+            k_pt_direct<FIRST, false><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);                     \
+            k_pt_exact<FIRST, false><<<c->sms * 8, 256, 0, c->stream>>>(A);                               \
+        }                                                                                                 \
+    } while (0)
     if (v == 0) {
         k_pt_open<<<(unsigned)std::max<size_t>(1, std::min<size_t>((size_t)c->sms * 8, (t->n_w + 1023) / 1024)), 256, 0, c->stream>>>(A, (int64_t)t->n_w);
-        if (many) k_pt_direct<true, true><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
-        else k_pt_direct<true, false><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
+        SG_PT_DIRECT(true);
     } else {
-        if (many) k_pt_direct<false, true><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
-        else k_pt_direct<false, false><<<c->sms * 8, 256, 0, c->stream>>>(A, c->tc32);
+        SG_PT_DIRECT(false);
     }
-    c->stats.launches += 3 + (v == 0);
+#undef SG_PT_DIRECT
+    c->stats.launches += 4 + (v == 0);
     // a launch that was refused leaves the last step's keys: waiting alone would not tell
     sisso_status st = check_cuda(c, cudaGetLastError(), "pair scores");
     if (st) return st;
