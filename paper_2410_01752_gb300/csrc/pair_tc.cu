@@ -328,17 +328,21 @@ __device__ __forceinline__ size_t w_index(const PtArgs& A, int op, int64_t i, in
 }
 
 // key and 1/sd from the variance, its error bound dv, the covariance and its bound dc (both
-// relative to the target's deviation).  Rejected (w = -inf) only where the FP64 rules must
-// reject: |v(sample 0)| > 1e12, a root mean square above 1e12, or a deviation that even at the
-// upper end of its bound is <= 1e-6 max(|v0|, |mean|).  Open (w = -dc) where the bounds could
-// move the key by more than a quarter of the FP32 screening margin (2e-4) each, or decide the
-// validity test.
-__device__ __forceinline__ PtKey pt_key(float var, float dv, float cov, float dc, float v0, float mean, bool v0_ok,
+// relative to the target's deviation) and the mean and its bound dm.  Rejected (w = -inf) only where
+// the FP64 rules must reject: |v(sample 0)| > 1e12, a root mean square that even at the lower end of
+// its bounds is above 1e12, or a deviation that even at the upper end of its bound is <= 1e-6
+// max(|v0|, |mean|) with the mean at its lower end.  (Operands that span many decades and cancel,
+// as a quotient of two of them does, leave a variance and a mean that are mostly rounding.)  Open
+// (w = -dc) where the bounds could move the key by more than a quarter of the FP32 screening margin
+// (2e-4) each, or decide the validity tests.
+__device__ __forceinline__ PtKey pt_key(float var, float dv, float cov, float dc, float v0, float mean, float dm, bool v0_ok,
                                         float rms2_max, float tol, float inv_sdr) {
-    const float lim = (float)kConstRel * fmaxf(fabsf(v0), fabsf(mean)), lim2 = lim * lim;
-    if (!v0_ok || !(var + mean * mean <= rms2_max) || !(var + dv > lim2)) return PtKey{-1.f, -INFINITY};
+    const float am = fabsf(mean), lo = fmaxf(am - dm, 0.f), hi = am + dm;
+    const float lim_lo = (float)kConstRel * fmaxf(fabsf(v0), lo), lim_hi = (float)kConstRel * fmaxf(fabsf(v0), hi);
+    if (!v0_ok || !(var - dv + lo * lo <= rms2_max) || !(var + dv > lim_lo * lim_lo)) return PtKey{-1.f, -INFINITY};
     const float w = __frsqrt_rn(var);
-    if (!(dv <= tol * var) || !(var - dv > lim2) || !(dc * w <= 0.5f * tol)) return PtKey{-1.f, -fmaxf(dc, 1e-30f)};
+    if (!(dv <= tol * var) || !(var - dv > lim_hi * lim_hi) || !(var + dv + hi * hi <= rms2_max) || !(dc * w <= 0.5f * tol))
+        return PtKey{-1.f, -fmaxf(dc, 1e-30f)};
     return PtKey{fabsf(cov) * w * inv_sdr, w};
 }
 
@@ -357,7 +361,8 @@ __device__ __forceinline__ PtKey pt_product(const PtArgs& A, const PtSide& a, co
     const float cov = a.m * b.R + b.m * a.R + T;
     const float dc = A.eps * q + 20.f * kU * (fa * b.s + fb * a.s + q) + fl * (1.f + fa + fb);
     const float lg = a.lg + b.lg;
-    return pt_key(var, dv, cov, dc, a.x0 * b.x0, AB + P1, lg <= kLogCap, exp2f(kLogRms - 2.f * (float)(a.ex + b.ex)),
+    const float dm = A.eps * q + 4.f * kU * (fabsf(AB) + fabsf(P1)) + 0.5f * fl;
+    return pt_key(var, dv, cov, dc, a.x0 * b.x0, AB + P1, dm, lg <= kLogCap, exp2f(kLogRms - 2.f * (float)(a.ex + b.ex)),
                   A.tol, inv_sdr);
 }
 
@@ -373,7 +378,8 @@ __device__ __forceinline__ PtKey pt_sum(const PtArgs& A, const PtSide& a, const 
     const float dv = 2.f * A.eps * sa * sb + 6.f * kU * (va + vb + fabsf(c2)) + 2.f * kFloor * fa * fabsf(fb) * (a.s + b.s);
     const float v0 = fa * a.x0 + fb * b.x0, mean = fa * a.m + fb * b.m;
     const bool ok = a.lg < INFINITY && b.lg < INFINITY && fabsf(v0) * pow2f(em) <= (float)kValueCap;
-    return pt_key(var, dv, fa * a.R + fb * b.R, 20.f * kU * (sa + sb), v0, mean, ok, exp2f(kLogRms - 2.f * (float)em),
+    return pt_key(var, dv, fa * a.R + fb * b.R, 20.f * kU * (sa + sb), v0, mean,
+                  3.f * kU * (fa * fabsf(a.m) + fabsf(fb * b.m)), ok, exp2f(kLogRms - 2.f * (float)em),
                   A.tol, inv_sdr);
 }
 
@@ -891,7 +897,7 @@ __global__ void __launch_bounds__(256) k_pt_direct(PtArgs A, const float* __rest
             const float v0 = ca * a.x0 + cb * b.x0;
             t1 *= inv_n;
             const float var = t2 * inv_n - t1 * t1;
-            k = pt_key(var, 0.f, tr * inv_n, 0.f, v0, ca * a.m + cb * b.m,
+            k = pt_key(var, 0.f, tr * inv_n, 0.f, v0, ca * a.m + cb * b.m, 0.f,
                        a.lg < INFINITY && b.lg < INFINITY && fabsf(v0) * pow2f(em) <= (float)kValueCap,
                        exp2f(kLogRms - 2.f * (float)em), A.tol, inv_sdr);
             // values 3 2^-24 and 2^-39 off, in the sums of v r and of v^2

@@ -1,6 +1,6 @@
 """Keys of pairs whose terms nearly cancel: differences and quotients of operands that agree to
-1e-4 .. 1e-7.  Every key lies within the screening margin of the oracle's score, for a context's
-first target and for a later one."""
+1e-4 .. 1e-7, and quotients of operands that span many decades together.  Every key lies within the
+screening margin of the oracle's score, for a context's first target and for a later one."""
 import numpy as np
 import pytest
 
@@ -33,3 +33,14 @@ def test_nearly_equal_operands(orc, delta, N, rung, prec):
     X = np.stack([x, x + delta * n, r.uniform(1, 5, size=N)], 1)
     targets = [n + 0.1 * r.normal(size=N), n / x + 0.1 * r.normal(size=N)]
     _check(orc, X, targets, ["+", "-", "*", "/"], rung, prec)
+
+
+@pytest.mark.parametrize("seed", range(6))
+@pytest.mark.parametrize("N", [60, 500, 5000])
+@pytest.mark.parametrize("prec", [1, 3])
+def test_operands_over_many_decades(orc, seed, N, prec):
+    r = np.random.default_rng([N, seed])
+    x = 10.0 ** r.uniform(-9, 9, size=N)
+    a, b = r.normal(size=N), r.normal(size=N)
+    X = np.stack([x, x * np.exp(0.1 * a), np.exp(0.1 * b) / x], 1)
+    _check(orc, X, [a + 0.3 * b, b - a], ["*", "/"], 1, prec)
