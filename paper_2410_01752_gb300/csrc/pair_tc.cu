@@ -15,7 +15,7 @@
 // every candidate and the later steps run the T sum alone.
 //
 // Precision: every row is scaled by a power of two and split into two FP16 parts hi + lo
-// (|x - hi - lo| <= 2^-24 |x|, the rounding of an FP32 copy, down to 2^-39 of the row's
+// (|x - hi - lo| <= 2^-23 |x| beside the 2^-24 of its FP32 copy, down to 2^-39 of the row's
 // largest value), and the products hi lo, lo hi, hi hi are accumulated in FP32.  The tensor
 // cores drop up to about one unit in the last place of the accumulator per MMA, so a run is
 // only 64 samples (the four hi hi MMAs of a run come last, on an accumulator that until then
@@ -79,8 +79,19 @@ constexpr int kPtThreads = kPtEpiWarps * 32 + 64;   // then a TMA and an MMA war
 constexpr int kPtI5 = 48, kPtI1 = 240;     // largest i tile of the two shapes (240 accumulator columns)
 constexpr int kMaxRuns = 32;               // runs added in FP32 (2048 samples)
 constexpr float kU = 5.9604645e-8f;        // 2^-24
-constexpr float kTolMany = 1e-4f;          // largest relative variance bound of a final key (score: half)
-constexpr float kTolFew = 2.5e-5f;         // ... up to kFewRuns runs: FP32 sums that short are better than that
+// largest errors, in units of 2^-24 and relative to the value: a row's x' as hi + lo (its FP32 copy
+// and the parts), x'^2 (two copies, the square, the parts), x'r (hi + lo, the target's copy, the
+// product, the parts), the part product lo lo that is left out, and a row's mean square V (the
+// squares, four accumulators of up to four pairs, their sum, the warp's)
+constexpr int kErrRow = 3, kErrSquare = 5, kErrTarget = 7, kErrLoLo = 4, kErrV = 17;
+// ... of a sum of products over runs of 64: its two rows and lo lo at most (x'^2 g'^2 and x'r g'), one
+// last-place unit of the accumulator at each of a run's four hi hi MMAs, the chunks and the scale;
+// the additions of the runs come on top
+constexpr int kErrSum = 2 * kErrSquare + kErrLoLo + 8 + 3;
+static_assert(kErrTarget + kErrRow <= 2 * kErrSquare, "the largest pair of rows");
+constexpr float kTolMany = 1.5e-4f;        // largest relative variance bound of a final key (score: half)
+constexpr float kTolFew = 4e-5f;           // ... up to kFewRuns runs: FP32 sums that short are better than that
+constexpr float kTolDirect = 1e-4f;        // ... of a key from the direct FP32 sums (k_pt_direct)
 constexpr int kFewRuns = 4;
 constexpr float kFloor = 1.82e-12f;        // 2^-39: parts below FP16's range, relative to a row's largest value
 
@@ -234,31 +245,31 @@ k_pt_rows(const double* __restrict__ val, const double* __restrict__ inv, const 
         __half* r0 = rows + (size_t)(set * 4) * P * Kpad + (size_t)f * Kpad;
         const size_t lo = (size_t)P * Kpad;
         __half* r1 = r0 + 2 * lo;
-        float run = 0.f;
+        float run[4] = {0.f, 0.f, 0.f, 0.f};
         double V = 0.0;
-        auto put = [&](int i, double x, double y) {
+        auto put = [&](int i, double x, double y, float& sum) {
             const float a = bad ? 0.f : scaled_f32(x, 15 - e), b = bad ? 0.f : scaled_f32(y, 15 - e);
             const float a2 = a * a * 3.0517578125e-5f, b2 = b * b * 3.0517578125e-5f;      // times 2^15
             put_parts2(a, b, r0 + i, r0 + lo + i);
             put_parts2(a2, b2, r1 + i, r1 + lo + i);
-            run += a2 + b2;
+            sum += a2 + b2;
         };
         if constexpr (IT > 0) {
 #pragma unroll
             for (int q = 0; q < IT; ++q) {
                 const int i = 2 * (t + q * nt);
-                if (i < Kpad) put(i, c[2 * q], c[2 * q + 1]);
+                if (i < Kpad) put(i, c[2 * q], c[2 * q + 1], run[q & 3]);
             }
         } else {
             int q = 0;
             for (int i = 2 * t; i < Kpad; i += 2 * nt) {
-                put(i, i < N ? load(i) - mean : 0.0, i + 1 < N ? load(i + 1) - mean : 0.0);
-                if ((++q & 7) == 0) { V += (double)run; run = 0.f; }
+                put(i, i < N ? load(i) - mean : 0.0, i + 1 < N ? load(i + 1) - mean : 0.0, run[0]);
+                if ((++q & 7) == 0) { V += (double)run[0]; run[0] = 0.f; }
             }
         }
         float Vs;
-        if constexpr (IT > 0) Vs = warp_sum(run);
-        else Vs = (float)group_sum<CTA>(V + (double)run, shd);
+        if constexpr (IT > 0) Vs = warp_sum((run[0] + run[1]) + (run[2] + run[3]));
+        else Vs = (float)group_sum<CTA>(V + (double)run[0], shd);
         if (t == 0) {
             const double x0 = load(0);
             const float g = 3.0517578125e-5f;
@@ -333,8 +344,8 @@ __device__ __forceinline__ size_t w_index(const PtArgs& A, int op, int64_t i, in
 // its bounds is above 1e12, or a deviation that even at the upper end of its bound is <= 1e-6
 // max(|v0|, |mean|) with the mean at its lower end.  (Operands that span many decades and cancel,
 // as a quotient of two of them does, leave a variance and a mean that are mostly rounding.)  Open
-// (w = -dc) where the bounds could move the key by more than a quarter of the FP32 screening margin
-// (2e-4) each, or decide the validity tests.
+// (w = -dc) where the bounds could move the key by more than 7.5e-5 each (the selection's margin is
+// 2e-4), or decide the validity tests.
 __device__ __forceinline__ PtKey pt_key(float var, float dv, float cov, float dc, float v0, float mean, float dm, bool v0_ok,
                                         float rms2_max, float tol, float inv_sdr) {
     const float am = fabsf(mean), lo = fmaxf(am - dm, 0.f), hi = am + dm;
@@ -353,13 +364,18 @@ __device__ __forceinline__ PtKey pt_product(const PtArgs& A, const PtSide& a, co
     const float t1 = a.m * a.m * b.V, t2 = b.m * b.m * a.V, t3 = 2.f * AB * P1, t4 = 2.f * a.m * P3, t5 = 2.f * b.m * P4;
     const float p11 = P1 * P1;
     const float var = ((t1 + t2) + (P2 - p11)) + (t3 + (t4 + t5));
-    const float q = sqrtf(fmaxf(P2, 0.f)), fa = fabsf(a.m), fb = fabsf(b.m);
+    const float fa = fabsf(a.m), fb = fabsf(b.m);
     const float S = t1 + t2 + P2 + p11 + fabsf(t3) + fabsf(t4) + fabsf(t5);
     const float fl = 2.f * kFloor * (a.s + b.s);
-    const float dv = A.eps * (2.f * q * (fabsf(AB) + fabsf(P1) + fa * b.s + fb * a.s) + P2) + 10.f * kU * S +
+    const float q = sqrtf(fmaxf(P2, 0.f) + fl);              // >= root of E x'^2 g'^2 >= E |x'g'|
+    // the sums' errors (E |x'g'^2| <= q s_g), V's and this expression's, the parts' floor
+    const float dv = A.eps * (2.f * q * (fabsf(AB) + fabsf(P1) + fa * b.s + fb * a.s) + P2) + (kErrV + 8.f) * kU * S +
                      fl * (2.f + (1.f + 2.f * fa) * (1.f + 2.f * fb));
     const float cov = a.m * b.R + b.m * a.R + T;
-    const float dc = A.eps * q + 20.f * kU * (fa * b.s + fb * a.s + q) + fl * (1.f + fa + fb);
+    // T's error, R's (19 2^-24 E |x'r|) and the additions', the floors of x', g' and x'r: the last
+    // is one of the target scaled into [-1, 1], whose deviation there is 1 / inv_sdr
+    const float dc = A.eps * q + 20.f * kU * (fa * b.s + fb * a.s + q) +
+                     2.f * kFloor * (a.s + b.s * (1.f + inv_sdr) + fa + fb);
     const float lg = a.lg + b.lg;
     const float dm = A.eps * q + 4.f * kU * (fabsf(AB) + fabsf(P1)) + 0.5f * fl;
     return pt_key(var, dv, cov, dc, a.x0 * b.x0, AB + P1, dm, lg <= kLogCap, exp2f(kLogRms - 2.f * (float)(a.ex + b.ex)),
@@ -375,10 +391,10 @@ __device__ __forceinline__ PtKey pt_sum(const PtArgs& A, const PtSide& a, const 
     const float var = va + vb + c2;
     const float sa = fa * a.s, sb = fabsf(fb) * b.s;
     // E |x_i' x_j'| <= s_i s_j
-    const float dv = 2.f * A.eps * sa * sb + 6.f * kU * (va + vb + fabsf(c2)) + 2.f * kFloor * fa * fabsf(fb) * (a.s + b.s);
+    const float dv = 2.f * A.eps * sa * sb + (kErrV + 4.f) * kU * (va + vb + fabsf(c2)) + 2.f * kFloor * fa * fabsf(fb) * (a.s + b.s);
     const float v0 = fa * a.x0 + fb * b.x0, mean = fa * a.m + fb * b.m;
     const bool ok = a.lg < INFINITY && b.lg < INFINITY && fabsf(v0) * pow2f(em) <= (float)kValueCap;
-    return pt_key(var, dv, fa * a.R + fb * b.R, 20.f * kU * (sa + sb), v0, mean,
+    return pt_key(var, dv, fa * a.R + fb * b.R, 20.f * kU * (sa + sb) + 2.f * kFloor * (fa + fabsf(fb)), v0, mean,
                   3.f * kU * (fa * fabsf(a.m) + fabsf(fb * b.m)), ok, exp2f(kLogRms - 2.f * (float)em),
                   A.tol, inv_sdr);
 }
@@ -900,9 +916,9 @@ __global__ void __launch_bounds__(256) k_pt_direct(PtArgs A, const float* __rest
             k = pt_key(var, 0.f, tr * inv_n, 0.f, v0, ca * a.m + cb * b.m, 0.f,
                        a.lg < INFINITY && b.lg < INFINITY && fabsf(v0) * pow2f(em) <= (float)kValueCap,
                        exp2f(kLogRms - 2.f * (float)em), A.tol, inv_sdr);
-            // values 3 2^-24 and 2^-39 off, in the sums of v r and of v^2
-            const float off = 6.f * kU * (ca * a.s + fabsf(cb) * b.s) + 4.f * kFloor * (ca + fabsf(cb));
-            sure = k.key >= 0.f && off * off <= kTolMany * kTolMany * var;
+            // values kErrRow 2^-24 and 2^-39 off, in the sums of v r and of v^2
+            const float off = 2.f * kErrRow * kU * (ca * a.s + fabsf(cb) * b.s) + 4.f * kFloor * (ca + fabsf(cb));
+            sure = k.key >= 0.f && off * off <= kTolDirect * kTolDirect * var;
         } else {
             const bool quot = op > 2;
             const float* xa = A.val32 + (size_t)(op == 4 ? j : i) * A.Kpad;      // numerator
@@ -920,11 +936,11 @@ __global__ void __launch_bounds__(256) k_pt_direct(PtArgs A, const float* __rest
             if (k.key >= 0.f) {
                 t1 *= inv_n;
                 t2 *= inv_n;
-                const float var = t2 - t1 * t1, mean = v0 + t1, half = 0.5f * kTolMany;
+                const float var = t2 - t1 * t1, mean = v0 + t1, half = 0.5f * kTolDirect;
                 k.w = __frsqrt_rn(var) * pow2f(scale / 2) * pow2f(scale - scale / 2);
                 // values 3 2^-24 off (two operands, the reciprocal), in the sums of v r and of v^2; sums of
                 // u = v - v0 about 40 2^-24 of E u^2 off
-                sure = k.w > 0.f && 36.f * kU * kU * (var + mean * mean) <= kTolMany * kTolMany * var && 60.f * kU * t2 <= half * var;
+                sure = k.w > 0.f && 36.f * kU * kU * (var + mean * mean) <= kTolDirect * kTolDirect * var && 60.f * kU * t2 <= half * var;
             }
         }
         if (lane == 0) {
@@ -1169,9 +1185,7 @@ sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow) {
     A.N = c->N; A.Kpad = t->Kpad; A.rows = t->rows; A.val32 = t->val32;
     A.val64 = c->opval64; A.inv64 = c->opinv64; A.tc64 = c->tc64; A.inv_n = 1.0 / c->N;
     A.scale = (float)(1.0 / (1073741824.0 * c->N));
-    // a run's sums: at most four last-place units from its hi hi MMAs (2^-23 each), the parts'
-    // rounding and the dropped lo lo (3 2^-24); one rounding per run added
-    A.eps = (float)((16 + t->run_len[v]) * std::ldexp(1.0, -24));
+    A.eps = (float)((kErrSum + t->run_len[v]) * std::ldexp(1.0, -24));
     A.tol = t->runs <= kFewRuns ? kTolFew : kTolMany;
     A.par = t->par; A.ex = t->ex; A.R = t->R; A.w = t->w; A.scores = c->scores; A.st = c->tstats;
     A.list = t->list; A.count = t->count; A.cap = t->cap; A.part = t->part;
