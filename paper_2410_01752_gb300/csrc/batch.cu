@@ -1558,11 +1558,16 @@ sisso_status sisso_batch_create(const sisso_task* tasks, int n_tasks, uint32_t o
             f.AR[t] = region(sizeof(double) * P.P);
         }
     }
-    // the pair tiles' kept values behind the rest, left out when they do not fit
+    // the pair tiles' kept values behind the rest, left out where they would take more than half of
+    // the memory that the rest leaves: the buffers below and the caller's later ones need some too
     std::vector<size_t> keep_off(n_tasks);
     const size_t without = total;
-    if (max_dim > 1)
+    if (max_dim > 1) {
         for (int i = 0; i < n_tasks; ++i) keep_off[i] = region(sizeof(float) * kPairKeepTile * plans[i].tiles.size());
+        size_t left = 0, all = 0;
+        if (cudaMemGetInfo(&left, &all) != cudaSuccess) { cudaGetLastError(); left = 0; }
+        if (left < without || total - without > (left - without) / 2) total = without;
+    }
     sisso_status st;
     if (total > without && cudaMalloc(&b->arena, total) != cudaSuccess) {
         cudaGetLastError();

@@ -128,3 +128,22 @@ def test_gram_digits_that_do_not_fit():
         ref = _fit(c)
     with S.Sisso(X, y, inputs.OPS9, 2, 200, 3) as c, _Held(S, GB // 3):
         _same(_fit(c), ref)
+
+
+def test_batch_values_that_do_not_fit():
+    """The deviations that a batch keeps for later steps take most of what its other buffers leave."""
+    from paper_2410_01752_gb300 import sisso as S
+    problems = [_problem(2000, 9, seed) for seed in range(96)]
+
+    def make():
+        return S.Batch(problems, inputs.OPS9, 2, 20, 2)
+
+    with make() as b:
+        b.run()
+        ref = b.results()
+    base = _memory_of(S, make)
+    inputs_bytes = 96 * 2000 * 10 * 8
+    with _Held(S, base - inputs_bytes // 2), make() as b:
+        b.run()
+        for (st0, a), (st1, g) in zip(ref, b.results()):
+            assert st0 == st1 == 0 and [m.ids for m in a] == [m.ids for m in g]
