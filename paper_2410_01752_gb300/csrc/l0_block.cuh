@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(128) k_l0_confirm(const __grid_constant__ Tile
         int pos[D];
 #pragma unroll
         for (int m = 0; m < D; ++m) pos[m] = (int)((k >> (12 * m)) & 4095u);
-        const double B = okey_inv(*(volatile unsigned long long*)A.ub_key);
+        const double B = fmin((double)INFINITY, okey_inv(*(volatile unsigned long long*)A.ub_key));    // (NaN: not set)
         block_exact<D>(A, pos, B, B + A.tie64);
     }
 }
