@@ -138,17 +138,17 @@ def cpu_baseline_sample(P, seconds: float, seed: int = 0, threads: int = 0):
 
 
 def captured_traffic():
-    """DRAM bytes per launch of the pair kernel from the committed ncu summary, or None
-    when the kernel's source has changed since that capture."""
+    """DRAM bytes per launch of k_pair_tc, averaged over a fit's steps, from the committed ncu
+    summary, or None when the kernel's source has changed since that capture."""
     import hashlib
-    path = os.path.join(ROOT, "profiles", "k_score_pairs_rung3_N1000_d10_traffic.md")
+    path = os.path.join(ROOT, "profiles", "k_pair_tc_rung3_N1000_d10_traffic.md")
     try:
         txt = open(path).read()
     except OSError:
         return None
     vals = dict(l.split(":", 1) for l in txt.splitlines() if l.startswith(("traffic_bytes", "source_sha256")))
     h = hashlib.sha256()
-    for f in ("sis.cu", "sis_device.cuh"):        # the kernel, its device code and its tile list
+    for f in ("pair_tc.cu", "tc_device.cuh", "sis_device.cuh"):        # the kernel and its device code
         with open(os.path.join(ROOT, "paper_2410_01752_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     sha = next((v.strip() for k, v in vals.items() if k.startswith("source_sha256")), "")
