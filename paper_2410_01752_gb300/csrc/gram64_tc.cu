@@ -3,15 +3,19 @@
 // GB300's FP64 pipe bounds the plain kernel (k_gram_rows): 600 features over 65 536 samples are
 // 1.2e10 fused multiply-adds, 20 ms.  Here every row is rounded once to a 55-bit integer
 //     q = rint(z 2^(54 - e)),  |z| < 2^e for the whole row,
-// written in base 256 with digits d0 .. d6 in [-128, 127] (d0 the leading one), and the digit
-// products are summed on the tensor cores as FP16 integers: a product is at most 2^14 and an
+// written in base 256 with digits d0 .. d6 in [-128, 127] (d0 the leading one; the error-free slicing of
+// Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication", 2012), and the
+// digit products are summed on the tensor cores as FP16 integers: a product is at most 2^14 and an
 // accumulator takes at most 7 x 64 of them between two reads, so every partial sum is an integer
 // below 2^23, which FP32 holds exactly whatever the order of the additions.  The sums S_w of equal
 // weight w = i + j <= 7 (34 of the 49 products) are added as 64-bit integers, exactly again, also
 // across CTAs.  What is left out, the products of weight 8 and more, is below 2^-61 of
-// 2^(ei + ej) a sample at random signs; the rounding of q is half a unit of 2^(e - 54).  Both are
-// averaged over the samples, so the result is the Gram rounded once or twice to FP64: its error
-// against longer sums is below that of the FP64 accumulation it replaces.
+// 2^(ei + ej) a sample at random signs, but of one sign between a row and itself, where it is
+// 2^-63.6 4^e of the Gram's 1; the rounding of q is half a unit of 2^(e - 54).  Both are averaged over
+// the samples, so the result is the Gram rounded once or twice to FP64: its error against longer
+// sums is below that of the FP64 accumulation it replaces.  A pair of rows with ei + ej above
+// kGWide, largest values of 45 deviations and more, would lose more than an FP64 rounding (5e-15 at
+// 250 deviations: reciprocals of near-equal columns) and is summed in FP64 (k_gram64_wide).
 //
 // One CTA takes a 128 x 64 tile of the lower triangle and a run of 64-sample blocks: one warp
 // streams the seven slices of both sides with TMA (two stages of 32 samples), one issues the 68
@@ -38,6 +42,7 @@ constexpr int kGK = 32;                   // samples of a stage (64-byte rows)
 constexpr int kGBlock = 64;               // samples between two reads of the accumulators
 constexpr int kGStages = 2;
 constexpr int kGThreads = 10 * 32;
+constexpr int kGWide = 11;
 constexpr uint32_t kGTileA = kGM * kGK * 2, kGTileB = kGN * kGK * 2;
 
 struct Gram64Smem {
@@ -225,28 +230,48 @@ k_gram64_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 }
 
 // G from the integer sums: sum q_i q_j = 2^72 (256^3 S_0 + .. + S_3) + 2^40 (256^3 S_4 + .. + S_7).
-// A wait that ran out (err) leaves the sums unusable: the entry is then summed in FP64 here.
+// Pairs with too wide a range, and all of them where a wait ran out (err: the sums are unusable), go
+// to the list instead.
 __global__ void k_gram64_finish(const unsigned long long* __restrict__ acc, size_t plane, int n_pad, const int* __restrict__ ex,
-                                const int* __restrict__ err, const double* __restrict__ Z, int N, int row0, int n, int ld,
-                                double* __restrict__ G, float* __restrict__ G32) {
+                                const int* __restrict__ err, int N, int row0, int n, int ld, double* __restrict__ G,
+                                float* __restrict__ G32, int2* __restrict__ list, unsigned* __restrict__ count) {
     const bool bad = *err != 0;
     const int64_t total = (int64_t)(n - row0) * n;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int r = (int)(e / n), j = (int)(e % n), i = row0 + r;
         if (j > i) continue;
-        double s;
-        if (bad) {
-            s = 0.0;
-            for (int t = 0; t < N; ++t) s += Z[(size_t)i * N + t] * Z[(size_t)j * N + t];
-        } else {
-            const long long hi = (long long)acc[(size_t)r * n_pad + j], lo = (long long)acc[plane + (size_t)r * n_pad + j];
-            s = scalbn((double)hi * 4294967296.0 + (double)lo, ex[i] + ex[j] - 68);
-        }
-        s /= N;
+        if (bad || ex[i] + ex[j] > kGWide) { list[atomicAdd(count, 1u)] = make_int2(i, j); continue; }
+        const long long hi = (long long)acc[(size_t)r * n_pad + j], lo = (long long)acc[plane + (size_t)r * n_pad + j];
+        const double s = scalbn((double)hi * 4294967296.0 + (double)lo, ex[i] + ex[j] - 68) / N;
         G[(size_t)i * ld + j] = s;
         G[(size_t)j * ld + i] = s;
         G32[(size_t)i * ld + j] = (float)s;
         G32[(size_t)j * ld + i] = (float)s;
+    }
+}
+
+// the listed entries, one CTA each
+__global__ void __launch_bounds__(256) k_gram64_wide(const double* __restrict__ Z, int N, int ld, const int2* __restrict__ list,
+                                                     const unsigned* __restrict__ count, double* __restrict__ G,
+                                                     float* __restrict__ G32) {
+    __shared__ double red[8];
+    const unsigned m = *count;
+    for (unsigned e = blockIdx.x; e < m; e += gridDim.x) {
+        const int2 p = list[e];
+        const double *a = Z + (size_t)p.x * N, *b = Z + (size_t)p.y * N;
+        double s = 0.0;
+        for (int t = threadIdx.x; t < N; t += 256) s += a[t] * b[t];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int q = 1; q < 8; ++q) s += red[q];
+            s /= N;
+            G[(size_t)p.x * ld + p.y] = G[(size_t)p.y * ld + p.x] = s;
+            G32[(size_t)p.x * ld + p.y] = G32[(size_t)p.y * ld + p.x] = (float)s;
+        }
+        __syncthreads();
     }
 }
 
@@ -312,10 +337,13 @@ sisso_status gram64_tc(sisso_ctx* c, const double* Z, const double* yc, int N, i
     A.per = (A.blocks + A.splits - 1) / A.splits;
     A.n_pad = A.tiles_n * kGN;
     A.plane = (size_t)tiles_m * kGM * A.n_pad;
-    sisso_status st = tmp_alloc(c, (void**)&A.acc, sizeof(unsigned long long) * (2 * A.plane + 1), "gram sums");
+    // sums, the error flag and the list's length, the list
+    sisso_status st = tmp_alloc(c, (void**)&A.acc, sizeof(unsigned long long) * (2 * A.plane + 1 + (size_t)n_new * n), "gram sums");
     if (st) return st;
     cudaMemsetAsync(A.acc, 0, sizeof(unsigned long long) * (2 * A.plane + 1), c->stream);
     A.err = reinterpret_cast<int*>(A.acc + 2 * A.plane);
+    unsigned* wide = reinterpret_cast<unsigned*>(A.err + 1);
+    int2* list = reinterpret_cast<int2*>(A.acc + 2 * A.plane + 1);
     CUtensorMap ma, mb;
     if (!gram64_map(&ma, slices, (int64_t)kSl * n_cap, Kpad, kGM) || !gram64_map(&mb, slices, (int64_t)kSl * n_cap, Kpad, kGN)) {
         cudaFreeAsync(A.acc, c->stream);
@@ -326,9 +354,10 @@ sisso_status gram64_tc(sisso_ctx* c, const double* Z, const double* yc, int N, i
     cudaFuncSetAttribute(k_gram64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     k_gram64_tc<<<tiles * A.splits, kGThreads, sm, c->stream>>>(ma, mb, A);
     k_gram64_finish<<<std::max(1, std::min(c->sms * 4, (int)(((int64_t)n_new * n + 255) / 256))), 256, 0, c->stream>>>(
-        A.acc, A.plane, A.n_pad, ex, A.err, Z, N, n_old, n, ld, G, G32);
+        A.acc, A.plane, A.n_pad, ex, A.err, N, n_old, n, ld, G, G32, list, wide);
+    k_gram64_wide<<<c->sms * 8, 256, 0, c->stream>>>(Z, N, ld, list, wide, G, G32);
     k_gram64_b<<<n_new, 256, 0, c->stream>>>(Z, yc, N, n_old, b, b32);
-    c->stats.launches += 4;
+    c->stats.launches += 5;
     cudaFreeAsync(A.acc, c->stream);
     return check_cuda(c, cudaGetLastError(), "gram64_tc");
 }
