@@ -198,9 +198,11 @@ typedef struct {
     int l0_enum_launches;        /* launches of the tiled FP32 enumeration kernel */
     int64_t l0_candidates;       /* subsets its filter sent to the exact FP32/FP64 test */
     int64_t certified_prefixes;  /* learned D = 5 step: 3-prefixes its certificate left to enumerate */
-    int screen_tc;               /* 1 if the top level's pairs were scored on the tensor cores */
-    int64_t tc_keys_raised;      /* ... keys raised to their error bound (0: keys with a wide
-                                    bound are scored directly, see pm_keys_direct) */
+    int screen_tc;               /* mixed forms: 1 if the top level's pairs were scored on the tensor
+                                    cores, for AUTO only where they lie within phi_{L-1} (see
+                                    opts.screen); 0 in the other precisions, whatever ran */
+    int64_t tc_keys_raised;      /* 0: keys with a wide error bound are scored directly, see
+                                    pm_keys_direct (kept for the layout) */
     int64_t pm_keys_direct;      /* top-level binary candidates whose key from per-operand and
                                     pair sums was left open (terms that nearly cancel) and
                                     scored from the direct sums instead, all steps */

@@ -709,9 +709,10 @@ sisso_status append_subspace(sisso_ctx* c, int n_old, int n_new, bool gram64) {
             k_std_write<<<grid, 256, 0, c->stream>>>(c->N, n_old, c->Z, run, part, c->Zmean, c->Zsd);
             c->stats.launches += 2;
             cudaFreeAsync(part, c->stream);
-        } else
-        k_standardise<<<n_new, 256, 0, c->stream>>>(c->space_dev, c->Xc64, c->N, c->S_dev, n_old, c->opval64, c->Z,
-                                                     c->Zmean, c->Zsd);
+        } else {
+            k_standardise<<<n_new, 256, 0, c->stream>>>(c->space_dev, c->Xc64, c->N, c->S_dev, n_old, c->opval64, c->Z,
+                                                         c->Zmean, c->Zsd);
+        }
         c->stats.launches++;
     }
     if (n_old < c->gram_rows) c->gram_rows = n_old;
@@ -1171,9 +1172,10 @@ sisso_status winner_model_z(sisso_ctx* c, int n, int D, Winner& w) {
         k_model_resid<<<kModelBlocks, 256, 0, c->stream>>>(c->N, c->syy, D, c->Z, c->Zmean, c->Zsd, c->yc64, c->ybar, c->S_dev,
                                                            c->win, c->resid, c->mpart, done + 1);
         c->stats.launches++;
-    } else
-    k_model_z<<<1, 1024, 0, c->stream>>>(c->Z, c->Zmean, c->Zsd, c->yc64, c->ybar, c->N, c->syy, D, c->S_dev, c->win,
-                                         c->resid);
+    } else {
+        k_model_z<<<1, 1024, 0, c->stream>>>(c->Z, c->Zmean, c->Zsd, c->yc64, c->ybar, c->N, c->syy, D, c->S_dev, c->win,
+                                             c->resid);
+    }
     c->stats.launches++;
     cudaMemcpyAsync(c->win_h, c->win, sizeof(Winner), cudaMemcpyDeviceToHost, c->stream);
     sisso_status st = check_cuda(c, cudaGetLastError(), "winner_model_z");
@@ -1192,9 +1194,10 @@ sisso_status winner_model(sisso_ctx* c, int n, int D, Winner& w) {
         k_model_resid<<<kModelBlocks, 256, 0, c->stream>>>(c->N, c->syy, D, c->Z, c->Zmean, c->Zsd, c->yc64, c->ybar, c->S_dev,
                                                            c->win, c->resid, c->mpart, done + 1);
         c->stats.launches++;
-    } else
-    k_model<<<1, 1024, 0, c->stream>>>(c->G64, c->b64, c->n_cap, c->syy, c->N, D, c->Z, c->Zmean, c->Zsd, c->yc64,
-                                       c->ybar, c->S_dev, c->win, c->resid);
+    } else {
+        k_model<<<1, 1024, 0, c->stream>>>(c->G64, c->b64, c->n_cap, c->syy, c->N, D, c->Z, c->Zmean, c->Zsd, c->yc64,
+                                           c->ybar, c->S_dev, c->win, c->resid);
+    }
     c->stats.launches++;
     cudaMemcpyAsync(c->win_h, c->win, sizeof(Winner), cudaMemcpyDeviceToHost, c->stream);
     sisso_status st = check_cuda(c, cudaGetLastError(), "winner_model");

@@ -262,7 +262,6 @@ __device__ __noinline__ BlockQueue block_take(const TileArgs& A, const BlockPre*
     return BlockQueue{B, qn, taken};
 }
 
-// prefixes item0 .. of the colex order, M the most features right of one of them
 // the FP64 Gram and moments in the order of perm
 __global__ void k_l0_reorder(const double* __restrict__ G, const double* __restrict__ b, int ld, int n,
                              const int* __restrict__ perm, double* __restrict__ Gq, double* __restrict__ bq) {
@@ -273,6 +272,7 @@ __global__ void k_l0_reorder(const double* __restrict__ G, const double* __restr
     }
 }
 
+// prefixes item0 .. of the colex order, M the most features right of one of them
 template <int DC, int W>
 __global__ void __launch_bounds__(W * 32, 16 / W) k_l0_block(const __grid_constant__ TileArgs A, int slices, int item0, int M) {
     extern __shared__ __align__(16) unsigned char block_smem[];

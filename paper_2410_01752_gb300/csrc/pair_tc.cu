@@ -23,13 +23,15 @@
 // kMaxRuns runs are added in FP32, longer ones in chunks whose totals are added with compensation.
 // Each key carries a bound of its error (pt_key); a key whose bound could matter next to the
 // screening margin, where the candidate's terms nearly cancel, is left open and scored by
-// k_pt_direct from the sums the definition writes, sample by sample.
+// k_pt_direct from the sums the definition writes, sample by sample, in FP32, or, where those are not
+// sure either, by k_pt_exact in FP64.
 //
 // Measured against the CUDA-core kernel it replaced: 2.9e8 rung-3 candidates (1000 samples, 10 primaries), 40.6 ms
-// a step -> 5.6 ms (first step), 2.4 ms (later ones) and 2.7 ms of open keys; 402 operands over
-// 65 536 samples, 7.9 ms a step -> 0.77 and 0.18 ms.  The mixed forms had their own split
-// products (FP64 rows, chunk sums and scores): 4.9 ms a step there.  The rows, target rows and
-// partials bound the long samples (HBM), the epilogue's FP32 adds the short ones.
+// a step -> 6.0 ms (first step), 2.4 ms (later ones), and 2.6 ms of open keys in the first step with 0.5 of
+// those left to FP64; 402 operands over 65 536 samples, 7.9 ms a step -> 0.80 and 0.18 ms.  The mixed forms had their own split
+// products (FP64 rows, chunk sums and scores): 4.9 ms a step there, and keys raised to their
+// bound where they nearly cancel.  The rows, target rows and partials bound the long samples
+// (HBM), the epilogue's FP32 adds the short ones.
 #include "sis_device.cuh"
 #include "tc_device.cuh"
 

@@ -1,8 +1,9 @@
 // sis.cu — sure independence screening (§2.2, Eqs. 5-6) on the device.
 //
 //  1. The top level's binary sections (almost all of phi_L): pair_tc.cu's tensor-core products
-//     for the FP32 and mixed forms; k_score_pairs otherwise (FP64, SISSO_SCREEN_CORES, operands
-//     too large for the rows or the cache, or too many open keys).  A CTA of k_score_pairs owns a
+//     for the FP32 and mixed forms; k_score_pairs otherwise (FP64, the mixed forms with
+//     SISSO_SCREEN_CORES, operands beyond the cache, buffers beyond the memory left, or too many
+//     open keys).  A CTA of k_score_pairs owns a
 //     32 x 32 tile of operand pairs, stages 32 samples of both sides at a time (from the operand
 //     cache, or rebuilt from the primaries by postfix programs), and every thread accumulates, for
 //     4 pairs x 5 operators (+, -, *, a/b, b/a), the shifted sums S1 = sum v', S2 = sum v'^2,
@@ -1838,8 +1839,8 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
     // the default window holds thousands of candidates so that it proves dense selections too; the
     // FP64 work of most steps needs the best few hundred: walks visit 1.2 to 4.4 k candidates, so
     // rank 5 k (at 3 k one step in twelve was repeated); half of that for long samples, whose FP64
-    // work dwarfs a repeated step's kernels (65 536 samples, k = 200: 1.6 -> 0.9 ms a step).  1013 samples, k = 50: 12 438 -> 636 candidates
-    // re-scored over three steps, 3.1 -> 2.6 ms a fit
+    // work dwarfs a repeated step's kernels (65 536 samples, k = 200: 1.6 -> 0.9 ms a step).  1013
+    // samples, k = 50: 12 438 -> 636 candidates re-scored over three steps, 3.1 -> 2.6 ms a fit
     bool narrow = c->opts.survivors <= 0;
     const int64_t n = c->n_feat;
     const int gridS = std::max(1, c->sms * 8);
@@ -1907,9 +1908,9 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
             k_rank_keys<<<(n_pad + 255) / 256, 256, 0, c->stream>>>(c->surv_ids, c->surv_score, c->surv_valid, ns, c->S_sorted,
                                                                     n_prev, c->unit_mask, c->rank_key, c->rank_id, c->dup_np);
         else
-        k_sort_keys<<<(n_pad + 255) / 256, 256, 0, c->stream>>>(c->surv_ids, c->surv_score, c->surv_valid, ns,
-                                                                 c->S_sorted, n_prev, n_pad, c->unit_mask,
-                                                                 c->sort_score, c->sort_id, c->sort_src, c->dup_np);
+            k_sort_keys<<<(n_pad + 255) / 256, 256, 0, c->stream>>>(c->surv_ids, c->surv_score, c->surv_valid, ns,
+                                                                     c->S_sorted, n_prev, n_pad, c->unit_mask,
+                                                                     c->sort_score, c->sort_id, c->sort_src, c->dup_np);
         c->stats.launches += 2;
         cudaEventRecord(q[2], c->stream);
         if (ranked) {
@@ -1933,9 +1934,10 @@ sisso_status sis_select(sisso_ctx* c, int k, const int64_t* S_prev_host, int n_p
             k_dup_confirm_cta<<<(int)std::min<int64_t>((int64_t)c->sms * 8, std::max<int64_t>(1, (int64_t)n_pad * n_confirm(c->N))), 256, 0,
                                 c->stream>>>(c->N, c->sort_src, zc, c->dup_list, c->dup_pairs, c->dup_np, c->dup_ok);
         else
-        k_dup_confirm<<<(int)std::max<int64_t>(1, std::min<int64_t>((int64_t)c->sms * 8, ((int64_t)n_pad + 7) / 8)), 256, 0, c->stream>>>(
-            c->space_dev, c->Xc64, c->N, c->sort_src, c->sort_id, c->surv_ids, c->surv_mean, c->surv_sd, zc,
-            c->opval64, c->dup_list, c->dup_pairs, c->dup_np, c->dup_ok, c->opinv64);
+            k_dup_confirm<<<(int)std::max<int64_t>(1, std::min<int64_t>((int64_t)c->sms * 8, ((int64_t)n_pad + 7) / 8)), 256, 0,
+                            c->stream>>>(c->space_dev, c->Xc64, c->N, c->sort_src, c->sort_id, c->surv_ids, c->surv_mean,
+                                         c->surv_sd, zc, c->opval64, c->dup_list, c->dup_pairs, c->dup_np, c->dup_ok,
+                                         c->opinv64);
         cudaFuncSetAttribute(k_walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkSmem);
         const size_t wsm = n_pad <= kWalkStage && ns <= kWalkStage ? kWalkSmem : 0;
         k_walk<<<1, kWalkThreads, wsm, c->stream>>>(c->space_dev, c->Xc64, c->N, c->sort_score, c->sort_id, c->sort_src,
