@@ -347,15 +347,13 @@ __device__ __forceinline__ size_t w_index(const PtArgs& A, int op, int64_t i, in
 // max(|v0|, |mean|) with the mean at its lower end.  (Operands that span many decades and cancel,
 // as a quotient of two of them does, leave a variance and a mean that are mostly rounding.)  Open
 // (w = -dc) where the bounds could move the key by more than 7.5e-5 each (the selection's margin is
-// 2e-4), or decide the validity tests.
+// 2e-4).  A key that only its bounds could reject is final: the FP64 re-score applies the rules.
 __device__ __forceinline__ PtKey pt_key(float var, float dv, float cov, float dc, float v0, float mean, float dm, bool v0_ok,
                                         float rms2_max, float tol, float inv_sdr) {
-    const float am = fabsf(mean), lo = fmaxf(am - dm, 0.f), hi = am + dm;
-    const float lim_lo = (float)kConstRel * fmaxf(fabsf(v0), lo), lim_hi = (float)kConstRel * fmaxf(fabsf(v0), hi);
-    if (!v0_ok || !(var - dv + lo * lo <= rms2_max) || !(var + dv > lim_lo * lim_lo)) return PtKey{-1.f, -INFINITY};
+    const float lo = fmaxf(fabsf(mean) - dm, 0.f), lim = (float)kConstRel * fmaxf(fabsf(v0), lo);
+    if (!v0_ok || !(fmaf(lo, lo, var - dv) <= rms2_max) || !(var + dv > lim * lim)) return PtKey{-1.f, -INFINITY};
     const float w = __frsqrt_rn(var);
-    if (!(dv <= tol * var) || !(var - dv > lim_hi * lim_hi) || !(var + dv + hi * hi <= rms2_max) || !(dc * w <= 0.5f * tol))
-        return PtKey{-1.f, -fmaxf(dc, 1e-30f)};
+    if (!(dv <= tol * var) || !(dc * w <= 0.5f * tol)) return PtKey{-1.f, -fmaxf(dc, 1e-30f)};
     return PtKey{fabsf(cov) * w * inv_sdr, w};
 }
 
@@ -982,15 +980,34 @@ __global__ void __launch_bounds__(256) k_pt_exact(PtArgs A) {
          e += CTA ? (int64_t)gridDim.x / kExactCtas : ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const unsigned long long word = A.list[2 * A.cap + e];
         const PtOpen o = pt_open(word);
-        const OpRef ref{o.op == 4 ? o.j : o.i, o.op == 4 ? o.i : o.j, o.op < 3 ? o.op : DIV, A.inv64};
-        double mag;
-        const double v0 = opref_val(ref, A.val64, A.N, 0, mag);
+        const int64_t a = o.op == 4 ? o.j : o.i, b = o.op == 4 ? o.i : o.j;
+        const bool inv = o.op > 2 && A.inv64;
+        const double *xa = A.val64 + (size_t)a * A.N, *vb = A.val64 + (size_t)b * A.N, *xb = inv ? A.inv64 + (size_t)b * A.N : vb;
+        auto value = [&](double x, double y, int s) {          // as the FP64 re-score's (opref_val)
+            if (o.op == 0) return x + y;
+            if (o.op == 1) return x - y;
+            if (o.op == 2) return x * y;
+            if (!inv) return x / y;
+            return (__double2hiint(y) & 0x7ff00000) != 0x7ff00000 ? x * y : x / vb[s];
+        };
+        const double v0 = value(xa[0], xb[0], 0);
         double s1 = 0.0, s2 = 0.0, sr = 0.0;
-        for (int s = t; s < A.N; s += nt) {
-            const double u = opref_val(ref, A.val64, A.N, s, mag) - v0;
-            s1 += u;
-            s2 = fma(u, u, s2);
-            sr = fma(u, A.tc64[s], sr);
+        for (int s0 = t; s0 < A.N; s0 += 4 * nt) {            // four samples' loads in flight
+            double x[4], y[4], r[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int s = min(s0 + q * nt, A.N - 1);
+                x[q] = xa[s]; y[q] = xb[s]; r[q] = A.tc64[s];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int s = s0 + q * nt;
+                if (s >= A.N) break;
+                const double u = value(x[q], y[q], s) - v0;
+                s1 += u;
+                s2 = fma(u, u, s2);
+                sr = fma(u, r[q], sr);
+            }
         }
         s1 = group_sum<CTA>(s1, sh); s2 = group_sum<CTA>(s2, sh); sr = group_sum<CTA>(sr, sh);
         if constexpr (CTA) {
@@ -1010,6 +1027,7 @@ __global__ void __launch_bounds__(256) k_pt_exact(PtArgs A) {
 // ids below the top level: |E x'r| / sqrt(E x'^2) of the operand itself
 __global__ void __launch_bounds__(256) k_pt_low(PtArgs A, const unsigned char* __restrict__ valid) {
     const int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (f == 0) A.count[3] = 0u;               // (this step's keys left to FP64 are listed later)
     if (f >= A.P) return;
     const float4 p = A.par[f];
     A.scores[f] = valid[f] && p.w < INFINITY ? fabsf(A.R[f]) * __frsqrt_rn(p.y) * A.st->inv_sdr : -1.f;
@@ -1191,7 +1209,6 @@ sisso_status pair_tc_scores(sisso_ctx* c, const int sec[4], bool* overflow) {
     A.tol = t->runs <= kFewRuns ? kTolFew : kTolMany;
     A.par = t->par; A.ex = t->ex; A.R = t->R; A.w = t->w; A.scores = c->scores; A.st = c->tstats;
     A.list = t->list; A.count = t->count; A.cap = t->cap; A.part = t->part;
-    cudaMemsetAsync(t->count + 3, 0, sizeof(unsigned), c->stream);
     if (v == 0) {
         cudaMemsetAsync(t->count, 0, sizeof(unsigned) * 4, c->stream);
         // entries no unit writes (pairs i >= j of one set, disabled operators) read as not open
