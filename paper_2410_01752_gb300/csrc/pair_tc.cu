@@ -27,7 +27,7 @@
 // sure either, by k_pt_exact in FP64.
 //
 // Measured against the CUDA-core kernel it replaced: 2.9e8 rung-3 candidates (1000 samples, 10 primaries), 40.6 ms
-// a step -> 6.0 ms (first step), 2.4 ms (later ones), and 2.6 ms of open keys in the first step with 0.5 of
+// a step -> 5.7 ms (first step), 2.4 ms (later ones), and 2.6 ms of open keys in the first step with 0.6 of
 // those left to FP64; 402 operands over 65 536 samples, 7.9 ms a step -> 0.80 and 0.18 ms.  The mixed forms had their own split
 // products (FP64 rows, chunk sums and scores): 4.9 ms a step there, and keys raised to their
 // bound where they nearly cancel.  The rows, target rows and partials bound the long samples
